@@ -3,7 +3,7 @@
 ``listed()`` names one workload per way of using the library, ``draw(rng)`` gives another of the same ranges,
 ``prepare`` makes a workload's inputs and buffers, ``run`` is one call through the public binding and returns the
 whole output tensor.  ``work`` counts what the operation cannot do without; ``tolerance`` is what another correct
-implementation at the same precision would differ by.
+implementation at the same precision would differ by; ``exact`` is the result in 64 bits.
 
 A case is a dict of
   entry   "single" | "general" | "16bit" | "padded" | "strided" | "noalloc" | "host"
@@ -172,18 +172,25 @@ def _algo(c):
     return {"auto": lib.ALGO_AUTO, "fp32": lib.ALGO_FFMA}[c["algo"]]
 
 
-def prepare(case, seed):
-    c = case
+def _inputs(c, seed):
     gen = torch.Generator(device="cuda")
     gen.manual_seed(int(seed))
     N, C, H, W, K, R, S = (c[k] for k in "NCHWKRS")
-    P, Q = _out_hw(c)
     x = _values((N, C, H, W), c["data"], gen)
     w = torch.empty((K, C, R, S), device="cuda").normal_(0.0, (2.0 / (C * R * S)) ** 0.5, generator=gen)
-    st = {"case": c, "y": torch.empty((N, K, P, Q), device="cuda"), "workspace": None, "bytes": 0}
     if c["entry"] == "16bit":
         kind = torch.bfloat16 if c["operand"] == "bf16" else torch.float16
         x, w = x.to(kind), w.to(kind)
+    return x, w
+
+
+def prepare(case, seed):
+    c = case
+    N, C, H, W, K, R, S = (c[k] for k in "NCHWKRS")
+    P, Q = _out_hw(c)
+    x, w = _inputs(c, seed)
+    st = {"case": c, "y": torch.empty((N, K, P, Q), device="cuda"), "workspace": None, "bytes": 0}
+    if c["entry"] == "16bit":
         st["bytes"] = lib.conv2d_fwd_workspace_size(N, C, H, W, K, R, S, lib.ALGO_16BIT)
     elif c["entry"] in ("general", "host"):
         st["bytes"] = lib.conv2d_fwd_workspace_size(N, C, H, W, K, R, S, _algo(c))
@@ -204,6 +211,25 @@ def prepare(case, seed):
         run(st)                                             # the first call leaves the re-ordered filters in the workspace
         st["flags"] = lib.FLAG_WEIGHTS_PACKED
     return st
+
+
+def exact(case, seed):
+    """The same convolution in float64, an image or a few at a time: one tap's plane of products after the other."""
+    c = case
+    x, w = _inputs(c, seed)
+    P, Q = _out_hw(c)
+    pad, st, C, R, S = (c[k] for k in ("pad", "stride", "C", "R", "S"))
+    wd = w.double()
+    out = torch.empty((c["N"], c["K"], P, Q), dtype=torch.float64, device="cuda")
+    for n in range(c["N"]):
+        xd = torch.nn.functional.pad(x[n].double(), (pad, pad, pad, pad))
+        y = torch.zeros((c["K"], P * Q), dtype=torch.float64, device="cuda")
+        for r in range(R):
+            for s in range(S):
+                taps = xd[:, r:r + st * (P - 1) + 1:st, s:s + st * (Q - 1) + 1:st].reshape(C, P * Q)
+                y += wd[:, :, r, s] @ taps
+        out[n] = y.view(c["K"], P, Q)
+    return out
 
 
 def run(state):
