@@ -948,8 +948,37 @@ cudaError_t consume_device_timeout(bool* raised)
     return e;
 }
 
+// Which kernel.  The flat kernel (single_channel_flat.cu) stores aligned quads whatever the alignment of the rows and takes
+// any filter height, so it has most shapes; measured against the kernels of this file (old -> flat, us):
+//   3 x 3: 3 x 1083 x 1917, 16 maps 205 -> 73; 4096 x 4096, 32 maps 471 -> 413; 512 x 512, 32 maps 16.9 -> 14.4
+//   1 x 1: 2048 x 2048, 32 maps 96 -> 82        7 x 7: 2048 x 2048, 32 maps 267 -> 256; 7 x 187 x 1674, 14 maps 84 -> 72
+//   5 x 5: 2049 x 2049, 32 maps 217 -> 165; 1000 x 600, 16 maps 33.2 -> 32.3 -- but with rows that are whole quads, where
+//   the kernels here lose nothing on their stores, two rows per tap read pay: 4096 x 4096, 32 maps 467 -> 563,
+//   1000 x 1000, 16 maps 38 -> 47 (1000 x 1200, 30 maps 53 either way)
+//   5 x 3: 2 x 1500 x 700, 24 maps 722 -> 56 (only the shape-agnostic kernel took filters that are not square)
+// A few maps of a short wide image stay with the shifted kernel: 200 x 2048, 16 maps of 3 x 3 11.2 -> 12.6, 40 x 1032, 4
+// maps 8.8 -> 8.6.
+static bool take_flat(const Shape& sh)
+{
+    const int forced = env_int("CONV2D_B200_SC_FLAT", -1);
+    if (forced >= 0) return forced != 0;
+    static const char* const other_kernels[] = {"CONV2D_B200_SC_UNIT", "CONV2D_B200_SC_PACKED", "CONV2D_B200_SC_TILE_H",
+                                                "CONV2D_B200_SC_ROWS", "CONV2D_B200_SC_WIDE", "CONV2D_B200_SC_SHIFT",
+                                                "CONV2D_B200_SC_BAND_H", "CONV2D_B200_SC_WSRC", "CONV2D_B200_SC_WIDE_MINQ"};
+    for (const char* name : other_kernels)
+        if (env_int(name, -1) != -1) return false;                   // (a switch of the kernels of this file is set)
+    if (sh.R == 5 && sh.S == 5 && sh.Q % 4 == 0 && sh.Q >= 640) return false;
+    if (sh.R == 3 && sh.S == 3 && sh.W % 4 == 0 && sh.P % 2 == 0 && sh.Q >= 1024 && sh.N == 1 && sh.P >= 32 && sh.P <= 256 && sh.K <= 16)
+        return false;
+    return true;
+}
+
 conv2d_status_t launch_single_channel(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream)
 {
+    if (take_flat(sh)) {
+        const conv2d_status_t st = launch_single_channel_flat(x, w, y, sh, stream);
+        if (st != CONV2D_ERR_UNSUPPORTED) return st;
+    }
     if (sh.R == 1 && sh.S == 1) return dispatch_rs<1, 1>(x, w, y, sh, stream);
     if (sh.R == 3 && sh.S == 3) return dispatch_rs<3, 3>(x, w, y, sh, stream);
     if (sh.R == 5 && sh.S == 5) return dispatch_rs<5, 5>(x, w, y, sh, stream);
