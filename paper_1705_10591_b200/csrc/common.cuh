@@ -110,6 +110,7 @@ cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
 
 // Launchers.  Each returns CONV2D_OK, CONV2D_ERR_UNSUPPORTED (no instance) or CONV2D_ERR_CUDA.
 conv2d_status_t launch_single_channel(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream);
+double single_channel_flat_cost(const Shape& sh);      // estimated scheduler cycles of a warp for four outputs of all maps
 conv2d_status_t launch_single_channel_flat(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream);
 conv2d_status_t launch_general_ffma(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream);
 conv2d_status_t launch_direct_fallback(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream);

@@ -952,12 +952,15 @@ cudaError_t consume_device_timeout(bool* raised)
 // any filter height, so it has most shapes; measured against the kernels of this file (old -> flat, us):
 //   3 x 3: 3 x 1083 x 1917, 16 maps 205 -> 73; 4096 x 4096, 32 maps 471 -> 413; 512 x 512, 32 maps 16.9 -> 14.4
 //   1 x 1: 2048 x 2048, 32 maps 96 -> 82        7 x 7: 2048 x 2048, 32 maps 267 -> 256; 7 x 187 x 1674, 14 maps 84 -> 72
-//   5 x 5: 2049 x 2049, 32 maps 217 -> 165; 1000 x 600, 16 maps 33.2 -> 32.3 -- but with rows that are whole quads, where
-//   the kernels here lose nothing on their stores, two rows per tap read pay: 4096 x 4096, 32 maps 467 -> 563,
-//   1000 x 1000, 16 maps 38 -> 47 (1000 x 1200, 30 maps 53 either way)
+//   5 x 5: 2049 x 2049, 32 maps 217 -> 165; 3000 x 3001, 2 maps 47 -> 41
 //   5 x 3: 2 x 1500 x 700, 24 maps 722 -> 56 (only the shape-agnostic kernel took filters that are not square)
-// A few maps of a short wide image stay with the shifted kernel: 200 x 2048, 16 maps of 3 x 3 11.2 -> 12.6, 40 x 1032, 4
-// maps 8.8 -> 8.6.
+// The kernels here keep
+//   * rows that are whole quads and fill most of a 512-column tile: nothing is lost on their stores, and two rows per tap
+//     read pay: 4096 x 4096, 32 maps of 5 x 5 467 -> 563, 1000 x 1000, 16 of 5 x 5 38 -> 47, 12 x 115 x 662, 26 of 3 x 3 25 -> 31;
+//   * 5 x 5 on a few maps of different alignment, whose classes the flat kernel computes one by one, where strided stores
+//     of all maps cost less: 14 x 375 x 1439, 4 maps 60 -> 64, 6 x 383 x 805, 5 maps 25 -> 33, 2 x 749 x 2938, 2 maps 24 -> 27
+//     (238 cycles of a scheduler for a warp's pair of maps, 130 for the strided stores of a map);
+//   * a few maps of a short wide image, on the shifted kernel: 200 x 2048, 16 maps of 3 x 3 11.2 -> 12.6, 40 x 1032, 4 maps 8.8 -> 8.6.
 static bool take_flat(const Shape& sh)
 {
     const int forced = env_int("CONV2D_B200_SC_FLAT", -1);
@@ -967,7 +970,12 @@ static bool take_flat(const Shape& sh)
                                                 "CONV2D_B200_SC_BAND_H", "CONV2D_B200_SC_WSRC", "CONV2D_B200_SC_WIDE_MINQ"};
     for (const char* name : other_kernels)
         if (env_int(name, -1) != -1) return false;                   // (a switch of the kernels of this file is set)
-    if (sh.R == 5 && sh.S == 5 && sh.Q % 4 == 0 && sh.Q >= 640) return false;
+    const double full = (double)sh.Q / ((sh.Q + kTileW - 1) / kTileW * kTileW);      // of a tile's columns
+    if (sh.R == sh.S && (sh.R == 3 || sh.R == 5) && sh.Q % 4 == 0 && full >= 0.6) return false;
+    if (sh.R == 5 && sh.S == 5 && sh.Q >= kTileW / 2) {
+        const double pairs = (sh.K + 1) / 2 * 238.0, stores = sh.K * 130.0;
+        if ((pairs > stores ? pairs : stores) / full < 0.76 * single_channel_flat_cost(sh)) return false;
+    }
     if (sh.R == 3 && sh.S == 3 && sh.W % 4 == 0 && sh.P % 2 == 0 && sh.Q >= 1024 && sh.N == 1 && sh.P >= 32 && sh.P <= 256 && sh.K <= 16)
         return false;
     return true;

@@ -49,7 +49,9 @@ template <int M>
 struct Residency { static constexpr int kBlocks = M <= 2 ? 4 : (M <= 8 ? 3 : 2); };
 
 // RT: filter rows, 0 = a.R.  M: maps accumulated together (1, or an even number).
-template <int RT, int S, int M>
+// TURN: maps of every alignment together (one class).  All outputs of a thread start at column 4t; a map whose row starts m
+// floats past a boundary is turned into aligned quads at the store, with the last m outputs of the lane to the left.
+template <int RT, int S, int M, bool TURN>
 __global__ void __launch_bounds__(kMaxThreads, Residency<M>::kBlocks)
 single_channel_flat_kernel(const FlatArgs a)
 {
@@ -103,6 +105,7 @@ single_channel_flat_kernel(const FlatArgs a)
     const int col0 = 4 * ct * a.cq;
     float* const band_out = a.y + (size_t)n * a.K * map + (size_t)row0 * a.Q;
     const unsigned band_m = (unsigned)n * (unsigned)a.K * (unsigned)map + (unsigned)row0 * (unsigned)a.Q;      // (only its value modulo 4 is used)
+    const int units = th * a.cq, lane = tid & 31;
     const float* wt = taps;
 #pragma unroll 1
     for (int cb = cb0; cb < cb0 + ncb; ++cb, wt += rs * TF) {
@@ -110,14 +113,17 @@ single_channel_flat_kernel(const FlatArgs a)
         float* const map_out = band_out + (size_t)k0 * map;
         const unsigned map_m = band_m + (unsigned)k0 * (unsigned)map;
         const int live = (a.K - k0 + cmask) >> a.class_shift;                 // maps of this block that exist (or more)
+        // (with TURN all lanes of a warp stay together: lanes past the end repeat the last unit and store nothing)
 #pragma unroll 1
-        for (int u = tid; u < th * a.cq; u += nthr) {
+        for (int u0 = tid & ~31; u0 < units; u0 += nthr) {
+            const bool exists = u0 + lane < units;
+            const int u = exists ? u0 + lane : units - 1;
             int t;
             const int row = a.div_cq.divmod(u, t);
             const int row_off = row * a.Q;
-            const int m = (int)((map_m + (unsigned)row_off) & 3u);
+            const int m = TURN ? 0 : (int)((map_m + (unsigned)row_off) & 3u);
             const int q0 = col0 + 4 * t - m;
-            if (q0 >= a.Q) continue;
+            if (!TURN && (!exists || q0 >= a.Q)) continue;
             const float* base = tile + row * pitch + t;
             // window column i is staged column 4t + 4 - m + i
             const float* win_at[4];
@@ -146,8 +152,9 @@ single_channel_flat_kernel(const FlatArgs a)
                             acc[0][j] = __ffma2_rn(make_float2(v[s + 2 * j], v[s + 2 * j + 1]), tap, acc[0][j]);
                     } else {
                         float2 tap[NB];
-                        if constexpr (PB == 1) {
-                            tap[0] = *reinterpret_cast<const float2*>(wr + s * TF);
+                        if constexpr (PB % 2 == 1) {
+#pragma unroll
+                            for (int b = 0; b < NB; ++b) tap[b] = *reinterpret_cast<const float2*>(wr + s * TF + 2 * b);
                         } else {
 #pragma unroll
                             for (int b = 0; b < PB / 2; ++b) {
@@ -174,7 +181,34 @@ single_channel_flat_kernel(const FlatArgs a)
                 for (int j = 0; j < 4; ++j)
                     o[j] = M == 1 ? ((j & 1) ? acc[0][(j / 2) % NA].y : acc[0][(j / 2) % NA].x)
                                   : ((e & 1) ? acc[e / 2][j % NA].y : acc[e / 2][j % NA].x);
-                if (whole) {
+                if constexpr (TURN) {
+                    const int me = (int)((map_m + (unsigned)e * (unsigned)map + (unsigned)row_off) & 3u);
+                    float l[3];                            // outputs 1, 2, 3 of the lane to the left
+#pragma unroll
+                    for (int j = 0; j < 3; ++j) l[j] = __shfl_up_sync(0xffffffffu, o[j + 1], 1);
+                    if (!exists) continue;
+                    const bool left = lane > 0 && t > 0;   // that lane holds the quad to the left
+                    const bool right = lane < 31 && t + 1 < a.cq && u + 1 < units;      // the next lane takes this quad's end along
+                    const float s1[6] = {me & 1 ? l[0] : l[1], me & 1 ? l[1] : l[2], me & 1 ? l[2] : o[0],
+                                         me & 1 ? o[0] : o[1], me & 1 ? o[1] : o[2], me & 1 ? o[2] : o[3]};
+                    const float4 v = make_float4(me & 2 ? s1[0] : s1[2], me & 2 ? s1[1] : s1[3], me & 2 ? s1[2] : s1[4], me & 2 ? s1[3] : s1[5]);
+                    const int qa = q0 - me;                // first column of the aligned quad
+                    float* const at = out - me;
+                    if ((left || me == 0) && qa + 3 < a.Q) {
+                        __stcs(reinterpret_cast<float4*>(at), v);
+                    } else {
+                        if (left && qa < a.Q) __stcs(at, v.x);                           // (me > 0 or the row's last quad)
+                        if ((left || me <= 1) && qa + 1 >= 0 && qa + 1 < a.Q) __stcs(at + 1, v.y);
+                        if ((left || me <= 2) && qa + 2 >= 0 && qa + 2 < a.Q) __stcs(at + 2, v.z);
+                        if (qa + 3 >= 0 && qa + 3 < a.Q) __stcs(at + 3, v.w);
+                        if (!left && me == 0 && qa < a.Q) __stcs(at, v.x);
+                    }
+                    if (!right) {                          // outputs 4 - me .. 3
+#pragma unroll
+                        for (int j = 1; j < 4; ++j)
+                            if (j + me >= 4 && q0 + j < a.Q) __stcs(out + j, o[j]);
+                    }
+                } else if (whole) {
                     __stcs(reinterpret_cast<float4*>(out), make_float4(o[0], o[1], o[2], o[3]));
                 } else {
 #pragma unroll
@@ -187,12 +221,12 @@ single_channel_flat_kernel(const FlatArgs a)
 }
 
 // Cycles of a scheduler for one warp's (quad, map block).
-inline double unit_cycles(int maps, int R, int S)
+inline double unit_cycles(int maps, int R, int S, bool turn)
 {
-    return (maps == 1 ? 4.0 : 4.0 * maps) * R * S + R * (S + 3) * 2.5 + 60;
+    return (maps == 1 ? 4.0 : 4.0 * maps) * R * S + R * (S + 3) * 2.5 + 60 + (turn ? 75.0 * maps : 0.0);
 }
 
-template <int RT, int S, int M>
+template <int RT, int S, int M, bool TURN>
 conv2d_status_t launch_flat(FlatArgs& a, const Shape& sh, cudaStream_t stream)
 {
     constexpr int TF = M == 1 ? 2 : M;
@@ -201,7 +235,7 @@ conv2d_status_t launch_flat(FlatArgs& a, const Shape& sh, cudaStream_t stream)
     const int whole = sh.K / (classes * M), left = sh.K - whole * classes * M;
     a.cbs = whole * classes + (left < classes ? left : classes);
     const int sms = sm_count();
-    const int nq = (sh.Q + (a.class_shift == 0 && sh.Q % 4 == 0 ? 0 : 3) + 3) / 4;
+    const int nq = (sh.Q + (TURN || (a.class_shift == 0 && sh.Q % 4 == 0) ? 0 : 3) + 3) / 4;
     a.col_tiles = (nq + kMaxQuads - 1) / kMaxQuads;
     a.cq = (nq + a.col_tiles - 1) / a.col_tiles;
     a.div_cq = FastDiv(a.cq);
@@ -218,7 +252,8 @@ conv2d_status_t launch_flat(FlatArgs& a, const Shape& sh, cudaStream_t stream)
         const int per = (a.cbs + splits - 1) / splits, used = (a.cbs + per - 1) / per;
         const size_t tap_bytes = (size_t)per * sh.R * S * TF * sizeof(float);
         if (tap_bytes > 64 * 1024) continue;
-        for (int bh = 1; bh <= 32 && bh <= sh.P; ++bh) {
+        for (int bh : {1, 2, 3, 4, 5, 6, 8, 12, 16}) {                       // (the search is on the path of every call)
+            if (bh > sh.P) break;
             const size_t smem = tap_bytes + (size_t)(bh + sh.R - 1) * 4 * a.plane * sizeof(float);
             if (smem > (bh == 1 ? (size_t)200 : (size_t)72) * 1024) break;
             const int threads = bh * a.cq >= kMaxThreads ? kMaxThreads : (bh * a.cq + 31) / 32 * 32;
@@ -229,7 +264,7 @@ conv2d_status_t launch_flat(FlatArgs& a, const Shape& sh, cudaStream_t stream)
             const double res = by_regs < by_smem ? by_regs : by_smem;
             // one block on a scheduler: what its warps issue, beside what it writes at an SM's share of the memory rate
             const double staging = (bh + sh.R - 1) * (4.0 * a.npos / 32.0) * 20.0 + (double)per * sh.R * S * TF / 32.0 * 20.0;
-            const double issue = ((threads / 32) * (passes * per * unit_cycles(M, sh.R, S)) + staging) / 4 + kBlockCycles;
+            const double issue = ((threads / 32) * (passes * per * unit_cycles(M, sh.R, S, TURN)) + staging) / 4 + kBlockCycles;
             const double write = (double)(sh.K < per * M ? sh.K : per * M) * bh * a.cq * 16.0 / 23.0;
             const double work = issue > write ? issue + 0.3 * write : write + 0.3 * issue;
             const double per_sm = (double)blocks / sms, each = (kLatency + work) / res;
@@ -246,7 +281,7 @@ conv2d_status_t launch_flat(FlatArgs& a, const Shape& sh, cudaStream_t stream)
     a.bands = (sh.P + a.band_h - 1) / a.band_h;
     const long long blocks = (long long)sh.N * a.col_tiles * a.bands * a.splits;
     if (blocks > 0x7fffffffLL) return CONV2D_ERR_UNSUPPORTED;
-    auto kern = single_channel_flat_kernel<RT, S, M>;
+    auto kern = single_channel_flat_kernel<RT, S, M, TURN>;
     static size_t smem_done[64] = {};
     if (best_smem > 48 * 1024 && raise_smem_limit(reinterpret_cast<const void*>(kern), best_smem, smem_done) != cudaSuccess)
         return CONV2D_ERR_CUDA;
@@ -258,48 +293,87 @@ conv2d_status_t launch_flat(FlatArgs& a, const Shape& sh, cudaStream_t stream)
 // Maps accumulated together: as many as a class fills.  More of them share the reads of a window row; empty ones cost
 // as much as full ones.  16 maps leave two blocks on an SM: they pay from 9 taps on (2048 x 2048, 32 maps: 7 x 7 267 us
 // with 8, 255 with 16; 4096 x 4096, 32 maps of 3 x 3 439 and 412; 2048 x 2048, 1 x 1 82 and 84 to 95).
-template <int RT, int S>
-conv2d_status_t pick_maps(FlatArgs& a, const Shape& sh, cudaStream_t stream)
+// Classes or turned quads: where a class would have one or two maps only, each class reads the windows anew, which costs
+// more than turning the quads of all maps at the store (14 x 375 x 1439, 4 maps of 5 x 5: 83 us in classes, 64 turned;
+// 15 x 2463 x 567, 8 maps of 5 x 5 242 and 269; 7 x 1623 x 488, 6 maps of 3 x 3 36 and 49).
+struct MapChoice { int maps; bool turn; double cost; };      // cost: cycles of a scheduler for one warp's quads of all maps
+MapChoice choose_maps(const Shape& sh, int class_shift)
 {
-    const int per_class = (sh.K + (1 << a.class_shift) - 1) >> a.class_shift;
-    auto cost = [&](int m) { return ((per_class + m - 1) / m) * unit_cycles(m, sh.R, S); };
-    int best = 1;
-    for (int m = 2; m <= (sh.R * S >= 9 ? 16 : 8); m *= 2)
-        if (cost(m) <= cost(best)) best = m;
-    switch (best) {
-    case 16: return launch_flat<RT, S, 16>(a, sh, stream);
-    case 8: return launch_flat<RT, S, 8>(a, sh, stream);
-    case 4: return launch_flat<RT, S, 4>(a, sh, stream);
-    case 2: return launch_flat<RT, S, 2>(a, sh, stream);
-    default: return launch_flat<RT, S, 1>(a, sh, stream);
+    auto cost = [&](int m, int classes, bool turn) {
+        const int per_class = (sh.K + classes - 1) / classes, used = sh.K < classes ? sh.K : classes;
+        return (double)used * ((per_class + m - 1) / m) * unit_cycles(m, sh.R, sh.S, turn);
+    };
+    MapChoice best{1, false, cost(1, 1 << class_shift, false)};
+    for (int m : {2, 4, 6, 8, 12, 16}) {
+        const double c = cost(m, 1 << class_shift, false);
+        if ((m <= 8 || sh.R * sh.S >= 9) && c <= best.cost) best = MapChoice{m, false, c};
+    }
+    const int forced = env_int("CONV2D_B200_SC_TURN", -1);
+    if (class_shift == 0 || forced == 0) return best;
+    MapChoice turned{1, true, cost(1, 1, true)};
+    for (int m : {2, 4, 8}) {
+        const double c = cost(m, 1, true);
+        if (c <= turned.cost) turned = MapChoice{m, true, c};
+    }
+    return forced > 0 || turned.cost < best.cost ? turned : best;
+}
+
+template <int RT, int S>
+conv2d_status_t launch_maps(FlatArgs& a, const Shape& sh, cudaStream_t stream)
+{
+    const MapChoice c = choose_maps(sh, a.class_shift);
+    if (c.turn) {
+        a.class_shift = 0;
+        switch (c.maps) {
+        case 8: return launch_flat<RT, S, 8, true>(a, sh, stream);
+        case 4: return launch_flat<RT, S, 4, true>(a, sh, stream);
+        case 2: return launch_flat<RT, S, 2, true>(a, sh, stream);
+        default: return launch_flat<RT, S, 1, true>(a, sh, stream);
+        }
+    }
+    switch (c.maps) {
+    case 16: return launch_flat<RT, S, 16, false>(a, sh, stream);
+    case 12: return launch_flat<RT, S, 12, false>(a, sh, stream);
+    case 8: return launch_flat<RT, S, 8, false>(a, sh, stream);
+    case 6: return launch_flat<RT, S, 6, false>(a, sh, stream);
+    case 4: return launch_flat<RT, S, 4, false>(a, sh, stream);
+    case 2: return launch_flat<RT, S, 2, false>(a, sh, stream);
+    default: return launch_flat<RT, S, 1, false>(a, sh, stream);
     }
 }
 
+int class_shift_of(const Shape& sh)
+{
+    const long long map = (long long)sh.P * sh.Q;
+    return map % 4 == 0 ? 0 : (map % 2 == 0 ? 1 : 2);
+}
+
 }  // namespace
+
+double single_channel_flat_cost(const Shape& sh) { return choose_maps(sh, class_shift_of(sh)).cost; }
 
 conv2d_status_t launch_single_channel_flat(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream)
 {
     FlatArgs a{};
     a.x = x; a.w = w; a.y = y;
     a.H = sh.H; a.W = sh.W; a.K = sh.K; a.R = sh.R; a.P = sh.P; a.Q = sh.Q;
-    const long long map = (long long)sh.P * sh.Q;
-    a.class_shift = map % 4 == 0 ? 0 : (map % 2 == 0 ? 1 : 2);
+    a.class_shift = class_shift_of(sh);
     if (sh.R == sh.S) {
         switch (sh.R) {
-        case 1: return pick_maps<1, 1>(a, sh, stream);
-        case 3: return pick_maps<3, 3>(a, sh, stream);
-        case 5: return pick_maps<5, 5>(a, sh, stream);
-        case 7: return pick_maps<7, 7>(a, sh, stream);
+        case 1: return launch_maps<1, 1>(a, sh, stream);
+        case 3: return launch_maps<3, 3>(a, sh, stream);
+        case 5: return launch_maps<5, 5>(a, sh, stream);
+        case 7: return launch_maps<7, 7>(a, sh, stream);
         }
     }
     switch (sh.S) {
-    case 1: return pick_maps<0, 1>(a, sh, stream);
-    case 2: return pick_maps<0, 2>(a, sh, stream);
-    case 3: return pick_maps<0, 3>(a, sh, stream);
-    case 4: return pick_maps<0, 4>(a, sh, stream);
-    case 5: return pick_maps<0, 5>(a, sh, stream);
-    case 6: return pick_maps<0, 6>(a, sh, stream);
-    case 7: return pick_maps<0, 7>(a, sh, stream);
+    case 1: return launch_maps<0, 1>(a, sh, stream);
+    case 2: return launch_maps<0, 2>(a, sh, stream);
+    case 3: return launch_maps<0, 3>(a, sh, stream);
+    case 4: return launch_maps<0, 4>(a, sh, stream);
+    case 5: return launch_maps<0, 5>(a, sh, stream);
+    case 6: return launch_maps<0, 6>(a, sh, stream);
+    case 7: return launch_maps<0, 7>(a, sh, stream);
     }
     return CONV2D_ERR_UNSUPPORTED;
 }

@@ -20,10 +20,12 @@ SHAPES += [
 ]
 
 
+@pytest.mark.parametrize("turn", [0, 1])      # maps in classes of equal alignment / quads turned at the store
 @pytest.mark.parametrize("dims", SHAPES)
-def test_exact_on_integers(oracle, monkeypatch, dims):
+def test_exact_on_integers(oracle, monkeypatch, dims, turn):
     N, H, W, K, R, S = dims
     monkeypatch.setenv("CONV2D_B200_SC_FLAT", "1")
+    monkeypatch.setenv("CONV2D_B200_SC_TURN", str(turn))
     x, w = small_integers((N, 1, H, W), 1401), small_integers((K, 1, R, S), 1402)
     y_ref, _ = oracle.conv2d_oracle(x, w)
     np.testing.assert_array_equal(run_library(x, w, entry="single").astype(np.float64), y_ref)
