@@ -13,7 +13,8 @@ namespace conv2d_b200 {
 // Problem extents, library symbols (N images, C channels, H x W image, K filters, R x S taps).
 struct Shape {
     int N, C, H, W, K, R, S, P, Q;
-    int pad_h = 0, pad_w = 0;   // zero padding; only the tensor-core path with patch addressing takes it natively
+    int pad_h = 0, pad_w = 0;   // zero padding and stride; only the tensor-core path takes them natively
+    int stride = 1;
 };
 
 // Capacity of the per-device constant-memory filter bank of the single-channel kernel, in floats.

@@ -324,6 +324,16 @@ conv2d_status_t conv2d_fwd_general_strided(const float* x, const float* w, float
     if (st != CONV2D_OK) return st;
     st = check_device();
     if (st != CONV2D_OK) return st;
+    // The tensor-core kernel computes strided convolutions on virtual images, straight from x and with as many
+    // multiplications as the definition has, wherever the rewritten problem would run there as well (inner > 0).
+    if (algo != CONV2D_ALGO_FFMA && inner > 0 && (long long)C * H * W <= 0x7fffffffLL) {
+        Shape shp{N, C, H, W, K, R, S, g.P, g.Q};
+        shp.pad_h = pad_h; shp.pad_w = pad_w; shp.stride = stride;
+        const conv2d_status_t native = launch_general_tf32(x, w, y, shp, workspace, workspace_bytes,
+                                                           (flags & CONV2D_FLAG_WEIGHTS_PACKED) != 0,
+                                                           static_cast<cudaStream_t>(cuda_stream));
+        if (native != CONV2D_ERR_UNSUPPORTED && native != CONV2D_ERR_WORKSPACE) return native;
+    }
     const bool own_status = inner < kStatusBytes;
     unsigned char* base = static_cast<unsigned char*>(workspace);
     float* x2 = reinterpret_cast<float*>(base + round_up_256(own_status ? kStatusBytes : inner));

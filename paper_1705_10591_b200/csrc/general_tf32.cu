@@ -121,7 +121,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
 {
     const float* x = static_cast<const float*>(x_any);   // 16-bit operands: re-read as such inside the kernel
     const float* w = static_cast<const float*>(w_any);
-    {
+    if (sh.stride == 1 && sh.pad_h == 0 && sh.pad_w == 0) {
         // 1 x 1 filters on suitably aligned tensors: the kernel whose operands and output all move by tensor-map copies
         const conv2d_status_t st = launch_pointwise_tma(x_any, w_any, y, sh, b16, fp16, workspace, workspace_bytes, weights_packed, stream);
         if (st != CONV2D_ERR_UNSUPPORTED) return st;
@@ -141,30 +141,38 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
 
     if (!weights_packed) {
         const long long total = (long long)packed_floats(p);
-        const FoldedFilter ff{sh.C, sh.R, sh.S, p.fold_r, p.fold_s};
+        const FoldedFilter ff{sh.C, sh.R, sh.S, p.fold_r, p.fold_s, p.mixed ? sh.stride : 1};
         const long long lanes = (long long)p.n_blocks * p.cblks * kChunks * p.n_tile * (b16 ? 8 : 4);   // one thread per element of a tap's slice
         long long blocks = (lanes + 255) / 256;
         if (blocks > sm_count() * 16LL) blocks = sm_count() * 16LL;
-        const size_t tile_bytes = (size_t)8 * kCB * 4 * p.taps;       // 8 filters x one channel block x taps
-        if (p.fold_r * p.fold_s == 1 && tile_bytes <= 48 * 1024 && p.n_tile % 8 == 0 && !p.pair_taps) {
-            const dim3 grid((unsigned)(p.n_blocks * p.n_tile / 8), (unsigned)p.cblks);
-            int threads = (8 * kChunks * p.taps + 31) / 32 * 32;          // one 16-byte unit per thread in the store phase
+        // few blocks: the taps are shared out, too (64 filters of 3 x 7 x 7 with stride 2: 16 blocks whose threads walked
+        // over 16 taps took 7.6 us)
+        unsigned tap_rows = 1;
+        while (p.pair_compact == 0 && tap_rows * 2 <= (unsigned)p.taps && blocks * tap_rows * 2 <= sm_count() * 4LL) tap_rows *= 2;
+        const int all_taps = p.phases > 1 ? sh.R * sh.S : p.taps;
+        const int bank_blocks = p.cblks / p.phases;
+        const size_t tile_bytes = (size_t)8 * kCB * 4 * all_taps;     // 8 filters x one channel block x taps
+        const bool tiled = p.fold_r * p.fold_s == 1 && !p.mixed && tile_bytes <= 48 * 1024 && p.n_tile % 8 == 0 && !p.pair_taps;
+        if (p.phases > 1 && !tiled) return CONV2D_ERR_UNSUPPORTED;
+        if (tiled) {
+            const dim3 grid((unsigned)(p.n_blocks * p.n_tile / 8), (unsigned)bank_blocks);
+            int threads = (8 * kChunks * all_taps + 31) / 32 * 32;        // one 16-byte unit per thread in the store phase
             threads = threads < 128 ? 128 : (threads > 1024 ? 1024 : threads);
             // (launched the ordinary way: it starts only when the previous call's kernel, which may still
             // be reading the workspace, has finished; measured no gain from overlapping its launch)
             if (b16)
                 repack_filters_tiled_kernel<unsigned short, 8><<<grid, threads, tile_bytes, stream>>>(
                     static_cast<const unsigned short*>(w_any), reinterpret_cast<unsigned short*>(wp), status, sh.K, sh.C,
-                    p.taps, p.n_tile, p.cblks);
+                    all_taps, p.n_tile, bank_blocks, sh.S, 1);
             else
-                repack_filters_tiled_kernel<float, 4><<<grid, threads, tile_bytes, stream>>>(w, wp, status, sh.K, sh.C, p.taps,
-                                                                                             p.n_tile, p.cblks);
+                repack_filters_tiled_kernel<float, 4><<<grid, threads, tile_bytes, stream>>>(w, wp, status, sh.K, sh.C, all_taps,
+                                                                                             p.n_tile, bank_blocks, sh.S, p.phases > 1 ? sh.stride : 1);
         } else if (b16)
-            repack_filters_kernel<unsigned short, 8><<<(unsigned)blocks, 256, 0, stream>>>(
+            repack_filters_kernel<unsigned short, 8><<<dim3((unsigned)blocks, tap_rows), 256, 0, stream>>>(
                 static_cast<const unsigned short*>(w_any), reinterpret_cast<unsigned short*>(wp), status, sh.K, ff,
                 p.taps, p.n_tile, p.cblks, lanes, p.pair_taps + p.pair_compact);
         else
-            repack_filters_kernel<float, 4><<<(unsigned)blocks, 256, 0, stream>>>(w, wp, status, sh.K, ff, p.taps,
+            repack_filters_kernel<float, 4><<<dim3((unsigned)blocks, tap_rows), 256, 0, stream>>>(w, wp, status, sh.K, ff, p.taps,
                                                                                   p.n_tile, p.cblks, lanes, p.pair_taps + p.pair_compact);
         count_launch();
         if (cudaGetLastError() != cudaSuccess) return CONV2D_ERR_CUDA;
@@ -182,7 +190,9 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
                                      general_tc_kernel<false, false, true, false>,  general_tc_kernel<true, false, true, false>,
                                      general_tc_kernel<false, false, false, true>,  general_tc_kernel<true, false, false, true>,
                                      general_tc_kernel<false, false, true, true>,   general_tc_kernel<true, false, true, true>,
-                                     general_tc_kernel<false, false, false, false, true>, general_tc_kernel<true, false, false, false, true>};
+                                     general_tc_kernel<false, false, false, false, true>, general_tc_kernel<true, false, false, false, true>,
+                                     general_tc_kernel<false, false, false, false, false, true>, general_tc_kernel<false, false, false, true, false, true>,
+                                     general_tc_kernel<false, false, false, false, true, true>};
         for (auto k : all)
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess)
             return CONV2D_ERR_CUDA;
@@ -192,23 +202,27 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     a.x = x; a.wp = wp; a.y = y; a.status = status;
     a.N = sh.N; a.C = sh.C; a.H = sh.H; a.W = sh.W; a.K = sh.K; a.P = sh.P; a.Q = sh.Q;
     a.patch_w = p.patch_w; a.patch_tw = p.patch_tw; a.patch_rows = p.patch_rows; a.patch_cols = p.patch_cols;
-    a.row_pitch = p.patch_w ? p.patch_w : sh.W;
+    a.row_pitch = p.patch_w ? p.patch_w : (p.virt ? p.virt_w : sh.W);
     a.pad_h = sh.pad_h; a.pad_w = sh.pad_w;
     a.fold_r = p.fold_r; a.fold_s = p.fold_s; a.R = sh.R / p.fold_r; a.S = sh.S / p.fold_s;
     a.HW = sh.H * sh.W;
-    a.total_pix = sh.N * sh.H * sh.W;
+    const int plan_h = p.virt ? p.virt_h : sh.H, plan_w = p.virt ? p.virt_w : sh.W;       // rows and columns of the flat pixel sequence
+    a.total_pix = sh.N * plan_h * plan_w;
+    a.st = sh.stride; a.off_h = p.off_h; a.off_w = p.off_w; a.shift0 = p.shift0;
+    a.phases = p.phases; a.phase_cols = p.phase_cols; a.cblks_c = p.cblks / p.phases; a.div_phases = FastDiv(p.phases);
+    a.mixed = p.mixed; a.mix_c = sh.C; a.mix_st2 = sh.stride * sh.stride;
     a.n_tile = p.n_tile; a.n_blocks = p.n_blocks; a.mt = p.mt; a.tile_px = p.tile_px; a.px_groups = p.px_groups; a.nbuf = p.nbuf; a.npix = p.npix; a.cstride = chunk_stride(p.npix);
     a.cblks = p.cblks; a.taps = p.taps;
     a.a_stages = p.a_stages; a.b_stages = p.b_stages; a.tps = p.tps;
     a.cbg = p.cbg; a.groups = (p.cblks + p.cbg - 1) / p.cbg; a.resident = p.resident; a.swap = p.swap;
     a.vec = 1;
     for (int v = 4; v >= 2; v >>= 1)       // v adjacent accumulator columns must be v adjacent, aligned outputs of one row
-        if ((p.patch_w ? p.patch_tw : sh.W) % v == 0 && sh.Q % v == 0 && ((long long)sh.P * sh.Q) % v == 0 &&
+        if ((p.patch_w ? p.patch_tw : plan_w) % v == 0 && sh.Q % v == 0 && ((long long)sh.P * sh.Q) % v == 0 &&
             reinterpret_cast<uintptr_t>(y) % (4 * v) == 0) { a.vec = v; break; }
     a.vec_shift = a.vec == 4 ? 2 : (a.vec == 2 ? 1 : 0);
     a.pair_compact = p.pair_compact; a.cb_bytes = (int)p.cb_bytes;
     a.pair_taps = p.pair_taps; a.s_slots = p.s_slots; a.s_step = p.pair_taps ? 2 : 1; a.item_stride = p.tile_px - p.ovl;
-    a.div_HW = FastDiv(a.HW); a.div_W = FastDiv(sh.W); a.div_npix = FastDiv(p.npix);
+    a.div_HW = FastDiv(plan_h * plan_w); a.div_W = FastDiv(plan_w); a.div_npix = FastDiv(p.npix);
     a.div_qn = FastDiv(p.npix / 4 > 0 ? p.npix / 4 : 1); a.div_patch_w = FastDiv(p.patch_w ? p.patch_w : 1);
     a.xchg_slots = p.xchg_slots;
     a.xchg_bytes = (int)xchg_area_bytes(p.xchg_slots);
@@ -216,7 +230,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     // per block is short: 34.0 us without them, 35.4 us with them on 32 x 256 x 14 x 14 -> 256 maps)
     a.helpers = (p.swap && !p.cluster && (size_t)p.a_stages * p.cbg * kCB * chunk_stride(p.npix) * 4 >= 2 * kXposeBytes &&
                  env_int("CONV2D_B200_TF32_HELPERS", 1) != 0) ? 1 : 0;
-    a.quad = ((p.patch_w ? (sh.W % 4 == 0 && sh.pad_w % 4 == 0) : (sh.H * sh.W) % 4 == 0) && p.fold_r * p.fold_s == 1 && env_int("CONV2D_B200_TF32_QUAD", 1) != 0) ? 1 : 0;
+    a.quad = ((p.virt ? (sh.stride == 1 && sh.W % 4 == 0) : p.patch_w ? (sh.W % 4 == 0 && sh.pad_w % 4 == 0) : (sh.H * sh.W) % 4 == 0) && p.fold_r * p.fold_s == 1 && env_int("CONV2D_B200_TF32_QUAD", 1) != 0) ? 1 : 0;
     {
         // as many producer groups as can each still cover a stage in one pass (one memory round trip)
         const long long per_pass = a.quad ? kProducers : (long long)kProducers * kUnitsPerThread;
@@ -250,13 +264,15 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     // tail of whatever kernel precedes it on the stream; it waits for that kernel before it touches global memory.
     const bool fold = p.fold_r * p.fold_s > 1;
     void (*kernel)(KernelArgs);
-    if (p.pair_taps && p.patch_w) kernel = b16 ? general_tc_kernel<true, false, true, true> : general_tc_kernel<false, false, true, true>;
+    if (p.virt) kernel = p.pair_taps ? general_tc_kernel<false, false, false, true, false, true> : general_tc_kernel<false, false, false, false, false, true>;
+    else if (p.pair_taps && p.patch_w) kernel = b16 ? general_tc_kernel<true, false, true, true> : general_tc_kernel<false, false, true, true>;
     else if (p.pair_taps) kernel = b16 ? general_tc_kernel<true, false, false, true> : general_tc_kernel<false, false, false, true>;
     else if (p.patch_w) kernel = b16 ? general_tc_kernel<true, false, true, false> : general_tc_kernel<false, false, true, false>;
     else if (fold) kernel = b16 ? general_tc_kernel<true, true, false, false> : general_tc_kernel<false, true, false, false>;
     else kernel = b16 ? general_tc_kernel<true, false, false, false> : general_tc_kernel<false, false, false, false>;
     if (p.cluster) {
-        kernel = b16 ? general_tc_kernel<true, false, false, false, true> : general_tc_kernel<false, false, false, false, true>;
+        kernel = p.virt ? general_tc_kernel<false, false, false, false, true, true>
+               : b16 ? general_tc_kernel<true, false, false, false, true> : general_tc_kernel<false, false, false, false, true>;
         if (launch_pdl_cluster(kernel, dim3((unsigned)p.grid), dim3(kThreads), p.smem_bytes, stream, 2u, a) != cudaSuccess)
             return CONV2D_ERR_CUDA;
     } else if (launch_pdl(kernel, dim3((unsigned)p.grid), dim3(kThreads), p.smem_bytes, stream, a) != cudaSuccess) return CONV2D_ERR_CUDA;

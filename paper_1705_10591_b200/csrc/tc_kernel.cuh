@@ -75,6 +75,15 @@ struct KernelArgs {
     int test_drop_stage;    // test hook: the filter copy with this ordinal is armed but never issued (-1: none)
     int early_x;            // 1: this call's filter re-ordering kernel directly precedes on the stream, so the image is
                             // final already and the producers need not wait for that kernel
+    // Virtual images (VIRT kernels): zero padding and strides, see staged_pixel_virtual.  H, W, HW are those of the image
+    // in memory; div_HW and div_W divide by the virtual plane and row, total_pix counts virtual pixels.
+    int st, off_h, off_w;   // stride; rows and columns of zeros before the image in the virtual one (before the stride)
+    int shift0;             // staged pixels between an output and its tap (0, 0)
+    int phases, phase_cols; // phases with taps of their own (1 where the taps are the same for all channels); columns of them
+    int cblks_c;            // 16-channel blocks of one phase
+    int mixed;              // 1: the phases of a channel are adjacent staged channels (few input channels), every tap for all
+    int mix_c, mix_st2;     // ... channels of the image, stride * stride
+    FastDiv div_phases;
     int items;              // work items = supertiles x n_blocks
     unsigned tmem_cols;
 };
@@ -126,11 +135,49 @@ __device__ __forceinline__ bool output_pixel(const KernelArgs& a, const ItemGeom
     return p < a.P && q < a.Q;
 }
 
+// Virtual images.  A padded convolution is computed on images that carry their zeros: rows of W + off_w columns, the
+// first off_w of them zero (a multiple of four where the producers load quads), of which the zeros to the right of one
+// row are those to the left of the next; in the same way the rows of zeros above an image are those below the one before.
+// With a stride st the virtual pixel (h, w) of phase (a, b) is pixel (st*h + a - off_h, st*w + b - off_w) of the image:
+// a stride-1 convolution whose taps (r, s) with r % st == a, s % st == b read phase (a, b) shifted by (r / st, s / st).
+// Every staged channel block belongs to one phase and meets only that phase's taps: as many multiplications as the
+// definition has (a rewritten image of st*st times as many channels has ceil(R/st)*ceil(S/st) taps on all of them).
+struct Phase {
+    int cblk, a, b;         // channel block of the image, phase
+    int taps, cols;         // its taps, and how many of them lie in a row
+    int base;               // taps of the phases before it
+};
+__device__ __forceinline__ Phase phase_of(const KernelArgs& a, int cb)
+{
+    Phase p;
+    int idx;
+    p.cblk = a.div_phases.divmod(cb, idx);
+    p.a = idx / a.phase_cols;
+    p.b = idx - p.a * a.phase_cols;
+    const int rows = (a.R - p.a + a.st - 1) / a.st;
+    p.cols = (a.S - p.b + a.st - 1) / a.st;
+    p.taps = rows * p.cols;
+    const int rows_before = p.a * (a.R / a.st) + min(p.a, a.R % a.st), cols_before = p.b * (a.S / a.st) + min(p.b, a.S % a.st);
+    p.base = rows_before * a.S + rows * cols_before;
+    return p;
+}
+// Staged pixel -> image n and the image row and column of phase (0, 0), which may lie outside the image.
+__device__ __forceinline__ bool staged_pixel_virtual(const KernelArgs& a, const ItemGeom& g, int jj, int& n, int& h, int& wc)
+{
+    const int j = g.j0 + jj;
+    int rem;
+    n = a.div_HW.divmod(j, rem);
+    h = a.div_W.divmod(rem, wc);
+    h = h * a.st - a.off_h;
+    wc = wc * a.st - a.off_w;
+    return j < a.total_pix;
+}
+
 // Producer helpers.  A stage holds `cbg` channel blocks of kCB channels for npix pixels, laid out
 // [channel block][chunk][pixel] in 16-byte units.  A work unit is (channel block g, pixel jj), numbered
 // i = g * npix + jj; thread t of the 256 producers owns units first + t, first + t + 256, ...  Consecutive
 // lanes read consecutive pixels of one channel (coalesced) and write consecutive 16-byte units.
-template <bool B16, bool FOLD, bool PATCH, int CNT>
+template <bool B16, bool FOLD, bool PATCH, bool VIRT, int CNT>
 __device__ __forceinline__ void load_units(float (&v)[CNT][kCB], const KernelArgs& a, const ItemGeom& geom, int cb0, int first, int wtid, int nthr)
 {
     const int units = a.npix * a.cbg;
@@ -142,6 +189,36 @@ __device__ __forceinline__ void load_units(float (&v)[CNT][kCB], const KernelArg
         if (i < units) {
             int jj;
             const int g = a.div_npix.divmod(i, jj);
+            if (VIRT) {
+                int n, h, wc;
+                if (!staged_pixel_virtual(a, geom, jj, n, h, wc)) continue;
+                const float* img = a.x + (size_t)n * a.C * a.HW;
+                if (a.mixed) {
+                    // staged channel (c, a, b): one pixel of every phase of a channel after the other
+                    int vc = (cb0 + g) * kCB;
+                    int c = vc / a.mix_st2, ph = vc - c * a.mix_st2;
+                    int pa = ph / a.st, pb = ph - pa * a.st;
+                    const float* src = img + (size_t)c * a.HW + h * a.W + wc;
+#pragma unroll
+                    for (int e = 0; e < kCB; ++e) {
+                        if (c < a.mix_c && (unsigned)(h + pa) < (unsigned)a.H && (unsigned)(wc + pb) < (unsigned)a.W)
+                            v[u][e] = __ldg(src + pa * a.W + pb);
+                        if (++pb == a.st) { pb = 0; if (++pa == a.st) { pa = 0; ++c; src += a.HW; } }
+                    }
+                } else {
+                    const Phase p = phase_of(a, cb0 + g);
+                    h += p.a;
+                    wc += p.b;
+                    const int c0 = p.cblk * kCB;
+                    if ((unsigned)h < (unsigned)a.H && (unsigned)wc < (unsigned)a.W) {
+                        const float* src = img + (size_t)c0 * a.HW + h * a.W + wc;
+#pragma unroll
+                        for (int e = 0; e < kCB; ++e)
+                            if (c0 + e < a.C) v[u][e] = __ldg(src + (size_t)e * a.HW);
+                    }
+                }
+                continue;
+            }
             if (FOLD) {
                 // Folded taps: staged channel vc = (c, r, s) of pixel j is x[c] at pixel j + r*W + s (zero beyond
                 // the image: such windows belong to outputs that are dropped anyway).
@@ -312,7 +389,8 @@ __device__ __forceinline__ void issue_tap(uint32_t d, uint32_t px_lo, uint32_t f
 // peer's shared memory (distributed shared memory, plain stores) and adds what the peer sent to its own
 // accumulators before the ordinary write-back.  No zero-fill of y, no atomic adds, and a + b = b + a keeps the
 // result independent of timing.
-template <bool B16, bool FOLD, bool PATCH, bool STACK, bool CLUSTER = false>
+// VIRT: zero padding and strides on virtual images (staged_pixel_virtual); flat addressing, fp32 operands.
+template <bool B16, bool FOLD, bool PATCH, bool STACK, bool CLUSTER = false, bool VIRT = false>
 __global__ void __launch_bounds__(kThreads, 1)
 general_tc_kernel(const KernelArgs a)
 {
@@ -323,7 +401,8 @@ general_tc_kernel(const KernelArgs a)
     const uint32_t b_stage_bytes = b_chunk_bytes * (uint32_t)a.tps;
     unsigned char* a_smem = smem;
     unsigned char* b_smem = smem + (size_t)a.a_stages * a_stage_bytes;
-    const size_t b_region_bytes = a.resident ? (size_t)a.cblks * a.cb_bytes : (size_t)a.b_stages * b_stage_bytes;
+    const int bank_blocks = VIRT ? a.cblks_c : a.cblks;                 // pieces of cb_bytes in a filter block's bank
+    const size_t b_region_bytes = a.resident ? (size_t)bank_blocks * a.cb_bytes : (size_t)a.b_stages * b_stage_bytes;
     float* xpose = reinterpret_cast<float*>(b_smem + b_region_bytes);            // only present (and used) when a.swap
     unsigned char* after_xpose = b_smem + b_region_bytes + (a.swap ? kXposeBytes : 0);
     float* xchg = reinterpret_cast<float*>(after_xpose);     // CLUSTER: [4 quarters][xchg_slots][8 column groups][32 lanes][4 floats] partial sums from the peer
@@ -344,6 +423,14 @@ general_tc_kernel(const KernelArgs a)
     volatile unsigned long long* t_entry = reinterpret_cast<volatile unsigned long long*>(tmem_slot + 2);
     uint32_t* tap_shift = tmem_slot + 4;                   // [taps] r * row_pitch + s of every tap, in staged pixels
     // (bit 31: the slot is a lone tap held as a 64-row slice, see pair_compact)
+    if (VIRT && a.phases > 1) {
+        // one table per phase, behind one another in the order of the filter bank
+        for (int t = tid; t < a.R * a.S; t += kThreads) {
+            const int r = t / a.S, sx = t - r * a.S, r2 = r / a.st, s2 = sx / a.st;
+            const Phase p = phase_of(a, (r - r2 * a.st) * a.phase_cols + sx - s2 * a.st);
+            tap_shift[p.base + r2 * p.cols + s2] = (uint32_t)(r2 * a.row_pitch + s2);
+        }
+    } else
     for (int t = tid; t < a.taps; t += kThreads)
         tap_shift[t] = (uint32_t)((t / a.s_slots) * a.row_pitch + (t % a.s_slots) * a.s_step) |
                        ((a.pair_compact && (a.S & 1) && t % a.s_slots == a.s_slots - 1) ? 0x80000000u : 0u);
@@ -391,8 +478,8 @@ general_tc_kernel(const KernelArgs a)
                 // block, all on one barrier
                 const unsigned char* src = reinterpret_cast<const unsigned char*>(a.wp);
                 const uint32_t piece = (uint32_t)a.cb_bytes;
-                mbar_arrive_expect_tx(&b_full[0], piece * (uint32_t)a.cblks);
-                for (int cb = 0; cb < a.cblks; ++cb)
+                mbar_arrive_expect_tx(&b_full[0], piece * (uint32_t)bank_blocks);
+                for (int cb = 0; cb < bank_blocks; ++cb)
                     bulk_g2s(b_smem + (size_t)cb * piece, src + (size_t)cb * piece, piece, &b_full[0]);
                 alive = false;          // nothing to stream
                 if (*abort_flag) { uint32_t dummy = 0; mbar_wait_bounded(&b_full[0], 0u, &dummy, 1u << 16); }
@@ -401,7 +488,7 @@ general_tc_kernel(const KernelArgs a)
                 const ItemInfo ii = decode_item(a, item);
                 const int nb = ii.nb;
                 const unsigned char* src = reinterpret_cast<const unsigned char*>(a.wp)
-                                         + (size_t)nb * a.cblks * a.taps * b_chunk_bytes;
+                                         + (size_t)nb * bank_blocks * (VIRT ? (size_t)a.cb_bytes : (size_t)a.taps * b_chunk_bytes);
                 for (int grp = 0; grp < ii.n_groups && alive; ++grp) {
                     int gr = grp + ii.rot;
                     if (gr >= ii.n_groups) gr -= ii.n_groups;
@@ -409,13 +496,20 @@ general_tc_kernel(const KernelArgs a)
                     for (int g = 0; g < a.cbg && alive; ++g) {
                         const int cbr = gr * a.cbg + g;
                         if (cbr >= a.cblks) break;
-                        for (int t0 = 0; t0 < a.taps; t0 += a.tps) {
-                            const int nt = min(a.tps, a.taps - t0);
+                        int taps = a.taps;
+                        size_t cb_at = (size_t)cbr * a.taps;            // taps of the bank before this channel block's
+                        if (VIRT && a.phases > 1) {
+                            const Phase p = phase_of(a, cbr);
+                            taps = p.taps;
+                            cb_at = (size_t)p.cblk * (a.R * a.S) + p.base;
+                        }
+                        for (int t0 = 0; t0 < taps; t0 += a.tps) {
+                            const int nt = min(a.tps, taps - t0);
                             if (!mbar_wait_bounded(&b_empty[s], ph ^ 1u, abort_flag, a.max_polls)) { alive = false; break; }
                             const uint32_t bytes = b_chunk_bytes * (uint32_t)nt;
                             mbar_arrive_expect_tx(&b_full[s], bytes);
                             if (issued != a.test_drop_stage)     // (test hook: a dropped copy makes the consumer's wait expire)
-                                bulk_g2s(b_smem + (size_t)s * b_stage_bytes, src + ((size_t)cbr * a.taps + t0) * b_chunk_bytes,
+                                bulk_g2s(b_smem + (size_t)s * b_stage_bytes, src + (cb_at + t0) * b_chunk_bytes,
                                          bytes, &b_full[s]);
                             ++issued;
                             if (++s == a.b_stages) { s = 0; ph ^= 1u; }
@@ -493,13 +587,20 @@ general_tc_kernel(const KernelArgs a)
                     uint32_t a_lo_block = a_lo_fixed | ((smem_u32(a_smem + (size_t)as * a_stage_bytes) >> 4) & 0x3FFFu);
                     for (int g = 0; g < a.cbg && alive; ++g, a_lo_block += a_block_bytes >> 4) {
                         if (gr * a.cbg + g >= a.cblks) break;
-                        uint32_t row_shift = 0;                                  // r * row pitch, in pixels (= 16-byte units)
+                        uint32_t row_shift = VIRT ? (uint32_t)a.shift0 : 0u;     // r * row pitch, in pixels (= 16-byte units)
                         int sx = 0, sc = 0;
-                        for (int t0 = 0; t0 < a.taps; t0 += a.tps) {
-                            const int nt = min(a.tps, a.taps - t0);
+                        int taps = a.taps, s_slots = a.s_slots, tap0 = 0;
+                        size_t bank_at = (size_t)(gr * a.cbg + g) * a.cb_bytes;   // (resident filters)
+                        if (VIRT && a.phases > 1) {
+                            const Phase p = phase_of(a, gr * a.cbg + g);
+                            taps = p.taps; s_slots = p.cols; tap0 = p.base;
+                            bank_at = (size_t)p.cblk * a.cb_bytes + (size_t)p.base * b_chunk_bytes;
+                        }
+                        for (int t0 = 0; t0 < taps; t0 += a.tps) {
+                            const int nt = min(a.tps, taps - t0);
                             uint32_t b_lo;
                             if (a.resident) {
-                                b_lo = b_lo_fixed | ((smem_u32(b_smem + (size_t)(gr * a.cbg + g) * a.cb_bytes) >> 4) & 0x3FFFu);
+                                b_lo = b_lo_fixed | ((smem_u32(b_smem + bank_at) >> 4) & 0x3FFFu);
                             } else {
                                 if (!mbar_wait_bounded(&b_full[bs], b_phase, abort_flag, a.max_polls)) { alive = false; break; }
                                 tc_fence_after_sync();
@@ -511,7 +612,7 @@ general_tc_kernel(const KernelArgs a)
                                 // issue it with loop and address arithmetic around it (~230 cycles per MMA that
                                 // way), so a tap is one block of straight-line code and its shift comes from a
                                 // table, fetched one tap ahead.
-                                const uint32_t* shift = tap_shift + t0;
+                                const uint32_t* shift = tap_shift + tap0 + t0;
                                 uint32_t cur = shift[0];
                                 if (STACK && a.pair_compact) {
                                     // pairs of taps as M = 128 slices, a lone last tap as an M = 64 slice of half the size
@@ -533,7 +634,7 @@ general_tc_kernel(const KernelArgs a)
                                 } else
 #pragma unroll 3
                                 for (int t = 0; t < nt; ++t, b_lo += b_chunk_bytes >> 4) {
-                                    const uint32_t a_lo = a_lo_block + cur;
+                                    const uint32_t a_lo = (VIRT ? a_lo_block + (uint32_t)a.shift0 : a_lo_block) + cur;
                                     cur = shift[t + 1 < nt ? t + 1 : t];
                                     issue_tap<B16, 1>(d0, a_lo, b_lo, a_kstep, b_kstep, n_mma, desc_hi, idesc, accumulate);
                                     accumulate = 1;
@@ -559,7 +660,7 @@ general_tc_kernel(const KernelArgs a)
                                     }
                                     accumulate = 1;
                                     sx += a.s_step;
-                                    if (++sc == a.s_slots) { sc = 0; sx = 0; row_shift += (uint32_t)a.row_pitch; }
+                                    if (++sc == s_slots) { sc = 0; sx = 0; row_shift += (uint32_t)a.row_pitch; }
                                 }
                             }
                             if (!a.resident) {
@@ -641,7 +742,15 @@ general_tc_kernel(const KernelArgs a)
 #pragma unroll
                         for (int e = 0; e < kCB; ++e) v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
                         int n, off;
-                        if (staged_pixel<PATCH>(a, ii.geom, 4 * pq, n, off) && c0 < a.C) {
+                        bool in;
+                        if (VIRT) {             // (stride 1: four columns of a row lie in the image together or not at all)
+                            int h, wc;
+                            in = staged_pixel_virtual(a, ii.geom, 4 * pq, n, h, wc) && (unsigned)h < (unsigned)a.H && (unsigned)wc < (unsigned)a.W;
+                            off = h * a.W + wc;
+                        } else {
+                            in = staged_pixel<PATCH>(a, ii.geom, 4 * pq, n, off);
+                        }
+                        if (in && c0 < a.C) {
                             const float* src = a.x + ((size_t)n * a.C + c0) * a.HW + off;
 #pragma unroll
                             for (int ch = 0; ch < kChunks; ++ch) {
@@ -708,7 +817,7 @@ general_tc_kernel(const KernelArgs a)
                 } else
                 for (int first = 0; first < units; first += nthr * kUnitsPerThread) {
                     float v[kUnitsPerThread][kCB];
-                    load_units<B16, FOLD, PATCH>(v, a, ii.geom, gr * a.cbg, first, wtid, nthr);
+                    load_units<B16, FOLD, PATCH, VIRT>(v, a, ii.geom, gr * a.cbg, first, wtid, nthr);
                     store_units<B16>(v, dst, a, first, wtid, nthr);
                 }
                 fence_proxy_async_smem();

@@ -76,6 +76,11 @@ struct Plan {
     int supertiles;   // work-item rows over the flat pixel sequence
     int grid;
     size_t smem_bytes;
+    int virt;         // 1: virtual images (zero padding, strides)
+    int virt_h, virt_w, off_h, off_w, shift0, phases, phase_cols, mixed;     // see KernelArgs
+    long long pairs;  // (tap, channel block) pairs of a filter block
+    size_t bank_bytes;   // re-ordered filters of one filter block
+    double staged_ratio; // staged pixels per output of a 448-pixel item
     double makespan;  // MMA work of the busiest block, in item pixels x taps x channel blocks (to compare patch widths)
     bool ok;
 };
@@ -95,10 +100,40 @@ size_t smem_need(int a_stages, int npix, int n_tile, int b_stages, int tps, int 
 
 // b16: the operands are 16-bit floats, bf16 or fp16 (16-byte unit = 8 channels, 32 channels per staged block, K = 16 per MMA); the
 // byte layout of every stage is the same as for TF32 (16 channels of 4 bytes).
-Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool allow_compact = true)
+Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool allow_compact = true, bool virt = false)
 {
     Plan p{};
     p.ok = false;
+    Shape sh = shape;                                      // (virtual images: the extents of the virtual plane)
+    const int st = sh.stride;
+    if (st > 1 && !virt) return p;
+    p.phases = p.phase_cols = 1;
+    if (virt) {
+        if (b16) return p;
+        p.virt = 1;
+        p.off_h = sh.pad_h;
+        if (st == 1) {
+            // zeros to the left of a row serve the row before as well; a multiple of four keeps quads of the image aligned
+            p.off_w = sh.W % 4 == 0 ? (sh.pad_w + 3) / 4 * 4 : sh.pad_w;
+            p.shift0 = p.off_w - sh.pad_w;
+            p.virt_h = sh.H + sh.pad_h > sh.P ? sh.H + sh.pad_h : sh.P;
+            p.virt_w = sh.W + p.off_w > sh.Q ? sh.W + p.off_w : sh.Q;
+        } else {
+            p.off_w = sh.pad_w;
+            p.virt_h = sh.P + (sh.R + st - 1) / st - 1;
+            p.virt_w = sh.Q + (sh.S + st - 1) / st - 1;
+            p.phase_cols = st < sh.S ? st : sh.S;
+            p.phases = p.phase_cols * (st < sh.R ? st : sh.R);
+        }
+        // outputs that can be stored as quads or pairs start on such a column of the accumulators, too
+        const int unit = (st == 1 && sh.W % 4 == 0) || (sh.Q % 4 == 0 && (long long)sh.P * sh.Q % 4 == 0) ? 4 : (sh.Q % 2 == 0 && (long long)sh.P * sh.Q % 2 == 0 ? 2 : 1);
+        p.virt_w = (p.virt_w + unit - 1) / unit * unit;
+        if ((long long)p.virt_h * p.virt_w >= 1LL << 30) return p;
+        sh.H = p.virt_h;
+        sh.W = p.virt_w;
+        sh.pad_h = sh.pad_w = 0;
+        if (sh.R * sh.S > kMaxTaps) return p;
+    }
     const long long total_pix = (long long)sh.N * sh.H * sh.W;
     if (total_pix >= (1LL << 31) - (1LL << 20)) return p;     // flat pixel indices stay within int32
     const int kp16 = (sh.K + 15) / 16 * 16;
@@ -130,7 +165,7 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
     p.fold_r = p.fold_s = 1;
     const bool padded = sh.pad_h != 0 || sh.pad_w != 0;      // needs patch addressing: no folding, filters as M
     if (padded && !p.swap) return p;
-    const int fold_mode = padded ? 0 : env_int("CONV2D_B200_TF32_FOLD", 1);
+    const int fold_mode = padded || virt ? 0 : env_int("CONV2D_B200_TF32_FOLD", 1);
     if (sh.C < cbc && (fold_mode == 2 || (fold_mode == 1 && sh.C <= 3))) {
         long long best = (long long)sh.R * sh.S * ((sh.C + cbc - 1) / cbc);
         const int cand[3][2] = {{1, sh.S}, {sh.R, 1}, {sh.R, sh.S}};
@@ -142,8 +177,22 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
         }
     }
     const int c_eff = sh.C * p.fold_r * p.fold_s;
-    const int r_eff = sh.R / p.fold_r, s_eff = sh.S / p.fold_s;
+    const int r_eff = st > 1 ? (sh.R + st - 1) / st : sh.R / p.fold_r, s_eff = st > 1 ? (sh.S + st - 1) / st : sh.S / p.fold_s;
     p.cblks = (c_eff + cbc - 1) / cbc;
+    if (st > 1) {
+        // Channel blocks: all phases of a 16-channel block after one another, each with its own taps -- or, with few
+        // channels, the phases of every channel as staged channels with all ceil(R/st) x ceil(S/st) taps (zero filters
+        // where a phase has none), where that takes fewer MMAs: 3 channels, 7 x 7, stride 2: 16 pairs instead of 49.
+        const long long apart = (long long)p.cblks * sh.R * sh.S;
+        const long long together = ((long long)sh.C * st * st + cbc - 1) / cbc * r_eff * s_eff;
+        if (together < apart) {
+            p.mixed = 1;
+            p.phases = p.phase_cols = 1;
+            p.cblks = (int)(((long long)sh.C * st * st + cbc - 1) / cbc);
+        } else {
+            p.cblks *= p.phases;
+        }
+    }
     // Stacked taps.  With at most 64 filters an M = 64 instruction runs the tensor pipe at half its rate.  Instead
     // half of the rows of an M = 128 operand hold the filters' tap (r, s) and the other half their tap (r, s + 1),
     // both multiplied with the pixels shifted for (r, s): the accumulator row of tap (r, s + 1), column j + 1, then
@@ -158,7 +207,7 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
     // 24.3 -> 20.8 us; 64 channels 3 x 3 on 56 x 56 (36 pairs): 27.6 -> 30.6 us.  Hence from 48 (tap, channel block)
     // pairs on.  CONV2D_B200_TF32_PAIR_TAPS = 0 / 2: never / whenever possible.
     const int pair_mode = env_int("CONV2D_B200_TF32_PAIR_TAPS", 1);
-    p.pair_taps = (p.swap && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
+    p.pair_taps = (p.swap && st == 1 && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
                    (pair_mode == 2 || (long long)r_eff * s_eff * p.cblks >= 48)) ? 1 : 0;
     // Compact stacking for banks that can stay in shared memory: pairs of taps as 128-row slices, the lone last tap of
     // an odd filter row as a 64-row slice that an M = 64 instruction adds onto the same accumulator lanes.  The bank
@@ -171,7 +220,7 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
     p.pair_compact = 0;
     const size_t compact_cb_bytes = (size_t)r_eff * ((s_eff / 2) * 128 + (s_eff & 1) * 64) * kCB * 4;
     if (allow_compact && !p.pair_taps && p.swap && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
-        !padded && (size_t)((c_eff + cbc - 1) / cbc) * compact_cb_bytes <= 152 * 1024 && env_int("CONV2D_B200_TF32_PAIR_COMPACT", 0) != 0) {
+        !padded && !virt && (size_t)((c_eff + cbc - 1) / cbc) * compact_cb_bytes <= 152 * 1024 && env_int("CONV2D_B200_TF32_PAIR_COMPACT", 0) != 0) {
         p.pair_taps = 1;
         p.pair_compact = 1;
     }
@@ -185,8 +234,8 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
     // first patch_tw produce outputs), whose halo is (R-1) patch rows.  The patch width with the least staged
     // pixels per output wins.
     p.patch_w = p.patch_tw = p.patch_rows = p.patch_cols = 0;
-    const long long flat_halo = (long long)(r_eff - 1) * sh.W + (s_eff - 1);
-    const int patch_mode = padded ? 2 : env_int("CONV2D_B200_TF32_PATCH", 1);       // 0 never, 1 when the flat halo is large, 2 always
+    const long long flat_halo = (long long)(r_eff - 1) * sh.W + (s_eff - 1) + p.shift0;
+    const int patch_mode = virt ? 0 : padded ? 2 : env_int("CONV2D_B200_TF32_PATCH", 1);       // 0 never, 1 when the flat halo is large, 2 always
     if (p.swap && p.fold_r * p.fold_s == 1 && patch_mode != 0) {
         double best_ratio = 0;
         const int forced_wp = want_patch_w ? want_patch_w : env_int("CONV2D_B200_TF32_PATCH_W", 0);
@@ -204,8 +253,10 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
         // 7 x 7 on 224 x 224, 4.2 vs 2.2, 20 % faster in patches).
         const double flat_ratio = (448.0 + flat_halo) / 448.0 * ((double)sh.H * sh.W) / ((double)sh.P * sh.Q);
         if (patch_mode == 1 && !(flat_ratio > 1.75 * best_ratio)) p.patch_w = p.patch_tw = 0;
+        p.staged_ratio = best_ratio;
         if (p.patch_w) p.patch_cols = (sh.Q + p.patch_tw - 1) / p.patch_tw;
     }
+    if (virt) p.staged_ratio = (448.0 + flat_halo) / 448.0 * ((double)sh.H * sh.W) / ((double)sh.P * sh.Q);
     if (padded && !p.patch_w) return p;
     p.ovl = (p.pair_taps && !p.patch_w) ? 4 : 0;
     const long long halo = p.patch_w ? (long long)(r_eff - 1) * p.patch_w + (s_eff - 1) : flat_halo;
@@ -221,8 +272,10 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
     const int sms = sm_count();
 
     const int forced_mt = env_int("CONV2D_B200_TF32_MT", 0);      // benchmark ablations only
-    p.cb_bytes = p.pair_compact ? compact_cb_bytes : (size_t)p.taps * chunk;
-    const size_t wbytes = (size_t)p.cblks * p.cb_bytes;            // re-ordered filters of one filter block
+    p.cb_bytes = p.pair_compact ? compact_cb_bytes : (p.phases > 1 ? (size_t)sh.R * sh.S : (size_t)p.taps) * chunk;
+    p.pairs = p.phases > 1 ? (long long)(p.cblks / p.phases) * sh.R * sh.S : (long long)p.taps * p.cblks;
+    const size_t wbytes = (size_t)(p.cblks / p.phases) * p.cb_bytes;   // re-ordered filters of one filter block
+    p.bank_bytes = wbytes;
     auto npix_of = [&](int tile_px) { return (int)(((long long)tile_px + halo + 7) / 8 * 8); };
 
     // Light problems (1x1-like: few taps x channel blocks) with a small filter bank keep it resident in
@@ -234,7 +287,7 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
     p.resident = 0;
     const int resident_mode = env_int("CONV2D_B200_TF32_RESIDENT", 2);      // 0 never, 1 light problems only, 2 whenever it fits
     if (resident_mode != 0 && p.n_blocks == 1 && wbytes <= 152 * 1024 &&
-        ((long long)p.taps * p.cblks <= 16 || resident_mode == 2)) {
+        (p.pairs <= 16 || resident_mode == 2)) {
         const int mt = forced_mt ? forced_mt : (p.swap ? 2 : 1);
         int res_px = mt * kTileM;
         if (p.swap && !p.patch_w && !forced_mt) {
@@ -295,7 +348,7 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
                 const long long rounds = (items + sms - 1) / sms;
                 const int nbuf = 2 * px <= 512 ? 2 : 1;
                 const double mma_step = groups * ((px / groups) / 2.0 > 64.0 ? (px / groups) / 2.0 : 64.0);
-                const double tile_time = (double)p.taps * p.cblks * (2 * mma_step + stage_cycles);
+                const double tile_time = (double)p.pairs * (2 * mma_step + stage_cycles);
                 const double writeback = (nbuf == 1 ? 1.0 : 0.15) * (px / 128.0) * (3000.0 * p.n_tile / 128.0);
                 double cost = rounds * (tile_time + 0.5 * writeback);
                 // With one accumulator set the MMAs of an item wait for the whole write-back of the item before it
@@ -318,7 +371,7 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
                 const long long items = (tiles + mt - 1) / mt * p.n_blocks;
                 const long long rounds = (items + sms - 1) / sms;
                 const int nbuf = (2 * mt * set_cols <= 512) ? 2 : 1;
-                const double tile_time = (double)p.taps * p.cblks * (mt * 2 * mma_cycles + stage_cycles);
+                const double tile_time = (double)p.pairs * (mt * 2 * mma_cycles + stage_cycles);
                 const double writeback = (nbuf == 1 ? 1.0 : 0.15) * mt * (3000.0 * p.n_tile / 128.0);
                 const double cost = rounds * (tile_time + 0.5 * writeback);
                 if (best_px == 0 || cost < best_cost) { best_px = mt * kTileM; best_cost = cost; }
@@ -392,7 +445,7 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
     int cols = p.nbuf * item_cols;
     p.tmem_cols = 32;
     while (p.tmem_cols < cols) p.tmem_cols <<= 1;
-    p.makespan = (double)((items + sms - 1) / sms) * p.tile_px * p.taps * p.cblks;
+    p.makespan = (double)((items + sms - 1) / sms) * p.tile_px * p.pairs;
     p.ok = true;
     return p;
 }
@@ -404,7 +457,14 @@ Plan plan_with_patch_width(const Shape& sh, bool b16, int want_patch_w, bool all
 // where both take two rounds of equal items).
 Plan make_plan(const Shape& sh, bool b16 = false)
 {
+    if (sh.stride > 1) return plan_with_patch_width(sh, b16, 0, true, true);
     Plan best = plan_with_patch_width(sh, b16, 0);
+    if (sh.pad_h != 0 || sh.pad_w != 0) {
+        // Padding: virtual images, unless their rows are so wide that patches stage far fewer pixels.
+        const int mode = env_int("CONV2D_B200_TF32_VIRT", 1);             // 0 never, 1 by the rule, 2 always
+        const Plan v = plan_with_patch_width(sh, b16, 0, true, true);
+        if (v.ok && mode != 0 && (mode == 2 || !best.ok || !(v.staged_ratio > 1.75 * best.staged_ratio))) return v;
+    }
     if (!best.ok || !best.patch_w || env_int("CONV2D_B200_TF32_PATCH_W", 0) != 0) return best;
     const int first = best.patch_w;
     for (int wp = 32; wp <= 128; wp *= 2) {
@@ -417,7 +477,7 @@ Plan make_plan(const Shape& sh, bool b16 = false)
 
 size_t packed_floats(const Plan& p)
 {
-    return (size_t)p.n_blocks * p.cblks * (p.cb_bytes / 4);
+    return (size_t)p.n_blocks * (p.bank_bytes / 4);
 }
 
 }  // namespace

@@ -13,11 +13,18 @@ using namespace ptx;
 // wp[nb][cb][t][chunk][f][e] = tf32(w[nb*n_tile + f][cb*kCB + 4*chunk + e][t]), zero outside K, C.
 // With folded taps, channel index vc = (c*fold_r + r_in)*fold_s + s_in and tap index t = r_out*(S/fold_s) + s_out
 // stand for filter element w[k][c][r_out*fold_r + r_in][s_out*fold_s + s_in].
+// With a stride (st > 1) staged channel vc = (c, a, b) and tap t = (r2, s2) stand for element [st*r2 + a][st*s2 + b].
 struct FoldedFilter {
-    int C, R, S, fold_r, fold_s;
+    int C, R, S, fold_r, fold_s, st;
     // offset of that element inside filter k's C*R*S block, or -1 for channel padding
     __device__ __forceinline__ int offset(int vc, int t) const
     {
+        if (st > 1) {
+            const int c = vc / (st * st), ph = vc - c * st * st;
+            const int s_eff = (S + st - 1) / st, r2 = t / s_eff;
+            const int r = r2 * st + ph / st, s = (t - r2 * s_eff) * st + ph % st;
+            return r < R && s < S ? (c * R + r) * S + s : -1;
+        }
         const int frs = fold_r * fold_s;
         const int c = vc / frs, rem = vc - c * frs;
         if (c >= C) return -1;
@@ -44,7 +51,7 @@ __global__ void repack_filters_kernel(const T* __restrict__ w, T* __restrict__ w
     grid_dep_launch();      // the convolution kernel may set itself up while this one runs
     // the status block in front of the filters starts every (non-prepacked) call cleared
     if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / sizeof(unsigned)) status[threadIdx.x] = 0u;
-    const bool folded = ff.fold_r * ff.fold_s > 1;
+    const bool folded = ff.fold_r * ff.fold_s > 1 || ff.st > 1;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < threads_total; i += stride) {
         long long r = i;
@@ -63,8 +70,8 @@ __global__ void repack_filters_kernel(const T* __restrict__ w, T* __restrict__ w
         const T* src = w + (size_t)k * ff.C * ff.R * ff.S;
         T* dst = wp + ((((size_t)nb * cblks + cb) * taps * kChunks + chunk) * n_tile + f) * EPC + e;
         const size_t tap_stride = (size_t)kChunks * n_tile * EPC;
-        const bool live = k < K && (folded ? vc < ff.C * ff.fold_r * ff.fold_s : vc < ff.C);
-        if (stacked == 2) {
+        const bool live = k < K && (folded ? vc < ff.C * ff.fold_r * ff.fold_s * ff.st * ff.st : vc < ff.C);
+        if (stacked == 2) {                                // (one row of blocks)
             // compact bank of one filter block: per filter row `pairs` slices of 128 rows, then the lone tap's 64 rows
             const int pairs = ff.S / 2, odd = ff.S & 1;
             const size_t row_elems = (size_t)(pairs * n_tile + odd * (n_tile / 2)) * kChunks * EPC;
@@ -90,7 +97,8 @@ __global__ void repack_filters_kernel(const T* __restrict__ w, T* __restrict__ w
             }
             continue;
         }
-        for (int t = 0; t < taps; ++t, dst += tap_stride) {
+        dst += blockIdx.y * tap_stride;                    // (the taps are shared out over the grid's second dimension)
+        for (int t = blockIdx.y; t < taps; t += gridDim.y, dst += gridDim.y * tap_stride) {
             T v = T(0);
             if (live) {
                 int o = folded ? ff.offset(vc, t) : vc * taps + t;
@@ -108,12 +116,12 @@ __global__ void repack_filters_kernel(const T* __restrict__ w, T* __restrict__ w
     }
 }
 
-// Re-ordering through shared memory for unfolded filters: a block takes 8 filters x one channel block x all
+// Re-ordering through shared memory for unfolded filters (taps: all R x S of them, also with a stride): a block takes 8 filters x one channel block x all
 // taps.  Its reads are runs of (channels per block) x taps contiguous elements per filter, its writes runs of
 // 8 filters x EPC elements (128 bytes with fp32) per (tap, chunk): both sides coalesced.
 template <typename T, int EPC>
 __global__ void repack_filters_tiled_kernel(const T* __restrict__ w, T* __restrict__ wp, unsigned* __restrict__ status,
-                                            int K, int C, int taps, int n_tile, int cblks)
+                                            int K, int C, int taps, int n_tile, int cblks, int S, int st)
 {
     extern __shared__ __align__(16) unsigned char repack_smem[];
     T* tile = reinterpret_cast<T*>(repack_smem);                 // [8][cpb * taps]
@@ -173,7 +181,13 @@ __global__ void repack_filters_tiled_kernel(const T* __restrict__ w, T* __restri
             v = make_uint4((unsigned)u[0] | ((unsigned)u[1] << 16), (unsigned)u[2 % EPC] | ((unsigned)u[3 % EPC] << 16),
                            (unsigned)u[4 % EPC] | ((unsigned)u[5 % EPC] << 16), (unsigned)u[6 % EPC] | ((unsigned)u[7 % EPC] << 16));
         }
-        *reinterpret_cast<uint4*>(dst + (((size_t)t * kChunks + chunk) * n_tile + f0 + kk) * EPC) = v;
+        int tt = t;                                       // place of the tap in the bank
+        if (st > 1) {                                     // grouped by phase (r % st, s % st), see phase_of
+            const int r = t / S, s = t - r * S, R = taps / S, pa = r % st, pb = s % st;
+            const int rows = (R - pa + st - 1) / st, cols = (S - pb + st - 1) / st;
+            tt = (pa * (R / st) + min(pa, R % st)) * S + rows * (pb * (S / st) + min(pb, S % st)) + (r / st) * cols + s / st;
+        }
+        *reinterpret_cast<uint4*>(dst + (((size_t)tt * kChunks + chunk) * n_tile + f0 + kk) * EPC) = v;
     }
 }
 
