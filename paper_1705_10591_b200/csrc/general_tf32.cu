@@ -141,7 +141,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
 
     if (!weights_packed) {
         const long long total = (long long)packed_floats(p);
-        const FoldedFilter ff{sh.C, sh.R, sh.S, p.fold_r, p.fold_s, p.mixed ? sh.stride : 1};
+        const FoldedFilter ff{sh.C, sh.R, sh.S, p.fold_r, p.fold_s, p.mixed ? sh.stride : 1, p.ext};
         const long long lanes = (long long)p.n_blocks * p.cblks * kChunks * p.n_tile * (b16 ? 8 : 4);   // one thread per element of a tap's slice
         long long blocks = (lanes + 255) / 256;
         if (blocks > sm_count() * 16LL) blocks = sm_count() * 16LL;
@@ -163,10 +163,10 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
             if (b16)
                 repack_filters_tiled_kernel<unsigned short, 8><<<grid, threads, tile_bytes, stream>>>(
                     static_cast<const unsigned short*>(w_any), reinterpret_cast<unsigned short*>(wp), status, sh.K, sh.C,
-                    all_taps, p.n_tile, bank_blocks, sh.S, 1);
+                    all_taps, p.n_tile, bank_blocks, sh.S, 1, 0);
             else
                 repack_filters_tiled_kernel<float, 4><<<grid, threads, tile_bytes, stream>>>(w, wp, status, sh.K, sh.C, all_taps,
-                                                                                             p.n_tile, bank_blocks, sh.S, p.phases > 1 ? sh.stride : 1);
+                                                                                             p.n_tile, bank_blocks, sh.S, p.phases > 1 ? sh.stride : 1, p.ext);
         } else if (b16)
             repack_filters_kernel<unsigned short, 8><<<dim3((unsigned)blocks, tap_rows), 256, 0, stream>>>(
                 static_cast<const unsigned short*>(w_any), reinterpret_cast<unsigned short*>(wp), status, sh.K, ff,
@@ -208,7 +208,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     a.HW = sh.H * sh.W;
     const int plan_h = p.virt ? p.virt_h : sh.H, plan_w = p.virt ? p.virt_w : sh.W;       // rows and columns of the flat pixel sequence
     a.total_pix = sh.N * plan_h * plan_w;
-    a.st = sh.stride; a.off_h = p.off_h; a.off_w = p.off_w; a.shift0 = p.shift0;
+    a.st = sh.stride; a.off_h = p.off_h; a.off_w = p.off_w; a.shift0 = p.shift0; a.ext = p.ext; a.quad2 = p.quad2;
     a.phases = p.phases; a.phase_cols = p.phase_cols; a.cblks_c = p.cblks / p.phases; a.div_phases = FastDiv(p.phases);
     a.mixed = p.mixed; a.mix_c = sh.C; a.mix_st2 = sh.stride * sh.stride;
     a.n_tile = p.n_tile; a.n_blocks = p.n_blocks; a.mt = p.mt; a.tile_px = p.tile_px; a.px_groups = p.px_groups; a.nbuf = p.nbuf; a.npix = p.npix; a.cstride = chunk_stride(p.npix);
@@ -223,7 +223,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     a.pair_compact = p.pair_compact; a.cb_bytes = (int)p.cb_bytes;
     a.pair_taps = p.pair_taps; a.s_slots = p.s_slots; a.s_step = p.pair_taps ? 2 : 1; a.item_stride = p.tile_px - p.ovl;
     a.div_HW = FastDiv(plan_h * plan_w); a.div_W = FastDiv(plan_w); a.div_npix = FastDiv(p.npix);
-    a.div_qn = FastDiv(p.npix / 4 > 0 ? p.npix / 4 : 1); a.div_patch_w = FastDiv(p.patch_w ? p.patch_w : 1);
+    a.div_qn = FastDiv(p.quad2 ? p.npix / 2 : (p.npix / 4 > 0 ? p.npix / 4 : 1)); a.div_patch_w = FastDiv(p.patch_w ? p.patch_w : 1);
     a.xchg_slots = p.xchg_slots;
     a.xchg_bytes = (int)xchg_area_bytes(p.xchg_slots);
     // (the helper warps of the last item's write-back: measured no gain for the two-block cluster, whose single item
@@ -233,8 +233,8 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     a.quad = ((p.virt ? (sh.stride == 1 && sh.W % 4 == 0) : p.patch_w ? (sh.W % 4 == 0 && sh.pad_w % 4 == 0) : (sh.H * sh.W) % 4 == 0) && p.fold_r * p.fold_s == 1 && env_int("CONV2D_B200_TF32_QUAD", 1) != 0) ? 1 : 0;
     {
         // as many producer groups as can each still cover a stage in one pass (one memory round trip)
-        const long long per_pass = a.quad ? kProducers : (long long)kProducers * kUnitsPerThread;
-        const long long stage_work = (long long)(a.quad ? p.npix / 4 : p.npix) * p.cbg;
+        const long long per_pass = a.quad || p.quad2 ? kProducers : (long long)kProducers * kUnitsPerThread;
+        const long long stage_work = p.quad2 ? (long long)(p.npix / 2) * (p.mixed ? p.cbg : p.cbg / 2) : (long long)(a.quad ? p.npix / 4 : p.npix) * p.cbg;
         int g = 1;
         while (g < 4 && g * 2 <= p.a_stages && stage_work * (g * 2) <= per_pass) g *= 2;
         a.pgroups = env_int("CONV2D_B200_TF32_PGROUPS", g);

@@ -56,6 +56,7 @@ struct KernelArgs {
     int fold_r, fold_s;  // taps folded into the channel dimension (1, 1: none); R, S below are what is left as shifts
     int helpers;      // 1: warps 8-15 share the write-back of a block's last item (operand-swap layout only)
     int pgroups;      // producer groups (1, 2 or 4): stage k is filled by group k % pgroups
+    int quad2;        // 1: stride 2, producers load four adjacent pixels (two virtual pixels of both phases of a row) per word
     int quad;         // producers load four adjacent pixels per 128-bit (fp32) or 64-bit (16-bit operands) word (needs H*W % 4 == 0)
     int pair;         // 16-bit operands only: producers load two adjacent pixels per 32-bit word (needs H*W even)
     int cbg, groups;        // channel blocks per activation stage, number of such groups
@@ -78,7 +79,7 @@ struct KernelArgs {
     // Virtual images (VIRT kernels): zero padding and strides, see staged_pixel_virtual.  H, W, HW are those of the image
     // in memory; div_HW and div_W divide by the virtual plane and row, total_pix counts virtual pixels.
     int st, off_h, off_w;   // stride; rows and columns of zeros before the image in the virtual one (before the stride)
-    int shift0;             // staged pixels between an output and its tap (0, 0)
+    int shift0, ext;        // staged pixels between an output and its first tap; columns by which the taps start later in their phases
     int phases, phase_cols; // phases with taps of their own (1 where the taps are the same for all channels); columns of them
     int cblks_c;            // 16-channel blocks of one phase
     int mixed;              // 1: the phases of a channel are adjacent staged channels (few input channels), every tap for all
@@ -145,6 +146,7 @@ __device__ __forceinline__ bool output_pixel(const KernelArgs& a, const ItemGeom
 struct Phase {
     int cblk, a, b;         // channel block of the image, phase
     int taps, cols;         // its taps, and how many of them lie in a row
+    int col0;               // virtual columns before the first of them
     int base;               // taps of the phases before it
 };
 __device__ __forceinline__ Phase phase_of(const KernelArgs& a, int cb)
@@ -155,9 +157,12 @@ __device__ __forceinline__ Phase phase_of(const KernelArgs& a, int cb)
     p.a = idx / a.phase_cols;
     p.b = idx - p.a * a.phase_cols;
     const int rows = (a.R - p.a + a.st - 1) / a.st;
-    p.cols = (a.S - p.b + a.st - 1) / a.st;
+    p.col0 = p.b < a.ext ? 1 : 0;
+    p.cols = (a.S + a.ext - p.b + a.st - 1) / a.st - p.col0;
     p.taps = rows * p.cols;
-    const int rows_before = p.a * (a.R / a.st) + min(p.a, a.R % a.st), cols_before = p.b * (a.S / a.st) + min(p.b, a.S % a.st);
+    const int end = a.S + a.ext;                                  // (taps in columns ext .. end - 1)
+    const int rows_before = p.a * (a.R / a.st) + min(p.a, a.R % a.st);
+    const int cols_before = p.b * (end / a.st) + min(p.b, end % a.st) - min(p.b, a.ext);
     p.base = rows_before * a.S + rows * cols_before;
     return p;
 }
@@ -426,9 +431,9 @@ general_tc_kernel(const KernelArgs a)
     if (VIRT && a.phases > 1) {
         // one table per phase, behind one another in the order of the filter bank
         for (int t = tid; t < a.R * a.S; t += kThreads) {
-            const int r = t / a.S, sx = t - r * a.S, r2 = r / a.st, s2 = sx / a.st;
+            const int r = t / a.S, sx = t - r * a.S + a.ext, r2 = r / a.st, s2 = sx / a.st;
             const Phase p = phase_of(a, (r - r2 * a.st) * a.phase_cols + sx - s2 * a.st);
-            tap_shift[p.base + r2 * p.cols + s2] = (uint32_t)(r2 * a.row_pitch + s2);
+            tap_shift[p.base + r2 * p.cols + s2 - p.col0] = (uint32_t)(r2 * a.row_pitch + s2);
         }
     } else
     for (int t = tid; t < a.taps; t += kThreads)
@@ -589,11 +594,11 @@ general_tc_kernel(const KernelArgs a)
                         if (gr * a.cbg + g >= a.cblks) break;
                         uint32_t row_shift = VIRT ? (uint32_t)a.shift0 : 0u;     // r * row pitch, in pixels (= 16-byte units)
                         int sx = 0, sc = 0;
-                        int taps = a.taps, s_slots = a.s_slots, tap0 = 0;
+                        int taps = a.taps, s_slots = a.s_slots, tap0 = 0, sx0 = 0;
                         size_t bank_at = (size_t)(gr * a.cbg + g) * a.cb_bytes;   // (resident filters)
                         if (VIRT && a.phases > 1) {
                             const Phase p = phase_of(a, gr * a.cbg + g);
-                            taps = p.taps; s_slots = p.cols; tap0 = p.base;
+                            taps = p.taps; s_slots = p.cols; tap0 = p.base; sx0 = sx = p.col0;
                             bank_at = (size_t)p.cblk * a.cb_bytes + (size_t)p.base * b_chunk_bytes;
                         }
                         for (int t0 = 0; t0 < taps; t0 += a.tps) {
@@ -660,7 +665,7 @@ general_tc_kernel(const KernelArgs a)
                                     }
                                     accumulate = 1;
                                     sx += a.s_step;
-                                    if (++sc == s_slots) { sc = 0; sx = 0; row_shift += (uint32_t)a.row_pitch; }
+                                    if (++sc == s_slots) { sc = 0; sx = sx0; row_shift += (uint32_t)a.row_pitch; }
                                 }
                             }
                             if (!a.resident) {
@@ -724,7 +729,60 @@ general_tc_kernel(const KernelArgs a)
                 int gr = grp + ii.rot;
                 if (gr >= ii.n_groups) gr -= ii.n_groups;
                 gr += ii.g_begin;
-                if (!B16 && !FOLD && a.quad) {
+                if (VIRT && a.quad2) {
+                    // Stride 2: four adjacent pixels of an image row are two virtual pixels of both phases of that row.
+                    const int qn = a.npix >> 1;
+                    const int c_step = a.mixed ? 1 : 2;                  // staged channel blocks of a unit
+                    for (int i = wtid; i * c_step < qn * a.cbg; i += nthr) {
+                        int pq;
+                        const int g = a.div_qn.divmod(i, pq) * c_step, cb = gr * a.cbg + g;
+                        float4 v[kCB];
+#pragma unroll
+                        for (int e = 0; e < kCB; ++e) v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        int n, h, wc;
+                        const bool in = staged_pixel_virtual(a, ii.geom, 2 * pq, n, h, wc) && (unsigned)wc < (unsigned)a.W && cb < a.cblks;
+                        float4* d = dst + (size_t)g * kChunks * a.cstride + 2 * pq;
+                        if (a.mixed) {
+                            // a chunk holds the four phases of a channel: two rows of the image
+                            const int c0 = cb * kChunks;
+                            if (in) {
+                                const float* src = a.x + ((size_t)n * a.C + c0) * a.HW + h * a.W + wc;
+#pragma unroll
+                                for (int c = 0; c < kChunks; ++c) {
+                                    if (c0 + c >= a.C) break;
+                                    if ((unsigned)h < (unsigned)a.H) v[2 * c] = __ldg(reinterpret_cast<const float4*>(src + (size_t)c * a.HW));
+                                    if ((unsigned)(h + 1) < (unsigned)a.H) v[2 * c + 1] = __ldg(reinterpret_cast<const float4*>(src + (size_t)c * a.HW + a.W));
+                                }
+                            }
+#pragma unroll
+                            for (int c = 0; c < kChunks; ++c) {
+                                const float4 r0 = v[2 * c], r1 = v[2 * c + 1];
+                                d[c * a.cstride] = make_float4(to_tf32_rna(r0.x), to_tf32_rna(r0.y), to_tf32_rna(r1.x), to_tf32_rna(r1.y));
+                                d[c * a.cstride + 1] = make_float4(to_tf32_rna(r0.z), to_tf32_rna(r0.w), to_tf32_rna(r1.z), to_tf32_rna(r1.w));
+                            }
+                        } else {
+                            const Phase p = phase_of(a, cb);
+                            const int c0 = p.cblk * kCB;
+                            h += p.a;
+                            if (in && (unsigned)h < (unsigned)a.H) {
+                                const float* src = a.x + ((size_t)n * a.C + c0) * a.HW + h * a.W + wc;
+#pragma unroll
+                                for (int e = 0; e < kCB; ++e)
+                                    if (c0 + e < a.C) v[e] = __ldg(reinterpret_cast<const float4*>(src + (size_t)e * a.HW));
+                            }
+#pragma unroll
+                            for (int ch = 0; ch < kChunks; ++ch) {
+                                float4* dc = d + ch * a.cstride;
+                                const float4 v0 = v[4 * ch], v1 = v[4 * ch + 1], v2 = v[4 * ch + 2], v3 = v[4 * ch + 3];
+                                dc[0] = make_float4(to_tf32_rna(v0.x), to_tf32_rna(v1.x), to_tf32_rna(v2.x), to_tf32_rna(v3.x));
+                                dc[1] = make_float4(to_tf32_rna(v0.z), to_tf32_rna(v1.z), to_tf32_rna(v2.z), to_tf32_rna(v3.z));
+                                dc += kChunks * a.cstride;                     // the block of the phase one column to the right
+                                dc[0] = make_float4(to_tf32_rna(v0.y), to_tf32_rna(v1.y), to_tf32_rna(v2.y), to_tf32_rna(v3.y));
+                                dc[1] = make_float4(to_tf32_rna(v0.w), to_tf32_rna(v1.w), to_tf32_rna(v2.w), to_tf32_rna(v3.w));
+                            }
+                        }
+                    }
+                } else if (!B16 && !FOLD && a.quad) {
                     // H*W a multiple of 4: a thread fetches 4 adjacent pixels of each of the 16 channels with
                     // 128-bit loads (a quarter of the load instructions, which otherwise crowd the SM's memory
                     // pipeline that the MMA instructions pass through as well) and writes four 16-channel units.

@@ -77,7 +77,7 @@ struct Plan {
     int grid;
     size_t smem_bytes;
     int virt;         // 1: virtual images (zero padding, strides)
-    int virt_h, virt_w, off_h, off_w, shift0, phases, phase_cols, mixed;     // see KernelArgs
+    int virt_h, virt_w, off_h, off_w, shift0, ext, phases, phase_cols, mixed, quad2;     // see KernelArgs
     long long pairs;  // (tap, channel block) pairs of a filter block
     size_t bank_bytes;   // re-ordered filters of one filter block
     double staged_ratio; // staged pixels per output of a 448-pixel item
@@ -119,14 +119,20 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
             p.virt_h = sh.H + sh.pad_h > sh.P ? sh.H + sh.pad_h : sh.P;
             p.virt_w = sh.W + p.off_w > sh.Q ? sh.W + p.off_w : sh.Q;
         } else {
-            p.off_w = sh.pad_w;
+            // Stride 2 with whole quads of columns: the zeros in front of a row are a multiple of four columns, so that four
+            // adjacent pixels of the image are two virtual pixels of both phases of a row.  The taps then start `ext`
+            // columns into their phases, and `shift0` virtual pixels further on.
+            p.quad2 = st == 2 && sh.W % 4 == 0 && sh.S >= 2 && sh.R >= 2 && env_int("CONV2D_B200_TF32_QUAD", 1) != 0 ? 1 : 0;
+            p.off_w = p.quad2 ? (sh.pad_w + 3) / 4 * 4 : sh.pad_w;
+            p.ext = (p.off_w - sh.pad_w) % st;
+            p.shift0 = (p.off_w - sh.pad_w) / st;
             p.virt_h = sh.P + (sh.R + st - 1) / st - 1;
-            p.virt_w = sh.Q + (sh.S + st - 1) / st - 1;
+            p.virt_w = sh.Q + p.shift0 + (sh.S + p.ext + st - 1) / st - 1;
             p.phase_cols = st < sh.S ? st : sh.S;
             p.phases = p.phase_cols * (st < sh.R ? st : sh.R);
         }
         // outputs that can be stored as quads or pairs start on such a column of the accumulators, too
-        const int unit = (st == 1 && sh.W % 4 == 0) || (sh.Q % 4 == 0 && (long long)sh.P * sh.Q % 4 == 0) ? 4 : (sh.Q % 2 == 0 && (long long)sh.P * sh.Q % 2 == 0 ? 2 : 1);
+        const int unit = (st == 1 && sh.W % 4 == 0) || p.quad2 || (sh.Q % 4 == 0 && (long long)sh.P * sh.Q % 4 == 0) ? 4 : (sh.Q % 2 == 0 && (long long)sh.P * sh.Q % 2 == 0 ? 2 : 1);
         p.virt_w = (p.virt_w + unit - 1) / unit * unit;
         if ((long long)p.virt_h * p.virt_w >= 1LL << 30) return p;
         sh.H = p.virt_h;
@@ -177,7 +183,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         }
     }
     const int c_eff = sh.C * p.fold_r * p.fold_s;
-    const int r_eff = st > 1 ? (sh.R + st - 1) / st : sh.R / p.fold_r, s_eff = st > 1 ? (sh.S + st - 1) / st : sh.S / p.fold_s;
+    const int r_eff = st > 1 ? (sh.R + st - 1) / st : sh.R / p.fold_r, s_eff = st > 1 ? (sh.S + p.ext + st - 1) / st : sh.S / p.fold_s;
     p.cblks = (c_eff + cbc - 1) / cbc;
     if (st > 1) {
         // Channel blocks: all phases of a 16-channel block after one another, each with its own taps -- or, with few
@@ -188,6 +194,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         if (together < apart) {
             p.mixed = 1;
             p.phases = p.phase_cols = 1;
+            if (st != 2) p.quad2 = 0;
             p.cblks = (int)(((long long)sh.C * st * st + cbc - 1) / cbc);
         } else {
             p.cblks *= p.phases;
@@ -302,12 +309,12 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
             if (p.swap && want >= 64 && want <= (p.pair_compact ? 256 : 512) && want % 32 == 0 && pixel_items(want) > 0) res_px = want;
         }
         const int npix = npix_of(res_px);
-        if ((p.swap ? res_px : mt * set_cols) <= 512 && npix <= 16000 && wbytes + extra + (size_t)2 * kCB * chunk_stride(npix) * 4 + kBookBytes <= kSmemLimit) {
+        if ((p.swap ? res_px : mt * set_cols) <= 512 && npix <= 16000 && wbytes + extra + (size_t)2 * (p.quad2 && !p.mixed ? 2 : 1) * kCB * chunk_stride(npix) * 4 + kBookBytes <= kSmemLimit) {
             p.resident = 1;
             p.mt = p.swap ? (res_px + kTileM - 1) / kTileM : mt;
             p.tile_px = res_px;
             p.npix = npix;
-            p.cbg = 1;
+            p.cbg = p.quad2 && !p.mixed ? 2 : 1;                       // (both phases of a row of pixels in one stage)
             p.a_stages = 2;
             p.b_stages = 1;
             p.tps = p.taps;
@@ -327,6 +334,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         // second accumulator set (hidden write-back) and balance better.  Cost in units of one tile's MMA
         // time: rounds x mt x (1 + stage cost / MMA time) + exposed write-back.
         const size_t kLimit = kSmemLimit - extra;
+        const int stage_blocks = p.quad2 && !p.mixed ? 2 : 1;    // channel blocks of an activation stage
         const double stage_cycles = chunk / 66.0;           // one (tap, channel block) of filters through L2
         const int forced_px = env_int("CONV2D_B200_TF32_TILE_PX", 0);
         const bool ksplit_allowed = env_int("CONV2D_B200_TF32_KSPLIT", 1) != 0;
@@ -342,7 +350,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
                 const int groups = (px + 255) / 256;
                 if (px % (16 * groups)) continue;
                 const int npix = npix_of(px);
-                if (npix > 16000 || smem_need(2, npix, p.n_tile, 2, 1, 1) > kLimit) continue;
+                if (npix > 16000 || smem_need(2, npix, p.n_tile, 2, 1, stage_blocks) > kLimit) continue;
                 if (pixel_items(px) == 0) continue;
                 const long long items = pixel_items(px) * p.n_blocks;
                 const long long rounds = (items + sms - 1) / sms;
@@ -386,20 +394,21 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         // by varying the stage size) once per 16-48 MMAs; the ring should hold
         // 64-128 KB in flight to cover the L2 latency.
         p.a_stages = 2;
-        p.cbg = 1;
+        p.cbg = stage_blocks;
         p.tps = env_int("CONV2D_B200_TF32_STAGE_KB", 48) * 1024 / chunk;
         if (p.tps < 1) p.tps = 1;
         if (p.tps > p.taps) p.tps = p.taps;
         p.b_stages = 2;
-        while (p.tps > 1 && smem_need(p.a_stages, p.npix, p.n_tile, 3, p.tps, 1) > kLimit) --p.tps;
+        while (p.tps > 1 && smem_need(p.a_stages, p.npix, p.n_tile, 3, p.tps, p.cbg) > kLimit) --p.tps;
         // equal stages: 6 taps as 3 + 3 instead of 5 + 1 (the short stage's MMAs would end long before the next
         // long stage has arrived)
         {
             const int per_block = (p.taps + p.tps - 1) / p.tps;
             p.tps = (p.taps + per_block - 1) / per_block;
         }
-        while (p.b_stages < 4 && smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages + 1, p.tps, 1) <= kLimit) ++p.b_stages;
-        while (p.a_stages < kMaxAStages && p.taps <= 3 &&
+        while (p.b_stages < 4 && smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages + 1, p.tps, p.cbg) <= kLimit) ++p.b_stages;
+        // (few MMAs per stage: more stages have to be on their way)
+        while (p.a_stages < kMaxAStages && (p.taps <= 3 || st > 1) &&
                smem_need(p.a_stages + 1, p.npix, p.n_tile, p.b_stages, p.tps, p.cbg) <= kLimit - 32 * 1024) ++p.a_stages;
         while (p.b_stages < kMaxBStages && smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages + 1, p.tps, p.cbg) <= kLimit &&
                (size_t)p.b_stages * p.tps * chunk < 128 * 1024) ++p.b_stages;

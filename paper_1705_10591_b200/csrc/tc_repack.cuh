@@ -13,17 +13,17 @@ using namespace ptx;
 // wp[nb][cb][t][chunk][f][e] = tf32(w[nb*n_tile + f][cb*kCB + 4*chunk + e][t]), zero outside K, C.
 // With folded taps, channel index vc = (c*fold_r + r_in)*fold_s + s_in and tap index t = r_out*(S/fold_s) + s_out
 // stand for filter element w[k][c][r_out*fold_r + r_in][s_out*fold_s + s_in].
-// With a stride (st > 1) staged channel vc = (c, a, b) and tap t = (r2, s2) stand for element [st*r2 + a][st*s2 + b].
+// With a stride (st > 1) staged channel vc = (c, a, b) and tap t = (r2, s2) stand for element [st*r2 + a][st*s2 + b - ext].
 struct FoldedFilter {
-    int C, R, S, fold_r, fold_s, st;
+    int C, R, S, fold_r, fold_s, st, ext;
     // offset of that element inside filter k's C*R*S block, or -1 for channel padding
     __device__ __forceinline__ int offset(int vc, int t) const
     {
         if (st > 1) {
             const int c = vc / (st * st), ph = vc - c * st * st;
-            const int s_eff = (S + st - 1) / st, r2 = t / s_eff;
-            const int r = r2 * st + ph / st, s = (t - r2 * s_eff) * st + ph % st;
-            return r < R && s < S ? (c * R + r) * S + s : -1;
+            const int s_eff = (S + ext + st - 1) / st, r2 = t / s_eff;
+            const int r = r2 * st + ph / st, s = (t - r2 * s_eff) * st + ph % st - ext;
+            return r < R && s >= 0 && s < S ? (c * R + r) * S + s : -1;
         }
         const int frs = fold_r * fold_s;
         const int c = vc / frs, rem = vc - c * frs;
@@ -121,7 +121,7 @@ __global__ void repack_filters_kernel(const T* __restrict__ w, T* __restrict__ w
 // 8 filters x EPC elements (128 bytes with fp32) per (tap, chunk): both sides coalesced.
 template <typename T, int EPC>
 __global__ void repack_filters_tiled_kernel(const T* __restrict__ w, T* __restrict__ wp, unsigned* __restrict__ status,
-                                            int K, int C, int taps, int n_tile, int cblks, int S, int st)
+                                            int K, int C, int taps, int n_tile, int cblks, int S, int st, int ext)
 {
     extern __shared__ __align__(16) unsigned char repack_smem[];
     T* tile = reinterpret_cast<T*>(repack_smem);                 // [8][cpb * taps]
@@ -183,9 +183,11 @@ __global__ void repack_filters_tiled_kernel(const T* __restrict__ w, T* __restri
         }
         int tt = t;                                       // place of the tap in the bank
         if (st > 1) {                                     // grouped by phase (r % st, s % st), see phase_of
-            const int r = t / S, s = t - r * S, R = taps / S, pa = r % st, pb = s % st;
-            const int rows = (R - pa + st - 1) / st, cols = (S - pb + st - 1) / st;
-            tt = (pa * (R / st) + min(pa, R % st)) * S + rows * (pb * (S / st) + min(pb, S % st)) + (r / st) * cols + s / st;
+            const int r = t / S, s = t - r * S + ext, R = taps / S, pa = r % st, pb = s % st, end = S + ext;
+            const int first = pb < ext ? 1 : 0;
+            const int rows = (R - pa + st - 1) / st, cols = (end - pb + st - 1) / st - first;
+            tt = (pa * (R / st) + min(pa, R % st)) * S + rows * (pb * (end / st) + min(pb, end % st) - min(pb, ext))
+               + (r / st) * cols + s / st - first;
         }
         *reinterpret_cast<uint4*>(dst + (((size_t)tt * kChunks + chunk) * n_tile + f0 + kk) * EPC) = v;
     }
