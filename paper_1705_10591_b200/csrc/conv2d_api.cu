@@ -1,5 +1,6 @@
 // C-ABI boundary: argument validation, dispatch and the host-buffer convenience path.
 #include <atomic>
+#include <mutex>
 
 #include "common.cuh"
 
@@ -369,6 +370,96 @@ conv2d_status_t conv2d_fwd_general_noalloc(const float* x, const float* w, float
     return launch_general_tf32_noalloc(x, w, y, sh, wait != 0, static_cast<cudaStream_t>(cuda_stream));
 }
 
+// ---------------------------------------------------------------- host buffers
+namespace {
+// Streams and events of a call that copies in both directions at once.  Sets are kept between calls (making one costs tens
+// of microseconds), at most kKeptSets per device; a set serves one call at a time and goes back with nothing pending.
+constexpr int kMaxChunks = 5;
+constexpr int kKeptSets = 4;
+struct CopySet {
+    cudaStream_t in = nullptr, out = nullptr;
+    cudaEvent_t begin = nullptr, end = nullptr, arrived[kMaxChunks] = {}, done[kMaxChunks] = {};
+    bool make()
+    {
+        bool ok = cudaStreamCreateWithFlags(&in, cudaStreamNonBlocking) == cudaSuccess &&
+                  cudaStreamCreateWithFlags(&out, cudaStreamNonBlocking) == cudaSuccess;
+        auto event = [&](cudaEvent_t& e) { ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess; };
+        event(begin); event(end);
+        for (int i = 0; i < kMaxChunks; ++i) { event(arrived[i]); event(done[i]); }
+        if (!ok) destroy();
+        return ok;
+    }
+    void destroy()
+    {
+        for (int i = 0; i < kMaxChunks; ++i) { if (arrived[i]) cudaEventDestroy(arrived[i]); if (done[i]) cudaEventDestroy(done[i]); }
+        if (begin) cudaEventDestroy(begin);
+        if (end) cudaEventDestroy(end);
+        if (in) cudaStreamDestroy(in);
+        if (out) cudaStreamDestroy(out);
+        *this = CopySet();
+    }
+};
+std::mutex g_sets_mu;
+CopySet g_sets[64][kKeptSets];
+int g_sets_kept[64] = {};
+
+bool take_set(int dev, CopySet* set)
+{
+    {
+        std::lock_guard<std::mutex> lock(g_sets_mu);
+        if (g_sets_kept[dev] > 0) { *set = g_sets[dev][--g_sets_kept[dev]]; return true; }
+    }
+    return set->make();
+}
+void give_set(int dev, CopySet* set)
+{
+    {
+        std::lock_guard<std::mutex> lock(g_sets_mu);
+        if (g_sets_kept[dev] < kKeptSets) { g_sets[dev][g_sets_kept[dev]++] = *set; return; }
+    }
+    set->destroy();
+}
+}  // namespace
+
+// Convolves some images of a call with host buffers; *status_in_workspace as in general_dispatch.
+static conv2d_status_t host_images(const float* x, const float* w, float* y, int N, int C, int H, int W, int K, int R, int S,
+                                   conv2d_algo_t algo, void* workspace, size_t workspace_bytes, void* cuda_stream, bool* status_in_workspace)
+{
+    *status_in_workspace = false;
+    if (C == 1 && algo != CONV2D_ALGO_TF32)
+        return conv2d_fwd_single_channel(x, w, y, N, H, W, K, R, S, nullptr, 0, 0, cuda_stream);
+    return general_dispatch(x, w, y, N, C, H, W, K, R, S, algo, workspace, workspace_bytes, 0, cuda_stream, status_in_workspace);
+}
+
+// How many images a call with host buffers copies at a time; N: all at once.  The copies take nearly all of such a call,
+// and the link carries both directions at once, so the images are copied in, convolved and copied out in groups:
+// 32 x 64 x 56 x 56, 64 filters: 1020 us at once, 856 in two groups, 777 in four or five, 863 in
+// eight (every copy costs 4.5 us beside its bytes; 538 us is what both copies take when nothing orders them).  A group
+// is at least 4 MB of copies, keeps x and y 16-byte aligned, and runs the same algorithm as the whole call would.
+static int images_per_copy(const Shape& sh, conv2d_algo_t algo, const void* workspace, size_t workspace_bytes)
+{
+    const long long in = (long long)sh.C * sh.H * sh.W, out = (long long)sh.K * sh.P * sh.Q;      // floats of an image
+    long long chunks = sh.N * (in + out) * 4 / (4 << 20);
+    if (chunks > kMaxChunks) chunks = kMaxChunks;
+    if (chunks > sh.N) chunks = sh.N;
+    if (chunks < 2) return sh.N;
+    long long per = (sh.N + chunks - 1) / chunks;
+    while (per < sh.N && (per * in % 4 != 0 || per * out % 4 != 0)) ++per;
+    if (per >= sh.N) return sh.N;
+    if (algo != CONV2D_ALGO_FFMA && !(sh.C == 1 && algo != CONV2D_ALGO_TF32) && workspace) {
+        // tensor cores for all groups or for none, and room for the filters of each
+        auto fits = [&](int n) {
+            Shape s = sh;
+            s.N = n;
+            return tf32_supported(s) && tf32_workspace_bytes(s) <= workspace_bytes;
+        };
+        const int last = sh.N % (int)per;
+        const bool whole = fits(sh.N);
+        if (fits((int)per) != whole || (last && fits(last) != whole)) return sh.N;
+    }
+    return (int)per;
+}
+
 conv2d_status_t conv2d_fwd_host(const float* x_host, const float* w_host, float* y_host,
                                 float* x, float* w, float* y,
                                 int N, int C, int H, int W, int K, int R, int S,
@@ -380,20 +471,48 @@ conv2d_status_t conv2d_fwd_host(const float* x_host, const float* w_host, float*
     conv2d_status_t st = make_shape(N, C, H, W, K, R, S, &sh);
     if (st != CONV2D_OK) return st;
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    const size_t xb = (size_t)N * C * H * W * sizeof(float);
-    const size_t wb = (size_t)K * C * R * S * sizeof(float);
-    const size_t yb = (size_t)N * K * sh.P * sh.Q * sizeof(float);
-    if (cudaMemcpyAsync(x, x_host, xb, cudaMemcpyHostToDevice, stream) != cudaSuccess) return CONV2D_ERR_CUDA;
-    if (cudaMemcpyAsync(w, w_host, wb, cudaMemcpyHostToDevice, stream) != cudaSuccess) return CONV2D_ERR_CUDA;
+    const size_t xn = (size_t)C * H * W, yn = (size_t)K * sh.P * sh.Q, wb = (size_t)K * C * R * S * sizeof(float);
     // Only the tensor-core launcher clears and uses the status block in the workspace; after any other kernel the
     // workspace (which may be NULL, of size 0, or never written) must not be read for a status.
     bool status_in_workspace = false;
-    if (C == 1 && algo != CONV2D_ALGO_TF32)
-        st = conv2d_fwd_single_channel(x, w, y, N, H, W, K, R, S, nullptr, 0, 0, cuda_stream);
-    else
-        st = general_dispatch(x, w, y, N, C, H, W, K, R, S, algo, workspace, workspace_bytes, 0, cuda_stream, &status_in_workspace);
+    const int per = images_per_copy(sh, algo, workspace, workspace_bytes);
+    int dev = 0;
+    CopySet set;
+    if (per >= N || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || !take_set(dev, &set)) {
+        if (cudaMemcpyAsync(x, x_host, N * xn * sizeof(float), cudaMemcpyHostToDevice, stream) != cudaSuccess) return CONV2D_ERR_CUDA;
+        if (cudaMemcpyAsync(w, w_host, wb, cudaMemcpyHostToDevice, stream) != cudaSuccess) return CONV2D_ERR_CUDA;
+        st = host_images(x, w, y, N, C, H, W, K, R, S, algo, workspace, workspace_bytes, cuda_stream, &status_in_workspace);
+        if (st != CONV2D_OK) return st;
+        if (cudaMemcpyAsync(y_host, y, N * yn * sizeof(float), cudaMemcpyDeviceToHost, stream) != cudaSuccess) return CONV2D_ERR_CUDA;
+        return conv2d_get_status(status_in_workspace ? workspace : nullptr, cuda_stream);
+    }
+    // Copies in on one stream, convolutions on the caller's, copies out on another; everything after what the caller's
+    // stream holds already, and the caller's stream ends after the last copy.
+    bool ok = cudaEventRecord(set.begin, stream) == cudaSuccess && cudaStreamWaitEvent(set.in, set.begin, 0) == cudaSuccess &&
+              cudaMemcpyAsync(w, w_host, wb, cudaMemcpyHostToDevice, set.in) == cudaSuccess;
+    int chunks = 0;
+    for (int n0 = 0; n0 < N && ok; n0 += per, ++chunks) {
+        const size_t images = N - n0 < per ? N - n0 : per;
+        ok = cudaMemcpyAsync(x + n0 * xn, x_host + n0 * xn, images * xn * sizeof(float), cudaMemcpyHostToDevice, set.in) == cudaSuccess &&
+             cudaEventRecord(set.arrived[chunks], set.in) == cudaSuccess;
+    }
+    for (int i = 0, n0 = 0; i < chunks && ok && st == CONV2D_OK; ++i, n0 += per) {
+        const int images = N - n0 < per ? N - n0 : per;
+        ok = cudaStreamWaitEvent(stream, set.arrived[i], 0) == cudaSuccess;
+        if (!ok) break;
+        st = host_images(x + n0 * xn, w, y + n0 * yn, images, C, H, W, K, R, S, algo, workspace, workspace_bytes, cuda_stream, &status_in_workspace);
+        if (st != CONV2D_OK) break;
+        ok = (!status_in_workspace || latch_status(workspace, stream) == cudaSuccess) &&
+             cudaEventRecord(set.done[i], stream) == cudaSuccess && cudaStreamWaitEvent(set.out, set.done[i], 0) == cudaSuccess &&
+             cudaMemcpyAsync(y_host + n0 * yn, y + n0 * yn, images * yn * sizeof(float), cudaMemcpyDeviceToHost, set.out) == cudaSuccess;
+    }
+    ok = cudaEventRecord(set.end, set.out) == cudaSuccess && cudaStreamWaitEvent(stream, set.end, 0) == cudaSuccess && ok;
+    // (nothing of the call is pending when it returns, after an error either)
+    ok = cudaStreamSynchronize(set.in) == cudaSuccess && ok;
+    ok = cudaStreamSynchronize(set.out) == cudaSuccess && ok;
+    give_set(dev, &set);
     if (st != CONV2D_OK) return st;
-    if (cudaMemcpyAsync(y_host, y, yb, cudaMemcpyDeviceToHost, stream) != cudaSuccess) return CONV2D_ERR_CUDA;
+    if (!ok) return CONV2D_ERR_CUDA;
     return conv2d_get_status(status_in_workspace ? workspace : nullptr, cuda_stream);
 }
 

@@ -149,21 +149,34 @@ struct Phase {
     int col0;               // virtual columns before the first of them
     int base;               // taps of the phases before it
 };
-__device__ __forceinline__ Phase phase_of(const KernelArgs& a, int cb)
+// Phase number idx (once per block: the divisions would take a thread that runs alone some 1000 cycles per channel block,
+// 32 x 128 x 56 x 56 with stride 2: 43 us with them on the way of the MMA thread, @@PH@@ without).
+__device__ __forceinline__ uint2 describe_phase(const KernelArgs& a, int idx)
+{
+    const int pa = idx / a.phase_cols, pb = idx - pa * a.phase_cols;
+    const int rows = (a.R - pa + a.st - 1) / a.st, end = a.S + a.ext;          // (taps in columns ext .. end - 1)
+    const int col0 = pb < a.ext ? 1 : 0;
+    const int cols = (end - pb + a.st - 1) / a.st - col0;
+    const int rows_before = pa * (a.R / a.st) + min(pa, a.R % a.st);
+    const int cols_before = pb * (end / a.st) + min(pb, end % a.st) - min(pb, a.ext);
+    return make_uint2((unsigned)(rows * cols) | ((unsigned)cols << 16),
+                      (unsigned)(rows_before * a.S + rows * cols_before) | ((unsigned)pa << 16) | ((unsigned)pb << 20) | ((unsigned)col0 << 24));
+}
+__device__ __forceinline__ Phase unpack_phase(uint2 v)
 {
     Phase p;
+    p.cblk = 0;
+    p.taps = (int)(v.x & 0xffffu); p.cols = (int)(v.x >> 16);
+    p.base = (int)(v.y & 0xffffu); p.a = (int)(v.y >> 16) & 15; p.b = (int)(v.y >> 20) & 15; p.col0 = (int)(v.y >> 24);
+    return p;
+}
+// Channel block cb, from the block's table of phases.
+__device__ __forceinline__ Phase phase_of(const KernelArgs& a, const uint2* phase_table, int cb)
+{
     int idx;
-    p.cblk = a.div_phases.divmod(cb, idx);
-    p.a = idx / a.phase_cols;
-    p.b = idx - p.a * a.phase_cols;
-    const int rows = (a.R - p.a + a.st - 1) / a.st;
-    p.col0 = p.b < a.ext ? 1 : 0;
-    p.cols = (a.S + a.ext - p.b + a.st - 1) / a.st - p.col0;
-    p.taps = rows * p.cols;
-    const int end = a.S + a.ext;                                  // (taps in columns ext .. end - 1)
-    const int rows_before = p.a * (a.R / a.st) + min(p.a, a.R % a.st);
-    const int cols_before = p.b * (end / a.st) + min(p.b, end % a.st) - min(p.b, a.ext);
-    p.base = rows_before * a.S + rows * cols_before;
+    const int cblk = a.div_phases.divmod(cb, idx);
+    Phase p = unpack_phase(phase_table[idx]);
+    p.cblk = cblk;
     return p;
 }
 // Staged pixel -> image n and the image row and column of phase (0, 0), which may lie outside the image.
@@ -183,7 +196,7 @@ __device__ __forceinline__ bool staged_pixel_virtual(const KernelArgs& a, const 
 // i = g * npix + jj; thread t of the 256 producers owns units first + t, first + t + 256, ...  Consecutive
 // lanes read consecutive pixels of one channel (coalesced) and write consecutive 16-byte units.
 template <bool B16, bool FOLD, bool PATCH, bool VIRT, int CNT>
-__device__ __forceinline__ void load_units(float (&v)[CNT][kCB], const KernelArgs& a, const ItemGeom& geom, int cb0, int first, int wtid, int nthr)
+__device__ __forceinline__ void load_units(float (&v)[CNT][kCB], const KernelArgs& a, const uint2* phase_table, const ItemGeom& geom, int cb0, int first, int wtid, int nthr)
 {
     const int units = a.npix * a.cbg;
 #pragma unroll
@@ -211,7 +224,7 @@ __device__ __forceinline__ void load_units(float (&v)[CNT][kCB], const KernelArg
                         if (++pb == a.st) { pb = 0; if (++pa == a.st) { pa = 0; ++c; src += a.HW; } }
                     }
                 } else {
-                    const Phase p = phase_of(a, cb0 + g);
+                    const Phase p = phase_of(a, phase_table, cb0 + g);
                     h += p.a;
                     wc += p.b;
                     const int c0 = p.cblk * kCB;
@@ -428,11 +441,15 @@ general_tc_kernel(const KernelArgs a)
     volatile unsigned long long* t_entry = reinterpret_cast<volatile unsigned long long*>(tmem_slot + 2);
     uint32_t* tap_shift = tmem_slot + 4;                   // [taps] r * row_pitch + s of every tap, in staged pixels
     // (bit 31: the slot is a lone tap held as a 64-row slice, see pair_compact)
+    // (behind the tap shifts; the planner keeps kMaxTaps entries for both)
+    uint2* phase_table = reinterpret_cast<uint2*>(tap_shift + ((VIRT ? a.R * a.S : 0) + 1) / 2 * 2);
+    if (VIRT)
+        for (int i = tid; i < a.phases; i += kThreads) phase_table[i] = describe_phase(a, i);
     if (VIRT && a.phases > 1) {
         // one table per phase, behind one another in the order of the filter bank
         for (int t = tid; t < a.R * a.S; t += kThreads) {
             const int r = t / a.S, sx = t - r * a.S + a.ext, r2 = r / a.st, s2 = sx / a.st;
-            const Phase p = phase_of(a, (r - r2 * a.st) * a.phase_cols + sx - s2 * a.st);
+            const Phase p = unpack_phase(describe_phase(a, (r - r2 * a.st) * a.phase_cols + sx - s2 * a.st));
             tap_shift[p.base + r2 * p.cols + s2 - p.col0] = (uint32_t)(r2 * a.row_pitch + s2);
         }
     } else
@@ -504,7 +521,7 @@ general_tc_kernel(const KernelArgs a)
                         int taps = a.taps;
                         size_t cb_at = (size_t)cbr * a.taps;            // taps of the bank before this channel block's
                         if (VIRT && a.phases > 1) {
-                            const Phase p = phase_of(a, cbr);
+                            const Phase p = phase_of(a, phase_table, cbr);
                             taps = p.taps;
                             cb_at = (size_t)p.cblk * (a.R * a.S) + p.base;
                         }
@@ -597,7 +614,7 @@ general_tc_kernel(const KernelArgs a)
                         int taps = a.taps, s_slots = a.s_slots, tap0 = 0, sx0 = 0;
                         size_t bank_at = (size_t)(gr * a.cbg + g) * a.cb_bytes;   // (resident filters)
                         if (VIRT && a.phases > 1) {
-                            const Phase p = phase_of(a, gr * a.cbg + g);
+                            const Phase p = phase_of(a, phase_table, gr * a.cbg + g);
                             taps = p.taps; s_slots = p.cols; tap0 = p.base; sx0 = sx = p.col0;
                             bank_at = (size_t)p.cblk * a.cb_bytes + (size_t)p.base * b_chunk_bytes;
                         }
@@ -624,7 +641,7 @@ general_tc_kernel(const KernelArgs a)
                                     // (its chunk stride and K step are half as long too) onto the same accumulator lanes
                                     const uint32_t idesc64 = B16 ? idesc_b16(64u, n_cols, a.fp16 != 0) : idesc_tf32(64u, n_cols);
                                     for (int t = 0; t < nt; ++t) {
-                                        const uint32_t a_lo = a_lo_block + (cur & 0x7FFFFFFFu);
+                                        const uint32_t a_lo = (VIRT ? a_lo_block + (uint32_t)a.shift0 : a_lo_block) + (cur & 0x7FFFFFFFu);
                                         const bool lone = (cur >> 31) != 0u;
                                         cur = shift[t + 1 < nt ? t + 1 : t];
                                         if (lone) {
@@ -761,7 +778,7 @@ general_tc_kernel(const KernelArgs a)
                                 d[c * a.cstride + 1] = make_float4(to_tf32_rna(r0.z), to_tf32_rna(r0.w), to_tf32_rna(r1.z), to_tf32_rna(r1.w));
                             }
                         } else {
-                            const Phase p = phase_of(a, cb);
+                            const Phase p = phase_of(a, phase_table, cb);
                             const int c0 = p.cblk * kCB;
                             h += p.a;
                             if (in && (unsigned)h < (unsigned)a.H) {
@@ -875,7 +892,7 @@ general_tc_kernel(const KernelArgs a)
                 } else
                 for (int first = 0; first < units; first += nthr * kUnitsPerThread) {
                     float v[kUnitsPerThread][kCB];
-                    load_units<B16, FOLD, PATCH, VIRT>(v, a, ii.geom, gr * a.cbg, first, wtid, nthr);
+                    load_units<B16, FOLD, PATCH, VIRT>(v, a, phase_table, ii.geom, gr * a.cbg, first, wtid, nthr);
                     store_units<B16>(v, dst, a, first, wtid, nthr);
                 }
                 fence_proxy_async_smem();

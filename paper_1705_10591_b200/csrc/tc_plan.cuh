@@ -138,7 +138,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         sh.H = p.virt_h;
         sh.W = p.virt_w;
         sh.pad_h = sh.pad_w = 0;
-        if (sh.R * sh.S > kMaxTaps) return p;
+        if ((long long)sh.R * sh.S + 1 + 2 * p.phases > kMaxTaps) return p;      // (tap shifts and the table of phases)
     }
     const long long total_pix = (long long)sh.N * sh.H * sh.W;
     if (total_pix >= (1LL << 31) - (1LL << 20)) return p;     // flat pixel indices stay within int32
@@ -227,7 +227,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     p.pair_compact = 0;
     const size_t compact_cb_bytes = (size_t)r_eff * ((s_eff / 2) * 128 + (s_eff & 1) * 64) * kCB * 4;
     if (allow_compact && !p.pair_taps && p.swap && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
-        !padded && !virt && (size_t)((c_eff + cbc - 1) / cbc) * compact_cb_bytes <= 152 * 1024 && env_int("CONV2D_B200_TF32_PAIR_COMPACT", 0) != 0) {
+        !padded && (size_t)((c_eff + cbc - 1) / cbc) * compact_cb_bytes <= 152 * 1024 && env_int("CONV2D_B200_TF32_PAIR_COMPACT", 0) != 0) {
         p.pair_taps = 1;
         p.pair_compact = 1;
     }
@@ -326,7 +326,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         }
     }
 
-    if (p.pair_compact && !p.resident) return plan_with_patch_width(sh, b16, want_patch_w, false);    // compact stacking needs the resident bank
+    if (p.pair_compact && !p.resident) return plan_with_patch_width(shape, b16, want_patch_w, false, virt);    // compact stacking needs the resident bank
     if (!p.resident) {
         // Streamed filters.  Measured: all SMs together draw filter stages from L2 at no more than
         // ~5-6 TB/s, i.e. a 8 KB stage costs ~120 cycles on top of the MMAs that consume it unless it is
@@ -406,9 +406,10 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
             const int per_block = (p.taps + p.tps - 1) / p.tps;
             p.tps = (p.taps + per_block - 1) / per_block;
         }
+        // (phases have few MMAs per stage: stages of the image are worth more than filters far ahead)
+        while (st > 1 && p.a_stages < kMaxAStages && smem_need(p.a_stages + 1, p.npix, p.n_tile, p.b_stages, p.tps, p.cbg) <= kLimit) ++p.a_stages;
         while (p.b_stages < 4 && smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages + 1, p.tps, p.cbg) <= kLimit) ++p.b_stages;
-        // (few MMAs per stage: more stages have to be on their way)
-        while (p.a_stages < kMaxAStages && (p.taps <= 3 || st > 1) &&
+        while (p.a_stages < kMaxAStages && p.taps <= 3 &&
                smem_need(p.a_stages + 1, p.npix, p.n_tile, p.b_stages, p.tps, p.cbg) <= kLimit - 32 * 1024) ++p.a_stages;
         while (p.b_stages < kMaxBStages && smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages + 1, p.tps, p.cbg) <= kLimit &&
                (size_t)p.b_stages * p.tps * chunk < 128 * 1024) ++p.b_stages;
