@@ -1097,6 +1097,67 @@ general_tc_kernel(const KernelArgs a)
                     continue;
                 }
                 uint32_t va0[16], va1[16], vb0[16], vb1[16], vax[1], vbx[1];
+                if (!STACK && !CLUSTER && rpq == 16 && a.vec >= 2 && !add) {
+                    // At most 64 filters (a quarter holds 16 maps): two 32-pixel blocks share the tile and one pass over it,
+                    // each half of the warp stores one of them.  A block at a time the warps, not the MMAs or the memory,
+                    // set the pace of short contractions (900 cycles per block, most of them the latency of the steps).
+                    const int half = lane >> 4, lanes_per_row = 32 >> a.vec_shift;
+                    const int row_sub = (lane & 15) >> (5 - a.vec_shift), pg = lane & (lanes_per_row - 1);
+                    const int pairs = (blocks + 1) / 2, p_step = split ? 3 : 1;
+                    const int kmax = min(16, a.K - nb * a.n_tile - quarter * 16);      // maps of this quarter that exist
+                    auto load_pair = [&](int bp) {
+                        tmem_ld16(lane_base + (uint32_t)(bp * 64), va0);
+                        tmem_ld16(lane_base + (uint32_t)(bp * 64 + 16), va1);
+                        if (2 * bp + 1 < blocks) {
+                            tmem_ld16(lane_base + (uint32_t)(bp * 64 + 32), vb0);
+                            tmem_ld16(lane_base + (uint32_t)(bp * 64 + 48), vb1);
+                        }
+                    };
+                    int bp = split ? share : 0;
+                    if (bp < pairs) load_pair(bp);
+                    while (bp < pairs) {
+                        tmem_ld_wait();
+                        __syncwarp();                               // the previous pair has been read out
+                        if (lane < 16) {
+                            float4* ra = reinterpret_cast<float4*>(tile + lane * kXposePitch);
+                            float4* rb = reinterpret_cast<float4*>(tile + (lane + 16) * kXposePitch);
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                ra[i] = make_float4(__uint_as_float(va0[4 * i]), __uint_as_float(va0[4 * i + 1]), __uint_as_float(va0[4 * i + 2]), __uint_as_float(va0[4 * i + 3]));
+                                ra[4 + i] = make_float4(__uint_as_float(va1[4 * i]), __uint_as_float(va1[4 * i + 1]), __uint_as_float(va1[4 * i + 2]), __uint_as_float(va1[4 * i + 3]));
+                            }
+                            if (2 * bp + 1 < blocks) {
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) {
+                                    rb[i] = make_float4(__uint_as_float(vb0[4 * i]), __uint_as_float(vb0[4 * i + 1]), __uint_as_float(vb0[4 * i + 2]), __uint_as_float(vb0[4 * i + 3]));
+                                    rb[4 + i] = make_float4(__uint_as_float(vb1[4 * i]), __uint_as_float(vb1[4 * i + 1]), __uint_as_float(vb1[4 * i + 2]), __uint_as_float(vb1[4 * i + 3]));
+                                }
+                            }
+                        }
+                        __syncwarp();
+                        const int b = 2 * bp + half;
+                        bp += p_step;
+                        if (bp < pairs) load_pair(bp);
+                        int n, p, q;                                // this lane's first pixel of its block
+                        if (b < blocks && output_pixel<PATCH>(a, ii.geom, b * 32 + pg * a.vec, n, p, q)) {
+                            float* o = a.y + (((size_t)n * a.K + nb * a.n_tile + quarter * 16 + row_sub) * a.P + p) * a.Q + q;
+                            const float* src = tile + (16 * half + row_sub) * kXposePitch + pg * a.vec;
+                            if (a.vec == 4) {
+#pragma unroll
+                                for (int r = 0; r < 16; r += 2, o += 2 * plane, src += 2 * kXposePitch)
+                                    if (r + row_sub < kmax) *reinterpret_cast<float4*>(o) = *reinterpret_cast<const float4*>(src);
+                            } else {
+#pragma unroll
+                                for (int r = 0; r < 16; ++r, o += plane, src += kXposePitch)
+                                    if (r < kmax) *reinterpret_cast<float2*>(o) = *reinterpret_cast<const float2*>(src);
+                            }
+                        }
+                    }
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0 && !helper) mbar_arrive(&acc_empty[buf]);
+                    continue;
+                }
                 const int b_step = split ? 3 : 1;
                 int b = split ? share : 0;
                 if (b < blocks) load_block(va0, va1, vax, b);
