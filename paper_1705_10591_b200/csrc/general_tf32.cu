@@ -234,7 +234,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     {
         // as many producer groups as can each still cover a stage in one pass (one memory round trip)
         const long long per_pass = a.quad || p.quad2 ? kProducers : (long long)kProducers * kUnitsPerThread;
-        const long long stage_work = p.quad2 ? (long long)(p.npix / 2) * (p.mixed ? p.cbg : p.cbg / 2) : (long long)(a.quad ? p.npix / 4 : p.npix) * p.cbg;
+        const long long stage_work = p.quad2 ? (long long)(p.npix / 2) * p.cbg : (long long)(a.quad ? p.npix / 4 : p.npix) * p.cbg;
         int g = 1;
         while (g < 4 && g * 2 <= p.a_stages && stage_work * (g * 2) <= per_pass) g *= 2;
         a.pgroups = env_int("CONV2D_B200_TF32_PGROUPS", g);

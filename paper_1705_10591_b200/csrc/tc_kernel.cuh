@@ -149,6 +149,8 @@ struct Phase {
     int col0;               // virtual columns before the first of them
     int base;               // taps of the phases before it
 };
+// (quad2: the phases are those of the rows, a.phase_cols = 1; each has the taps of both column phases, first those of
+// column phase 0, and a channel block is two 16-channel blocks, one per column phase.)
 // Phase number idx (once per block: the divisions would take a thread that runs alone some 1000 cycles per channel block,
 // 32 x 128 x 56 x 56 with stride 2: 43 us with them on the way of the MMA thread, @@PH@@ without).
 __device__ __forceinline__ uint2 describe_phase(const KernelArgs& a, int idx)
@@ -158,6 +160,8 @@ __device__ __forceinline__ uint2 describe_phase(const KernelArgs& a, int idx)
     const int col0 = pb < a.ext ? 1 : 0;
     const int cols = (end - pb + a.st - 1) / a.st - col0;
     const int rows_before = pa * (a.R / a.st) + min(pa, a.R % a.st);
+    if (a.quad2 && a.phases > 1)
+        return make_uint2((unsigned)(rows * a.S) | ((unsigned)a.S << 16), (unsigned)(rows_before * a.S) | ((unsigned)pa << 16));
     const int cols_before = pb * (end / a.st) + min(pb, end % a.st) - min(pb, a.ext);
     return make_uint2((unsigned)(rows * cols) | ((unsigned)cols << 16),
                       (unsigned)(rows_before * a.S + rows * cols_before) | ((unsigned)pa << 16) | ((unsigned)pb << 20) | ((unsigned)col0 << 24));
@@ -413,7 +417,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 general_tc_kernel(const KernelArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    const uint32_t a_block_bytes = (uint32_t)kCB * a.cstride * 4;       // one channel block of a stage
+    const uint32_t a_block_bytes = (uint32_t)kCB * a.cstride * 4 * (VIRT && a.quad2 && !a.mixed ? 2 : 1);       // one channel block of a stage
     const uint32_t a_stage_bytes = a_block_bytes * (uint32_t)a.cbg;
     const uint32_t b_chunk_bytes = (uint32_t)kCB * a.n_tile * 4;        // one (channel block, tap)
     const uint32_t b_stage_bytes = b_chunk_bytes * (uint32_t)a.tps;
@@ -449,6 +453,15 @@ general_tc_kernel(const KernelArgs a)
         // one table per phase, behind one another in the order of the filter bank
         for (int t = tid; t < a.R * a.S; t += kThreads) {
             const int r = t / a.S, sx = t - r * a.S + a.ext, r2 = r / a.st, s2 = sx / a.st;
+            if (a.quad2) {
+                // taps of column phase 1 read the second 16-channel block of the channel block
+                const int pa = r - r2 * a.st, pb = sx - s2 * a.st, rows = (a.R - pa + 1) / 2;
+                const int cols0 = (a.S + a.ext + 1) / 2 - a.ext, cols1 = a.S - cols0;
+                const int base = (pa * (a.R / 2) + min(pa, a.R % 2)) * a.S + (pb ? rows * cols0 : 0);
+                tap_shift[base + r2 * (pb ? cols1 : cols0) + (pb ? s2 : s2 - a.ext)] =
+                    (uint32_t)(r2 * a.row_pitch + s2) + (pb ? (uint32_t)(kChunks * a.cstride) : 0u);
+                continue;
+            }
             const Phase p = unpack_phase(describe_phase(a, (r - r2 * a.st) * a.phase_cols + sx - s2 * a.st));
             tap_shift[p.base + r2 * p.cols + s2 - p.col0] = (uint32_t)(r2 * a.row_pitch + s2);
         }
@@ -664,6 +677,7 @@ general_tc_kernel(const KernelArgs a)
                             } else {
                                 for (int t = 0; t < nt; ++t, b_lo += b_chunk_bytes >> 4) {
                                     uint32_t a_lo = a_lo_block + row_shift + (uint32_t)sx;
+                                    if (VIRT && a.quad2 && a.phases > 1) a_lo = a_lo_block + (uint32_t)a.shift0 + tap_shift[tap0 + t0 + t];
                                     uint32_t d = d0;
                                     if (a.swap) {
                                         // two pixel groups: four MMAs per tap keep the pipe busy (measured faster
@@ -749,16 +763,15 @@ general_tc_kernel(const KernelArgs a)
                 if (VIRT && a.quad2) {
                     // Stride 2: four adjacent pixels of an image row are two virtual pixels of both phases of that row.
                     const int qn = a.npix >> 1;
-                    const int c_step = a.mixed ? 1 : 2;                  // staged channel blocks of a unit
-                    for (int i = wtid; i * c_step < qn * a.cbg; i += nthr) {
+                    for (int i = wtid; i < qn * a.cbg; i += nthr) {
                         int pq;
-                        const int g = a.div_qn.divmod(i, pq) * c_step, cb = gr * a.cbg + g;
+                        const int g = a.div_qn.divmod(i, pq), cb = gr * a.cbg + g;
                         float4 v[kCB];
 #pragma unroll
                         for (int e = 0; e < kCB; ++e) v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
                         int n, h, wc;
                         const bool in = staged_pixel_virtual(a, ii.geom, 2 * pq, n, h, wc) && (unsigned)wc < (unsigned)a.W && cb < a.cblks;
-                        float4* d = dst + (size_t)g * kChunks * a.cstride + 2 * pq;
+                        float4* d = dst + (size_t)g * (a_block_bytes >> 4) + 2 * pq;
                         if (a.mixed) {
                             // a chunk holds the four phases of a channel: two rows of the image
                             const int c0 = cb * kChunks;

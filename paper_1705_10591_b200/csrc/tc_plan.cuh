@@ -197,9 +197,12 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
             if (st != 2) p.quad2 = 0;
             p.cblks = (int)(((long long)sh.C * st * st + cbc - 1) / cbc);
         } else {
+            // (with quad2 the two phases of a row are one block of 32 staged channels with the taps of both)
+            if (p.quad2) { p.phases /= p.phase_cols; p.phase_cols = 1; }
             p.cblks *= p.phases;
         }
     }
+    const int stage_blocks = p.quad2 && !p.mixed ? 2 : 1;    // 16-channel blocks of a channel block
     // Stacked taps.  With at most 64 filters an M = 64 instruction runs the tensor pipe at half its rate.  Instead
     // half of the rows of an M = 128 operand hold the filters' tap (r, s) and the other half their tap (r, s + 1),
     // both multiplied with the pixels shifted for (r, s): the accumulator row of tap (r, s + 1), column j + 1, then
@@ -233,7 +236,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     }
     if (p.pair_taps) p.n_tile = 128;
     p.s_slots = p.pair_taps ? (s_eff + 1) / 2 : s_eff;
-    p.taps = r_eff * p.s_slots;
+    p.taps = stage_blocks == 2 ? r_eff * sh.S : r_eff * p.s_slots;          // (with phases: of the phase that has most)
     if (p.taps > kMaxTaps) return p;
     const size_t extra = p.swap ? kXposeBytes : 0;       // epilogue transposition tile
     // Addressing mode.  In the flat pixel run the staged halo is (R-1) whole image rows; once that exceeds a
@@ -309,17 +312,17 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
             if (p.swap && want >= 64 && want <= (p.pair_compact ? 256 : 512) && want % 32 == 0 && pixel_items(want) > 0) res_px = want;
         }
         const int npix = npix_of(res_px);
-        if ((p.swap ? res_px : mt * set_cols) <= 512 && npix <= 16000 && wbytes + extra + (size_t)2 * (p.quad2 && !p.mixed ? 2 : 1) * kCB * chunk_stride(npix) * 4 + kBookBytes <= kSmemLimit) {
+        if ((p.swap ? res_px : mt * set_cols) <= 512 && npix <= 16000 && wbytes + extra + (size_t)2 * stage_blocks * kCB * chunk_stride(npix) * 4 + kBookBytes <= kSmemLimit) {
             p.resident = 1;
             p.mt = p.swap ? (res_px + kTileM - 1) / kTileM : mt;
             p.tile_px = res_px;
             p.npix = npix;
-            p.cbg = p.quad2 && !p.mixed ? 2 : 1;                       // (both phases of a row of pixels in one stage)
+            p.cbg = 1;
             p.a_stages = 2;
             p.b_stages = 1;
             p.tps = p.taps;
-            auto need = [&](int a_stages, int cbg) { return wbytes + extra + (size_t)a_stages * cbg * kCB * chunk_stride(npix) * 4 + kBookBytes; };
-            while (p.cbg * 2 <= p.cblks && npix * p.cbg * 2 <= kProducers * kUnitsPerThread &&
+            auto need = [&](int a_stages, int cbg) { return wbytes + extra + (size_t)a_stages * cbg * stage_blocks * kCB * chunk_stride(npix) * 4 + kBookBytes; };
+            while (p.cbg * 2 <= p.cblks && npix * p.cbg * stage_blocks * 2 <= kProducers * kUnitsPerThread &&
                    need(p.a_stages, p.cbg * 2) <= kSmemLimit) p.cbg *= 2;
             while (p.a_stages < kMaxAStages && need(p.a_stages + 1, p.cbg) <= kSmemLimit) ++p.a_stages;
             p.smem_bytes = need(p.a_stages, p.cbg);
@@ -334,7 +337,6 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         // second accumulator set (hidden write-back) and balance better.  Cost in units of one tile's MMA
         // time: rounds x mt x (1 + stage cost / MMA time) + exposed write-back.
         const size_t kLimit = kSmemLimit - extra;
-        const int stage_blocks = p.quad2 && !p.mixed ? 2 : 1;    // channel blocks of an activation stage
         const double stage_cycles = chunk / 66.0;           // one (tap, channel block) of filters through L2
         const int forced_px = env_int("CONV2D_B200_TF32_TILE_PX", 0);
         const bool ksplit_allowed = env_int("CONV2D_B200_TF32_KSPLIT", 1) != 0;
@@ -394,12 +396,12 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         // by varying the stage size) once per 16-48 MMAs; the ring should hold
         // 64-128 KB in flight to cover the L2 latency.
         p.a_stages = 2;
-        p.cbg = stage_blocks;
+        p.cbg = 1;
         p.tps = env_int("CONV2D_B200_TF32_STAGE_KB", 48) * 1024 / chunk;
         if (p.tps < 1) p.tps = 1;
         if (p.tps > p.taps) p.tps = p.taps;
         p.b_stages = 2;
-        while (p.tps > 1 && smem_need(p.a_stages, p.npix, p.n_tile, 3, p.tps, p.cbg) > kLimit) --p.tps;
+        while (p.tps > 1 && smem_need(p.a_stages, p.npix, p.n_tile, 3, p.tps, p.cbg * stage_blocks) > kLimit) --p.tps;
         // equal stages: 6 taps as 3 + 3 instead of 5 + 1 (the short stage's MMAs would end long before the next
         // long stage has arrived)
         {
@@ -407,13 +409,13 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
             p.tps = (p.taps + per_block - 1) / per_block;
         }
         // (phases have few MMAs per stage: stages of the image are worth more than filters far ahead)
-        while (st > 1 && p.a_stages < kMaxAStages && smem_need(p.a_stages + 1, p.npix, p.n_tile, p.b_stages, p.tps, p.cbg) <= kLimit) ++p.a_stages;
-        while (p.b_stages < 4 && smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages + 1, p.tps, p.cbg) <= kLimit) ++p.b_stages;
+        while (st > 1 && p.a_stages < kMaxAStages && smem_need(p.a_stages + 1, p.npix, p.n_tile, p.b_stages, p.tps, p.cbg * stage_blocks) <= kLimit) ++p.a_stages;
+        while (p.b_stages < 4 && smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages + 1, p.tps, p.cbg * stage_blocks) <= kLimit) ++p.b_stages;
         while (p.a_stages < kMaxAStages && p.taps <= 3 &&
-               smem_need(p.a_stages + 1, p.npix, p.n_tile, p.b_stages, p.tps, p.cbg) <= kLimit - 32 * 1024) ++p.a_stages;
-        while (p.b_stages < kMaxBStages && smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages + 1, p.tps, p.cbg) <= kLimit &&
+               smem_need(p.a_stages + 1, p.npix, p.n_tile, p.b_stages, p.tps, p.cbg * stage_blocks) <= kLimit - 32 * 1024) ++p.a_stages;
+        while (p.b_stages < kMaxBStages && smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages + 1, p.tps, p.cbg * stage_blocks) <= kLimit &&
                (size_t)p.b_stages * p.tps * chunk < 128 * 1024) ++p.b_stages;
-        p.smem_bytes = smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages, p.tps, p.cbg) + extra;
+        p.smem_bytes = smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages, p.tps, p.cbg * stage_blocks) + extra;
     }
 
     const int item_cols = p.swap ? p.tile_px : p.mt * p.n_tile;     // tensor-memory columns of one accumulator set
@@ -444,12 +446,12 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         const int slots = (p.tile_px / 32 + 1) / 2;
         const size_t xb = xchg_area_bytes(slots);
         int bs = p.b_stages;
-        while (bs > 2 && smem_need(p.a_stages, p.npix, p.n_tile, bs, p.tps, p.cbg) + extra + xb > kSmemLimit) --bs;
-        if (smem_need(p.a_stages, p.npix, p.n_tile, bs, p.tps, p.cbg) + extra + xb <= kSmemLimit) {
+        while (bs > 2 && smem_need(p.a_stages, p.npix, p.n_tile, bs, p.tps, p.cbg * stage_blocks) + extra + xb > kSmemLimit) --bs;
+        if (smem_need(p.a_stages, p.npix, p.n_tile, bs, p.tps, p.cbg * stage_blocks) + extra + xb <= kSmemLimit) {
             p.cluster = 1;
             p.xchg_slots = slots;
             p.b_stages = bs;
-            p.smem_bytes = smem_need(p.a_stages, p.npix, p.n_tile, bs, p.tps, p.cbg) + extra + xb;
+            p.smem_bytes = smem_need(p.a_stages, p.npix, p.n_tile, bs, p.tps, p.cbg * stage_blocks) + extra + xb;
         }
     }
     int cols = p.nbuf * item_cols;
