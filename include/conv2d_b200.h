@@ -199,10 +199,11 @@ conv2d_status_t conv2d_fwd_general_padded(const float* x, const float* w, float*
  * General case with zero padding and a stride (not in the paper, which has stride 1):
  *   y[n,k,p,q] = sum_{c,r,s} xz[n,c,stride*p+r-pad_h,stride*q+s-pad_w] * w[k,c,r,s],
  *   P = (H + 2*pad_h - R) / stride + 1, Q = (W + 2*pad_w - S) / stride + 1 (integer division), y [N][K][P][Q].
- * The call rewrites the problem as a stride-1 convolution over stride*stride times as many channels
- * ("space to depth": channel (c,a,b) of the rewritten image holds the pixels whose row is a and whose column
- * is b modulo the stride; the filters are split the same way) with two extra kernels into the workspace and
- * then runs conv2d_fwd_general on it: the same multiply-adds as the definition plus zeros, every algorithm.
+ * With the tensor-core algorithms the kernel stages the phases of the stride straight from x and multiplies each
+ * with its own taps.  Otherwise (fp32, or no such instance) the call rewrites the problem as a stride-1 convolution
+ * over stride*stride times as many channels ("space to depth": channel (c,a,b) of the rewritten image holds the pixels
+ * whose row is a and whose column is b modulo the stride; the filters are split the same way) with two extra kernels
+ * into the workspace and then runs conv2d_fwd_general on it: the same multiply-adds as the definition plus zeros.
  * 1 <= stride <= 8.  Workspace from conv2d_fwd_strided_workspace_size; required, 16-byte aligned, status
  * block first.  With CONV2D_FLAG_WEIGHTS_PACKED the rewritten filters of the previous call are reused too.
  * algo is AUTO, FFMA or TF32; N * C must not exceed 65535 (CONV2D_ERR_UNSUPPORTED otherwise, checked before
@@ -258,6 +259,9 @@ conv2d_status_t conv2d_fwd_general_noalloc(const float* x, const float* w, float
  * w_host are copied to the caller's device buffers x, w on the stream, the
  * convolution runs (single-channel kernel when C == 1, else conv2d_fwd_general
  * with `algo`), y is copied back into y_host and the stream is synchronised.
+ * Large calls (from 8 MB of copies on) do this in up to five groups of images, with the
+ * copies in both directions on streams of the library's own while the caller's stream
+ * convolves; they start after what the caller's stream holds and have ended on return.
  * Host buffers should be page-locked for the copies to run at full speed.
  * Returns the first error met, or the device status after synchronising
  * (CONV2D_ERR_DEVICE_TIMEOUT if a bounded on-device wait expired).  The
