@@ -875,8 +875,8 @@ conv2d_status_t dispatch_rs(const float* x, const float* w, float* y, const Shap
     const bool rows_ok = sh.W % 4 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
     if (rows_ok && env_int("CONV2D_B200_SC_WIDE", 1) != 0) {
         // Rows per work item: 8, or another height (4..16, as far as the double buffer fits) when that fills the last
-        // round of work items over the SMs clearly better (2048 x 2048, 1 x 1: 256 items of 8 rows are 1.73 rounds
-        // on 148 SMs, 146 items of 14 rows one round).  Every row below 8 costs a little (more halo rows, more
+        // round of work items over the SMs clearly better (3072 x 3072, 5 x 5: 768 items of 8 rows are 5.2 rounds
+        // on 148 SMs, 1024 items of 6 rows 6.9: 409 -> 359 us).  Every row below 8 costs a little (more halo rows, more
         // per-item set-up), hence the 1.5 % per row.
         // (Heights are multiples of the rows a step produces: an odd height would compute its last row twice.)
         auto pick_band = [&](int step, int item_factor, size_t pitch_bytes) {
@@ -907,10 +907,12 @@ conv2d_status_t dispatch_rs(const float* x, const float* w, float* y, const Shap
             const conv2d_status_t st = try_rows_shift<R, S>(x, w, y, sh, forced_band > 0 ? band_h : pick_band(2, 2, kShiftPitch * sizeof(float)), stream);
             if (st != CONV2D_ERR_UNSUPPORTED) return st;
         }
-        if (sh.Q >= env_int("CONV2D_B200_SC_WIDE_MINQ", 1024)) {
-            const conv2d_status_t st = (tr == 1 || R >= 7) ? launch_rows<R, S, 1>(x, w, y, sh, band_h, stream)
-                                                           : launch_rows<R, S, 2>(x, w, y, sh, band_h, stream);
-            if (st != CONV2D_ERR_UNSUPPORTED) return st;
+        if constexpr (R == 3 || R == 5) {                    // (the flat kernel has the wide images of the other sizes)
+            if (sh.Q >= env_int("CONV2D_B200_SC_WIDE_MINQ", 1024)) {
+                const conv2d_status_t st = tr == 1 ? launch_rows<R, S, 1>(x, w, y, sh, band_h, stream)
+                                                   : launch_rows<R, S, 2>(x, w, y, sh, band_h, stream);
+                if (st != CONV2D_ERR_UNSUPPORTED) return st;
+            }
         }
     }
     if (env_int("CONV2D_B200_SC_PACKED", 1) != 0 &&
