@@ -192,7 +192,11 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
                                      general_tc_kernel<false, false, true, true>,   general_tc_kernel<true, false, true, true>,
                                      general_tc_kernel<false, false, false, false, true>, general_tc_kernel<true, false, false, false, true>,
                                      general_tc_kernel<false, false, false, false, false, true>, general_tc_kernel<false, false, false, true, false, true>,
-                                     general_tc_kernel<false, false, false, false, true, true>};
+                                     general_tc_kernel<false, false, false, false, true, true>,
+                                     general_tc_kernel<false, false, false, false, false, false, true>, general_tc_kernel<true, false, false, false, false, false, true>,
+                                     general_tc_kernel<false, true, false, false, false, false, true>, general_tc_kernel<true, true, false, false, false, false, true>,
+                                     general_tc_kernel<false, false, true, false, false, false, true>, general_tc_kernel<true, false, true, false, false, false, true>,
+                                     general_tc_kernel<false, false, false, false, false, true, true>};
         for (auto k : all)
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess)
             return CONV2D_ERR_CUDA;
@@ -264,7 +268,13 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     // tail of whatever kernel precedes it on the stream; it waits for that kernel before it touches global memory.
     const bool fold = p.fold_r * p.fold_s > 1;
     void (*kernel)(KernelArgs);
-    if (p.virt) kernel = p.pair_taps ? general_tc_kernel<false, false, false, true, false, true> : general_tc_kernel<false, false, false, false, false, true>;
+    if (p.swap && p.n_tile == 64 && !p.pair_taps) {
+        if (p.virt) kernel = general_tc_kernel<false, false, false, false, false, true, true>;
+        else if (p.patch_w) kernel = b16 ? general_tc_kernel<true, false, true, false, false, false, true> : general_tc_kernel<false, false, true, false, false, false, true>;
+        else if (fold) kernel = b16 ? general_tc_kernel<true, true, false, false, false, false, true> : general_tc_kernel<false, true, false, false, false, false, true>;
+        else kernel = b16 ? general_tc_kernel<true, false, false, false, false, false, true> : general_tc_kernel<false, false, false, false, false, false, true>;
+    }
+    else if (p.virt) kernel = p.pair_taps ? general_tc_kernel<false, false, false, true, false, true> : general_tc_kernel<false, false, false, false, false, true>;
     else if (p.pair_taps && p.patch_w) kernel = b16 ? general_tc_kernel<true, false, true, true> : general_tc_kernel<false, false, true, true>;
     else if (p.pair_taps) kernel = b16 ? general_tc_kernel<true, false, false, true> : general_tc_kernel<false, false, false, true>;
     else if (p.patch_w) kernel = b16 ? general_tc_kernel<true, false, true, false> : general_tc_kernel<false, false, true, false>;

@@ -412,7 +412,9 @@ __device__ __forceinline__ void issue_tap(uint32_t d, uint32_t px_lo, uint32_t f
 // accumulators before the ordinary write-back.  No zero-fill of y, no atomic adds, and a + b = b + a keeps the
 // result independent of timing.
 // VIRT: zero padding and strides on virtual images (staged_pixel_virtual); flat addressing, fp32 operands.
-template <bool B16, bool FOLD, bool PATCH, bool STACK, bool CLUSTER = false, bool VIRT = false>
+// M64: at most 64 filters without stacked taps (the write-back takes two blocks at a time; in instances of its own, since as
+// run-time code it cost the 128-filter layers 1 %: more spills in roles that are at the register limit).
+template <bool B16, bool FOLD, bool PATCH, bool STACK, bool CLUSTER = false, bool VIRT = false, bool M64 = false>
 __global__ void __launch_bounds__(kThreads, 1)
 general_tc_kernel(const KernelArgs a)
 {
@@ -1110,7 +1112,7 @@ general_tc_kernel(const KernelArgs a)
                     continue;
                 }
                 uint32_t va0[16], va1[16], vb0[16], vb1[16], vax[1], vbx[1];
-                if (!STACK && !CLUSTER && rpq == 16 && a.vec >= 2 && !add) {
+                if (M64 && a.vec >= 2 && !add) {
                     // At most 64 filters (a quarter holds 16 maps): two 32-pixel blocks share the tile and one pass over it,
                     // each half of the warp stores one of them.  A block at a time the warps, not the MMAs or the memory,
                     // set the pace of short contractions (900 cycles per block, most of them the latency of the steps).
