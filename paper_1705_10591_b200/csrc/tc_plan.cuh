@@ -100,7 +100,7 @@ size_t smem_need(int a_stages, int npix, int n_tile, int b_stages, int tps, int 
 
 // b16: the operands are 16-bit floats, bf16 or fp16 (16-byte unit = 8 channels, 32 channels per staged block, K = 16 per MMA); the
 // byte layout of every stage is the same as for TF32 (16 channels of 4 bytes).
-Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool allow_compact = true, bool virt = false)
+Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool allow_compact = true, bool virt = false, bool narrow = false)
 {
     Plan p{};
     p.ok = false;
@@ -133,7 +133,8 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         }
         // outputs that can be stored as quads or pairs start on such a column of the accumulators, too
         const int unit = (st == 1 && sh.W % 4 == 0) || p.quad2 || (sh.Q % 4 == 0 && (long long)sh.P * sh.Q % 4 == 0) ? 4 : (sh.Q % 2 == 0 && (long long)sh.P * sh.Q % 2 == 0 ? 2 : 1);
-        p.virt_w = (p.virt_w + unit - 1) / unit * unit;
+        const int cols = narrow && unit == 4 ? 2 : unit;
+        p.virt_w = (p.virt_w + cols - 1) / cols * cols;
         if ((long long)p.virt_h * p.virt_w >= 1LL << 30) return p;
         sh.H = p.virt_h;
         sh.W = p.virt_w;
@@ -469,7 +470,14 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
 // where both take two rounds of equal items).
 Plan make_plan(const Shape& sh, bool b16 = false)
 {
-    if (sh.stride > 1) return plan_with_patch_width(sh, b16, 0, true, true);
+    if (sh.stride > 1) {
+        // Rows of a multiple of four columns allow 128-bit stores; where two columns less let the busiest block do a tenth
+        // less (28 columns of output need 30: 145 items of 192 pixels instead of 133 of 224), pairs are the better cut.
+        const Plan p = plan_with_patch_width(sh, b16, 0, true, true);
+        if (!p.ok || sh.stride != 2 || env_int("CONV2D_B200_TF32_NARROW", 1) == 0) return p;
+        const Plan q = plan_with_patch_width(sh, b16, 0, true, true, true);
+        return q.ok && q.makespan < 0.9 * p.makespan ? q : p;
+    }
     Plan best = plan_with_patch_width(sh, b16, 0);
     if (sh.pad_h != 0 || sh.pad_w != 0) {
         // Padding: virtual images, unless their rows are so wide that patches stage far fewer pixels.

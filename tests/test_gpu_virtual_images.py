@@ -26,6 +26,7 @@ STRIDED = [
     (2, 1, 40, 36, 5, 5, 5, 2, 2, 4), (1, 64, 9, 9, 32, 1, 1, 0, 0, 3), (1, 18, 12, 14, 12, 2, 5, 0, 2, 4),
     (16, 256, 14, 14, 256, 3, 3, 1, 1, 2), (2, 24, 33, 8, 100, 3, 1, 1, 0, 2), (1, 16, 20, 20, 8, 3, 3, 0, 0, 8),
     (1, 9, 64, 70, 12, 5, 3, 2, 1, 5),
+    (32, 16, 56, 56, 20, 3, 3, 1, 1, 2),     # rows of 30 columns instead of 32: fewer, smaller items
 ]
 
 
