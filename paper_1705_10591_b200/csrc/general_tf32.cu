@@ -151,9 +151,8 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
         while (p.pair_compact == 0 && tap_rows * 2 <= (unsigned)p.taps && blocks * tap_rows * 2 <= sm_count() * 4LL) tap_rows *= 2;
         const int all_taps = p.phases > 1 ? sh.R * sh.S : p.taps;
         const int bank_blocks = p.cblks / p.phases;
-        const size_t tile_bytes = (size_t)8 * kCB * 4 * all_taps;     // 8 filters x one channel block x taps
-        const bool tiled = p.fold_r * p.fold_s == 1 && !p.mixed && tile_bytes <= 48 * 1024 && p.n_tile % 8 == 0 && !p.pair_taps;
-        if (p.phases > 1 && !tiled) return CONV2D_ERR_UNSUPPORTED;
+        const size_t tile_bytes = repack_tile_bytes(all_taps);
+        const bool tiled = p.fold_r * p.fold_s == 1 && !p.mixed && tile_bytes <= kRepackTileLimit && p.n_tile % 8 == 0 && !p.pair_taps;
         if (tiled) {
             const dim3 grid((unsigned)(p.n_blocks * p.n_tile / 8), (unsigned)bank_blocks);
             int threads = (8 * kChunks * all_taps + 31) / 32 * 32;        // one 16-byte unit per thread in the store phase

@@ -92,6 +92,10 @@ struct Plan {
 // at the same time (each lane rotates its chunk order), and the eight lanes of a store phase cover all banks.
 inline int chunk_stride(int npix) { return npix + 1; }
 
+// Shared memory of the re-ordering kernel that works in tiles (8 filters x one channel block x `taps`), and its limit.
+constexpr size_t kRepackTileLimit = 48 * 1024;
+inline size_t repack_tile_bytes(int taps) { return (size_t)8 * kCB * 4 * taps; }
+
 // b_stages counts filter stages of `tps` taps each; an activation stage holds `cbg` channel blocks.
 size_t smem_need(int a_stages, int npix, int n_tile, int b_stages, int tps, int cbg)
 {
@@ -201,6 +205,9 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
             // (with quad2 the two phases of a row are one block of 32 staged channels with the taps of both)
             if (p.quad2) { p.phases /= p.phase_cols; p.phase_cols = 1; }
             p.cblks *= p.phases;
+            // (only the tiled re-ordering kernel groups the taps by phase; refused here and not where the filters are
+            // re-ordered, so that a call that finds them packed takes the same path as the call that packed them)
+            if (p.phases > 1 && repack_tile_bytes(sh.R * sh.S) > kRepackTileLimit) return p;
         }
     }
     const int stage_blocks = p.quad2 && !p.mixed ? 2 : 1;    // 16-channel blocks of a channel block
@@ -230,7 +237,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     // (CONV2D_B200_TF32_PAIR_COMPACT = 1 turns it on) until the write-back is faster than the MMAs.
     p.pair_compact = 0;
     const size_t compact_cb_bytes = (size_t)r_eff * ((s_eff / 2) * 128 + (s_eff & 1) * 64) * kCB * 4;
-    if (allow_compact && !p.pair_taps && p.swap && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
+    if (allow_compact && !p.pair_taps && p.swap && st == 1 && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
         !padded && (size_t)((c_eff + cbc - 1) / cbc) * compact_cb_bytes <= 152 * 1024 && env_int("CONV2D_B200_TF32_PAIR_COMPACT", 0) != 0) {
         p.pair_taps = 1;
         p.pair_compact = 1;

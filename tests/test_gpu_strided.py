@@ -64,10 +64,18 @@ def test_strided_matches_subsampled_oracle(oracle, case, algo, tol):
     np.testing.assert_array_equal(_run(xi, wi, ph, pw, st, algo)[0].astype(np.float64), yi_ref)
 
 
-def test_strided_prepacked_filters(oracle):
+@pytest.mark.parametrize("case", [
+    (2, 16, 20, 20, 130, 3, 3, 1, 1, 2),
+    # around 96 taps, beyond which the phases of a stride cannot be re-ordered apart: both calls have to take the same path
+    (1, 16, 24, 24, 20, 8, 12, 0, 0, 2), (2, 16, 32, 32, 32, 11, 11, 5, 5, 2), (1, 16, 35, 31, 24, 11, 11, 2, 2, 4),
+    (1, 64, 20, 24, 40, 10, 10, 0, 0, 2),
+])
+def test_strided_prepacked_filters(oracle, case):
     import paper_1705_10591_b200 as lib
-    N, C, H, W, K, R, S, ph, pw, st = 2, 16, 20, 20, 130, 3, 3, 1, 1, 2
+    N, C, H, W, K, R, S, ph, pw, st = case
     x, w = uniform((N, C, H, W), 485), uniform((K, C, R, S), 486)
     y1, ws = _run(x, w, ph, pw, st, 2)
+    y_ref, yabs = _reference(oracle, x, w, ph, pw, st)
+    assert_parity(y1, y_ref, yabs, TF32_TOL, f"strided {case}")
     y2, _ = _run(x, w, ph, pw, st, 2, flags=lib.FLAG_WEIGHTS_PACKED, ws=ws)
     np.testing.assert_array_equal(y1, y2)
