@@ -1,7 +1,10 @@
 // Internal declarations shared by the translation units of libconv2d_b200.
 #pragma once
 
+#include <atomic>
 #include <cstdlib>
+#include <mutex>
+
 #include <cuda_runtime.h>
 #include <stddef.h>
 #include <stdint.h>
@@ -33,17 +36,31 @@ cudaError_t latch_status(const void* workspace, cudaStream_t stream);
 // Every kernel launch goes through this so that conv2d_launch_count() is exact.
 void count_launch(int launches = 1);
 
-// Raises a kernel's dynamic shared-memory limit to `bytes` unless this call site already did so on the
-// current device (`done`: one static array per call site, i.e. per kernel instance).  The runtime call costs a
-// few microseconds, which matters for kernels that run for ten.
-inline cudaError_t raise_smem_limit(const void* kernel, size_t bytes, size_t (&done)[64])
+// Largest dynamic shared-memory limit set so far for one kernel, per device: one static object per kernel instance.
+struct SmemLimit { std::atomic<size_t> set[64]; };
+
+// Raises a kernel's dynamic shared-memory limit to `bytes` unless it is there already on the current device.  The runtime
+// call costs a few microseconds, which matters for kernels that run for ten, and it would lower the limit as well: the
+// planners choose sizes by the shape, so threads with different shapes meet here on one kernel, and the test, the call and
+// the record are one step under a lock.
+inline cudaError_t raise_smem_limit(const void* kernel, size_t bytes, SmemLimit& limit)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64 && done[dev] >= bytes) return cudaSuccess;
+    const bool recorded = dev >= 0 && dev < 64;
+    if (recorded && limit.set[dev].load(std::memory_order_acquire) >= bytes) return cudaSuccess;
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    if (recorded) {
+        if (limit.set[dev].load(std::memory_order_relaxed) >= bytes) return cudaSuccess;
+    } else {
+        cudaFuncAttributes a{};
+        e = cudaFuncGetAttributes(&a, kernel);
+        if (e != cudaSuccess || a.maxDynamicSharedSizeBytes >= (int)bytes) return e;
+    }
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev] = bytes;
+    if (e == cudaSuccess && recorded) limit.set[dev].store(bytes, std::memory_order_release);
     return e;
 }
 

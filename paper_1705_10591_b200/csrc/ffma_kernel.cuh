@@ -304,7 +304,7 @@ template <int R, int S, int CB, int TQ, bool ALIGNED>
 conv2d_status_t launch_split(const float* x, const float* w, float* y, const Shape& sh, const FfmaSplit& f, cudaStream_t stream)
 {
     auto kern = general_ffma_kernel<R, S, CB, TQ, ALIGNED>;
-    static size_t smem_done[64] = {};
+    static SmemLimit smem_done;
     if (f.smem > 48 * 1024 && raise_smem_limit(reinterpret_cast<const void*>(kern), f.smem, smem_done) != cudaSuccess)
         return CONV2D_ERR_CUDA;
     FfmaArgs a{};

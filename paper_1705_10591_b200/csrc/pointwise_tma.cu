@@ -722,7 +722,7 @@ conv2d_status_t launch_pw(const void* x, const void* w, float* y, const Shape& s
         if (!encode_map(&map_y, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, y, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B))
             return CONV2D_ERR_UNSUPPORTED;
     }
-    static size_t smem_done[64] = {}, smem_done_pair[64] = {};
+    static SmemLimit smem_done, smem_done_pair;
     if ((p.pair ? raise_smem_limit(reinterpret_cast<const void*>(pointwise_tma_kernel<B16, true>), p.smem_bytes, smem_done_pair)
                 : raise_smem_limit(reinterpret_cast<const void*>(pointwise_tma_kernel<B16, false>), p.smem_bytes, smem_done)) != cudaSuccess)
         return CONV2D_ERR_CUDA;

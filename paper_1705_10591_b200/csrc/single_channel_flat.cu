@@ -282,7 +282,7 @@ conv2d_status_t launch_flat(FlatArgs& a, const Shape& sh, cudaStream_t stream)
     const long long blocks = (long long)sh.N * a.col_tiles * a.bands * a.splits;
     if (blocks > 0x7fffffffLL) return CONV2D_ERR_UNSUPPORTED;
     auto kern = single_channel_flat_kernel<RT, S, M, TURN>;
-    static size_t smem_done[64] = {};
+    static SmemLimit smem_done;
     if (best_smem > 48 * 1024 && raise_smem_limit(reinterpret_cast<const void*>(kern), best_smem, smem_done) != cudaSuccess)
         return CONV2D_ERR_CUDA;
     kern<<<(unsigned)blocks, best_threads, best_smem, stream>>>(a);
