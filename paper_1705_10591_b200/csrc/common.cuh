@@ -30,9 +30,6 @@ constexpr size_t kStatusBytes = 256;
 // Returns cudaSuccess and sets *raised, or the CUDA error.  The stream must already be idle.
 cudaError_t consume_device_timeout(bool* raised);
 
-// Raises that word if the status block at the start of `workspace` shows a time-out (stream-ordered).
-cudaError_t latch_status(const void* workspace, cudaStream_t stream);
-
 // Every kernel launch goes through this so that conv2d_launch_count() is exact.
 void count_launch(int launches = 1);
 

@@ -103,6 +103,19 @@ bool strided_geom(int C, int H, int W, int R, int S, int pad_h, int pad_w, int s
     return true;
 }
 
+// Keeps a time-out that the status block of one group shows beyond the next group's call, which clears the block: in a word
+// of this call's own, since another thread's status query reads and clears the device's words.
+__global__ void latch_status_kernel(const unsigned* status, unsigned* timed_out)
+{
+    if (*status != 0) *timed_out = 1u;
+}
+cudaError_t latch_status(const void* workspace, unsigned* timed_out, cudaStream_t stream)
+{
+    latch_status_kernel<<<1, 1, 0, stream>>>(static_cast<const unsigned*>(workspace), timed_out);
+    count_launch();
+    return cudaGetLastError();
+}
+
 conv2d_status_t check_device()
 {
     int dev = 0;
@@ -379,10 +392,12 @@ constexpr int kKeptSets = 4;
 struct CopySet {
     cudaStream_t in = nullptr, out = nullptr;
     cudaEvent_t begin = nullptr, end = nullptr, arrived[kMaxChunks] = {}, done[kMaxChunks] = {};
+    unsigned* timed_out = nullptr;      // page-locked: a group of this call gave up on a bounded wait
     bool make()
     {
         bool ok = cudaStreamCreateWithFlags(&in, cudaStreamNonBlocking) == cudaSuccess &&
-                  cudaStreamCreateWithFlags(&out, cudaStreamNonBlocking) == cudaSuccess;
+                  cudaStreamCreateWithFlags(&out, cudaStreamNonBlocking) == cudaSuccess &&
+                  cudaHostAlloc(reinterpret_cast<void**>(&timed_out), sizeof(unsigned), cudaHostAllocMapped) == cudaSuccess;
         auto event = [&](cudaEvent_t& e) { ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess; };
         event(begin); event(end);
         for (int i = 0; i < kMaxChunks; ++i) { event(arrived[i]); event(done[i]); }
@@ -396,6 +411,7 @@ struct CopySet {
         if (end) cudaEventDestroy(end);
         if (in) cudaStreamDestroy(in);
         if (out) cudaStreamDestroy(out);
+        if (timed_out) cudaFreeHost(timed_out);
         *this = CopySet();
     }
 };
@@ -488,6 +504,7 @@ conv2d_status_t conv2d_fwd_host(const float* x_host, const float* w_host, float*
     }
     // Copies in on one stream, convolutions on the caller's, copies out on another; everything after what the caller's
     // stream holds already, and the caller's stream ends after the last copy.
+    *set.timed_out = 0;
     bool ok = cudaEventRecord(set.begin, stream) == cudaSuccess && cudaStreamWaitEvent(set.in, set.begin, 0) == cudaSuccess &&
               cudaMemcpyAsync(w, w_host, wb, cudaMemcpyHostToDevice, set.in) == cudaSuccess;
     int chunks = 0;
@@ -502,7 +519,7 @@ conv2d_status_t conv2d_fwd_host(const float* x_host, const float* w_host, float*
         if (!ok) break;
         st = host_images(x + n0 * xn, w, y + n0 * yn, images, C, H, W, K, R, S, algo, workspace, workspace_bytes, cuda_stream, &status_in_workspace);
         if (st != CONV2D_OK) break;
-        ok = (!status_in_workspace || latch_status(workspace, stream) == cudaSuccess) &&
+        ok = (!status_in_workspace || latch_status(workspace, set.timed_out, stream) == cudaSuccess) &&
              cudaEventRecord(set.done[i], stream) == cudaSuccess && cudaStreamWaitEvent(set.out, set.done[i], 0) == cudaSuccess &&
              cudaMemcpyAsync(y_host + n0 * yn, y + n0 * yn, images * yn * sizeof(float), cudaMemcpyDeviceToHost, set.out) == cudaSuccess;
     }
@@ -510,10 +527,15 @@ conv2d_status_t conv2d_fwd_host(const float* x_host, const float* w_host, float*
     // (nothing of the call is pending when it returns, after an error either)
     ok = cudaStreamSynchronize(set.in) == cudaSuccess && ok;
     ok = cudaStreamSynchronize(set.out) == cudaSuccess && ok;
+    ok = cudaStreamSynchronize(stream) == cudaSuccess && ok;
+    const bool timed_out = *static_cast<volatile unsigned*>(set.timed_out) != 0;
     give_set(dev, &set);
     if (st != CONV2D_OK) return st;
     if (!ok) return CONV2D_ERR_CUDA;
-    return conv2d_get_status(status_in_workspace ? workspace : nullptr, cuda_stream);
+    // (the workspace shows the time-out of any group, as it does after a call that convolves all images at once)
+    if (timed_out && cudaMemsetAsync(workspace, 1, sizeof(unsigned), stream) != cudaSuccess) return CONV2D_ERR_CUDA;
+    st = conv2d_get_status(nullptr, cuda_stream);
+    return st == CONV2D_OK && timed_out ? CONV2D_ERR_DEVICE_TIMEOUT : st;
 }
 
 conv2d_status_t conv2d_get_status(const void* workspace, void* cuda_stream)

@@ -983,18 +983,6 @@ static bool take_flat(const Shape& sh)
     return true;
 }
 
-// Keeps a time-out that the status block of one call shows beyond the next call on the same block, which clears it.
-__global__ void latch_status_kernel(const unsigned* status)
-{
-    if (*status != 0) atomicExch(&g_device_timeout, 1u);
-}
-cudaError_t latch_status(const void* workspace, cudaStream_t stream)
-{
-    latch_status_kernel<<<1, 1, 0, stream>>>(static_cast<const unsigned*>(workspace));
-    count_launch();
-    return cudaGetLastError();
-}
-
 conv2d_status_t launch_single_channel(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream)
 {
     if (take_flat(sh)) {

@@ -47,3 +47,62 @@ def test_two_threads(oracle):
     for i in range(2):
         y_ref, _ = oracle.conv2d_oracle(*inputs[i])
         np.testing.assert_array_equal(results[i].astype(np.float64), y_ref)
+
+
+def test_time_out_of_an_early_group_reaches_its_own_call(oracle, monkeypatch):
+    """Host-side injection: the 37th filter copy of a block is armed but never issued, and the wait bound is short.  With
+    items of 64 pixels and one tap a copy, only blocks that get a second item come that far: those of the groups of two
+    images, not those of the last group of one.  Another thread asks for the device's status all the while: the time-out
+    belongs to the host call and must not reach that thread."""
+    import torch
+    import paper_1705_10591_b200 as lib
+    N, C, H, W, K = 9, 64, 96, 96, 128
+    x, w = small_integers((N, C, H, W), 1711), small_integers((K, C, 3, 3), 1712)
+    y_ref, _ = oracle.conv2d_oracle(x, w)
+    xh, wh = torch.from_numpy(x).pin_memory(), torch.from_numpy(w).pin_memory()
+    yh = torch.zeros((N, K, H - 2, W - 2)).pin_memory()
+    xd, wd, yd = (torch.empty(t.shape, device="cuda:0") for t in (xh, wh, yh))
+    nbytes = lib.conv2d_fwd_workspace_size(N, C, H, W, K, 3, 3, ALGO_TF32)
+    ws = torch.zeros(nbytes, dtype=torch.uint8, device="cuda:0")
+
+    def call():
+        lib.conv2d_fwd_host(xh.data_ptr(), wh.data_ptr(), yh.data_ptr(), xd.data_ptr(), wd.data_ptr(), yd.data_ptr(),
+                            N, C, H, W, K, 3, 3, ALGO_TF32, ws.data_ptr(), nbytes, torch.cuda.current_stream().cuda_stream)
+    monkeypatch.setenv("CONV2D_B200_TF32_TILE_PX", "64")
+    monkeypatch.setenv("CONV2D_B200_TF32_STAGE_KB", "8")
+    call()
+    np.testing.assert_array_equal(yh.numpy().astype(np.float64), y_ref)
+    stop, stolen, asked = threading.Event(), [], []
+
+    def ask():
+        stream = torch.cuda.Stream()
+        while not stop.is_set():
+            try:
+                lib.conv2d_get_status(0, stream.cuda_stream)
+                asked.append(1)
+            except lib.Conv2dError as e:
+                stolen.append(e.status)
+    thread = threading.Thread(target=ask)
+    thread.start()
+    monkeypatch.setenv("CONV2D_B200_TF32_MAX_POLLS", "20000")
+    monkeypatch.setenv("CONV2D_B200_TF32_TEST_DROP_STAGE", "36")
+    reported, shown = [], []
+    for _ in range(5):
+        yh.zero_()
+        try:
+            call()
+            reported.append(0)
+        except lib.Conv2dError as e:
+            reported.append(e.status)
+        shown.append(int(ws[:4].sum()))
+    monkeypatch.delenv("CONV2D_B200_TF32_MAX_POLLS")
+    monkeypatch.delenv("CONV2D_B200_TF32_TEST_DROP_STAGE")
+    stop.set()
+    thread.join()
+    np.testing.assert_array_equal(yh.numpy()[-1].astype(np.float64), y_ref[-1])       # (the last group did not time out)
+    assert asked and not stolen
+    assert reported == [8] * 5                      # CONV2D_ERR_DEVICE_TIMEOUT
+    assert all(shown)                               # and the status block shows it
+    call()
+    lib.conv2d_get_status(ws.data_ptr(), 0)
+    np.testing.assert_array_equal(yh.numpy().astype(np.float64), y_ref)
