@@ -454,6 +454,7 @@ static conv2d_status_t host_images(const float* x, const float* w, float* y, int
 // is at least 4 MB of copies, keeps x and y 16-byte aligned, and runs the same algorithm as the whole call would.
 static int images_per_copy(const Shape& sh, conv2d_algo_t algo, const void* workspace, size_t workspace_bytes)
 {
+    if (sh.C == 1 && algo != CONV2D_ALGO_TF32 && sh.N > 65535) return sh.N;       // (the single-channel entry refuses the call, not its groups)
     const long long in = (long long)sh.C * sh.H * sh.W, out = (long long)sh.K * sh.P * sh.Q;      // floats of an image
     long long chunks = sh.N * (in + out) * 4 / (4 << 20);
     if (chunks > kMaxChunks) chunks = kMaxChunks;

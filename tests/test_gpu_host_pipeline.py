@@ -29,6 +29,14 @@ def test_exact_on_integers(oracle, case, pinned):
     np.testing.assert_array_equal(_host_call(x, w, algo, pinned, workspace).astype(np.float64), y_ref)
 
 
+def test_a_batch_the_single_channel_entry_refuses_is_not_accepted_in_groups():
+    import paper_1705_10591_b200 as lib
+    x, w = np.zeros((70000, 1, 8, 8), np.float32), np.zeros((1, 1, 3, 3), np.float32)
+    with pytest.raises(lib.Conv2dError) as e:
+        _host_call(x, w, ALGO_AUTO, False, "none")
+    assert e.value.status == 5                      # CONV2D_ERR_UNSUPPORTED
+
+
 def test_two_threads(oracle):
     import torch
     xs, ws, algo, workspace = CASES[0]
