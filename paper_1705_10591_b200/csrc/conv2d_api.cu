@@ -492,7 +492,10 @@ conv2d_status_t conv2d_fwd_host(const float* x_host, const float* w_host, float*
     // Only the tensor-core launcher clears and uses the status block in the workspace; after any other kernel the
     // workspace (which may be NULL, of size 0, or never written) must not be read for a status.
     bool status_in_workspace = false;
-    const int per = images_per_copy(sh, algo, workspace, workspace_bytes);
+    int per = images_per_copy(sh, algo, workspace, workspace_bytes);
+    // (a call that waits for its stream fails while that stream is captured; the streams of a set must not join the capture)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (per < N && (cudaStreamIsCapturing(stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone)) per = N;
     int dev = 0;
     CopySet set;
     if (per >= N || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || !take_set(dev, &set)) {
@@ -530,7 +533,8 @@ conv2d_status_t conv2d_fwd_host(const float* x_host, const float* w_host, float*
     ok = cudaStreamSynchronize(set.out) == cudaSuccess && ok;
     ok = cudaStreamSynchronize(stream) == cudaSuccess && ok;
     const bool timed_out = *static_cast<volatile unsigned*>(set.timed_out) != 0;
-    give_set(dev, &set);
+    if (ok) give_set(dev, &set);
+    else set.destroy();                 // (what state its streams are in is not known)
     if (st != CONV2D_OK) return st;
     if (!ok) return CONV2D_ERR_CUDA;
     // (the workspace shows the time-out of any group, as it does after a call that convolves all images at once)

@@ -37,6 +37,44 @@ def test_a_batch_the_single_channel_entry_refuses_is_not_accepted_in_groups():
     assert e.value.status == 5                      # CONV2D_ERR_UNSUPPORTED
 
 
+def test_a_call_on_a_captured_stream_leaves_the_other_calls_alone(oracle):
+    """The call waits for its stream, so it fails under capture; until that capture ends, a call of another thread on a
+    stream of its own must neither fail nor be drawn into it."""
+    import torch
+    import paper_1705_10591_b200 as lib
+    rt = pytest.importorskip("cuda.bindings.runtime")
+    xs, ws, algo, workspace = CASES[1]
+    x, w = small_integers(xs, 1707), small_integers(ws, 1708)
+    y_ref, _ = oracle.conv2d_oracle(x, w)
+    N, C, H, W = xs
+    xh, wh = torch.from_numpy(x).pin_memory(), torch.from_numpy(w).pin_memory()
+    yh = torch.zeros(y_ref.shape).pin_memory()
+    xd, wd, yd = (torch.empty(t.shape, device="cuda:0") for t in (xh, wh, yh))
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    outcome = {}
+
+    def captured():
+        (err,) = rt.cudaStreamBeginCapture(stream.cuda_stream, rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed)
+        outcome["begin"] = int(err)
+        try:
+            lib.conv2d_fwd_host(xh.data_ptr(), wh.data_ptr(), yh.data_ptr(), xd.data_ptr(), wd.data_ptr(), yd.data_ptr(),
+                                N, C, H, W, ws[0], ws[2], ws[3], algo, 0, 0, stream.cuda_stream)
+        except lib.Conv2dError as e:
+            outcome["captured"] = e.status
+
+    def free():
+        with torch.cuda.stream(torch.cuda.Stream()):
+            outcome["free"] = _host_call(x, w, algo, True, workspace)
+    for part in (captured, free):                   # (threads: a runtime error stays with the thread that met it)
+        thread = threading.Thread(target=part)
+        thread.start()
+        thread.join()
+    rt.cudaStreamEndCapture(stream.cuda_stream)
+    assert outcome["begin"] == 0 and outcome["captured"] == 7                    # CONV2D_ERR_CUDA
+    np.testing.assert_array_equal(outcome["free"].astype(np.float64), y_ref)
+
+
 def test_two_threads(oracle):
     import torch
     xs, ws, algo, workspace = CASES[0]
