@@ -261,6 +261,7 @@ FfmaSplit split_ffma(const Shape& sh)
         if (kb > kgroups) continue;
         f.groups = (kgroups + kb - 1) / kb;
         f.kblocks = (kgroups + f.groups - 1) / f.groups;
+        if (f.kblocks > 65535) continue;
         // (warp w of every block sits on scheduler w % 4: other counts leave two schedulers with half the work, 64 x 128 x
         // 32 x 32, 128 filters of 3 x 3: 381 us with 4 warps, 407 with 8, 441 with 6)
         for (int warps : {2, 4, 8}) {
@@ -337,7 +338,7 @@ conv2d_status_t launch_instance(const float* x, const float* w, float* y, const 
     const int forced = env_int("CONV2D_B200_FFMA_TILE", -1);
     if (forced >= 0 && forced <= 6 && by_tile[forced]) tq = by_tile[forced];
     const FfmaSplit& f = tq == 6 ? f6 : (tq == 7 ? f7 : f8);
-    if (f.cost == 0 || f.seg_blocks > 0x7fffffffLL || f.kblocks > 65535) return CONV2D_ERR_UNSUPPORTED;
+    if (f.cost == 0 || f.seg_blocks > 0x7fffffffLL) return CONV2D_ERR_UNSUPPORTED;
     const bool x4 = f.x4 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
 #define CONV2D_FFMA_LAUNCH(TQ) \
     return x4 ? launch_split<R, S, CB, TQ, true>(x, w, y, sh, f, stream) : launch_split<R, S, CB, TQ, false>(x, w, y, sh, f, stream)

@@ -49,17 +49,27 @@ conv2d_status_t launch_direct_fallback(const float* x, const float* w, float* y,
     return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
 }
 
+namespace {
+conv2d_status_t launch_tuned(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream)
+{
+    if (sh.R != sh.S) return CONV2D_ERR_UNSUPPORTED;
+    switch (sh.R) {
+    case 1: return launch_ffma_1x1(x, w, y, sh, stream);
+    case 2: return launch_ffma_2x2(x, w, y, sh, stream);                          // (stride-2 rewriting of 3 x 3)
+    case 3: return launch_ffma_3x3(x, w, y, sh, stream);
+    case 4: return launch_ffma_4x4(x, w, y, sh, stream);                          // (stride-2 rewriting of 7 x 7)
+    case 5: return launch_ffma_5x5(x, w, y, sh, stream);
+    case 7: return launch_ffma_7x7(x, w, y, sh, stream);
+    }
+    return CONV2D_ERR_UNSUPPORTED;
+}
+}  // namespace
+
 conv2d_status_t launch_general_ffma(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream)
 {
-    constexpr int kFiltersPerBlock = 64;                     // (kTileK of the tuned kernel: grid.y counts blocks of 64 filters)
-    if (sh.N > 65535 || (sh.K + kFiltersPerBlock - 1) / kFiltersPerBlock > 65535) return launch_direct_fallback(x, w, y, sh, stream);
-    if (sh.R == 1 && sh.S == 1) return launch_ffma_1x1(x, w, y, sh, stream);
-    if (sh.R == 2 && sh.S == 2) return launch_ffma_2x2(x, w, y, sh, stream);      // (stride-2 rewriting of 3 x 3)
-    if (sh.R == 3 && sh.S == 3) return launch_ffma_3x3(x, w, y, sh, stream);
-    if (sh.R == 4 && sh.S == 4) return launch_ffma_4x4(x, w, y, sh, stream);      // (stride-2 rewriting of 7 x 7)
-    if (sh.R == 5 && sh.S == 5) return launch_ffma_5x5(x, w, y, sh, stream);
-    if (sh.R == 7 && sh.S == 7) return launch_ffma_7x7(x, w, y, sh, stream);
-    return launch_direct_fallback(x, w, y, sh, stream);
+    // (the tuned kernel numbers the rows of the whole batch in 32 bits: what does not fit is computed all the same)
+    const conv2d_status_t st = launch_tuned(x, w, y, sh, stream);
+    return st == CONV2D_ERR_UNSUPPORTED ? launch_direct_fallback(x, w, y, sh, stream) : st;
 }
 
 }  // namespace conv2d_b200

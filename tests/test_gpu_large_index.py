@@ -1,4 +1,5 @@
-"""Outputs with more than 2^31 elements: every kernel family must index y with 64 bits.
+"""Outputs with more than 2^31 elements: every kernel family must index y with 64 bits.  Batches with more rows or images than
+the fp32 kernel numbers.
 
 The output tensors here are 9-10 GB and stay on the device; only sampled rows are read back and compared with the
 oracle, among them rows at the very end of y and rows on both sides of element 2^31.
@@ -85,3 +86,32 @@ def test_general_output_beyond_2_to_31_elements(oracle, algo, tol):
     x, w = uniform((N, C, H, W), 443), uniform((K, C, R, S), 444)
     yd = _run_on_device(x, w, "general", algo)
     _check(oracle, x, w, yd, tol, f"general algo {algo}, 9.6 GB of output")
+
+
+@pytest.mark.parametrize("algo", [1, 0])
+def test_batch_with_more_rows_than_32_bits_number(algo):
+    """The tuned fp32 kernel numbers the image rows of the whole batch; beyond that the call is computed all the same."""
+    import torch
+    import paper_1705_10591_b200 as lib
+    if _free_bytes() < 22 * 2 ** 30:
+        pytest.skip("needs 22 GB of free device memory")
+    N, H = 40000, 53700
+    assert N * H > 2 ** 31
+    x = torch.arange(H, device="cuda:0", dtype=torch.float32).repeat(N, 1)
+    x += torch.arange(N, device="cuda:0", dtype=torch.float32)[:, None]          # (sums below 2^24: exact)
+    y = torch.full_like(x, float("nan"))
+    w = torch.full((1, 1, 1, 1), 0.5, device="cuda:0")
+    lib.conv2d_fwd_general(x.data_ptr(), w.data_ptr(), y.data_ptr(), N, 1, H, 1, 1, 1, 1, algo, 0, 0, 0,
+                           torch.cuda.current_stream().cuda_stream)
+    x *= 0.5
+    assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("dims", [(70000, 2, 4, 5, 9, 3, 3), (2, 3, 4, 4, 65536 * 8 + 5, 3, 3)])      # many images; many filters
+def test_fp32_kernel_takes_long_batches_and_banks(oracle, dims):
+    from helpers import run_library
+    from workloads import small_integers
+    N, C, H, W, K, R, S = dims
+    x, w = small_integers((N, C, H, W), 445), small_integers((K, C, R, S), 446)
+    y_ref, _ = oracle.conv2d_oracle(x, w)
+    np.testing.assert_array_equal(run_library(x, w, entry="general", algo=1).astype(np.float64), y_ref)
