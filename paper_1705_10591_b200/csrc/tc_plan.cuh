@@ -470,6 +470,39 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     return p;
 }
 
+// Rough cycles of the busiest block: its MMAs, its producers (7 cycles per staged pixel and channel block, 5 where they load
+// quads, a round trip to memory per block at least) and its write-back, which overlap for the most part; and the zero-fill
+// and adds of a contraction split without a cluster (4.5 us).  Fitted to the times of 2000 random padded layers on virtual
+// images and in patches (standard deviation 19 %).
+double estimated_cycles(const Plan& p, bool quads)
+{
+    const int sms = sm_count();
+    const double rounds = (double)(((long long)p.supertiles * p.n_blocks * p.ksplit + sms - 1) / sms);
+    const double load = p.npix * (quads ? 5.0 : 7.0);
+    const double mma = p.makespan / p.ksplit, stage = rounds * p.cblks / p.ksplit * (load > 1400.0 ? load : 1400.0);
+    const double store = rounds * p.tile_px / 32.0 * (p.n_tile == 128 && !p.pair_taps ? 800.0 : 500.0);
+    const double most = mma > stage ? (mma > store ? mma : store) : (stage > store ? stage : store);
+    return 0.6 * most + 0.4 * (mma + stage + store) + (p.ksplit == 2 && !p.cluster ? 9000.0 : 0.0);
+}
+
+// Where patches are the better cut for zero padding.  Of 2070 random layers 112 were slower by 4 % and more on virtual images
+// than in patches, 52 by more than 10 % (all layers together 14 % faster); with these rules it is about 70 and 23:
+bool patches_beat_virtual(const Plan& v, const Plan& patch, const Shape& sh)
+{
+    const int sms = sm_count();
+    const bool quads = sh.W % 4 == 0;
+    // a short contraction that only the virtual images split without a cluster: 5 x 80 x 65 x 33, 48 maps of 3 x 3 20.7 us
+    // on virtual images, 15.4 in patches (many channels earn the split back: 9 x 256 x 116 x 10, 6 of 2 x 2 18.6 and 26.1)
+    if (v.ksplit == 2 && !v.cluster && v.cblks <= 8 && patch.ksplit == 1 && patch.makespan < 10000.0) return true;
+    // clearly more staged pixels than the producers load in a pass (1024 in quads), stage after stage, or any of more than 1300:
+    // 55 x 44 x 66 x 170, 7 maps of 5 x 5 259 and 188 us; 21 x 16 x 37 x 184, 4 of 7 x 7 67 and 40; 11 of 13 layers
+    const long long stages = ((long long)v.supertiles * v.n_blocks * v.ksplit + sms - 1) / sms * v.cblks / v.ksplit;
+    if (v.npix > 1300 || (quads && v.npix > 1100 && stages >= 3)) return true;
+    // a clear difference of the estimates: 2 x 272 x 51 x 247, 11 maps of 3 x 3 48 and 35 us
+    const double ev = estimated_cycles(v, quads), ep = estimated_cycles(patch, quads && sh.pad_w % 4 == 0);
+    return ev > 1.25 * ep && ev - ep > 6000.0;
+}
+
 // The patch width with the fewest staged pixels per output is the first choice.  A wider patch has a larger valid
 // fraction (fewer MMA columns that only feed the next patch) and may need fewer rounds of items over the SMs: it is
 // taken when the busiest block then has at least 5 % less MMA work (7 x 7 on 224 x 224, 64 -> 128 channels: 73 -> 61
@@ -486,11 +519,11 @@ Plan make_plan(const Shape& sh, bool b16 = false)
         return q.ok && q.makespan < 0.9 * p.makespan ? q : p;
     }
     Plan best = plan_with_patch_width(sh, b16, 0);
-    if (sh.pad_h != 0 || sh.pad_w != 0) {
-        // Padding: virtual images, unless their rows are so wide that patches stage far fewer pixels.
-        const int mode = env_int("CONV2D_B200_TF32_VIRT", 1);             // 0 never, 1 by the rule, 2 always
+    const int mode = env_int("CONV2D_B200_TF32_VIRT", 1);                 // 0 never, 1 by the rule, 2 always
+    if (mode != 0 && (sh.pad_h != 0 || sh.pad_w != 0)) {
+        // Padding: virtual images, unless their rows are so wide that patches stage far fewer pixels (and see above).
         const Plan v = plan_with_patch_width(sh, b16, 0, true, true);
-        if (v.ok && mode != 0 && (mode == 2 || !best.ok || !(v.staged_ratio > 1.75 * best.staged_ratio))) return v;
+        if (v.ok && (mode == 2 || !best.ok || !(v.staged_ratio > 1.75 * best.staged_ratio || patches_beat_virtual(v, best, sh)))) return v;
     }
     if (!best.ok || !best.patch_w || env_int("CONV2D_B200_TF32_PATCH_W", 0) != 0) return best;
     const int first = best.patch_w;

@@ -40,6 +40,18 @@ def test_padded_exact_on_integers(oracle, monkeypatch, case):
         np.testing.assert_array_equal(run_padded(x, w, ph, pw, 2).astype(np.float64), y_ref)
 
 
+@pytest.mark.parametrize("case", [
+    (5, 80, 65, 33, 48, 3, 3, 1, 1),         # a contraction that only virtual images would split
+    (21, 16, 37, 184, 4, 7, 7, 3, 3),        # more staged pixels than the producers load in a pass
+    (2, 272, 51, 247, 11, 3, 3, 1, 1),       # a clear difference of the estimates
+])
+def test_padded_layers_left_to_patches(oracle, case):
+    N, C, H, W, K, R, S, ph, pw = case
+    x, w = small_integers((N, C, H, W), 1607), small_integers((K, C, R, S), 1608)
+    y_ref, _ = oracle.conv2d_oracle(np.pad(x, ((0, 0), (0, 0), (ph, ph), (pw, pw))), w)
+    np.testing.assert_array_equal(run_padded(x, w, ph, pw, 2).astype(np.float64), y_ref)
+
+
 @pytest.mark.parametrize("case", STRIDED)
 def test_strided_exact_on_integers(oracle, case):
     N, C, H, W, K, R, S, ph, pw, st = case
