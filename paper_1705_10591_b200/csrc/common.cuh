@@ -139,6 +139,9 @@ size_t tf32_workspace_bytes(const Shape& sh);   // includes the status block
 // (returns CONV2D_ERR_UNSUPPORTED without an instance, CONV2D_ERR_WORKSPACE when workspace_bytes is too small)
 conv2d_status_t launch_general_tf32(const float* x, const float* w, float* y, const Shape& sh,
                                     void* workspace, size_t workspace_bytes, bool weights_packed, cudaStream_t stream);
+// A strided layer, and the stride-1 layer on stride*stride times as many channels that computes the same: whether rewriting the
+// image for the latter is faster than the strided layer on virtual images.
+bool rewriting_beats_virtual(const Shape& strided, const Shape& rewritten);
 
 // 1 x 1 filters with every operand moved by tensor-map (TMA) copies; `workspace` holds the status block and, for fp32
 // shapes with more channels than a resident filter bank takes, the filters rounded to TF32 (`weights_packed`: they

@@ -3,6 +3,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "ptx.cuh"
 
 namespace conv2d_b200 {
 
@@ -50,6 +51,8 @@ size_t round_up_256(size_t v) { return (v + 255) / 256 * 256; }
 //   x2[n][(c*st + a)*st + b][h2][w2] = xz[n][c][st*h2 + a][st*w2 + b]      (xz = zero-padded x, 0 outside)
 //   w2[k][(c*st + a)*st + b][r2][s2] = w[k][c][st*r2 + a][st*s2 + b]       (0 where st*r2 + a >= R or st*s2 + b >= S)
 // so that sum_{c,r,s} xz[c][st*p + r][st*q + s] w[k][c][r][s] = sum over (c,a,b),(r2,s2) of x2[..][p + r2][q + s2] w2[..].
+// ROUND: the tensor cores multiply the result, so it is written rounded to the nearest TF32 (the 1 x 1 kernel would cut it off).
+template <bool ROUND>
 __global__ void space_to_depth_kernel(const float* __restrict__ x, float* __restrict__ x2, int H, int W,
                                       int pad_h, int pad_w, int st, int H2, int W2, unsigned* status_to_clear)
 {
@@ -64,9 +67,11 @@ __global__ void space_to_depth_kernel(const float* __restrict__ x, float* __rest
         const int a = ab / st, b = ab - a * st;
         const int h2 = rem / W2, w2 = rem - h2 * W2;
         const int h = st * h2 + a - pad_h, wc = st * w2 + b - pad_w;
-        dst[i] = (h >= 0 && h < H && wc >= 0 && wc < W) ? __ldg(src + h * W + wc) : 0.f;
+        const float v = (h >= 0 && h < H && wc >= 0 && wc < W) ? __ldg(src + h * W + wc) : 0.f;
+        dst[i] = ROUND ? ptx::to_tf32_rna(v) : v;
     }
 }
+template <bool ROUND>
 __global__ void filters_to_depth_kernel(const float* __restrict__ w, float* __restrict__ w2, int K, int C, int R, int S,
                                         int st, int R2, int S2)
 {
@@ -81,7 +86,8 @@ __global__ void filters_to_depth_kernel(const float* __restrict__ w, float* __re
         const int c = (int)(r % C); r /= C;
         const int k = (int)r;
         const int rr = st * r2 + a, ss = st * s2 + b;
-        w2[i] = (rr < R && ss < S) ? __ldg(w + (((size_t)k * C + c) * R + rr) * S + ss) : 0.f;
+        const float v = (rr < R && ss < S) ? __ldg(w + (((size_t)k * C + c) * R + rr) * S + ss) : 0.f;
+        w2[i] = ROUND ? ptx::to_tf32_rna(v) : v;
     }
 }
 
@@ -339,10 +345,13 @@ conv2d_status_t conv2d_fwd_general_strided(const float* x, const float* w, float
     st = check_device();
     if (st != CONV2D_OK) return st;
     // The tensor-core kernel computes strided convolutions on virtual images, straight from x and with as many
-    // multiplications as the definition has, wherever the rewritten problem would run there as well (inner > 0).
-    if (algo != CONV2D_ALGO_FFMA && inner > 0 && (long long)C * H * W <= 0x7fffffffLL) {
-        Shape shp{N, C, H, W, K, R, S, g.P, g.Q};
-        shp.pad_h = pad_h; shp.pad_w = pad_w; shp.stride = stride;
+    // multiplications as the definition has, wherever the rewritten problem would run there as well (inner > 0) and is not
+    // the faster one.
+    const bool tensor_cores = algo != CONV2D_ALGO_FFMA && inner > 0;
+    Shape shp{N, C, H, W, K, R, S, g.P, g.Q};
+    shp.pad_h = pad_h; shp.pad_w = pad_w; shp.stride = stride;
+    const Shape rewritten{N, g.C2, g.H2, g.W2, K, g.R2, g.S2, g.P, g.Q};
+    if (tensor_cores && (long long)C * H * W <= 0x7fffffffLL && !rewriting_beats_virtual(shp, rewritten)) {
         const conv2d_status_t native = launch_general_tf32(x, w, y, shp, workspace, workspace_bytes,
                                                            (flags & CONV2D_FLAG_WEIGHTS_PACKED) != 0,
                                                            static_cast<cudaStream_t>(cuda_stream));
@@ -357,12 +366,14 @@ conv2d_status_t conv2d_fwd_general_strided(const float* x, const float* w, float
     {
         const int work = stride * stride * g.H2 * g.W2;
         const dim3 grid((unsigned)((work + 1023) / 1024 > 64 ? 64 : (work + 1023) / 1024), (unsigned)(N * C));
-        space_to_depth_kernel<<<grid, 256, 0, stream>>>(x, x2, H, W, pad_h, pad_w, stride, g.H2, g.W2,
-                                                        own_status ? static_cast<unsigned*>(workspace) : nullptr);
+        auto kernel = tensor_cores ? space_to_depth_kernel<true> : space_to_depth_kernel<false>;
+        kernel<<<grid, 256, 0, stream>>>(x, x2, H, W, pad_h, pad_w, stride, g.H2, g.W2,
+                                         own_status ? static_cast<unsigned*>(workspace) : nullptr);
     }
     count_launch(1);
     if (!(flags & CONV2D_FLAG_WEIGHTS_PACKED)) {
-        filters_to_depth_kernel<<<blocks_for((long long)K * g.C2 * g.R2 * g.S2), 256, 0, stream>>>(w, w2, K, C, R, S, stride, g.R2, g.S2);
+        auto kernel = tensor_cores ? filters_to_depth_kernel<true> : filters_to_depth_kernel<false>;
+        kernel<<<blocks_for((long long)K * g.C2 * g.R2 * g.S2), 256, 0, stream>>>(w, w2, K, C, R, S, stride, g.R2, g.S2);
         count_launch(1);
     }
     if (cudaGetLastError() != cudaSuccess) return CONV2D_ERR_CUDA;

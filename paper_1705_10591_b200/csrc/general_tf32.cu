@@ -71,6 +71,25 @@ size_t tf32_workspace_bytes(const Shape& sh)
     return kStatusBytes + (general > pointwise ? general : pointwise);
 }
 
+// Windows that do not overlap (no filter larger than the stride) become 1 x 1 filters, and the 1 x 1 kernel moves the
+// rewritten image by tensor-map copies, while the virtual images of so many phases are gathered pixel by pixel, a phase a
+// stage.  Both estimated in us: launches, the re-ordering of the image and the longer contraction on one side (14 us, 1.4 a
+// MB, 1 per 200 channels, the output at 5.5 TB/s), the kernel's busiest block on the other.  Of 208 random layers of this
+// kind 33 were slower by 4 % and more on virtual images (3 x 352 x 54 x 54, 358 filters of 3 x 3, stride 3 77.0 us, rewritten 45.9;
+// 9 x 176 x 49 x 49, 16 of 5 x 5, stride 5 107 and 58), 8 are with this rule, by 8 % at most but for one; two lose 4 to 8 %.
+bool rewriting_beats_virtual(const Shape& strided, const Shape& rewritten)
+{
+    const int mode = env_int("CONV2D_B200_TF32_VIRT", 1);                 // 0 rewrite always, 1 by the rule, 2 never
+    if (mode != 1) return mode == 0;
+    if (rewritten.R != 1 || rewritten.S != 1 || !pointwise_tma_supported(rewritten, false)) return false;
+    const Plan p = make_plan(strided);
+    if (!p.ok) return true;
+    const double image_mb = 4e-6 * rewritten.N * rewritten.C * rewritten.H * rewritten.W;
+    const double output_mb = 4e-6 * strided.N * strided.K * strided.P * strided.Q;
+    const double virt_us = 10.0 + estimated_cycles(p, p.quad2 != 0) / 1900.0;
+    return virt_us > 1.1 * (14.0 + 1.4 * image_mb + rewritten.C / 200.0 + output_mb / 5.5);
+}
+
 bool b16_supported(const Shape& sh)
 {
     return make_plan(sh, true).ok || pointwise_tma_supported(sh, true);

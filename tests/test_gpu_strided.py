@@ -79,3 +79,26 @@ def test_strided_prepacked_filters(oracle, case):
     assert_parity(y1, y_ref, yabs, TF32_TOL, f"strided {case}")
     y2, _ = _run(x, w, ph, pw, st, 2, flags=lib.FLAG_WEIGHTS_PACKED, ws=ws)
     np.testing.assert_array_equal(y1, y2)
+
+
+@pytest.mark.parametrize("case", [
+    (2, 80, 30, 30, 48, 5, 5, 2, 2, 8), (3, 48, 24, 30, 40, 3, 3, 0, 0, 3), (5, 210, 33, 7, 32, 2, 2, 1, 1, 2),
+    (7, 128, 64, 8, 11, 3, 3, 1, 1, 4), (1, 600, 12, 16, 130, 2, 1, 0, 0, 2),
+])
+def test_windows_that_do_not_overlap(oracle, monkeypatch, case):
+    """By the rule, rewritten for the 1 x 1 kernel and on virtual images: exact on integers, and all of them round the operands
+    to the nearest TF32, so that they differ by the rounding of fp32 sums only."""
+    N, C, H, W, K, R, S, ph, pw, st = case
+    xi, wi = small_integers((N, C, H, W), 487), small_integers((K, C, R, S), 488)
+    yi_ref, _ = _reference(oracle, xi, wi, ph, pw, st)
+    x, w = uniform((N, C, H, W), 489), uniform((K, C, R, S), 490)
+    _, yabs = _reference(oracle, x, w, ph, pw, st)
+    results = []
+    for mode in ("1", "0", "2"):
+        monkeypatch.setenv("CONV2D_B200_TF32_VIRT", mode)
+        y, ws = _run(xi, wi, ph, pw, st, 2)
+        np.testing.assert_array_equal(y.astype(np.float64), yi_ref)
+        np.testing.assert_array_equal(_run(xi, wi, ph, pw, st, 2, flags=1, ws=ws)[0], y)
+        results.append(_run(x, w, ph, pw, st, 2)[0])
+    for y in results[1:]:
+        assert_parity(y, results[0].astype(np.float64), yabs, FFMA_TOL, f"{case}")
