@@ -17,12 +17,14 @@
 // filter reads had two-way bank conflicts (27 of 60 million wavefronts), and a 4-byte copy with three divisions for every
 // element of a row of odd width took a quarter of the issue slots.  Us, before -> now:
 //   32 x 96 x 27 x 35, 112 filters of 3 x 3: 282 -> 132 (38 of 74 TFLOP/s)   32 x 64 x 56 x 56, 64 of 3 x 3: 219 -> 159
-//   16 x 128 x 32 x 32, 128 of 7 x 7: 764 -> 414        64 x 128 x 32 x 32, 128 of 3 x 3: 430 -> 384, of 1 x 1 73 -> 77
+//   16 x 128 x 32 x 32, 128 of 7 x 7: 764 -> 414        64 x 128 x 32 x 32, 128 of 3 x 3: 430 -> 384, of 1 x 1 72 -> 70
 //   20 x 176 x 31 x 31, 32 of 7 x 7: 1077 -> 350        1 x 149 x 20 x 20, 80 of 3 x 3: 174 -> 71
 // What bounds it now: issue slots (0.6 other instructions per packed FMA) and, on small problems, the SMs' work per round.
 #pragma once
 #include "common.cuh"
 #include "fastdiv.cuh"
+
+#include <cmath>
 
 namespace conv2d_b200 {
 namespace {
@@ -235,6 +237,33 @@ struct FfmaSplit {
     double cost = 0;                  // estimated cycles; 0: no split
 };
 
+// Estimated cycles of a split for 1 x 1 filters.  Their contraction is short, so the latency of a block's stages and its
+// stores count as much as its multiplications, and smaller blocks pay, down to a few threads that multiply among many that
+// copy.  Fitted to 1300 random layers in all their splits: 5 % of them were slower by 4 % and more than in fixed tiles of
+// 32 x 8 outputs x 64 filters with the estimate of the other filter sizes, 1.5 % with this one, all together 9 % faster
+// (64 x 128 x 32 x 32, 128 filters 76 -> 70 us; 12 x 16 x 62 x 62, 384 filters 89 -> 49; 36 x 480 x 11 x 11, 7 filters 134 -> 61).
+template <int CB, int TQ>
+double pointwise_split_cost(const Shape& sh, const FfmaSplit& f, int resident, int sms)
+{
+    const double warps = f.threads / 32, stages = (sh.C + CB - 1) / CB, share = (double)f.seg_blocks * f.kblocks / sms;
+    const int width = f.sps * TQ < sh.W ? f.sps * TQ : sh.W, threads = f.threads;
+    const double pieces = stages * (double)(CB * f.rows * ((width + (f.x4 ? 0 : 3) + 3) / 4)) / threads;    // copies of a thread
+    const double filters = stages * (double)(CB * f.groups * kThrK) / threads;
+    const int unit = !f.x4 || TQ % 2 ? 1 : (TQ % 4 ? 2 : 4);                                               // floats of a read
+    const int store = sh.Q % 4 == 0 && unit == 4 ? 4 : (sh.Q % 2 == 0 && unit >= 2 ? 2 : 1);
+    const double issue = sh.C * (0.373 * kThrK * TQ + 1.34 + 0.233 * TQ / unit) + 237.0 * stages + 26.5 * pieces + 24.1 * filters
+                       + 27.8 * kThrK * TQ / store + 69.7;                                                 // slots of a warp
+    const double per_sm = ceil(share), conc = per_sm < resident ? per_sm : resident, beside = conc * warps / 4.0;
+    const double alone = issue * (warps > 4 ? warps / 4.0 : 1.0) * 2.26 + 142.0 * stages + 19.1 * (pieces + filters) + 3650.0;
+    double rounds = 1.0, count = per_sm;
+    if (per_sm > resident) {
+        rounds = share / conc + 6.75;
+        count = (per_sm > share + 0.5 * conc ? per_sm : share + 0.5 * conc) + 2.7 * conc;
+    }
+    const double latency = rounds * alone, slots = count * warps / 4.0 * issue * (1.0 + 3.86 / beside);
+    return latency > slots ? latency + 0.3 * slots : slots + 0.3 * latency;
+}
+
 template <int R, int S, int CB, int TQ>
 FfmaSplit split_ffma(const Shape& sh)
 {
@@ -258,15 +287,17 @@ FfmaSplit split_ffma(const Shape& sh)
     const int kb_min = (kgroups + kMaxGroups - 1) / kMaxGroups;
     const int kb_candidates[3] = {kb_min, kb_min * 2, kb_min * 4};
     for (int kb : kb_candidates) {
-        if (kb > kgroups) continue;
+        if (kb > kgroups || (R == 1 && kb > 2 * kb_min)) continue;
         f.groups = (kgroups + kb - 1) / kb;
         f.kblocks = (kgroups + f.groups - 1) / f.groups;
         if (f.kblocks > 65535) continue;
         // (warp w of every block sits on scheduler w % 4: other counts leave two schedulers with half the work, 64 x 128 x
         // 32 x 32, 128 filters of 3 x 3: 381 us with 4 warps, 407 with 8, 441 with 6)
-        for (int warps : {2, 4, 8}) {
+        // (1 x 1 filters, few of them: also a half and a quarter of the segments, the other threads only copy)
+        for (int choice = 0; choice < (R == 1 && f.groups <= 2 ? 5 : 3); ++choice) {
+            const int warps = choice < 3 ? 2 << choice : 4;
             f.threads = 32 * warps;
-            f.segs = f.threads / f.groups;
+            f.segs = f.threads / f.groups >> (choice < 3 ? 0 : choice - 2);
             // rows that the segments of a block can touch, and the halo rows of every image among them (many small
             // images with large filters: fewer segments than threads, until their rows fit)
             for (;; f.segs /= 2) {
@@ -282,6 +313,11 @@ FfmaSplit split_ffma(const Shape& sh)
             const long long blocks = f.seg_blocks * f.kblocks;
             const int by_regs = 512 / f.threads, by_smem = (int)(220 * 1024 / (f.smem + 1024));
             const int res = by_regs < by_smem ? by_regs : by_smem;
+            if constexpr (R == 1) {
+                const double t = pointwise_split_cost<CB, TQ>(sh, f, res, sms);
+                if (best.cost == 0 || t < best.cost) { best = f; best.cost = t; }
+                continue;
+            }
             // one warp's work on its scheduler, with its share of the copies of a channel block (an element of the image
             // rows or of the filters costs about 16 issue slots per 32 threads) and of the barrier at its end
             const double copies = CB * ((double)f.rows * f.pitch / 4 * 16.0 + (double)R * S * f.groups * kThrK * 8.0) / f.threads;
@@ -332,7 +368,8 @@ conv2d_status_t launch_instance(const float* x, const float* w, float* y, const 
     const FfmaSplit f7 = split_ffma<R, S, CB, 7>(sh);
     int tq = 8;
     double cost = f8.cost;
-    auto consider = [&](int len, const FfmaSplit& f) { if (f.cost > 0 && (cost == 0 || f.cost < 0.98 * cost)) { cost = f.cost; tq = len; } };
+    const double clearly = R == 1 ? 1.0 : 0.98;
+    auto consider = [&](int len, const FfmaSplit& f) { if (f.cost > 0 && (cost == 0 || f.cost < clearly * cost)) { cost = f.cost; tq = len; } };
     consider(6, f6); consider(7, f7);
     static const int by_tile[7] = {8, 8, 7, 0, 7, 7, 6};            // (the switch selects a shape of tile)
     const int forced = env_int("CONV2D_B200_FFMA_TILE", -1);

@@ -43,3 +43,14 @@ def test_non_finite_pixels_stay_in_their_windows(oracle):
     assert np.isnan(y[0][:, hit[0]]).all() and np.isposinf(y[1][:, hit[1]]).all()
     for n in range(2):
         np.testing.assert_array_equal(y[n][:, ~hit[n]], clean[n][:, ~hit[n]])
+
+
+@pytest.mark.parametrize("dims", [
+    (36, 480, 11, 11, 7), (9, 80, 21, 21, 16), (3, 33, 19, 18, 9),      # one or two groups: a part of the threads only copies
+    (2, 16, 31, 62, 384), (5, 5, 20, 47, 55), (1, 1, 3, 3, 1),           # one channel block
+])
+def test_pointwise_splits_exact_on_integers(oracle, dims):
+    N, C, H, W, K = dims
+    x, w = small_integers((N, C, H, W), 1505), small_integers((K, C, 1, 1), 1506)
+    y_ref, _ = oracle.conv2d_oracle(x, w)
+    np.testing.assert_array_equal(run_library(x, w, entry="general", algo=ALGO_FFMA).astype(np.float64), y_ref)
