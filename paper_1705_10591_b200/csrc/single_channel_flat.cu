@@ -256,9 +256,10 @@ conv2d_status_t launch_flat(FlatArgs& a, const Shape& sh, cudaStream_t stream)
             if (bh > sh.P) break;
             const size_t smem = tap_bytes + (size_t)(bh + sh.R - 1) * 4 * a.plane * sizeof(float);
             if (smem > (bh == 1 ? (size_t)200 : (size_t)72) * 1024) break;
-            const int threads = bh * a.cq >= kMaxThreads ? kMaxThreads : (bh * a.cq + 31) / 32 * 32;
-            const int passes = (bh * a.cq + threads - 1) / threads;
             const long long blocks = (long long)sh.N * a.col_tiles * ((sh.P + bh - 1) / bh) * used;
+            int threads = bh * a.cq >= kMaxThreads ? kMaxThreads : (bh * a.cq + 31) / 32 * 32;
+            if (threads < 128 && blocks <= sms) threads = 128;         // (few blocks: the other threads share the staging)
+            const int passes = (bh * a.cq + threads - 1) / threads;
             if (splits > 1 && best != 0 && blocks / used >= 2LL * sms) continue;      // (a share of the maps costs the whole staging)
             const int by_regs = Residency<M>::kBlocks * kMaxThreads / threads, by_smem = (int)(220 * 1024 / (smem + 1024));
             const double res = by_regs < by_smem ? by_regs : by_smem;
@@ -269,8 +270,14 @@ conv2d_status_t launch_flat(FlatArgs& a, const Shape& sh, cudaStream_t stream)
             const double work = issue > write ? issue + 0.3 * write : write + 0.3 * issue;
             const double per_sm = (double)blocks / sms, each = (kLatency + work) / res;
             double t = per_sm * (each > work ? each : work) + 0.7 * work;
+            // the time of one block with nothing beside it, whose few warps each sit on a scheduler of their own (without it
+            // and the threads that only stage, 14 x 17 x 21, 23 maps of 5 x 3 ran on 42 warps: 12.3 us, now 5.0)
+            const int units = (bh * a.cq + 31) / 32, deep = units < threads / 32 ? (units + 3) / 4 : (threads / 32 + 3) / 4;
+            const double copies = (bh + sh.R - 1) * (4.0 * a.npos / 32.0) * 32.0 * 60.0 + (double)per * sh.R * S * TF * 250.0;
+            const double alone = kLatency + deep * passes * per * unit_cycles(M, sh.R, S, TURN) * 1.3 + copies / threads;
             const double whole_blocks = (double)((blocks + sms - 1) / sms) * work;
             if (blocks <= 4LL * sms && t < whole_blocks) t = whole_blocks;
+            if (t < alone) t = alone;
             if (best == 0 || t < best) {
                 best = t; best_smem = smem; best_threads = threads;
                 a.band_h = bh; a.splits = used; a.cbs_per_split = per;
