@@ -34,24 +34,6 @@ constexpr int kPitch4 = kPitch / 4;
 
 __device__ __forceinline__ void store4(float* p, float4 v) { __stcs(reinterpret_cast<float4*>(p), v); }
 
-// Stores the n = 4 adjacent outputs of one thread at columns q0..q0+3 of a row of Q outputs with the
-// widest unit the row alignment allows: `unit` = 4 when Q % 4 == 0 (every row 16-byte aligned),
-// 2 when Q % 2 == 0, else 1.  q0 is a multiple of 4.
-__device__ __forceinline__ void store_outputs(float* o, float a0, float a1, float a2, float a3, int q0, int Q, int unit)
-{
-    if (unit == 4 && q0 + 3 < Q) {
-        store4(o, make_float4(a0, a1, a2, a3));
-    } else if (unit >= 2) {
-        if (q0 + 1 < Q) __stcs(reinterpret_cast<float2*>(o), make_float2(a0, a1));
-        if (q0 + 3 < Q) __stcs(reinterpret_cast<float2*>(o + 2), make_float2(a2, a3));
-    } else {
-        if (q0 + 0 < Q) __stcs(o + 0, a0);
-        if (q0 + 1 < Q) __stcs(o + 1, a1);
-        if (q0 + 2 < Q) __stcs(o + 2, a2);
-        if (q0 + 3 < Q) __stcs(o + 3, a3);
-    }
-}
-
 // WSRC: 0 = filter taps read from the constant bank, 1 = from a shared-memory copy (128-bit broadcast loads).
 template <int R, int S, int TR, int WSRC>
 __global__ void __launch_bounds__(kThreads)
@@ -459,7 +441,7 @@ constexpr int kRowsPitch4 = kRowsPitch / 4;
 template <int R, int S, int TR>
 __global__ void __launch_bounds__(kRowsThreads, 1)
 single_channel_rows_kernel(const float* __restrict__ x, const float* __restrict__ w, float* __restrict__ y,
-                           int N, int H, int W, int K, int P, int Q, int band_h, int col_tiles, int items, int unit,
+                           int N, int H, int W, int K, int P, int Q, int band_h, int col_tiles, int items,
                            unsigned max_polls, int test_short_item)
 {
     constexpr int NV = (S + kVec - 1 + 3) / 4;
@@ -592,10 +574,9 @@ single_channel_rows_kernel(const float* __restrict__ x, const float* __restrict_
 #pragma unroll
                 for (int tr = 0; tr < TR; ++tr) {
                     if (row_ok[tr]) {
-                        float* o = yout + (size_t)tr * Q;
-                        store_outputs(o, acc[tr][0].x, acc[tr][1].x, acc[tr][2].x, acc[tr][3].x, q0, Q, unit);
-                        if (second)
-                            store_outputs(o + plane, acc[tr][0].y, acc[tr][1].y, acc[tr][2].y, acc[tr][3].y, q0, Q, unit);
+                        float* o = yout + (size_t)tr * Q;                 // (Q % 4 == 0: whole aligned quads)
+                        store4(o, make_float4(acc[tr][0].x, acc[tr][1].x, acc[tr][2].x, acc[tr][3].x));
+                        if (second) store4(o + plane, make_float4(acc[tr][0].y, acc[tr][1].y, acc[tr][2].y, acc[tr][3].y));
                     }
                 }
             }
@@ -632,10 +613,9 @@ conv2d_status_t launch_rows(const float* x, const float* w, float* y, const Shap
     if (items > 0x7fffffffLL) return CONV2D_ERR_UNSUPPORTED;
     const int sms = sm_count();
     const int grid = (int)(items < sms ? items : sms);
-    const int unit = (reinterpret_cast<uintptr_t>(y) % 16 != 0) ? 1 : (sh.Q % 4 == 0 ? 4 : (sh.Q % 2 == 0 ? 2 : 1));
     // Failure-detection test hooks (host-side injection only): a short wait bound and one item whose barrier
     // expects a row that is never copied, so that the wait expires and the time-out path can be checked.
-    kern<<<grid, kRowsThreads, smem, stream>>>(x, w, y, sh.N, sh.H, sh.W, sh.K, sh.P, sh.Q, band_h, col_tiles, (int)items, unit,
+    kern<<<grid, kRowsThreads, smem, stream>>>(x, w, y, sh.N, sh.H, sh.W, sh.K, sh.P, sh.Q, band_h, col_tiles, (int)items,
                                                (unsigned)env_int("CONV2D_B200_SC_MAX_POLLS", 1 << 22),
                                                env_int("CONV2D_B200_SC_TEST_SHORT_ITEM", -1));
     count_launch();
@@ -836,17 +816,7 @@ conv2d_status_t launch_rows_shift(const float* x, const float* w, float* y, cons
     return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
 }
 
-// The shifted kernel pays for its aligned stores with one output row per step, which suits the memory-bound
-// 3 x 3 case (measured 0.652 -> 0.463 ms on 4096 x 4096, 32 filters); the FMA-bound 7 x 7 case measured
-// slightly slower with it and stays on the kernel above.
-template <int R, int S>
-conv2d_status_t try_rows_shift(const float*, const float*, float*, const Shape&, int, cudaStream_t) { return CONV2D_ERR_UNSUPPORTED; }
-template <>
-conv2d_status_t try_rows_shift<3, 3>(const float* x, const float* w, float* y, const Shape& sh, int band_h, cudaStream_t stream)
-{
-    return launch_rows_shift<3, 3>(x, w, y, sh, band_h, stream);
-}
-
+// 3 x 3 and 5 x 5 filters on the kernels of this file.
 template <int R, int S>
 conv2d_status_t dispatch_rs(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream)
 {
@@ -862,7 +832,7 @@ conv2d_status_t dispatch_rs(const float* x, const float* w, float* y, const Shap
     if (tile_h < 1) tile_h = 1;
     if (tile_h > 64) tile_h = 64;
     if (tile_h > sh.P) tile_h = sh.P;
-    const int tr = env_int("CONV2D_B200_SC_ROWS", R >= 7 ? 1 : 2);
+    const int tr = env_int("CONV2D_B200_SC_ROWS", 2);
     constexpr int RS2 = (R * S + 1) / 2;
     const int unit = env_int("CONV2D_B200_SC_UNIT", 0);      // per-thread unit ablation (benchmark only)
     if (unit == 1 || unit == 2 || unit == 4) {
@@ -871,7 +841,9 @@ conv2d_status_t dispatch_rs(const float* x, const float* w, float* y, const Shap
                                              : launch_unit<R, S, 4>(x, w, y, sh, tile_h, stream);
         if (st != CONV2D_ERR_UNSUPPORTED) return st;
     }
-    // Large images: the wide persistent kernels (they need 16-byte aligned input rows for the bulk copies).
+    // Large images: the wide persistent kernels (they need 16-byte aligned input rows for the bulk copies), for 5 x 5 filters the
+    // plain one (W % 4 == 0 makes its output rows whole quads), for 3 x 3 the one for rows that are only 8-byte aligned.  The
+    // shifted kernel pays for its aligned stores with one output row per step, which suits the memory-bound 3 x 3 case.
     const bool rows_ok = sh.W % 4 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
     if (rows_ok && env_int("CONV2D_B200_SC_WIDE", 1) != 0) {
         // Rows per work item: 8, or another height (4..16, as far as the double buffer fits) when that fills the last
@@ -896,29 +868,24 @@ conv2d_status_t dispatch_rs(const float* x, const float* w, float* y, const Shap
             return score8 >= best_score - 0.02 ? 8 : best;       // 8 rows unless another height is clearly better
         };
         const int forced_band = env_int("CONV2D_B200_SC_BAND_H", 0);
-        int band_h = forced_band > 0 ? forced_band : pick_band((tr == 1 || R >= 7) ? 1 : 2, 1, kRowsPitch * sizeof(float));
+        int band_h = forced_band > 0 ? forced_band : pick_band(tr == 1 ? 1 : 2, 1, kRowsPitch * sizeof(float));
         if (band_h < 1) band_h = 1;
         if (band_h > 16) band_h = 16;
-        // Rows that are only 8-byte aligned: the variant that shifts odd rows by two columns.  Its aligned
-        // 128-bit stores beat the tile kernel's 64-bit pairs already on mid-size images (3 x 3, 32 filters,
-        // 1024 x 1024: 75 -> 41 us; 512 x 512: 26 -> 20 us), although half of its 2048 columns are idle there.
-        if (sh.Q >= 384 && sh.Q % 4 == 2 && ((long long)sh.P * sh.Q) % 4 == 0 && reinterpret_cast<uintptr_t>(y) % 16 == 0 &&
-            env_int("CONV2D_B200_SC_SHIFT", 1) != 0) {
-            const conv2d_status_t st = try_rows_shift<R, S>(x, w, y, sh, forced_band > 0 ? band_h : pick_band(2, 2, kShiftPitch * sizeof(float)), stream);
-            if (st != CONV2D_ERR_UNSUPPORTED) return st;
-        }
-        if constexpr (R == 3 || R == 5) {                    // (the flat kernel has the wide images of the other sizes)
-            if (sh.Q >= env_int("CONV2D_B200_SC_WIDE_MINQ", 1024)) {
-                const conv2d_status_t st = tr == 1 ? launch_rows<R, S, 1>(x, w, y, sh, band_h, stream)
-                                                   : launch_rows<R, S, 2>(x, w, y, sh, band_h, stream);
+        if constexpr (R == 3) {
+            if (sh.Q >= 384 && sh.Q % 4 == 2 && ((long long)sh.P * sh.Q) % 4 == 0 && env_int("CONV2D_B200_SC_SHIFT", 1) != 0) {
+                const conv2d_status_t st = launch_rows_shift<R, S>(x, w, y, sh, forced_band > 0 ? band_h : pick_band(2, 2, kShiftPitch * sizeof(float)), stream);
                 if (st != CONV2D_ERR_UNSUPPORTED) return st;
             }
+        } else if (sh.Q >= env_int("CONV2D_B200_SC_WIDE_MINQ", 1024)) {
+            const conv2d_status_t st = tr == 1 ? launch_rows<R, S, 1>(x, w, y, sh, band_h, stream)
+                                               : launch_rows<R, S, 2>(x, w, y, sh, band_h, stream);
+            if (st != CONV2D_ERR_UNSUPPORTED) return st;
         }
     }
     if (env_int("CONV2D_B200_SC_PACKED", 1) != 0 &&
         (size_t)((sh.K + 1) / 2) * RS2 * sizeof(float4) <= 96 * 1024) {
-        return (tr == 1 || R >= 7) ? launch_packed<R, S, 1>(x, w, y, sh, tile_h, stream)
-                                   : launch_packed<R, S, 2>(x, w, y, sh, tile_h, stream);
+        return tr == 1 ? launch_packed<R, S, 1>(x, w, y, sh, tile_h, stream)
+                       : launch_packed<R, S, 2>(x, w, y, sh, tile_h, stream);
     }
     constexpr int RSP = (R * S + 3) / 4 * 4;
     int wsrc = env_int("CONV2D_B200_SC_WSRC", 1);
@@ -951,12 +918,14 @@ cudaError_t consume_device_timeout(bool* raised)
 }
 
 // Which kernel.  The flat kernel (single_channel_flat.cu) stores aligned quads whatever the alignment of the rows and takes
-// any filter height, so it has most shapes; measured against the kernels of this file (old -> flat, us):
-//   3 x 3: 3 x 1083 x 1917, 16 maps 205 -> 73; 4096 x 4096, 32 maps 471 -> 413; 512 x 512, 32 maps 16.9 -> 14.4
+// any filter height, so it has most shapes; measured against the kernels that were here or still are (old -> flat, us a call
+// among others unless a size says otherwise):
+//   3 x 3: 3 x 1083 x 1917, 16 maps 205 -> 85; 4096 x 4096, 32 maps 471 -> 413; 512 x 512, 32 maps 16.9 -> 14.4
 //   1 x 1: 2048 x 2048, 32 maps 96 -> 82        7 x 7: 2048 x 2048, 32 maps 267 -> 256; 7 x 187 x 1674, 14 maps 84 -> 72
 //   5 x 5: 2049 x 2049, 32 maps 217 -> 165; 3000 x 3001, 2 maps 47 -> 41
 //   5 x 3: 2 x 1500 x 700, 24 maps 722 -> 56 (only the shape-agnostic kernel took filters that are not square)
-// The kernels here keep
+// Of 1820 random shapes that it has 84 were faster before, most of them by one to two us or 7 x 7 on maps that fill no block
+// (6 x 85 x 1364, 44 maps 70 -> 92).  The kernels here keep
 //   * rows that are whole quads and fill most of a 512-column tile: nothing is lost on their stores, and two rows per tap
 //     read pay: 4096 x 4096, 32 maps of 5 x 5 467 -> 563, 1000 x 1000, 16 of 5 x 5 38 -> 47, 12 x 115 x 662, 26 of 3 x 3 25 -> 31;
 //   * 5 x 5 on a few maps of different alignment, whose classes the flat kernel computes one by one, where strided stores
@@ -967,20 +936,19 @@ static bool take_flat(const Shape& sh)
 {
     const int forced = env_int("CONV2D_B200_SC_FLAT", -1);
     if (forced >= 0) return forced != 0;
+    if (sh.R != sh.S || (sh.R != 3 && sh.R != 5)) return true;
     static const char* const other_kernels[] = {"CONV2D_B200_SC_UNIT", "CONV2D_B200_SC_PACKED", "CONV2D_B200_SC_TILE_H",
                                                 "CONV2D_B200_SC_ROWS", "CONV2D_B200_SC_WIDE", "CONV2D_B200_SC_SHIFT",
                                                 "CONV2D_B200_SC_BAND_H", "CONV2D_B200_SC_WSRC", "CONV2D_B200_SC_WIDE_MINQ"};
     for (const char* name : other_kernels)
         if (env_int(name, -1) != -1) return false;                   // (a switch of the kernels of this file is set)
     const double full = (double)sh.Q / ((sh.Q + kTileW - 1) / kTileW * kTileW);      // of a tile's columns
-    if (sh.R == sh.S && (sh.R == 3 || sh.R == 5) && sh.Q % 4 == 0 && full >= 0.6) return false;
-    if (sh.R == 5 && sh.S == 5 && sh.Q >= kTileW / 2) {
+    if (sh.Q % 4 == 0 && full >= 0.6) return false;
+    if (sh.R == 5 && sh.Q >= kTileW / 2) {
         const double pairs = (sh.K + 1) / 2 * 238.0, stores = sh.K * 130.0;
         if ((pairs > stores ? pairs : stores) / full < 0.76 * single_channel_flat_cost(sh)) return false;
     }
-    if (sh.R == 3 && sh.S == 3 && sh.W % 4 == 0 && sh.P % 2 == 0 && sh.Q >= 1024 && sh.N == 1 && sh.P >= 32 && sh.P <= 256 && sh.K <= 16)
-        return false;
-    return true;
+    return !(sh.R == 3 && sh.W % 4 == 0 && sh.P % 2 == 0 && sh.Q >= 1024 && sh.N == 1 && sh.P >= 32 && sh.P <= 256 && sh.K <= 16);
 }
 
 conv2d_status_t launch_single_channel(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream)
@@ -989,10 +957,8 @@ conv2d_status_t launch_single_channel(const float* x, const float* w, float* y, 
         const conv2d_status_t st = launch_single_channel_flat(x, w, y, sh, stream);
         if (st != CONV2D_ERR_UNSUPPORTED) return st;
     }
-    if (sh.R == 1 && sh.S == 1) return dispatch_rs<1, 1>(x, w, y, sh, stream);
     if (sh.R == 3 && sh.S == 3) return dispatch_rs<3, 3>(x, w, y, sh, stream);
     if (sh.R == 5 && sh.S == 5) return dispatch_rs<5, 5>(x, w, y, sh, stream);
-    if (sh.R == 7 && sh.S == 7) return dispatch_rs<7, 7>(x, w, y, sh, stream);
     return launch_direct_fallback(x, w, y, sh, stream);
 }
 

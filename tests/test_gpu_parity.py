@@ -60,7 +60,8 @@ def test_single_channel_within_tolerance(oracle, dims):
     dict(CONV2D_B200_SC_ROWS="1"), dict(CONV2D_B200_SC_TILE_H="5"),                       # packed-FMA kernel
     dict(CONV2D_B200_SC_UNIT="1"), dict(CONV2D_B200_SC_UNIT="2"), dict(CONV2D_B200_SC_UNIT="4"),   # unit ablation
     dict(CONV2D_B200_SC_WIDE="0"),                                                        # tile kernel on wide images
-    dict(CONV2D_B200_SC_SHIFT="0"),                                                       # wide kernel with 64-bit stores
+    dict(CONV2D_B200_SC_FLAT="0"),                                                        # shifted kernel, shape-agnostic kernel
+    dict(CONV2D_B200_SC_SHIFT="0"),                                                       # tile kernel instead of the shifted one
     dict(CONV2D_B200_SC_PACKED="0", CONV2D_B200_SC_WSRC="0"),                              # scalar-FMA kernel
     dict(CONV2D_B200_SC_PACKED="0", CONV2D_B200_SC_WSRC="1", CONV2D_B200_SC_ROWS="1"),
     dict(CONV2D_B200_SC_PACKED="0", CONV2D_B200_SC_TILE_H="5", CONV2D_B200_SC_WSRC="0", CONV2D_B200_SC_ROWS="1")])
