@@ -931,7 +931,9 @@ cudaError_t consume_device_timeout(bool* raised)
 //   * 5 x 5 on a few maps of different alignment, whose classes the flat kernel computes one by one, where strided stores
 //     of all maps cost less: 14 x 375 x 1439, 4 maps 60 -> 64, 6 x 383 x 805, 5 maps 25 -> 33, 2 x 749 x 2938, 2 maps 24 -> 27
 //     (238 cycles of a scheduler for a warp's pair of maps, 130 for the strided stores of a map);
-//   * a few maps of a short wide image, on the shifted kernel: 200 x 2048, 16 maps of 3 x 3 11.2 -> 12.6, 40 x 1032, 4 maps 8.8 -> 8.6.
+//   * one short wide image with 3 x 3 on up to 16 maps, from two million outputs on (eight below 192 rows), on the shifted kernel:
+//     200 x 2046 outputs of 16 maps 10.3 -> 12.3, 256 x 1402 of 16 8.2 -> 10.3, 128 x 4094 of 16 10.3 -> 14.4 (but 128 x 2046 of 16
+//     10.3 -> 9.2, 200 x 1030 of 4 6.0 -> 4.9; with more images or rows either kernel wins, as the maps fill the flat kernel's blocks).
 static bool take_flat(const Shape& sh)
 {
     const int forced = env_int("CONV2D_B200_SC_FLAT", -1);
@@ -948,7 +950,8 @@ static bool take_flat(const Shape& sh)
         const double pairs = (sh.K + 1) / 2 * 238.0, stores = sh.K * 130.0;
         if ((pairs > stores ? pairs : stores) / full < 0.76 * single_channel_flat_cost(sh)) return false;
     }
-    return !(sh.R == 3 && sh.W % 4 == 0 && sh.P % 2 == 0 && sh.Q >= 1024 && sh.N == 1 && sh.P >= 32 && sh.P <= 256 && sh.K <= 16);
+    return !(sh.R == 3 && sh.W % 4 == 0 && sh.P % 2 == 0 && sh.Q >= 1024 && sh.N == 1 && sh.P >= 128 && sh.P <= 256 && sh.K <= 16 &&
+             (long long)sh.K * sh.P * sh.Q >= (sh.P >= 192 ? 2000000 : 8000000));
 }
 
 conv2d_status_t launch_single_channel(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream)

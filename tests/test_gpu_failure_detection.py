@@ -59,6 +59,7 @@ def test_single_channel_wide_kernels_report_an_expired_wait(oracle, monkeypatch,
     xd, wd = torch.from_numpy(x).to(dev), torch.from_numpy(w).to(dev)
     y = torch.zeros((N, K, H - R + 1, W - S + 1), device=dev)
     stream = torch.cuda.current_stream().cuda_stream
+    monkeypatch.setenv("CONV2D_B200_SC_FLAT", "0")           # (the kernels with bounded waits, whatever the rule says)
     monkeypatch.setenv("CONV2D_B200_SC_MAX_POLLS", "4096")
     monkeypatch.setenv("CONV2D_B200_SC_TEST_SHORT_ITEM", "1")
     lib.conv2d_fwd_single_channel(xd.data_ptr(), wd.data_ptr(), y.data_ptr(), N, H, W, K, R, S, 0, 0, 0, stream)
