@@ -103,10 +103,12 @@ conv2d_status_t conv2d_fwd_plan_describe(int N, int C, int H, int W, int K, int 
  *   x [N][1][H][W], w [K][1][R][S], y [N][K][P][Q]; fp32 FMA arithmetic.
  * The filters are small in this case (Section 3.2) and are kept on chip for the
  * whole call: every thread block copies them into shared memory and reads them
- * with broadcast loads.  Tuned instances exist for R = S in {1, 3, 5, 7}; images
- * with W % 4 == 0 and at least 1024 output columns take the wide kernel that
- * stages input rows with bulk (TMA) copies; every other shape is computed by a
- * slower shape-agnostic kernel, never rejected.  N must not exceed 65535.
+ * with broadcast loads.  One kernel takes filters of any height and up to 7
+ * columns on images of any size and alignment; 3 x 3 and 5 x 5 filters on rows
+ * of whole 16-byte units, and a few shapes that a measured rule names, take
+ * kernels of their own (from 1024 output columns on with rows staged by bulk
+ * (TMA) copies).  Wider filters are computed by a slower shape-agnostic kernel,
+ * never rejected.  N must not exceed 65535.
  * (A benchmark-only variant selected by an environment switch keeps the filters
  * in a per-device constant-memory bank instead; calls using it on different
  * streams must not overlap.)
@@ -200,12 +202,15 @@ conv2d_status_t conv2d_fwd_general_padded(const float* x, const float* w, float*
  *   y[n,k,p,q] = sum_{c,r,s} xz[n,c,stride*p+r-pad_h,stride*q+s-pad_w] * w[k,c,r,s],
  *   P = (H + 2*pad_h - R) / stride + 1, Q = (W + 2*pad_w - S) / stride + 1 (integer division), y [N][K][P][Q].
  * With the tensor-core algorithms the kernel stages the phases of the stride straight from x and multiplies each
- * with its own taps.  Otherwise (fp32, or no such instance) the call rewrites the problem as a stride-1 convolution
+ * with its own taps.  Otherwise (fp32, no such instance, or windows that do not overlap where an estimate finds the
+ * 1 x 1 kernel faster on the rewritten image) the call rewrites the problem as a stride-1 convolution
  * over stride*stride times as many channels ("space to depth": channel (c,a,b) of the rewritten image holds the pixels
  * whose row is a and whose column is b modulo the stride; the filters are split the same way) with two extra kernels
- * into the workspace and then runs conv2d_fwd_general on it: the same multiply-adds as the definition plus zeros.
+ * into the workspace and then runs conv2d_fwd_general on it: the same multiply-adds as the definition plus zeros, on
+ * the tensor cores with operands rounded to the nearest TF32 either way.
  * 1 <= stride <= 8.  Workspace from conv2d_fwd_strided_workspace_size; required, 16-byte aligned, status
- * block first.  With CONV2D_FLAG_WEIGHTS_PACKED the rewritten filters of the previous call are reused too.
+ * block first; it has room for the rewritten image and filters whether or not the call needs them.  With
+ * CONV2D_FLAG_WEIGHTS_PACKED the rewritten filters of the previous call are reused too.
  * algo is AUTO, FFMA or TF32; N * C must not exceed 65535 (CONV2D_ERR_UNSUPPORTED otherwise, checked before
  * anything is enqueued).
  */

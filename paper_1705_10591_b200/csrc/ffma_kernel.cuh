@@ -360,7 +360,7 @@ conv2d_status_t launch_split(const float* x, const float* w, float* y, const Sha
 }
 
 // Length of the segments by estimated time (all of them give the same bits: an output's additions run over (c, r, s) in
-// the same order): 8 has the widest reads and stores, 9 and 10 leave less of 26-, 27- or 30-column maps idle, 6 less of 12.
+// the same order): 8 has the widest reads and stores, 7 leaves less of 14-, 27- or 33-column maps idle, 6 less of 12 or 30.
 template <int R, int S, int CB>
 conv2d_status_t launch_instance(const float* x, const float* w, float* y, const Shape& sh, cudaStream_t stream)
 {
@@ -371,9 +371,8 @@ conv2d_status_t launch_instance(const float* x, const float* w, float* y, const 
     const double clearly = R == 1 ? 1.0 : 0.98;
     auto consider = [&](int len, const FfmaSplit& f) { if (f.cost > 0 && (cost == 0 || f.cost < clearly * cost)) { cost = f.cost; tq = len; } };
     consider(6, f6); consider(7, f7);
-    static const int by_tile[7] = {8, 8, 7, 0, 7, 7, 6};            // (the switch selects a shape of tile)
-    const int forced = env_int("CONV2D_B200_FFMA_TILE", -1);
-    if (forced >= 0 && forced <= 6 && by_tile[forced]) tq = by_tile[forced];
+    const int forced = env_int("CONV2D_B200_FFMA_SEGMENT", 0);
+    if (forced >= 6 && forced <= 8) tq = forced;
     const FfmaSplit& f = tq == 6 ? f6 : (tq == 7 ? f7 : f8);
     if (f.cost == 0 || f.seg_blocks > 0x7fffffffLL) return CONV2D_ERR_UNSUPPORTED;
     const bool x4 = f.x4 && reinterpret_cast<uintptr_t>(x) % 16 == 0;

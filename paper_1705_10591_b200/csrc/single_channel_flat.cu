@@ -13,7 +13,7 @@
 // adjacent outputs where a class has one map only); row r of the window is read once for all of them, each tap as one
 // broadcast.  The additions of an output run over (r, s) in order.  Up to M = 8 few registers (about 80) leave 24 warps
 // on an SM, which hide the staging of a block behind the arithmetic of others.
-// Measured: 3 x 1083 x 1917, 16 maps of 3 x 3: 205 us with strided 32-bit stores, 73 us here (5.8 TB/s).  Two quads per
+// Measured: 3 x 1083 x 1917, 16 maps of 3 x 3: 205 us a call with strided 32-bit stores, 84 us here (5.0 TB/s).  Two quads per
 // thread and tap read (half the broadcasts, 16 warps) were slower everywhere: 2049 x 2049, 32 maps of 5 x 5 165 -> 214.
 #include "common.cuh"
 #include "fastdiv.cuh"

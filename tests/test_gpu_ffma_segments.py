@@ -21,12 +21,12 @@ SHAPES += [
 ]
 
 
-@pytest.mark.parametrize("tile", [None, "0", "2", "6"])      # chosen; segments of 8, 7 and 6
+@pytest.mark.parametrize("length", [None, "8", "7", "6"])      # chosen by the launcher; forced
 @pytest.mark.parametrize("dims", SHAPES)
-def test_exact_on_integers(oracle, monkeypatch, dims, tile):
+def test_exact_on_integers(oracle, monkeypatch, dims, length):
     N, C, H, W, K, R, S = dims
-    if tile is not None:
-        monkeypatch.setenv("CONV2D_B200_FFMA_TILE", tile)
+    if length is not None:
+        monkeypatch.setenv("CONV2D_B200_FFMA_SEGMENT", length)
     x, w = small_integers((N, C, H, W), 1501), small_integers((K, C, R, S), 1502)
     y_ref, _ = oracle.conv2d_oracle(x, w)
     np.testing.assert_array_equal(run_library(x, w, entry="general", algo=ALGO_FFMA).astype(np.float64), y_ref)

@@ -19,8 +19,8 @@ CASES = [
     (2, 6, 9, 9, 5, 2, 4, 1, 2, 2),          # rectangular, even taps
     (1, 5, 12, 12, 7, 3, 3, 1, 1, 1),        # stride 1 degenerates to the padded convolution
     (1, 2, 11, 11, 3, 3, 3, 0, 0, 4),        # stride larger than the filter
-    (2, 512, 14, 16, 96, 1, 1, 0, 0, 2),     # 1 x 1, stride 2: 2048 channels on 7 x 8 pixels after the rewriting (streamed, split contraction)
-    (1, 128, 16, 16, 200, 1, 1, 0, 0, 2),    # 512 channels, 200 filters after the rewriting (streamed filters, two-SM form)
+    (2, 512, 14, 16, 96, 1, 1, 0, 0, 2),     # 1 x 1, stride 2, many channels on few pixels
+    (1, 128, 16, 16, 200, 1, 1, 0, 0, 2),    # two filter blocks
 ]
 
 
@@ -84,6 +84,8 @@ def test_strided_prepacked_filters(oracle, case):
 @pytest.mark.parametrize("case", [
     (2, 80, 30, 30, 48, 5, 5, 2, 2, 8), (3, 48, 24, 30, 40, 3, 3, 0, 0, 3), (5, 210, 33, 7, 32, 2, 2, 1, 1, 2),
     (7, 128, 64, 8, 11, 3, 3, 1, 1, 4), (1, 600, 12, 16, 130, 2, 1, 0, 0, 2),
+    (2, 512, 14, 16, 96, 1, 1, 0, 0, 2),     # rewritten: 2048 channels on 7 x 8 pixels (streamed filters, split contraction)
+    (1, 128, 16, 16, 200, 1, 1, 0, 0, 2),    # rewritten: 512 channels, 200 filters (streamed filters, two-SM form)
 ])
 def test_windows_that_do_not_overlap(oracle, monkeypatch, case):
     """By the rule, rewritten for the 1 x 1 kernel and on virtual images: exact on integers, and all of them round the operands
