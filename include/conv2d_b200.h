@@ -264,10 +264,10 @@ conv2d_status_t conv2d_fwd_general_noalloc(const float* x, const float* w, float
  * w_host are copied to the caller's device buffers x, w on the stream, the
  * convolution runs (single-channel kernel when C == 1, else conv2d_fwd_general
  * with `algo`), y is copied back into y_host and the stream is synchronised.
- * Large calls (from 8 MB of copies on) do this in up to five groups of images, with the
- * copies in both directions on streams of the library's own while the caller's stream
- * convolves; they start after what the caller's stream holds and have ended on return.
- * Host buffers should be page-locked for the copies to run at full speed.
+ * Large calls (from 8 MB of copies on) between page-locked host buffers do this in up to
+ * five groups of images, with the copies in both directions on streams of the library's own
+ * while the caller's stream convolves; they start after what the caller's stream holds and
+ * have ended on return.  Other host buffers are copied at once, and more slowly.
  * Returns the first error met, or the device status after synchronising
  * (CONV2D_ERR_DEVICE_TIMEOUT if a bounded on-device wait expired).  The
  * workspace is the one conv2d_fwd_general would need for `algo`; it may be

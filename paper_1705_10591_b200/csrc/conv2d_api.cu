@@ -488,6 +488,16 @@ static int images_per_copy(const Shape& sh, conv2d_algo_t algo, const void* work
     return (int)per;
 }
 
+// Page-locked host memory.  Copies to and from other memory are staged by the calling thread, so that groups only add to them:
+// 32 x 64 x 56 x 56, 64 filters 2.74 ms at once, 3.00 in groups; 4 x 64 x 112 x 112, 32 filters 1.13 and 1.37.
+static bool page_locked(const void* p)
+{
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type != cudaMemoryTypeUnregistered;
+    (void)cudaGetLastError();
+    return false;
+}
+
 conv2d_status_t conv2d_fwd_host(const float* x_host, const float* w_host, float* y_host,
                                 float* x, float* w, float* y,
                                 int N, int C, int H, int W, int K, int R, int S,
@@ -504,6 +514,7 @@ conv2d_status_t conv2d_fwd_host(const float* x_host, const float* w_host, float*
     // workspace (which may be NULL, of size 0, or never written) must not be read for a status.
     bool status_in_workspace = false;
     int per = images_per_copy(sh, algo, workspace, workspace_bytes);
+    if (per < N && !(page_locked(x_host) && page_locked(y_host))) per = N;
     // (a call that waits for its stream fails while that stream is captured; the streams of a set must not join the capture)
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (per < N && (cudaStreamIsCapturing(stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone)) per = N;
