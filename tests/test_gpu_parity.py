@@ -25,22 +25,27 @@ SINGLE_SHAPES = [
     (3, 40, 520, 4, 7, 7),       # Q = 514: second column tile nearly empty
     (1, 33, 36, 1, 1, 1),        # 1x1: no data sharing at all
     (1, 5, 5, 7, 5, 5),          # filter as large as the image: one output per map
-    (2, 21, 24, 3, 3, 5),        # rectangular taps -> shape-agnostic kernel
+    (2, 21, 24, 3, 3, 5),        # rectangular taps
     (1, 70, 16, 6, 5, 5),        # more rows than one tile, Q = 12 (vector stores)
-    (1, 23, 2100, 3, 5, 5),      # wide persistent kernel: two column tiles (2048 + 48), 128-bit stores
-    (2, 11, 1032, 5, 3, 3),      # wide kernel, Q = 1030: 64-bit stores, odd filter count
-    (1, 9, 1028, 2, 7, 7),       # wide kernel, 7 x 7, band taller than the image's output rows
-    (1, 14, 1040, 4, 1, 1),      # wide kernel, 1 x 1
+    # what the comments say of the wide kernels holds with the flat kernel off; by the rule it has most of these
+    (1, 23, 2100, 3, 5, 5),      # wide persistent kernel (by the rule, too): two column tiles (2048 + 48), 128-bit stores
+    (2, 11, 1032, 5, 3, 3),      # tile kernel: rows of odd count, Q = 1030, odd filter count
+    (1, 9, 1028, 2, 7, 7),       # 7 x 7, few output rows
+    (1, 14, 1040, 4, 1, 1),      # 1 x 1, wide image
     (1, 12, 1032, 3, 3, 3),      # shifted wide kernel: Q = 1030 (8-byte aligned rows), odd filter count
     (1, 10, 388, 3, 3, 3),       # shifted wide kernel on a narrow image: Q = 386, most of the 2048 columns idle
     (2, 14, 520, 5, 3, 3),       # shifted wide kernel: Q = 518, two images, two bands
     (2, 20, 2100, 5, 3, 3),      # shifted wide kernel: Q = 2098, two column tiles, three bands
-    (1, 14, 1040, 4, 7, 7),      # wide kernel, 7 x 7, Q = 1034: 64-bit stores
+    (1, 202, 2048, 8, 3, 3),     # shifted wide kernel by the rule
+    (1, 14, 1040, 4, 7, 7),      # 7 x 7, Q = 1034
 ]
 
 
+@pytest.mark.parametrize("flat", [None, "0"])      # by the rule; with the flat kernel off
 @pytest.mark.parametrize("dims", SINGLE_SHAPES)
-def test_single_channel_exact_on_integers(oracle, dims):
+def test_single_channel_exact_on_integers(oracle, monkeypatch, dims, flat):
+    if flat is not None:
+        monkeypatch.setenv("CONV2D_B200_SC_FLAT", flat)
     N, H, W, K, R, S = dims
     x, w = small_integers((N, 1, H, W), 301), small_integers((K, 1, R, S), 302)
     y_ref, _ = oracle.conv2d_oracle(x, w)
