@@ -492,8 +492,9 @@ bool patches_beat_virtual(const Plan& v, const Plan& patch, const Shape& sh)
     const int sms = sm_count();
     const bool quads = sh.W % 4 == 0;
     // a short contraction that only the virtual images split without a cluster: 5 x 80 x 65 x 33, 48 maps of 3 x 3 20.7 us
-    // on virtual images, 15.4 in patches (many channels earn the split back: 9 x 256 x 116 x 10, 6 of 2 x 2 18.6 and 26.1)
-    if (v.ksplit == 2 && !v.cluster && v.cblks <= 8 && patch.ksplit == 1 && patch.makespan < 10000.0) return true;
+    // on virtual images, 15.4 in patches, 4 x 38 x 62 x 62, 115 of 7 x 3 26.8 and 16.8; 19 of 25 layers, none the other way (many
+    // channels earn the split back: 9 x 256 x 116 x 10, 6 of 2 x 2 18.6 and 26.1)
+    if (v.ksplit == 2 && !v.cluster && v.cblks <= 8 && patch.ksplit == 1 && patch.makespan < 16000.0) return true;
     // clearly more staged pixels than the producers load in a pass (1024 in quads), stage after stage, or any of more than 1300:
     // 55 x 44 x 66 x 170, 7 maps of 5 x 5 259 and 188 us; 21 x 16 x 37 x 184, 4 of 7 x 7 67 and 40; 11 of 13 layers
     const long long stages = ((long long)v.supertiles * v.n_blocks * v.ksplit + sms - 1) / sms * v.cblks / v.ksplit;
