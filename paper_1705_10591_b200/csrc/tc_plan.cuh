@@ -470,38 +470,37 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     return p;
 }
 
-// Rough cycles of the busiest block: its MMAs, its producers (7 cycles per staged pixel and channel block, 5 where they load
-// quads, a round trip to memory per block at least) and its write-back, which overlap for the most part; and the zero-fill
-// and adds of a contraction split without a cluster (4.5 us).  Fitted to the times of 2000 random padded layers on virtual
-// images and in patches (standard deviation 19 %).
+// Rough cycles of the busiest block: its MMAs with 400 for every filter stage that its one issuing thread hands over, its
+// producers (6 cycles per staged pixel and channel block, 5 where they load quads, a round trip to memory per block at
+// least) and its write-back, which overlap for the most part; and the zero-fill and adds of a contraction split without a
+// cluster (4.5 us).  Fitted to the times of 2070 random padded layers on virtual images and in patches (standard deviation
+// 16 %; 19 % without the filter stages, which long halos make smaller and more).
 double estimated_cycles(const Plan& p, bool quads)
 {
     const int sms = sm_count();
     const double rounds = (double)(((long long)p.supertiles * p.n_blocks * p.ksplit + sms - 1) / sms);
-    const double load = p.npix * (quads ? 5.0 : 7.0);
-    const double mma = p.makespan / p.ksplit, stage = rounds * p.cblks / p.ksplit * (load > 1400.0 ? load : 1400.0);
+    const double load = p.npix * (quads ? 5.0 : 6.0), blocks = rounds * p.cblks / p.ksplit;      // channel blocks in a row
+    const double mma = p.makespan / p.ksplit + (p.resident ? 0.0 : blocks * ((p.taps + p.tps - 1) / p.tps) * 400.0);
+    const double stage = blocks * (load > 1400.0 ? load : 1400.0);
     const double store = rounds * p.tile_px / 32.0 * (p.n_tile == 128 && !p.pair_taps ? 800.0 : 500.0);
     const double most = mma > stage ? (mma > store ? mma : store) : (stage > store ? stage : store);
     return 0.6 * most + 0.4 * (mma + stage + store) + (p.ksplit == 2 && !p.cluster ? 9000.0 : 0.0);
 }
 
 // Where patches are the better cut for zero padding.  Of 2070 random layers 112 were slower by 4 % and more on virtual images
-// than in patches, 52 by more than 10 % (all layers together 14 % faster); with these rules it is about 70 and 23:
+// than in patches, 52 by more than 10 % (all layers together 14 % faster); with these rules it is 69 and 21, and none is slower
+// by the rules:
 bool patches_beat_virtual(const Plan& v, const Plan& patch, const Shape& sh)
 {
-    const int sms = sm_count();
-    const bool quads = sh.W % 4 == 0;
     // a short contraction that only the virtual images split without a cluster: 5 x 80 x 65 x 33, 48 maps of 3 x 3 20.7 us
     // on virtual images, 15.4 in patches, 4 x 38 x 62 x 62, 115 of 7 x 3 26.8 and 16.8; 19 of 25 layers, none the other way (many
     // channels earn the split back: 9 x 256 x 116 x 10, 6 of 2 x 2 18.6 and 26.1)
     if (v.ksplit == 2 && !v.cluster && v.cblks <= 8 && patch.ksplit == 1 && patch.makespan < 16000.0) return true;
-    // clearly more staged pixels than the producers load in a pass (1024 in quads), stage after stage, or any of more than 1300:
-    // 55 x 44 x 66 x 170, 7 maps of 5 x 5 259 and 188 us; 21 x 16 x 37 x 184, 4 of 7 x 7 67 and 40; 11 of 13 layers
-    const long long stages = ((long long)v.supertiles * v.n_blocks * v.ksplit + sms - 1) / sms * v.cblks / v.ksplit;
-    if (v.npix > 1300 || (quads && v.npix > 1100 && stages >= 3)) return true;
-    // a clear difference of the estimates: 2 x 272 x 51 x 247, 11 maps of 3 x 3 48 and 35 us
+    // a clear difference of the estimates: 55 x 44 x 66 x 170, 7 maps of 5 x 5 259 and 188 us; 21 x 16 x 37 x 184, 4 of 7 x 7 67 and
+    // 40; 2 x 272 x 51 x 247, 11 of 3 x 3 48 and 35
+    const bool quads = sh.W % 4 == 0;
     const double ev = estimated_cycles(v, quads), ep = estimated_cycles(patch, quads && sh.pad_w % 4 == 0);
-    return ev > 1.25 * ep && ev - ep > 6000.0;
+    return ev > 1.2 * ep && ev - ep > 6000.0;
 }
 
 // The patch width with the fewest staged pixels per output is the first choice.  A wider patch has a larger valid
