@@ -42,8 +42,8 @@ def test_padded_exact_on_integers(oracle, monkeypatch, case):
 
 @pytest.mark.parametrize("case", [
     (5, 80, 65, 33, 48, 3, 3, 1, 1),         # a contraction that only virtual images would split
-    (21, 16, 37, 184, 4, 7, 7, 3, 3),        # more staged pixels than the producers load in a pass
-    (2, 272, 51, 247, 11, 3, 3, 1, 1),       # a clear difference of the estimates
+    (21, 16, 37, 184, 4, 7, 7, 3, 3),        # a clear difference of the estimates: a long halo
+    (2, 272, 51, 247, 11, 3, 3, 1, 1),       # ... rows staged pixel by pixel
 ])
 def test_padded_layers_left_to_patches(oracle, case):
     N, C, H, W, K, R, S, ph, pw = case
