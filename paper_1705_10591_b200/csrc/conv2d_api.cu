@@ -412,7 +412,7 @@ struct CopySet {
         auto event = [&](cudaEvent_t& e) { ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess; };
         event(begin); event(end);
         for (int i = 0; i < kMaxChunks; ++i) { event(arrived[i]); event(done[i]); }
-        if (!ok) destroy();
+        if (!ok) { destroy(); (void)cudaGetLastError(); }      // (the call goes on without a set: its launches must not find the error)
         return ok;
     }
     void destroy()
