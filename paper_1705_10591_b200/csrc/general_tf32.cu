@@ -116,9 +116,8 @@ int describe_tensor_core_plan(const Shape& sh, bool b16, char* text, size_t text
     if (!p.ok) return snprintf(text, text_bytes, "tensor_core=0");
     const double out_px = (double)sh.N * sh.P * sh.Q;
     const double cols = (double)p.supertiles * p.tile_px;
-    const double rows = p.swap ? p.n_tile : kTileM;                     // rows of the M operand
-    const double ncols = p.swap ? (double)p.supertiles * p.tile_px * p.n_blocks
-                                : (double)p.supertiles * p.mt * p.n_blocks * p.n_tile;
+    const double rows = p.n_tile;                                       // rows of the M operand
+    const double ncols = cols * p.n_blocks;
     const double kdim = (double)p.cblks * (b16 ? 2 * kCB : kCB) * p.taps;
     double issued = 2.0 * rows * ncols * kdim;
     if (p.pair_compact) issued *= (double)p.cb_bytes / ((double)p.taps * kCB * p.n_tile * 4);    // lone taps are 64-row MMAs
@@ -127,7 +126,7 @@ int describe_tensor_core_plan(const Shape& sh, bool b16, char* text, size_t text
                     "tensor_core=1 kernel=general_tc addressing=%s filters_as=%s m_rows=%d tile_px=%d px_groups=%d acc_sets=%d items=%lld grid=%d "
                     "ksplit=%d cluster=%d resident_filters=%d stacked_taps=%d stacked_compact=%d fold=%dx%d patch_w=%d smem_bytes=%zu "
                     "mma_useful_px=%.4f mma_useful_flops=%.4f",
-                    p.patch_w ? "patch" : "flat", p.swap ? "M" : "N", (int)rows, p.tile_px, p.px_groups, p.nbuf,
+                    p.patch_w ? "patch" : "flat", "M", (int)rows, p.tile_px, p.px_groups, p.nbuf,
                     (long long)p.supertiles * p.n_blocks * p.ksplit, p.grid, p.ksplit, p.cluster, p.resident, p.pair_taps, p.pair_compact,
                     p.fold_r, p.fold_s, p.patch_w, p.smem_bytes, out_px / cols, useful / issued);
 }
@@ -233,10 +232,10 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     a.st = sh.stride; a.off_h = p.off_h; a.off_w = p.off_w; a.shift0 = p.shift0; a.ext = p.ext; a.quad2 = p.quad2;
     a.phases = p.phases; a.phase_cols = p.phase_cols; a.cblks_c = p.cblks / p.phases; a.div_phases = FastDiv(p.phases);
     a.mixed = p.mixed; a.mix_c = sh.C; a.mix_st2 = sh.stride * sh.stride;
-    a.n_tile = p.n_tile; a.n_blocks = p.n_blocks; a.mt = p.mt; a.tile_px = p.tile_px; a.px_groups = p.px_groups; a.nbuf = p.nbuf; a.npix = p.npix; a.cstride = chunk_stride(p.npix);
+    a.n_tile = p.n_tile; a.n_blocks = p.n_blocks; a.tile_px = p.tile_px; a.px_groups = p.px_groups; a.nbuf = p.nbuf; a.npix = p.npix; a.cstride = chunk_stride(p.npix);
     a.cblks = p.cblks; a.taps = p.taps;
     a.a_stages = p.a_stages; a.b_stages = p.b_stages; a.tps = p.tps;
-    a.cbg = p.cbg; a.groups = (p.cblks + p.cbg - 1) / p.cbg; a.resident = p.resident; a.swap = p.swap;
+    a.cbg = p.cbg; a.groups = (p.cblks + p.cbg - 1) / p.cbg; a.resident = p.resident;
     a.vec = 1;
     for (int v = 4; v >= 2; v >>= 1)       // v adjacent accumulator columns must be v adjacent, aligned outputs of one row
         if ((p.patch_w ? p.patch_tw : plan_w) % v == 0 && sh.Q % v == 0 && ((long long)sh.P * sh.Q) % v == 0 &&
@@ -250,7 +249,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     a.xchg_bytes = (int)xchg_area_bytes(p.xchg_slots);
     // (the helper warps of the last item's write-back: measured no gain for the two-block cluster, whose single item
     // per block is short: 34.0 us without them, 35.4 us with them on 32 x 256 x 14 x 14 -> 256 maps)
-    a.helpers = (p.swap && !p.cluster && (size_t)p.a_stages * p.cbg * kCB * chunk_stride(p.npix) * 4 >= 2 * kXposeBytes &&
+    a.helpers = (!p.cluster && (size_t)p.a_stages * p.cbg * kCB * chunk_stride(p.npix) * 4 >= 2 * kXposeBytes &&
                  env_int("CONV2D_B200_TF32_HELPERS", 1) != 0) ? 1 : 0;
     a.quad = ((p.virt ? (sh.stride == 1 && sh.W % 4 == 0) : p.patch_w ? (sh.W % 4 == 0 && sh.pad_w % 4 == 0) : (sh.H * sh.W) % 4 == 0) && p.fold_r * p.fold_s == 1 && env_int("CONV2D_B200_TF32_QUAD", 1) != 0) ? 1 : 0;
     {
@@ -286,7 +285,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     // tail of whatever kernel precedes it on the stream; it waits for that kernel before it touches global memory.
     const bool fold = p.fold_r * p.fold_s > 1;
     void (*kernel)(KernelArgs);
-    if (p.swap && p.n_tile == 64 && !p.pair_taps) {
+    if (p.n_tile == 64 && !p.pair_taps) {
         if (p.virt) kernel = general_tc_kernel<false, false, false, false, false, true, true>;
         else if (p.patch_w) kernel = b16 ? general_tc_kernel<true, false, true, false, false, false, true> : general_tc_kernel<false, false, true, false, false, false, true>;
         else if (fold) kernel = b16 ? general_tc_kernel<true, true, false, false, false, false, true> : general_tc_kernel<false, true, false, false, false, false, true>;

@@ -118,14 +118,14 @@ struct Ops {
         if (PAIR) tmem_dealloc_pair(taddr, cols); else tmem_dealloc(taddr, cols);
     }
     template <bool B16>
-    static __device__ __forceinline__ void mma(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, bool accumulate)
+    static __device__ __forceinline__ void mma(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, bool accumulate, uint32_t elected)
     {
-        if (PAIR) { if (B16) mma_b16_pair(d, ad, bd, idesc, accumulate); else mma_tf32_pair(d, ad, bd, idesc, accumulate); }
-        else { if (B16) mma_b16(d, ad, bd, idesc, accumulate); else mma_tf32(d, ad, bd, idesc, accumulate); }
+        if (PAIR) { if (B16) mma_b16_pair(d, ad, bd, idesc, accumulate, elected); else mma_tf32_pair(d, ad, bd, idesc, accumulate, elected); }
+        else { if (B16) mma_b16(d, ad, bd, idesc, accumulate, elected); else mma_tf32(d, ad, bd, idesc, accumulate, elected); }
     }
     // arrives on `bar` (of both blocks of a pair) when the MMAs issued so far have completed
-    static __device__ __forceinline__ void commit(uint64_t* bar) { if (PAIR) mma_commit_pair_both(bar); else mma_commit(bar); }
-    static __device__ __forceinline__ void commit_local(uint64_t* bar) { if (PAIR) mma_commit_pair(bar); else mma_commit(bar); }
+    static __device__ __forceinline__ void commit(uint64_t* bar, uint32_t elected) { if (PAIR) mma_commit_pair_both(bar, elected); else mma_commit(bar, elected); }
+    static __device__ __forceinline__ void commit_local(uint64_t* bar, uint32_t elected) { if (PAIR) mma_commit_pair(bar, elected); else mma_commit(bar, elected); }
 };
 
 // PAIR = false: one block per work item (a pixel tile x one block of `m_rows` filters).
@@ -289,11 +289,14 @@ pointwise_tma_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
             }
         }
     } else if (warp == 1) {
-        // ---------------- MMA issue (one thread; of a pair: of its first block)
-        if (lane == 0 && first_block) {
+        // ---------------- MMA issue (the whole warp runs the loop, one elected lane issues, of a pair in its first block;
+        // the general kernel has the figures)
+        if (first_block) {
+            const uint32_t elected = elect_one();
+            const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);     // (warp-uniform for the compiler, too)
             const uint32_t a_base = smem_u32(a_smem), b_base = smem_u32(b_smem);
             int cur_bank = -1, slot = 0, buf = 0;
-            uint32_t ph = 0, a_waits = 0, acc_phase[2] = {0u, 0u};
+            uint32_t ph = 0, a_waits = 0, acc_phase = 0;              // (bit b: accumulator set b)
             bool alive = true;
             for (int item = worker; item < a.items && alive; item += n_workers) {
                 int bank, first, unit, c_lo, c_n;
@@ -302,17 +305,17 @@ pointwise_tma_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
                 const bool new_bank = !stream_a && bank != cur_bank;
                 cur_bank = bank;
                 // (of a pair: both blocks' write-back warps arrive here, the peer's with cluster-scope release)
-                if (!(PAIR ? mbar_wait_bounded_cluster(&acc_empty[buf], acc_phase[buf] ^ 1u, abort_flag, a.max_polls)
-                           : mbar_wait_bounded(&acc_empty[buf], acc_phase[buf] ^ 1u, abort_flag, a.max_polls))) { alive = false; break; }
+                if (!(PAIR ? mbar_wait_bounded_cluster_warp(&acc_empty[buf], (acc_phase >> buf & 1u) ^ 1u, abort_flag, a.max_polls)
+                           : mbar_wait_bounded_warp(&acc_empty[buf], (acc_phase >> buf & 1u) ^ 1u, abort_flag, a.max_polls))) { alive = false; break; }
                 tc_fence_after_sync();
                 const int groups = (PAIR && a.wide) ? 2 : 1;                 // MMA widths per item
                 const uint32_t n_cols = (uint32_t)((PAIR ? a.a_item / groups : min(a.a_item, a.total_atoms - first)) * kAtomPx);
                 const uint32_t m = PAIR ? 256u : (uint32_t)a.m_rows;
                 const uint32_t idesc = (B16 ? idesc_b16(m, n_cols, a.fp16 != 0) : idesc_tf32(m, n_cols)) | kIdescBMajorMN;
-                const uint32_t d = tmem + (uint32_t)(buf * kAccCols);
+                const uint32_t d = tmem_u + (uint32_t)(buf * kAccCols);
                 for (int st = 0; st < c_n && alive; ++st) {
-                    if (new_bank && !mbar_wait_bounded(&a_full[st], a_waits & 1u, abort_flag, a.max_polls)) { alive = false; break; }
-                    if (!mbar_wait_bounded(&b_full[slot], ph, abort_flag, a.max_polls)) { alive = false; break; }
+                    if (new_bank && !mbar_wait_bounded_warp(&a_full[st], a_waits & 1u, abort_flag, a.max_polls)) { alive = false; break; }
+                    if (!mbar_wait_bounded_warp(&b_full[slot], ph, abort_flag, a.max_polls)) { alive = false; break; }
                     tc_fence_after_sync();
                     const uint32_t stage = b_base + (uint32_t)slot * b_stage_bytes;
                     const uint32_t a_chunk = stream_a ? stage : a_base + (uint32_t)st * a_chunk_bytes;
@@ -326,23 +329,23 @@ pointwise_tma_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
                             const uint64_t a_desc = smem_desc_sw128(a_chunk + (uint32_t)kk * 32u, 16u, 1024u);
                             const uint64_t b_desc = B16 ? smem_desc_sw128(b_grp + (uint32_t)kk * 2048u, (uint32_t)kStageCh * 128u, 1024u)
                                                         : smem_desc_mn_sw128_32b(b_grp + (uint32_t)kk * 1024u, (uint32_t)kStageCh * 128u, 512u);
-                            Op::template mma<B16>(d + (uint32_t)(g * kAccCols), a_desc, b_desc, idesc, st > 0 || kk > 0);
+                            Op::template mma<B16>(d + (uint32_t)(g * kAccCols), a_desc, b_desc, idesc, st > 0 || kk > 0, elected);
                         }
                     }
-                    Op::commit(&b_empty[slot]);
+                    Op::commit(&b_empty[slot], elected);
                     if (++slot == a.stages) { slot = 0; ph ^= 1u; }
                 }
                 if (!alive) break;
                 if (new_bank) ++a_waits;
-                Op::commit(&acc_full[buf]);
+                Op::commit(&acc_full[buf], elected);
                 // the next item of this block uses another filter block: tell the loaders when this bank is free
                 const int next = item + n_workers;
-                if (!stream_a && next < a.items && a.div_tiles.div(next) != bank) Op::commit(a_empty);
-                acc_phase[buf] ^= 1u;
+                if (!stream_a && next < a.items && a.div_tiles.div(next) != bank) Op::commit(a_empty, elected);
+                acc_phase ^= 1u << buf;
                 if (!(PAIR && a.wide)) buf ^= 1;         // (a wide item uses both sets: one logical buffer)
             }
             if (!alive) {
-                Op::commit_local(drain_bar);
+                Op::commit_local(drain_bar, elected);
                 uint32_t dummy = 0;
                 mbar_wait_bounded(drain_bar, 0u, &dummy, 1u << 16);
             }

@@ -53,6 +53,26 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     return false;
 }
 
+// The warp forms below are for the warp that issues the MMAs: all 32 lanes run its loop and decide together, so that the
+// compiler sees warp-uniform values (a tcgen05.mma takes its operands from uniform registers; from the registers of one
+// diverged lane they are moved there for every instruction), and one elected lane's instructions take effect.
+// The lane that elect.sync picks (1 there, 0 elsewhere).
+__device__ __forceinline__ uint32_t elect_one()
+{
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ bool mbar_wait_bounded_warp(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag, uint32_t max_polls)
+{
+    for (uint32_t i = 0; i < max_polls; ++i) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if ((i & 63u) == 63u && __any_sync(0xffffffffu, *abort_flag != 0u)) return false;
+    }
+    *abort_flag = 1u;
+    return false;
+}
+
 // ---------------------------------------------------------------- thread-block clusters (distributed shared memory)
 __device__ __forceinline__ uint32_t cluster_ctarank()
 {
@@ -92,6 +112,16 @@ __device__ __forceinline__ bool mbar_wait_bounded_cluster(uint64_t* bar, uint32_
     for (uint32_t i = 0; i < max_polls; ++i) {
         if (mbar_try_wait_cluster(bar, parity)) return true;
         if ((i & 63u) == 63u && *abort_flag) return false;
+    }
+    *abort_flag = 1u;
+    return false;
+}
+__device__ __forceinline__ bool mbar_wait_bounded_cluster_warp(uint64_t* bar, uint32_t parity, volatile uint32_t* abort_flag,
+                                                               uint32_t max_polls)
+{
+    for (uint32_t i = 0; i < max_polls; ++i) {
+        if (__all_sync(0xffffffffu, mbar_try_wait_cluster(bar, parity))) return true;
+        if ((i & 63u) == 63u && __any_sync(0xffffffffu, *abort_flag != 0u)) return false;
     }
     *abort_flag = 1u;
     return false;
@@ -219,56 +249,60 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t colum
 __device__ __forceinline__ void tc_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// D[tmem] (+)= A[smem] * B[smem]^T, TF32 operands, fp32 accumulate; one thread issues.
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate)
+// D[tmem] (+)= A[smem] * B[smem]^T, TF32 operands, fp32 accumulate.  The whole warp executes it (and the commits below),
+// the lane with `elected` != 0 issues.
+__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate, uint32_t elected)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate), "r"(elected) : "memory");
 }
 // Same with 16-bit operands, bf16 or fp16 as the instruction descriptor says (kind::f16, K = 16 per instruction).
-__device__ __forceinline__ void mma_b16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate)
+__device__ __forceinline__ void mma_b16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate, uint32_t elected)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate), "r"(elected) : "memory");
 }
-// Arrives once on `bar` when all tcgen05.mma issued so far by this thread have completed.
-__device__ __forceinline__ void mma_commit(uint64_t* bar)
+// Arrives once on `bar` when all tcgen05.mma issued so far by the elected lane have completed.
+__device__ __forceinline__ void mma_commit(uint64_t* bar, uint32_t elected)
 {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                 ::"r"(smem_u32(bar)) : "memory");
+    asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t"
+                 "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 ::"r"(smem_u32(bar)), "r"(elected) : "memory");
 }
 // Two-SM MMAs, issued by one thread of the pair's first block.  D is 256 x N: rows 0-127 in the first block's tensor
 // memory, rows 128-255 in the second's, N columns in both.  The descriptors are offsets that hold in both blocks:
 // each block's shared memory holds its 128 rows of A and its half of B's N rows at the same addresses.
-__device__ __forceinline__ void mma_tf32_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate)
+__device__ __forceinline__ void mma_tf32_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate, uint32_t elected)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate), "r"(elected) : "memory");
 }
-__device__ __forceinline__ void mma_b16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate)
+__device__ __forceinline__ void mma_b16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate, uint32_t elected)
 {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
+        "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.ne.b32 e, %5, 0;\n\t"
+        "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate), "r"(elected) : "memory");
 }
 // Arrives once on `bar` of this block when all two-SM MMAs issued so far by this thread have completed ...
-__device__ __forceinline__ void mma_commit_pair(uint64_t* bar)
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar, uint32_t elected)
 {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                 ::"r"(smem_u32(bar)) : "memory");
+    asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t"
+                 "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+                 ::"r"(smem_u32(bar)), "r"(elected) : "memory");
 }
 // ... and on the barrier at the same offset in both blocks of the pair.
-__device__ __forceinline__ void mma_commit_pair_both(uint64_t* bar)
+__device__ __forceinline__ void mma_commit_pair_both(uint64_t* bar, uint32_t elected)
 {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(smem_u32(bar)), "h"((unsigned short)3) : "memory");
+    asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %2, 0;\n\t"
+                 "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n\t}"
+                 ::"r"(smem_u32(bar)), "h"((unsigned short)3), "r"(elected) : "memory");
 }
 // 32 lanes x 16 consecutive 32-bit columns: thread i of the warp receives lane (base lane + i).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16])

@@ -45,7 +45,7 @@ struct KernelArgs {
     int vec_shift;    // log2(vec)
     FastDiv div_ksplit, div_n_blocks, div_groups_lo, div_groups_hi, div_per_image, div_patch_cols;   // divisors of the item decoding
     int patch_item_rows;   // patch addressing: output rows of one item (tile_px / patch_w)
-    int n_tile, n_blocks, mt, tile_px, px_groups, nbuf, npix, cblks, taps, a_stages, b_stages, tps;
+    int n_tile, n_blocks, tile_px, px_groups, nbuf, npix, cblks, taps, a_stages, b_stages, tps;
     int rot;          // quad producers rotate their chunk order per lane (see there)
     int cstride;      // 16-byte units between the 4-channel chunks of a staged channel block (npix + 1: odd)
     int patch_w, patch_tw, patch_rows, patch_cols;   // patch addressing (PATCH kernels): staged row pitch, valid output
@@ -54,15 +54,14 @@ struct KernelArgs {
     int row_pitch;    // pixels between vertically adjacent taps in the staged sequence: W, or patch_w
     int fp16;         // 16-bit operands only: 1 = IEEE half, 0 = bf16
     int fold_r, fold_s;  // taps folded into the channel dimension (1, 1: none); R, S below are what is left as shifts
-    int helpers;      // 1: warps 8-15 share the write-back of a block's last item (operand-swap layout only)
+    int helpers;      // 1: warps 8-15 share the write-back of a block's last item
     int pgroups;      // producer groups (1, 2 or 4): stage k is filled by group k % pgroups
     int quad2;        // 1: stride 2, producers load four adjacent pixels (two virtual pixels of both phases of a row) per word
     int quad;         // producers load four adjacent pixels per 128-bit (fp32) or 64-bit (16-bit operands) word (needs H*W % 4 == 0)
     int pair;         // 16-bit operands only: producers load two adjacent pixels per 32-bit word (needs H*W even)
     int cbg, groups;        // channel blocks per activation stage, number of such groups
     int resident;           // filters loaded once per thread block instead of streamed
-    int swap;               // operand roles swapped: accumulator lanes = filters, columns = pixels
-    int vec;                // swap mode: adjacent pixels a lane stores as one unit (1, 2 or 4)
+    int vec;                // adjacent pixels a lane stores as one unit (1, 2 or 4)
     int pair_taps;          // stacked taps: accumulator lanes 64-127 hold the right-hand tap of each pair, one column to the right
     int s_slots, s_step;    // shift-table entries per filter row and the horizontal shift between them (2 with stacked taps)
     int pair_compact;       // stacked taps, resident bank: the odd last tap of a filter row is a 64-row slice of its own,
@@ -376,34 +375,30 @@ __device__ __forceinline__ ItemInfo decode_item(const KernelArgs& a, int item)
     return it;
 }
 
-// All MMAs of one tap of one channel block in the filters-as-M layout: K steps 0 and 1 for GROUPS pixel groups
-// of n_mma pixels.  d: accumulator column of group 0; px_lo / flt_lo: low words of the pixel and filter
-// descriptors of K step 0 (the K step and the group add constants to the start-address field); acc = 0 only
-// for the very first tap of an item.
+// All MMAs of one tap of one channel block: K steps 0 and 1 for GROUPS pixel groups of n_mma pixels.  d: accumulator
+// column of group 0; px_lo / flt_lo: low words of the pixel and filter descriptors of K step 0 (the K step and the group
+// add constants to the start-address field); acc = 0 only for the very first tap of an item.  The whole warp executes it,
+// the lane with `elected` != 0 issues.
 template <bool B16, int GROUPS>
 __device__ __forceinline__ void issue_tap(uint32_t d, uint32_t px_lo, uint32_t flt_lo, uint32_t px_kstep, uint32_t flt_kstep,
-                                          uint32_t n_mma, uint32_t desc_hi, uint32_t idesc, uint32_t acc)
+                                          uint32_t n_mma, uint32_t desc_hi, uint32_t idesc, uint32_t acc, uint32_t elected)
 {
-#define CONV2D_TAP_MMA(KIND)                                                                                  \
+#define CONV2D_GROUP_MMA(KIND, D, PX)                                                                         \
     asm volatile(                                                                                             \
-        "{\n\t.reg .pred p, q;\n\t.reg .b64 f0, f1, x;\n\t.reg .b32 t, dd;\n\t"                                 \
-        "setp.ne.b32 p, %8, 0;\n\tsetp.eq.b32 q, 0, 0;\n\t"                                                   \
-        "mov.b64 f0, {%2, %6};\n\tadd.u32 t, %2, %4;\n\tmov.b64 f1, {t, %6};\n\t"                             \
-        "mov.b64 x, {%1, %6};\n\t"                                                                            \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [%0], f0, x, %7, p;\n\t"                                      \
-        "add.u32 t, %1, %3;\n\tmov.b64 x, {t, %6};\n\t"                                                      \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [%0], f1, x, %7, q;\n\t"                                      \
-        "setp.ne.b32 q, %9, 0;\n\t"                                                                           \
-        "@!q bra DONE_%=;\n\t"                                                                                \
-        "add.u32 dd, %0, %5;\n\tadd.u32 t, %1, %5;\n\tmov.b64 x, {t, %6};\n\t"                               \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [dd], f0, x, %7, p;\n\t"                                      \
-        "add.u32 t, t, %3;\n\tmov.b64 x, {t, %6};\n\t"                                                       \
-        "tcgen05.mma.cta_group::1.kind::" KIND " [dd], f1, x, %7, q;\n\t"                                      \
-        "DONE_%=:\n\t}"                                                                                       \
-        ::"r"(d), "r"(px_lo), "r"(flt_lo), "r"(px_kstep), "r"(flt_kstep), "r"(n_mma), "r"(desc_hi), "r"(idesc), \
-          "r"(acc), "n"(GROUPS == 2 ? 1 : 0) : "memory")
-    if (B16) CONV2D_TAP_MMA("f16"); else CONV2D_TAP_MMA("tf32");
-#undef CONV2D_TAP_MMA
+        "{\n\t.reg .pred p, q, e;\n\t.reg .b64 f, x;\n\t.reg .b32 t;\n\t"                                 \
+        "setp.ne.b32 p, %7, 0;\n\tsetp.eq.b32 q, 0, 0;\n\tsetp.ne.b32 e, %8, 0;\n\t"                         \
+        "mov.b64 f, {%2, %5};\n\tmov.b64 x, {%1, %5};\n\t"                                                  \
+        "@e tcgen05.mma.cta_group::1.kind::" KIND " [%0], f, x, %6, p;\n\t"                                    \
+        "add.u32 t, %2, %4;\n\tmov.b64 f, {t, %5};\n\tadd.u32 t, %1, %3;\n\tmov.b64 x, {t, %5};\n\t"         \
+        "@e tcgen05.mma.cta_group::1.kind::" KIND " [%0], f, x, %6, q;\n\t}"                                   \
+        ::"r"(D), "r"(PX), "r"(flt_lo), "r"(px_kstep), "r"(flt_kstep), "r"(desc_hi), "r"(idesc), "r"(acc),    \
+          "r"(elected) : "memory")
+#pragma unroll
+    for (int g = 0; g < GROUPS; ++g) {
+        if (B16) CONV2D_GROUP_MMA("f16", d + g * n_mma, px_lo + g * n_mma);
+        else CONV2D_GROUP_MMA("tf32", d + g * n_mma, px_lo + g * n_mma);
+    }
+#undef CONV2D_GROUP_MMA
 }
 
 // CLUSTER: the two work items of a split contraction (ksplit = 2) run as a two-block cluster, one item per block.
@@ -427,8 +422,8 @@ general_tc_kernel(const KernelArgs a)
     unsigned char* b_smem = smem + (size_t)a.a_stages * a_stage_bytes;
     const int bank_blocks = VIRT ? a.cblks_c : a.cblks;                 // pieces of cb_bytes in a filter block's bank
     const size_t b_region_bytes = a.resident ? (size_t)bank_blocks * a.cb_bytes : (size_t)a.b_stages * b_stage_bytes;
-    float* xpose = reinterpret_cast<float*>(b_smem + b_region_bytes);            // only present (and used) when a.swap
-    unsigned char* after_xpose = b_smem + b_region_bytes + (a.swap ? kXposeBytes : 0);
+    float* xpose = reinterpret_cast<float*>(b_smem + b_region_bytes);
+    unsigned char* after_xpose = b_smem + b_region_bytes + kXposeBytes;
     float* xchg = reinterpret_cast<float*>(after_xpose);     // CLUSTER: [4 quarters][xchg_slots][8 column groups][32 lanes][4 floats] partial sums from the peer
     uint64_t* xbar = reinterpret_cast<uint64_t*>(after_xpose + (size_t)kEpilogueWarps * a.xchg_slots * kXchgBlockFloats * 4);   // [4][xchg_slots]
     uint64_t* bars = reinterpret_cast<uint64_t*>(after_xpose + (CLUSTER ? a.xchg_bytes : 0));
@@ -445,8 +440,7 @@ general_tc_kernel(const KernelArgs a)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     volatile unsigned long long* t_entry = reinterpret_cast<volatile unsigned long long*>(tmem_slot + 2);
-    uint32_t* tap_shift = tmem_slot + 4;                   // [taps] r * row_pitch + s of every tap, in staged pixels
-    // (bit 31: the slot is a lone tap held as a 64-row slice, see pair_compact)
+    uint32_t* tap_shift = tmem_slot + 4;                   // phases with taps of their own: [R * S] shift of every tap, in staged pixels
     // (behind the tap shifts; the planner keeps kMaxTaps entries for both)
     uint2* phase_table = reinterpret_cast<uint2*>(tap_shift + ((VIRT ? a.R * a.S : 0) + 1) / 2 * 2);
     if (VIRT)
@@ -467,10 +461,7 @@ general_tc_kernel(const KernelArgs a)
             const Phase p = unpack_phase(describe_phase(a, (r - r2 * a.st) * a.phase_cols + sx - s2 * a.st));
             tap_shift[p.base + r2 * p.cols + s2 - p.col0] = (uint32_t)(r2 * a.row_pitch + s2);
         }
-    } else
-    for (int t = tid; t < a.taps; t += kThreads)
-        tap_shift[t] = (uint32_t)((t / a.s_slots) * a.row_pitch + (t % a.s_slots) * a.s_step) |
-                       ((a.pair_compact && (a.S & 1) && t % a.s_slots == a.s_slots - 1) ? 0x80000000u : 0u);
+    }
     if (kDiag && tid == 0) *t_entry = wall_ns();
 
     if (tid == 0) {
@@ -502,7 +493,7 @@ general_tc_kernel(const KernelArgs a)
 
     // Work item -> (supertile, filter block); blocks rotate the order of the channel-block groups by the
     // item number, so that at any moment they stream different parts of the filter bank.
-    const int acc_cols = a.swap ? a.tile_px : a.mt * a.n_tile;   // tensor-memory columns of one accumulator set
+    const int acc_cols = a.tile_px;   // tensor-memory columns of one accumulator set
 
     if (warp == 0) {
         // ---------------- filters: global -> shared by bulk copy, up to `tps` taps of one channel block per stage
@@ -565,23 +556,16 @@ general_tc_kernel(const KernelArgs a)
             }
         }
     } else if (warp == 1) {
-        // ---------------- MMA issue (one thread)
-        if (lane == 0) {
-            // Per MMA this thread only adds small constants to the low word of a descriptor: everything
-            // that does not change is folded into a_lo_fixed / b_lo_fixed / desc_hi beforehand, because a
-            // single thread issuing ~40 dependent integer instructions per MMA was slower than the MMA.
-            const uint32_t m_rows = a.swap ? (uint32_t)a.n_tile : (uint32_t)kTileM;
-            const uint32_t n_mma = (uint32_t)(a.tile_px / a.px_groups);          // operand-swap layout: pixels per MMA
-            const uint32_t n_cols = a.swap ? n_mma : (uint32_t)a.n_tile;
-            const uint32_t idesc = B16 ? idesc_b16(m_rows, n_cols, a.fp16 != 0) : idesc_tf32(m_rows, n_cols);
-            auto pack64 = [](uint32_t lo, uint32_t hi) {
-                uint64_t r;
-                asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
-                return r;
-            };
-            auto mma = [](uint32_t d, uint64_t ad, uint64_t bd, uint32_t id, bool acc) {
-                if (B16) mma_b16(d, ad, bd, id, acc); else mma_tf32(d, ad, bd, id, acc);
-            };
+        // ---------------- MMA issue.  All 32 lanes run the loop and one elected lane issues: a tcgen05.mma takes its
+        // operands from uniform registers, which the compiler fills for nothing where the warp stays together, and with
+        // moves of their own for every instruction where one lane has gone its own way.  In a loop of this shape with a
+        // stage boundary every 6 to 10 MMAs, cycles per MMA of a lone lane / of the warp: N = 256 155 / 132, N = 224 (two
+        // groups) 122 / 114, N = 176 139 / 99, N = 96 161 / 93 (the pipe's own: 128, 112, 88, 64).
+        {
+            const uint32_t elected = elect_one();
+            const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);      // (warp-uniform for the compiler, too)
+            const uint32_t n_mma = (uint32_t)(a.tile_px / a.px_groups);          // pixels per MMA
+            const uint32_t idesc = B16 ? idesc_b16((uint32_t)a.n_tile, n_mma, a.fp16 != 0) : idesc_tf32((uint32_t)a.n_tile, n_mma);
             // (the start-address field of a descriptor holds bits 4-17 of the shared-memory address; the address of a
             // block that is not the first of its cluster has bits above those set, which must not leak into LBO)
             const uint32_t desc_hi = (128u >> 4) | (1u << 14);                  // SBO = 128 B, descriptor version 1
@@ -596,10 +580,10 @@ general_tc_kernel(const KernelArgs a)
             // free accumulator set, its total cycles, its item count
             long long wait_a = 0, wait_acc = 0, issue_cycles = 0;
             const long long t_begin = clock_now();
-            if (kDiag && blockIdx.x == 0) a.status[6] = (unsigned)(wall_ns() - *t_entry);   // ns from kernel entry to the start of the MMA loop
+            if (kDiag && blockIdx.x == 0 && lane == 0) a.status[6] = (unsigned)(wall_ns() - *t_entry);   // ns from kernel entry to the start of the MMA loop
             int n_items = 0;
             if (a.resident) {
-                if (!mbar_wait_bounded(&b_full[0], 0u, abort_flag, a.max_polls)) alive = false;
+                if (!mbar_wait_bounded_warp(&b_full[0], 0u, abort_flag, a.max_polls)) alive = false;
                 tc_fence_after_sync();
             }
             for (int item = blockIdx.x; item < a.items && alive; item += gridDim.x) {
@@ -607,14 +591,14 @@ general_tc_kernel(const KernelArgs a)
                 // the accumulator set must have been drained by the epilogue of its previous item
                 const uint32_t acc_phase = buf ? acc_phase1 : acc_phase0;
                 long long tw = clock_now();
-                if (!mbar_wait_bounded(&acc_empty[buf], acc_phase ^ 1u, abort_flag, a.max_polls)) { alive = false; break; }
+                if (!mbar_wait_bounded_warp(&acc_empty[buf], acc_phase ^ 1u, abort_flag, a.max_polls)) { alive = false; break; }
                 tc_fence_after_sync();
                 wait_acc += clock_now() - tw;
-                const uint32_t d0 = tmem + (uint32_t)(buf * acc_cols);
+                const uint32_t d0 = tmem_u + (uint32_t)(buf * acc_cols);
                 uint32_t accumulate = 0;
                 for (int grp = 0; grp < ii.n_groups && alive; ++grp) {
                     tw = clock_now();
-                    if (!mbar_wait_bounded(&a_full[as], a_phase, abort_flag, a.max_polls)) { alive = false; break; }
+                    if (!mbar_wait_bounded_warp(&a_full[as], a_phase, abort_flag, a.max_polls)) { alive = false; break; }
                     tc_fence_after_sync();
                     wait_a += clock_now() - tw;
                     const long long t_issue0 = clock_now();
@@ -624,13 +608,12 @@ general_tc_kernel(const KernelArgs a)
                     uint32_t a_lo_block = a_lo_fixed | ((smem_u32(a_smem + (size_t)as * a_stage_bytes) >> 4) & 0x3FFFu);
                     for (int g = 0; g < a.cbg && alive; ++g, a_lo_block += a_block_bytes >> 4) {
                         if (gr * a.cbg + g >= a.cblks) break;
-                        uint32_t row_shift = VIRT ? (uint32_t)a.shift0 : 0u;     // r * row pitch, in pixels (= 16-byte units)
-                        int sx = 0, sc = 0;
-                        int taps = a.taps, s_slots = a.s_slots, tap0 = 0, sx0 = 0;
+                        uint32_t row_shift = 0;                                  // r * row pitch, in pixels (= 16-byte units)
+                        int sx = 0, sc = 0, taps = a.taps, tap0 = 0;
                         size_t bank_at = (size_t)(gr * a.cbg + g) * a.cb_bytes;   // (resident filters)
                         if (VIRT && a.phases > 1) {
                             const Phase p = phase_of(a, phase_table, gr * a.cbg + g);
-                            taps = p.taps; s_slots = p.cols; tap0 = p.base; sx0 = sx = p.col0;
+                            taps = p.taps; tap0 = p.base;
                             bank_at = (size_t)p.cblk * a.cb_bytes + (size_t)p.base * b_chunk_bytes;
                         }
                         for (int t0 = 0; t0 < taps; t0 += a.tps) {
@@ -639,80 +622,61 @@ general_tc_kernel(const KernelArgs a)
                             if (a.resident) {
                                 b_lo = b_lo_fixed | ((smem_u32(b_smem + bank_at) >> 4) & 0x3FFFu);
                             } else {
-                                if (!mbar_wait_bounded(&b_full[bs], b_phase, abort_flag, a.max_polls)) { alive = false; break; }
+                                if (!mbar_wait_bounded_warp(&b_full[bs], b_phase, abort_flag, a.max_polls)) { alive = false; break; }
                                 tc_fence_after_sync();
                                 b_lo = b_lo_fixed | ((smem_u32(b_smem + (size_t)bs * b_stage_bytes) >> 4) & 0x3FFFu);
                             }
-                            if (a.swap && a.px_groups == 1) {
-                                // M operand = the 128 filters of this stage, N operand = n_mma staged pixels.
-                                // One MMA pair per tap carries less tensor-pipe work than this one thread needs to
-                                // issue it with loop and address arithmetic around it (~230 cycles per MMA that
-                                // way), so a tap is one block of straight-line code and its shift comes from a
-                                // table, fetched one tap ahead.
-                                const uint32_t* shift = tap_shift + tap0 + t0;
-                                uint32_t cur = shift[0];
-                                if (STACK && a.pair_compact) {
-                                    // pairs of taps as M = 128 slices, a lone last tap as an M = 64 slice of half the size
-                                    // (its chunk stride and K step are half as long too) onto the same accumulator lanes
-                                    const uint32_t idesc64 = B16 ? idesc_b16(64u, n_cols, a.fp16 != 0) : idesc_tf32(64u, n_cols);
-                                    for (int t = 0; t < nt; ++t) {
-                                        const uint32_t a_lo = (VIRT ? a_lo_block + (uint32_t)a.shift0 : a_lo_block) + (cur & 0x7FFFFFFFu);
-                                        const bool lone = (cur >> 31) != 0u;
-                                        cur = shift[t + 1 < nt ? t + 1 : t];
-                                        if (lone) {
-                                            issue_tap<B16, 1>(d0, a_lo, b_lo - (64u << 16), a_kstep, b_kstep >> 1, n_mma, desc_hi, idesc64, accumulate);
-                                            b_lo += b_chunk_bytes >> 5;
-                                        } else {
-                                            issue_tap<B16, 1>(d0, a_lo, b_lo, a_kstep, b_kstep, n_mma, desc_hi, idesc, accumulate);
-                                            b_lo += b_chunk_bytes >> 4;
-                                        }
-                                        accumulate = 1;
+                            // (the taps of a phase lie in its table; all others step through the rows)
+                            const bool table = VIRT && a.phases > 1;
+                            const uint32_t* shift = tap_shift + tap0 + t0;
+                            auto next_tap = [&](int t) {
+                                uint32_t px_lo = a_lo_block + (VIRT ? (uint32_t)a.shift0 : 0u);
+                                if (table) return px_lo + shift[t];
+                                px_lo += row_shift + (uint32_t)sx;
+                                sx += a.s_step;
+                                if (++sc == a.s_slots) { sc = 0; sx = 0; row_shift += (uint32_t)a.row_pitch; }
+                                return px_lo;
+                            };
+                            if (STACK && a.pair_compact) {
+                                // pairs of taps as M = 128 slices, a lone last tap as an M = 64 slice of half the size
+                                // (its chunk stride and K step are half as long too) onto the same accumulator lanes
+                                const uint32_t idesc64 = B16 ? idesc_b16(64u, n_mma, a.fp16 != 0) : idesc_tf32(64u, n_mma);
+                                for (int t = 0; t < nt; ++t) {
+                                    const bool lone = (a.S & 1) && sc == a.s_slots - 1;
+                                    const uint32_t a_lo = next_tap(t);
+                                    if (lone) {
+                                        issue_tap<B16, 1>(d0, a_lo, b_lo - (64u << 16), a_kstep, b_kstep >> 1, n_mma, desc_hi, idesc64, accumulate, elected);
+                                        b_lo += b_chunk_bytes >> 5;
+                                    } else {
+                                        issue_tap<B16, 1>(d0, a_lo, b_lo, a_kstep, b_kstep, n_mma, desc_hi, idesc, accumulate, elected);
+                                        b_lo += b_chunk_bytes >> 4;
                                     }
-                                } else
+                                    accumulate = 1;
+                                }
+                            } else if (a.px_groups == 1) {
 #pragma unroll 3
                                 for (int t = 0; t < nt; ++t, b_lo += b_chunk_bytes >> 4) {
-                                    const uint32_t a_lo = (VIRT ? a_lo_block + (uint32_t)a.shift0 : a_lo_block) + cur;
-                                    cur = shift[t + 1 < nt ? t + 1 : t];
-                                    issue_tap<B16, 1>(d0, a_lo, b_lo, a_kstep, b_kstep, n_mma, desc_hi, idesc, accumulate);
+                                    issue_tap<B16, 1>(d0, next_tap(t), b_lo, a_kstep, b_kstep, n_mma, desc_hi, idesc, accumulate, elected);
                                     accumulate = 1;
                                 }
                             } else {
                                 for (int t = 0; t < nt; ++t, b_lo += b_chunk_bytes >> 4) {
-                                    uint32_t a_lo = a_lo_block + row_shift + (uint32_t)sx;
-                                    if (VIRT && a.quad2 && a.phases > 1) a_lo = a_lo_block + (uint32_t)a.shift0 + tap_shift[tap0 + t0 + t];
-                                    uint32_t d = d0;
-                                    if (a.swap) {
-                                        // two pixel groups: four MMAs per tap keep the pipe busy (measured faster
-                                        // when the compiler schedules the address arithmetic between them)
-                                        const uint64_t bd0 = pack64(b_lo, desc_hi), bd1 = pack64(b_lo + b_kstep, desc_hi);
-                                        mma(d, bd0, pack64(a_lo, desc_hi), idesc, accumulate != 0);
-                                        mma(d, bd1, pack64(a_lo + a_kstep, desc_hi), idesc, true);
-                                        mma(d + n_mma, bd0, pack64(a_lo + n_mma, desc_hi), idesc, accumulate != 0);
-                                        mma(d + n_mma, bd1, pack64(a_lo + n_mma + a_kstep, desc_hi), idesc, true);
-                                    } else {
-                                        for (int m = 0; m < a.mt; ++m, a_lo += kTileM, d += (uint32_t)a.n_tile) {
-                                            mma(d, ((uint64_t)desc_hi << 32) | a_lo, ((uint64_t)desc_hi << 32) | b_lo, idesc, accumulate != 0);
-                                            mma(d, ((uint64_t)desc_hi << 32) | (a_lo + a_kstep),
-                                                     ((uint64_t)desc_hi << 32) | (b_lo + b_kstep), idesc, true);
-                                        }
-                                    }
+                                    issue_tap<B16, 2>(d0, next_tap(t), b_lo, a_kstep, b_kstep, n_mma, desc_hi, idesc, accumulate, elected);
                                     accumulate = 1;
-                                    sx += a.s_step;
-                                    if (++sc == s_slots) { sc = 0; sx = sx0; row_shift += (uint32_t)a.row_pitch; }
                                 }
                             }
                             if (!a.resident) {
-                                mma_commit(&b_empty[bs]);   // frees the filter stage when these MMAs have read it
+                                mma_commit(&b_empty[bs], elected);   // frees the filter stage when these MMAs have read it
                                 if (++bs == a.b_stages) { bs = 0; b_phase ^= 1u; }
                             }
                         }
                     }
                     issue_cycles += clock_now() - t_issue0;
-                    if (alive) mma_commit(&a_empty[as]);
+                    if (alive) mma_commit(&a_empty[as], elected);
                     if (++as == a.a_stages) { as = 0; a_phase ^= 1u; }
                 }
-                if (alive) mma_commit(&acc_full[buf]);
-                if (alive && item + (int)gridDim.x >= a.items) mma_commit(tail_full);
+                if (alive) mma_commit(&acc_full[buf], elected);
+                if (alive && item + (int)gridDim.x >= a.items) mma_commit(tail_full, elected);
                 if (buf) acc_phase1 ^= 1u; else acc_phase0 ^= 1u;
                 if (++buf == a.nbuf) buf = 0;
                 ++n_items;
@@ -720,11 +684,11 @@ general_tc_kernel(const KernelArgs a)
             if (!alive) {
                 // A wait ran out: MMAs issued before that may still be reading shared memory and writing tensor
                 // memory.  Let them finish (bounded) before the block frees its tensor memory and exits.
-                mma_commit(drain_bar);
+                mma_commit(drain_bar, elected);
                 uint32_t dummy = 0;
                 mbar_wait_bounded(drain_bar, 0u, &dummy, 1u << 16);
             }
-            if (kDiag && blockIdx.x == 0) {
+            if (kDiag && blockIdx.x == 0 && lane == 0) {
                 a.status[2] = (unsigned)wait_a;
                 a.status[3] = (unsigned)wait_acc;
                 a.status[4] = (unsigned)(clock_now() - t_begin);
@@ -883,8 +847,8 @@ general_tc_kernel(const KernelArgs a)
                                 const unsigned short* sc = src + (size_t)cc * a.HW;
                                 const int left = a.C - c0 - cc;
 #pragma unroll
-                                for (int j = 0; j < 8; ++j)
-                                    if (j < left) v[8 * ch + j] = __ldg(reinterpret_cast<const uint2*>(sc + (size_t)j * a.HW));
+                                for (int j = 0; j < 8; ++j, sc += a.HW)
+                                    if (j < left) v[8 * ch + j] = __ldg(reinterpret_cast<const uint2*>(sc));
                             }
                         }
                         float4* d = dst + (size_t)g * kChunks * a.cstride + 4 * pq;
@@ -925,8 +889,6 @@ general_tc_kernel(const KernelArgs a)
         const bool helper = warp >= 4 + kEpilogueWarps;
         const int share = helper ? 1 + ((warp - 8) >> 2) : 0;
         const size_t plane = (size_t)a.P * a.Q;
-        const int chunks_per_tile = a.n_tile / 16;
-        const int total_chunks = a.mt * chunks_per_tile;
         const int n_local = ((int)blockIdx.x < a.items) ? (a.items - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
         bool alive = true;
         for (int li = helper ? n_local - 1 : 0; li >= 0 && li < n_local; ++li) {
@@ -948,299 +910,253 @@ general_tc_kernel(const KernelArgs a)
             const long long t_busy0 = clock_now();
             if (kDiag && blockIdx.x == 0 && warp == 4 && lane == 0) a.status[10] += (unsigned)(t_busy0 - t_wait0);   // waited for accumulators
             const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * acc_cols);
-            if (a.swap) {
-                // Lanes are filters, columns pixels: this thread holds adjacent pixels of ONE map.  A
-                // warp-private shared-memory tile turns a 32-filter x 32-pixel block around so that each
-                // store instruction again writes 32 adjacent pixels of one map.
-                float* tile = helper ? reinterpret_cast<float*>(a_smem) + (size_t)(warp - 8) * 32 * kXposePitch
-                                     : xpose + (size_t)(warp - 4) * 32 * kXposePitch;
-                // Stacked taps: lanes 0-15 of the quarter hold 16 maps summed over the left-hand taps, lanes 16-31 the
-                // same maps over the right-hand taps, one column to the right: those lanes write their row shifted
-                // by one column (with the first column of the next block), and a map is the sum of two tile rows.
-                constexpr bool stacked = STACK;         // (a template parameter: as a run-time flag it slowed the ordinary epilogue by 15 %)
-                const int rpq = stacked ? 16 : a.n_tile / 4;    // maps per lane quarter: 32 (M = 128) or 16 (M = 64: lanes 0-15; stacked taps)
-                const int blocks = a.tile_px / 32;
-                auto load_block = [&](uint32_t (&v0)[16], uint32_t (&v1)[16], uint32_t (&vx)[1], int b) {
+            // Lanes are filters, columns pixels: this thread holds adjacent pixels of ONE map.  A
+            // warp-private shared-memory tile turns a 32-filter x 32-pixel block around so that each
+            // store instruction again writes 32 adjacent pixels of one map.
+            float* tile = helper ? reinterpret_cast<float*>(a_smem) + (size_t)(warp - 8) * 32 * kXposePitch
+                                 : xpose + (size_t)(warp - 4) * 32 * kXposePitch;
+            // Stacked taps: lanes 0-15 of the quarter hold 16 maps summed over the left-hand taps, lanes 16-31 the
+            // same maps over the right-hand taps, one column to the right: those lanes write their row shifted
+            // by one column (with the first column of the next block), and a map is the sum of two tile rows.
+            constexpr bool stacked = STACK;         // (a template parameter: as a run-time flag it slowed the ordinary epilogue by 15 %)
+            const int rpq = stacked ? 16 : a.n_tile / 4;    // maps per lane quarter: 32 (M = 128) or 16 (M = 64: lanes 0-15; stacked taps)
+            const int blocks = a.tile_px / 32;
+            auto load_block = [&](uint32_t (&v0)[16], uint32_t (&v1)[16], uint32_t (&vx)[1], int b) {
+                tmem_ld16(lane_base + (uint32_t)(b * 32), v0);
+                tmem_ld16(lane_base + (uint32_t)(b * 32 + 16), v1);
+                vx[0] = 0u;
+                if (stacked && b + 1 < blocks) tmem_ld1(lane_base + (uint32_t)(b * 32 + 32), vx);
+            };
+            auto store_block = [&](const uint32_t (&v0)[16], const uint32_t (&v1)[16], const uint32_t (&vx)[1], int b) {
+                __syncwarp();                                   // the previous block has been read out
+                float4* row = reinterpret_cast<float4*>(tile + lane * kXposePitch);
+                if (stacked) {
+                    const bool up = lane >= 16;
+                    auto sel = [&](uint32_t lo, uint32_t hi) { return __uint_as_float(up ? hi : lo); };
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        row[i] = make_float4(sel(v0[4 * i], v0[4 * i + 1]), sel(v0[4 * i + 1], v0[4 * i + 2]),
+                                             sel(v0[4 * i + 2], v0[4 * i + 3]), sel(v0[4 * i + 3], i < 3 ? v0[(4 * i + 4) & 15] : v1[0]));
+                        row[4 + i] = make_float4(sel(v1[4 * i], v1[4 * i + 1]), sel(v1[4 * i + 1], v1[4 * i + 2]),
+                                                 sel(v1[4 * i + 2], v1[4 * i + 3]), sel(v1[4 * i + 3], i < 3 ? v1[(4 * i + 4) & 15] : vx[0]));
+                    }
+                } else if (lane < rpq) {                        // M = 64: only lanes 0-15 of a quarter hold rows
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        row[i] = make_float4(__uint_as_float(v0[4 * i]), __uint_as_float(v0[4 * i + 1]),
+                                             __uint_as_float(v0[4 * i + 2]), __uint_as_float(v0[4 * i + 3]));
+                        row[4 + i] = make_float4(__uint_as_float(v1[4 * i]), __uint_as_float(v1[4 * i + 1]),
+                                                 __uint_as_float(v1[4 * i + 2]), __uint_as_float(v1[4 * i + 3]));
+                    }
+                }
+                __syncwarp();
+                // Each lane stores `vec` adjacent pixels of one map, so one instruction covers `vec` maps:
+                // per-warp store throughput is bounded by instructions in flight, not bytes (measured
+                // ~2.7 B/clk per warp with 4-byte lanes), hence the widest unit the alignment allows.
+                const int vec = a.vec;                          // 1, 2 or 4 (W, Q, P*Q multiples of vec)
+                const int lanes_per_row = 32 >> a.vec_shift;
+                const int row_sub = lane >> (5 - a.vec_shift), pg = lane & (lanes_per_row - 1);
+                int n, p, q;                                    // this lane's first pixel of the block
+                const bool ok = output_pixel<PATCH>(a, ii.geom, b * 32 + pg * vec, n, p, q);
+                float* o = a.y;
+                if (ok) o = a.y + (((size_t)n * a.K + nb * a.n_tile + quarter * rpq + row_sub) * a.P + p) * a.Q + q;
+                if (ok) {
+                    const int kmax = min(rpq, a.K - nb * a.n_tile - quarter * rpq);   // maps of this quarter that exist
+                    const float* src = tile + row_sub * kXposePitch + pg * vec;
+                    if (vec == 4) {
+#pragma unroll 4
+                        for (int r = 0; r < 32; r += 4, o += 4 * plane, src += 4 * kXposePitch)
+                            if (r + row_sub < kmax) {
+                                float4 t = *reinterpret_cast<const float4*>(src);
+                                if (stacked) {
+                                    const float4 u = *reinterpret_cast<const float4*>(src + 16 * kXposePitch);
+                                    t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+                                }
+                                if (add) { atomicAdd(o, t.x); atomicAdd(o + 1, t.y); atomicAdd(o + 2, t.z); atomicAdd(o + 3, t.w); }
+                                else *reinterpret_cast<float4*>(o) = t;
+                            }
+                    } else if (vec == 2) {
+#pragma unroll 8
+                        for (int r = 0; r < 32; r += 2, o += 2 * plane, src += 2 * kXposePitch)
+                            if (r + row_sub < kmax) {
+                                float2 t = *reinterpret_cast<const float2*>(src);
+                                if (stacked) {
+                                    const float2 u = *reinterpret_cast<const float2*>(src + 16 * kXposePitch);
+                                    t.x += u.x; t.y += u.y;
+                                }
+                                if (add) { atomicAdd(o, t.x); atomicAdd(o + 1, t.y); }
+                                else *reinterpret_cast<float2*>(o) = t;
+                            }
+                    } else {
+#pragma unroll 8
+                        for (int r = 0; r < 32; ++r, o += plane, src += kXposePitch)
+                            if (r < kmax) {
+                                const float t = stacked ? src[0] + src[16 * kXposePitch] : src[0];
+                                if (add) atomicAdd(o, t); else *o = t;
+                            }
+                    }
+                }
+            };
+            if (CLUSTER) {
+                const uint32_t rank = cluster_ctarank(), peer = rank ^ 1u;
+                // rows and barriers belong to a (lane quarter, block) pair; with the helper warps a quarter is
+                // drained by three warps, block b going to warp (b / 2) mod 3 of the quarter on both sides
+                float* my_rows = xchg + (size_t)quarter * a.xchg_slots * kXchgBlockFloats;
+                uint64_t* my_bars = xbar + quarter * a.xchg_slots;
+                const int nshare = a.helpers ? 3 : 1;
+                uint32_t v0[16], v1[16], vx[1];
+                vx[0] = 0u;
+                // the blocks the peer stores: this block's partial sums go into the peer's shared memory as
+                // [4-column group][lane][16 bytes], so that one store instruction of the warp writes 512 contiguous
+                // bytes over the cluster network (a row per lane, i.e. 16-byte pieces 144 bytes apart, took 2150 cycles
+                // per 32-pixel block, this layout 1290)
+                const long long t_x0 = clock_now();
+                long long t_xwait = 0;
+                for (int b = (int)peer; b < blocks; b += 2) {
+                    if ((b >> 1) % nshare != share) continue;
                     tmem_ld16(lane_base + (uint32_t)(b * 32), v0);
                     tmem_ld16(lane_base + (uint32_t)(b * 32 + 16), v1);
-                    vx[0] = 0u;
-                    if (stacked && b + 1 < blocks) tmem_ld1(lane_base + (uint32_t)(b * 32 + 32), vx);
-                };
-                auto store_block = [&](const uint32_t (&v0)[16], const uint32_t (&v1)[16], const uint32_t (&vx)[1], int b) {
-                    __syncwarp();                                   // the previous block has been read out
-                    float4* row = reinterpret_cast<float4*>(tile + lane * kXposePitch);
-                    if (stacked) {
-                        const bool up = lane >= 16;
-                        auto sel = [&](uint32_t lo, uint32_t hi) { return __uint_as_float(up ? hi : lo); };
+                    tmem_ld_wait();
+                    const int slot = b >> 1;
+                    const uint32_t dst = map_to_cta(smem_u32(my_rows + (size_t)slot * kXchgBlockFloats + lane * 4), peer);
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            row[i] = make_float4(sel(v0[4 * i], v0[4 * i + 1]), sel(v0[4 * i + 1], v0[4 * i + 2]),
-                                                 sel(v0[4 * i + 2], v0[4 * i + 3]), sel(v0[4 * i + 3], i < 3 ? v0[(4 * i + 4) & 15] : v1[0]));
-                            row[4 + i] = make_float4(sel(v1[4 * i], v1[4 * i + 1]), sel(v1[4 * i + 1], v1[4 * i + 2]),
-                                                     sel(v1[4 * i + 2], v1[4 * i + 3]), sel(v1[4 * i + 3], i < 3 ? v1[(4 * i + 4) & 15] : vx[0]));
-                        }
-                    } else if (lane < rpq) {                        // M = 64: only lanes 0-15 of a quarter hold rows
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            row[i] = make_float4(__uint_as_float(v0[4 * i]), __uint_as_float(v0[4 * i + 1]),
-                                                 __uint_as_float(v0[4 * i + 2]), __uint_as_float(v0[4 * i + 3]));
-                            row[4 + i] = make_float4(__uint_as_float(v1[4 * i]), __uint_as_float(v1[4 * i + 1]),
-                                                     __uint_as_float(v1[4 * i + 2]), __uint_as_float(v1[4 * i + 3]));
-                        }
+                    for (int i = 0; i < 4; ++i) {
+                        st_cluster_v4(dst + 512u * i, __uint_as_float(v0[4 * i]), __uint_as_float(v0[4 * i + 1]),
+                                      __uint_as_float(v0[4 * i + 2]), __uint_as_float(v0[4 * i + 3]));
+                        st_cluster_v4(dst + 2048u + 512u * i, __uint_as_float(v1[4 * i]), __uint_as_float(v1[4 * i + 1]),
+                                      __uint_as_float(v1[4 * i + 2]), __uint_as_float(v1[4 * i + 3]));
                     }
-                    __syncwarp();
-                    // Each lane stores `vec` adjacent pixels of one map, so one instruction covers `vec` maps:
-                    // per-warp store throughput is bounded by instructions in flight, not bytes (measured
-                    // ~2.7 B/clk per warp with 4-byte lanes), hence the widest unit the alignment allows.
-                    const int vec = a.vec;                          // 1, 2 or 4 (W, Q, P*Q multiples of vec)
-                    const int lanes_per_row = 32 >> a.vec_shift;
-                    const int row_sub = lane >> (5 - a.vec_shift), pg = lane & (lanes_per_row - 1);
-                    int n, p, q;                                    // this lane's first pixel of the block
-                    const bool ok = output_pixel<PATCH>(a, ii.geom, b * 32 + pg * vec, n, p, q);
-                    float* o = a.y;
-                    if (ok) o = a.y + (((size_t)n * a.K + nb * a.n_tile + quarter * rpq + row_sub) * a.P + p) * a.Q + q;
-                    if (ok) {
-                        const int kmax = min(rpq, a.K - nb * a.n_tile - quarter * rpq);   // maps of this quarter that exist
-                        const float* src = tile + row_sub * kXposePitch + pg * vec;
-                        if (vec == 4) {
-#pragma unroll 4
-                            for (int r = 0; r < 32; r += 4, o += 4 * plane, src += 4 * kXposePitch)
-                                if (r + row_sub < kmax) {
-                                    float4 t = *reinterpret_cast<const float4*>(src);
-                                    if (stacked) {
-                                        const float4 u = *reinterpret_cast<const float4*>(src + 16 * kXposePitch);
-                                        t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
-                                    }
-                                    if (add) { atomicAdd(o, t.x); atomicAdd(o + 1, t.y); atomicAdd(o + 2, t.z); atomicAdd(o + 3, t.w); }
-                                    else *reinterpret_cast<float4*>(o) = t;
-                                }
-                        } else if (vec == 2) {
-#pragma unroll 8
-                            for (int r = 0; r < 32; r += 2, o += 2 * plane, src += 2 * kXposePitch)
-                                if (r + row_sub < kmax) {
-                                    float2 t = *reinterpret_cast<const float2*>(src);
-                                    if (stacked) {
-                                        const float2 u = *reinterpret_cast<const float2*>(src + 16 * kXposePitch);
-                                        t.x += u.x; t.y += u.y;
-                                    }
-                                    if (add) { atomicAdd(o, t.x); atomicAdd(o + 1, t.y); }
-                                    else *reinterpret_cast<float2*>(o) = t;
-                                }
-                        } else {
-#pragma unroll 8
-                            for (int r = 0; r < 32; ++r, o += plane, src += kXposePitch)
-                                if (r < kmax) {
-                                    const float t = stacked ? src[0] + src[16 * kXposePitch] : src[0];
-                                    if (add) atomicAdd(o, t); else *o = t;
-                                }
-                        }
-                    }
-                };
-                if (CLUSTER) {
-                    const uint32_t rank = cluster_ctarank(), peer = rank ^ 1u;
-                    // rows and barriers belong to a (lane quarter, block) pair; with the helper warps a quarter is
-                    // drained by three warps, block b going to warp (b / 2) mod 3 of the quarter on both sides
-                    float* my_rows = xchg + (size_t)quarter * a.xchg_slots * kXchgBlockFloats;
-                    uint64_t* my_bars = xbar + quarter * a.xchg_slots;
-                    const int nshare = a.helpers ? 3 : 1;
-                    uint32_t v0[16], v1[16], vx[1];
-                    vx[0] = 0u;
-                    // the blocks the peer stores: this block's partial sums go into the peer's shared memory as
-                    // [4-column group][lane][16 bytes], so that one store instruction of the warp writes 512 contiguous
-                    // bytes over the cluster network (a row per lane, i.e. 16-byte pieces 144 bytes apart, took 2150 cycles
-                    // per 32-pixel block, this layout 1290)
-                    const long long t_x0 = clock_now();
-                    long long t_xwait = 0;
-                    for (int b = (int)peer; b < blocks; b += 2) {
-                        if ((b >> 1) % nshare != share) continue;
-                        tmem_ld16(lane_base + (uint32_t)(b * 32), v0);
-                        tmem_ld16(lane_base + (uint32_t)(b * 32 + 16), v1);
-                        tmem_ld_wait();
-                        const int slot = b >> 1;
-                        const uint32_t dst = map_to_cta(smem_u32(my_rows + (size_t)slot * kXchgBlockFloats + lane * 4), peer);
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            st_cluster_v4(dst + 512u * i, __uint_as_float(v0[4 * i]), __uint_as_float(v0[4 * i + 1]),
-                                          __uint_as_float(v0[4 * i + 2]), __uint_as_float(v0[4 * i + 3]));
-                            st_cluster_v4(dst + 2048u + 512u * i, __uint_as_float(v1[4 * i]), __uint_as_float(v1[4 * i + 1]),
-                                          __uint_as_float(v1[4 * i + 2]), __uint_as_float(v1[4 * i + 3]));
-                        }
-                    }
-                    // The arrivals come after the stores of all blocks (measured: the same time as arriving block by
-                    // block, ~1290 cycles per block either way: the remote stores themselves, ~150 cycles per 512-byte
-                    // instruction, are the cost; one arrival per warp behind a cluster-scope fence measured slower).
-                    for (int b = (int)peer; b < blocks; b += 2) {
-                        if ((b >> 1) % nshare != share) continue;
-                        mbar_arrive_remote(map_to_cta(smem_u32(&my_bars[b >> 1]), peer));
-                    }
-                    const long long t_x1 = clock_now();
-                    // this block's own blocks: accumulators + the peer's partial sums, then the ordinary write-back
-                    for (int b = (int)rank; b < blocks; b += 2) {
-                        if ((b >> 1) % nshare != share) continue;
-                        tmem_ld16(lane_base + (uint32_t)(b * 32), v0);
-                        tmem_ld16(lane_base + (uint32_t)(b * 32 + 16), v1);
-                        tmem_ld_wait();
-                        const int slot = b >> 1;
-                        const long long t_w0 = clock_now();
-                        alive = __all_sync(0xffffffffu, mbar_wait_bounded_cluster(&my_bars[slot], 0u, abort_flag, a.max_polls));
-                        t_xwait += clock_now() - t_w0;
-                        if (!alive) break;
-                        const float4* row = reinterpret_cast<const float4*>(my_rows + (size_t)slot * kXchgBlockFloats) + lane;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            const float4 t = row[32 * i], u = row[128 + 32 * i];
-                            v0[4 * i] = __float_as_uint(__uint_as_float(v0[4 * i]) + t.x);
-                            v0[4 * i + 1] = __float_as_uint(__uint_as_float(v0[4 * i + 1]) + t.y);
-                            v0[4 * i + 2] = __float_as_uint(__uint_as_float(v0[4 * i + 2]) + t.z);
-                            v0[4 * i + 3] = __float_as_uint(__uint_as_float(v0[4 * i + 3]) + t.w);
-                            v1[4 * i] = __float_as_uint(__uint_as_float(v1[4 * i]) + u.x);
-                            v1[4 * i + 1] = __float_as_uint(__uint_as_float(v1[4 * i + 1]) + u.y);
-                            v1[4 * i + 2] = __float_as_uint(__uint_as_float(v1[4 * i + 2]) + u.z);
-                            v1[4 * i + 3] = __float_as_uint(__uint_as_float(v1[4 * i + 3]) + u.w);
-                        }
-                        store_block(v0, v1, vx, b);
-                    }
+                }
+                // The arrivals come after the stores of all blocks (measured: the same time as arriving block by
+                // block, ~1290 cycles per block either way: the remote stores themselves, ~150 cycles per 512-byte
+                // instruction, are the cost; one arrival per warp behind a cluster-scope fence measured slower).
+                for (int b = (int)peer; b < blocks; b += 2) {
+                    if ((b >> 1) % nshare != share) continue;
+                    mbar_arrive_remote(map_to_cta(smem_u32(&my_bars[b >> 1]), peer));
+                }
+                const long long t_x1 = clock_now();
+                // this block's own blocks: accumulators + the peer's partial sums, then the ordinary write-back
+                for (int b = (int)rank; b < blocks; b += 2) {
+                    if ((b >> 1) % nshare != share) continue;
+                    tmem_ld16(lane_base + (uint32_t)(b * 32), v0);
+                    tmem_ld16(lane_base + (uint32_t)(b * 32 + 16), v1);
+                    tmem_ld_wait();
+                    const int slot = b >> 1;
+                    const long long t_w0 = clock_now();
+                    alive = __all_sync(0xffffffffu, mbar_wait_bounded_cluster(&my_bars[slot], 0u, abort_flag, a.max_polls));
+                    t_xwait += clock_now() - t_w0;
                     if (!alive) break;
-                    if (kDiag && blockIdx.x == 0 && warp == 4 && lane == 0) {     // cycles: sending, waiting for the peer, whole exchange
-                        a.status[13] = (unsigned)(t_x1 - t_x0);
-                        a.status[14] = (unsigned)t_xwait;
-                        a.status[15] = (unsigned)(clock_now() - t_x0);
+                    const float4* row = reinterpret_cast<const float4*>(my_rows + (size_t)slot * kXchgBlockFloats) + lane;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float4 t = row[32 * i], u = row[128 + 32 * i];
+                        v0[4 * i] = __float_as_uint(__uint_as_float(v0[4 * i]) + t.x);
+                        v0[4 * i + 1] = __float_as_uint(__uint_as_float(v0[4 * i + 1]) + t.y);
+                        v0[4 * i + 2] = __float_as_uint(__uint_as_float(v0[4 * i + 2]) + t.z);
+                        v0[4 * i + 3] = __float_as_uint(__uint_as_float(v0[4 * i + 3]) + t.w);
+                        v1[4 * i] = __float_as_uint(__uint_as_float(v1[4 * i]) + u.x);
+                        v1[4 * i + 1] = __float_as_uint(__uint_as_float(v1[4 * i + 1]) + u.y);
+                        v1[4 * i + 2] = __float_as_uint(__uint_as_float(v1[4 * i + 2]) + u.z);
+                        v1[4 * i + 3] = __float_as_uint(__uint_as_float(v1[4 * i + 3]) + u.w);
                     }
-                    tc_fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0 && !helper) mbar_arrive(&acc_empty[buf]);
-                    continue;
+                    store_block(v0, v1, vx, b);
                 }
-                uint32_t va0[16], va1[16], vb0[16], vb1[16], vax[1], vbx[1];
-                if (M64 && a.vec >= 2 && !add) {
-                    // At most 64 filters (a quarter holds 16 maps): two 32-pixel blocks share the tile and one pass over it,
-                    // each half of the warp stores one of them.  A block at a time the warps, not the MMAs or the memory,
-                    // set the pace of short contractions (900 cycles per block, most of them the latency of the steps).
-                    const int half = lane >> 4, lanes_per_row = 32 >> a.vec_shift;
-                    const int row_sub = (lane & 15) >> (5 - a.vec_shift), pg = lane & (lanes_per_row - 1);
-                    const int pairs = (blocks + 1) / 2, p_step = split ? 3 : 1;
-                    const int kmax = min(16, a.K - nb * a.n_tile - quarter * 16);      // maps of this quarter that exist
-                    auto load_pair = [&](int bp) {
-                        tmem_ld16(lane_base + (uint32_t)(bp * 64), va0);
-                        tmem_ld16(lane_base + (uint32_t)(bp * 64 + 16), va1);
-                        if (2 * bp + 1 < blocks) {
-                            tmem_ld16(lane_base + (uint32_t)(bp * 64 + 32), vb0);
-                            tmem_ld16(lane_base + (uint32_t)(bp * 64 + 48), vb1);
-                        }
-                    };
-                    int bp = split ? share : 0;
-                    if (bp < pairs) load_pair(bp);
-                    while (bp < pairs) {
-                        tmem_ld_wait();
-                        __syncwarp();                               // the previous pair has been read out
-                        if (lane < 16) {
-                            float4* ra = reinterpret_cast<float4*>(tile + lane * kXposePitch);
-                            float4* rb = reinterpret_cast<float4*>(tile + (lane + 16) * kXposePitch);
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                ra[i] = make_float4(__uint_as_float(va0[4 * i]), __uint_as_float(va0[4 * i + 1]), __uint_as_float(va0[4 * i + 2]), __uint_as_float(va0[4 * i + 3]));
-                                ra[4 + i] = make_float4(__uint_as_float(va1[4 * i]), __uint_as_float(va1[4 * i + 1]), __uint_as_float(va1[4 * i + 2]), __uint_as_float(va1[4 * i + 3]));
-                            }
-                            if (2 * bp + 1 < blocks) {
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) {
-                                    rb[i] = make_float4(__uint_as_float(vb0[4 * i]), __uint_as_float(vb0[4 * i + 1]), __uint_as_float(vb0[4 * i + 2]), __uint_as_float(vb0[4 * i + 3]));
-                                    rb[4 + i] = make_float4(__uint_as_float(vb1[4 * i]), __uint_as_float(vb1[4 * i + 1]), __uint_as_float(vb1[4 * i + 2]), __uint_as_float(vb1[4 * i + 3]));
-                                }
-                            }
-                        }
-                        __syncwarp();
-                        const int b = 2 * bp + half;
-                        bp += p_step;
-                        if (bp < pairs) load_pair(bp);
-                        int n, p, q;                                // this lane's first pixel of its block
-                        if (b < blocks && output_pixel<PATCH>(a, ii.geom, b * 32 + pg * a.vec, n, p, q)) {
-                            float* o = a.y + (((size_t)n * a.K + nb * a.n_tile + quarter * 16 + row_sub) * a.P + p) * a.Q + q;
-                            const float* src = tile + (16 * half + row_sub) * kXposePitch + pg * a.vec;
-                            if (a.vec == 4) {
-#pragma unroll
-                                for (int r = 0; r < 16; r += 2, o += 2 * plane, src += 2 * kXposePitch)
-                                    if (r + row_sub < kmax) *reinterpret_cast<float4*>(o) = *reinterpret_cast<const float4*>(src);
-                            } else {
-#pragma unroll
-                                for (int r = 0; r < 16; ++r, o += plane, src += kXposePitch)
-                                    if (r < kmax) *reinterpret_cast<float2*>(o) = *reinterpret_cast<const float2*>(src);
-                            }
-                        }
-                    }
-                    tc_fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0 && !helper) mbar_arrive(&acc_empty[buf]);
-                    continue;
+                if (!alive) break;
+                if (kDiag && blockIdx.x == 0 && warp == 4 && lane == 0) {     // cycles: sending, waiting for the peer, whole exchange
+                    a.status[13] = (unsigned)(t_x1 - t_x0);
+                    a.status[14] = (unsigned)t_xwait;
+                    a.status[15] = (unsigned)(clock_now() - t_x0);
                 }
-                const int b_step = split ? 3 : 1;
-                int b = split ? share : 0;
-                if (b < blocks) load_block(va0, va1, vax, b);
-                long long t_ld = 0;       // (diagnostics build: cycles spent waiting for tensor-memory loads)
-                while (b < blocks) {
-                    long long t0 = clock_now();
-                    tmem_ld_wait();
-                    t_ld += clock_now() - t0;
-                    if (b + b_step < blocks) load_block(vb0, vb1, vbx, b + b_step);
-                    store_block(va0, va1, vax, b);
-                    if ((b += b_step) >= blocks) break;
-                    t0 = clock_now();
-                    tmem_ld_wait();
-                    t_ld += clock_now() - t0;
-                    if (b + b_step < blocks) load_block(va0, va1, vax, b + b_step);
-                    store_block(vb0, vb1, vbx, b);
-                    b += b_step;
-                }
-                if (kDiag && blockIdx.x == 0 && warp == 4 && lane == 0) a.status[12] += (unsigned)t_ld;
                 tc_fence_before_sync();
                 __syncwarp();
                 if (lane == 0 && !helper) mbar_arrive(&acc_empty[buf]);
-                if (kDiag && blockIdx.x == 0 && warp == 4 && lane == 0) a.status[11] += (unsigned)(clock_now() - t_busy0);   // drained one item
                 continue;
             }
-            int cur_m = -1;
-            bool ok = false;
-            float* yb = a.y;
-            // Issues the tensor-memory load of 16-column chunk c (chunks are numbered tile-major).
-            auto load_chunk = [&](uint32_t (&v)[16], int c) {
-                const int m = c / chunks_per_tile, ch = c - m * chunks_per_tile;
-                tmem_ld16(lane_base + (uint32_t)(m * a.n_tile + ch * 16), v);
-            };
-            // Stores chunk c: this lane's pixel of 16 adjacent maps (the warp writes 32 adjacent pixels per map).
-            auto store_chunk = [&](const uint32_t (&v)[16], int c) {
-                const int m = c / chunks_per_tile, ch = c - m * chunks_per_tile;
-                if (m != cur_m) {
-                    cur_m = m;
-                    int n, p, q;
-                    ok = output_pixel<PATCH>(a, ii.geom, m * kTileM + quarter * 32 + lane, n, p, q);
-                    if (ok) yb = a.y + ((size_t)n * a.K * a.P + p) * a.Q + q;
-                }
-                const int k0 = nb * a.n_tile + ch * 16;
-                if (ok) {
-                    float* o = yb + (size_t)k0 * plane;
+            uint32_t va0[16], va1[16], vb0[16], vb1[16], vax[1], vbx[1];
+            if (M64 && a.vec >= 2 && !add) {
+                // At most 64 filters (a quarter holds 16 maps): two 32-pixel blocks share the tile and one pass over it,
+                // each half of the warp stores one of them.  A block at a time the warps, not the MMAs or the memory,
+                // set the pace of short contractions (900 cycles per block, most of them the latency of the steps).
+                const int half = lane >> 4, lanes_per_row = 32 >> a.vec_shift;
+                const int row_sub = (lane & 15) >> (5 - a.vec_shift), pg = lane & (lanes_per_row - 1);
+                const int pairs = (blocks + 1) / 2, p_step = split ? 3 : 1;
+                const int kmax = min(16, a.K - nb * a.n_tile - quarter * 16);      // maps of this quarter that exist
+                auto load_pair = [&](int bp) {
+                    tmem_ld16(lane_base + (uint32_t)(bp * 64), va0);
+                    tmem_ld16(lane_base + (uint32_t)(bp * 64 + 16), va1);
+                    if (2 * bp + 1 < blocks) {
+                        tmem_ld16(lane_base + (uint32_t)(bp * 64 + 32), vb0);
+                        tmem_ld16(lane_base + (uint32_t)(bp * 64 + 48), vb1);
+                    }
+                };
+                int bp = split ? share : 0;
+                if (bp < pairs) load_pair(bp);
+                while (bp < pairs) {
+                    tmem_ld_wait();
+                    __syncwarp();                               // the previous pair has been read out
+                    if (lane < 16) {
+                        float4* ra = reinterpret_cast<float4*>(tile + lane * kXposePitch);
+                        float4* rb = reinterpret_cast<float4*>(tile + (lane + 16) * kXposePitch);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i, o += plane)
-                        if (k0 + i < a.K) { if (add) atomicAdd(o, __uint_as_float(v[i])); else *o = __uint_as_float(v[i]); }
+                        for (int i = 0; i < 4; ++i) {
+                            ra[i] = make_float4(__uint_as_float(va0[4 * i]), __uint_as_float(va0[4 * i + 1]), __uint_as_float(va0[4 * i + 2]), __uint_as_float(va0[4 * i + 3]));
+                            ra[4 + i] = make_float4(__uint_as_float(va1[4 * i]), __uint_as_float(va1[4 * i + 1]), __uint_as_float(va1[4 * i + 2]), __uint_as_float(va1[4 * i + 3]));
+                        }
+                        if (2 * bp + 1 < blocks) {
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                rb[i] = make_float4(__uint_as_float(vb0[4 * i]), __uint_as_float(vb0[4 * i + 1]), __uint_as_float(vb0[4 * i + 2]), __uint_as_float(vb0[4 * i + 3]));
+                                rb[4 + i] = make_float4(__uint_as_float(vb1[4 * i]), __uint_as_float(vb1[4 * i + 1]), __uint_as_float(vb1[4 * i + 2]), __uint_as_float(vb1[4 * i + 3]));
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    const int b = 2 * bp + half;
+                    bp += p_step;
+                    if (bp < pairs) load_pair(bp);
+                    int n, p, q;                                // this lane's first pixel of its block
+                    if (b < blocks && output_pixel<PATCH>(a, ii.geom, b * 32 + pg * a.vec, n, p, q)) {
+                        float* o = a.y + (((size_t)n * a.K + nb * a.n_tile + quarter * 16 + row_sub) * a.P + p) * a.Q + q;
+                        const float* src = tile + (16 * half + row_sub) * kXposePitch + pg * a.vec;
+                        if (a.vec == 4) {
+#pragma unroll
+                            for (int r = 0; r < 16; r += 2, o += 2 * plane, src += 2 * kXposePitch)
+                                if (r + row_sub < kmax) *reinterpret_cast<float4*>(o) = *reinterpret_cast<const float4*>(src);
+                        } else {
+#pragma unroll
+                            for (int r = 0; r < 16; ++r, o += plane, src += kXposePitch)
+                                if (r < kmax) *reinterpret_cast<float2*>(o) = *reinterpret_cast<const float2*>(src);
+                        }
+                    }
                 }
-            };
-            // Two register buffers: the load of the next chunk is in flight while the current one is stored.
-            uint32_t va[16], vb[16];
-            int c = 0;
-            load_chunk(va, c);
-            while (c < total_chunks) {
-                tmem_ld_wait();
-                if (c + 1 < total_chunks) load_chunk(vb, c + 1);
-                store_chunk(va, c);
-                if (++c >= total_chunks) break;
-                tmem_ld_wait();
-                if (c + 1 < total_chunks) load_chunk(va, c + 1);
-                store_chunk(vb, c);
-                ++c;
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0 && !helper) mbar_arrive(&acc_empty[buf]);
+                continue;
             }
-            // all of this warp's reads of the accumulator set are complete: hand it back to the MMA thread
+            const int b_step = split ? 3 : 1;
+            int b = split ? share : 0;
+            if (b < blocks) load_block(va0, va1, vax, b);
+            long long t_ld = 0;       // (diagnostics build: cycles spent waiting for tensor-memory loads)
+            while (b < blocks) {
+                long long t0 = clock_now();
+                tmem_ld_wait();
+                t_ld += clock_now() - t0;
+                if (b + b_step < blocks) load_block(vb0, vb1, vbx, b + b_step);
+                store_block(va0, va1, vax, b);
+                if ((b += b_step) >= blocks) break;
+                t0 = clock_now();
+                tmem_ld_wait();
+                t_ld += clock_now() - t0;
+                if (b + b_step < blocks) load_block(va0, va1, vax, b + b_step);
+                store_block(vb0, vb1, vbx, b);
+                b += b_step;
+            }
+            if (kDiag && blockIdx.x == 0 && warp == 4 && lane == 0) a.status[12] += (unsigned)t_ld;
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[buf]);
+            if (lane == 0 && !helper) mbar_arrive(&acc_empty[buf]);
+            if (kDiag && blockIdx.x == 0 && warp == 4 && lane == 0) a.status[11] += (unsigned)(clock_now() - t_busy0);   // drained one item
         }
     }
     }

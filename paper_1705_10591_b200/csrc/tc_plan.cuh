@@ -8,7 +8,6 @@
 namespace conv2d_b200 {
 namespace {
 
-constexpr int kTileM = 128;                 // pixels per accumulator tile (UMMA M)
 constexpr int kCB = 16;                     // channels per staged block (two UMMA K steps of 8)
 constexpr int kChunks = kCB / 4;            // 16-byte channel chunks per block
 constexpr int kProducerWarps = 8;
@@ -47,11 +46,10 @@ constexpr int kXchgBlockFloats = 32 * 32;   // exchange area of a two-block clus
 constexpr size_t xchg_area_bytes(int slots) { return (size_t)kEpilogueWarps * slots * (kXchgBlockFloats * 4 + 8); }
 
 struct Plan {
-    int n_tile;       // filters per work item: 64 or 128 rows of the M operand (with the pixels as M: UMMA N, a multiple of 16)
+    int n_tile;       // filters per work item: 64 or 128 rows of the M operand
     int n_blocks;     // work-item columns over the filters
-    int mt;           // accumulator tiles per work item (pixels-as-M layout; informative otherwise)
-    int tile_px;      // pixels per work item: mt * 128, or any multiple of 32 up to 512 in the operand-swap layout
-    int px_groups;    // operand-swap layout: MMAs per K step (each covers n_mma = tile_px / px_groups pixels)
+    int tile_px;      // pixels per work item: any multiple of 32 up to 512
+    int px_groups;    // MMAs per K step (each covers n_mma = tile_px / px_groups pixels)
     int nbuf;         // accumulator sets in tensor memory (2: write-back overlaps the next item)
     int npix;         // staged pixel rows per channel chunk
     int cblks;        // channel blocks (of the folded channels, see fold_r/fold_s)
@@ -63,7 +61,6 @@ struct Plan {
     int tps;          // taps per filter stage
     int cbg;          // channel blocks per activation stage
     int resident;     // 1: the whole filter block stays in shared memory for the life of the thread block
-    int swap;         // 1: filters are the MMA's M operand, 256 pixels its N operand (K <= 128)
     int pair_taps;    // 1: at most 64 filters, horizontally adjacent taps stacked in one M = 128 operand (see make_plan)
     int pair_compact; // 1 (with pair_taps): a lone last tap of a filter row is a 64-row slice issued as M = 64 (resident bank only)
     size_t cb_bytes;  // bytes of one channel block of the re-ordered bank (all taps of one filter block)
@@ -148,8 +145,6 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     const long long total_pix = (long long)sh.N * sh.H * sh.W;
     if (total_pix >= (1LL << 31) - (1LL << 20)) return p;     // flat pixel indices stay within int32
     const int kp16 = (sh.K + 15) / 16 * 16;
-    p.n_blocks = (kp16 + 255) / 256;
-    p.n_tile = ((sh.K + p.n_blocks - 1) / p.n_blocks + 15) / 16 * 16;
     // Operand roles.  One tcgen05.mma costs its issuing thread ~60 cycles whatever its size (measured), so
     // an instruction must carry >= 128 cycles of tensor-pipe work to keep the pipe busy: N = 256.  For any
     // filter count that is possible with the pixels as the N operand: M = a block of 128 filters (zero
@@ -157,13 +152,8 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     // per pixel compared with 128 pixels x 256 filters.
     // Up to 64 filters use M = 64 (one tcgen05.mma then covers 64 filters x 256 pixels; its accumulator
     // occupies lanes 0-15 of each 32-lane quarter -- established with a probe).
-    p.swap = env_int("CONV2D_B200_TF32_SWAP", 1) != 0 ? 1 : 0;
-    if (p.swap && kp16 <= 64 && env_int("CONV2D_B200_TF32_M64", 1) == 0) p.swap = 0;
-    if (p.swap) {
-        p.n_tile = kp16 <= 64 ? 64 : 128;                  // filters per block = rows of the M operand
-        p.n_blocks = (kp16 + p.n_tile - 1) / p.n_tile;
-    }
-    const int set_cols = p.swap ? kTileM : p.n_tile;      // tensor-memory columns of one 128-pixel tile
+    p.n_tile = kp16 <= 64 ? 64 : 128;                      // filters per block = rows of the M operand
+    p.n_blocks = (kp16 + p.n_tile - 1) / p.n_tile;
     const int cbc = b16 ? 2 * kCB : kCB;                 // channels per staged block
     // Few input channels (first layers, the bridge between the one-channel and the many-channel case) would
     // leave most of a staged channel block as zero padding.  Then taps are folded into the channel dimension:
@@ -174,8 +164,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     // 3 channels 7 x 7 on 224 x 224: 0.91 ms folded, 1.06 ms not; 1 channel 5 x 5: 0.32 vs 0.40 ms; but
     // 8 channels 3 x 3 on 112 x 112: 0.175 vs 0.093 ms).  CONV2D_B200_TF32_FOLD = 2 folds whenever C < 16.
     p.fold_r = p.fold_s = 1;
-    const bool padded = sh.pad_h != 0 || sh.pad_w != 0;      // needs patch addressing: no folding, filters as M
-    if (padded && !p.swap) return p;
+    const bool padded = sh.pad_h != 0 || sh.pad_w != 0;      // needs patch addressing: no folding
     const int fold_mode = padded || virt ? 0 : env_int("CONV2D_B200_TF32_FOLD", 1);
     if (sh.C < cbc && (fold_mode == 2 || (fold_mode == 1 && sh.C <= 3))) {
         long long best = (long long)sh.R * sh.S * ((sh.C + cbc - 1) / cbc);
@@ -225,7 +214,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     // 24.3 -> 20.8 us; 64 channels 3 x 3 on 56 x 56 (36 pairs): 27.6 -> 30.6 us.  Hence from 48 (tap, channel block)
     // pairs on.  CONV2D_B200_TF32_PAIR_TAPS = 0 / 2: never / whenever possible.
     const int pair_mode = env_int("CONV2D_B200_TF32_PAIR_TAPS", 1);
-    p.pair_taps = (p.swap && st == 1 && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
+    p.pair_taps = (st == 1 && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
                    (pair_mode == 2 || (long long)r_eff * s_eff * p.cblks >= 48)) ? 1 : 0;
     // Compact stacking for banks that can stay in shared memory: pairs of taps as 128-row slices, the lone last tap of
     // an odd filter row as a 64-row slice that an M = 64 instruction adds onto the same accumulator lanes.  The bank
@@ -237,7 +226,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     // (CONV2D_B200_TF32_PAIR_COMPACT = 1 turns it on) until the write-back is faster than the MMAs.
     p.pair_compact = 0;
     const size_t compact_cb_bytes = (size_t)r_eff * ((s_eff / 2) * 128 + (s_eff & 1) * 64) * kCB * 4;
-    if (allow_compact && !p.pair_taps && p.swap && st == 1 && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
+    if (allow_compact && !p.pair_taps && st == 1 && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
         !padded && (size_t)((c_eff + cbc - 1) / cbc) * compact_cb_bytes <= 152 * 1024 && env_int("CONV2D_B200_TF32_PAIR_COMPACT", 0) != 0) {
         p.pair_taps = 1;
         p.pair_compact = 1;
@@ -246,7 +235,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     p.s_slots = p.pair_taps ? (s_eff + 1) / 2 : s_eff;
     p.taps = stage_blocks == 2 ? r_eff * sh.S : r_eff * p.s_slots;          // (with phases: of the phase that has most)
     if (p.taps > kMaxTaps) return p;
-    const size_t extra = p.swap ? kXposeBytes : 0;       // epilogue transposition tile
+    const size_t extra = kXposeBytes;                     // epilogue transposition tile
     // Addressing mode.  In the flat pixel run the staged halo is (R-1) whole image rows; once that exceeds a
     // 256-pixel item the item is cut as a rectangle of the image instead (patch_w columns wide, of which the
     // first patch_tw produce outputs), whose halo is (R-1) patch rows.  The patch width with the least staged
@@ -254,7 +243,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     p.patch_w = p.patch_tw = p.patch_rows = p.patch_cols = 0;
     const long long flat_halo = (long long)(r_eff - 1) * sh.W + (s_eff - 1) + p.shift0;
     const int patch_mode = virt ? 0 : padded ? 2 : env_int("CONV2D_B200_TF32_PATCH", 1);       // 0 never, 1 when the flat halo is large, 2 always
-    if (p.swap && p.fold_r * p.fold_s == 1 && patch_mode != 0) {
+    if (p.fold_r * p.fold_s == 1 && patch_mode != 0) {
         double best_ratio = 0;
         const int forced_wp = want_patch_w ? want_patch_w : env_int("CONV2D_B200_TF32_PATCH_W", 0);
         for (int wp = 32; wp <= 128; wp *= 2) {
@@ -285,11 +274,9 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         const int th = px / p.patch_w;
         return (long long)sh.N * ((sh.P + th - 1) / th) * p.patch_cols;
     };
-    const long long tiles = (total_pix + kTileM - 1) / kTileM;
     const int chunk = kCB * p.n_tile * 4;
     const int sms = sm_count();
 
-    const int forced_mt = env_int("CONV2D_B200_TF32_MT", 0);      // benchmark ablations only
     p.cb_bytes = p.pair_compact ? compact_cb_bytes : (p.phases > 1 ? (size_t)sh.R * sh.S : (size_t)p.taps) * chunk;
     p.pairs = p.phases > 1 ? (long long)(p.cblks / p.phases) * sh.R * sh.S : (long long)p.taps * p.cblks;
     const size_t wbytes = (size_t)(p.cblks / p.phases) * p.cb_bytes;   // re-ordered filters of one filter block
@@ -306,9 +293,8 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     const int resident_mode = env_int("CONV2D_B200_TF32_RESIDENT", 2);      // 0 never, 1 light problems only, 2 whenever it fits
     if (resident_mode != 0 && p.n_blocks == 1 && wbytes <= 152 * 1024 &&
         (p.pairs <= 16 || resident_mode == 2)) {
-        const int mt = forced_mt ? forced_mt : (p.swap ? 2 : 1);
-        int res_px = mt * kTileM;
-        if (p.swap && !p.patch_w && !forced_mt) {
+        int res_px = 256;
+        if (!p.patch_w) {
             // When all pixels fit in one round of items of at most 512 pixels, one item per block is the better
             // cut (64 x 32 x 32 pixels with 1 x 1 filters: 448 pixels per item 19.9 us, 256 per item 22.1 us).
             // (compact stacking issues one MMA per K step: at most 256 pixels per item)
@@ -317,12 +303,11 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         }
         {
             const int want = env_int("CONV2D_B200_TF32_TILE_PX", 0);
-            if (p.swap && want >= 64 && want <= (p.pair_compact ? 256 : 512) && want % 32 == 0 && pixel_items(want) > 0) res_px = want;
+            if (want >= 64 && want <= (p.pair_compact ? 256 : 512) && want % 32 == 0 && pixel_items(want) > 0) res_px = want;
         }
         const int npix = npix_of(res_px);
-        if ((p.swap ? res_px : mt * set_cols) <= 512 && npix <= 16000 && wbytes + extra + (size_t)2 * stage_blocks * kCB * chunk_stride(npix) * 4 + kBookBytes <= kSmemLimit) {
+        if (res_px <= 512 && npix <= 16000 && wbytes + extra + (size_t)2 * stage_blocks * kCB * chunk_stride(npix) * 4 + kBookBytes <= kSmemLimit) {
             p.resident = 1;
-            p.mt = p.swap ? (res_px + kTileM - 1) / kTileM : mt;
             p.tile_px = res_px;
             p.npix = npix;
             p.cbg = 1;
@@ -350,54 +335,36 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         const bool ksplit_allowed = env_int("CONV2D_B200_TF32_KSPLIT", 1) != 0;
         int best_px = 0;
         double best_cost = 0;
-        if (p.swap) {
-            // Any multiple of 32 pixels per item: the item size follows from the pixel count and the 148 SMs
-            // (64 x 32 x 32 pixels: 448 per item = 147 items in one round, where 512 would occupy 128 SMs).
-            // One or two MMAs of equal width cover the item per K step; an MMA narrower than 128 pixels is
-            // bound by its ~64-cycle issue cost.
-            for (int px = 512; px >= 64; px -= 32) {
-                if (forced_px ? px != forced_px : (forced_mt && px != forced_mt * kTileM)) continue;
-                const int groups = (px + 255) / 256;
-                if (px % (16 * groups)) continue;
-                const int npix = npix_of(px);
-                if (npix > 16000 || smem_need(2, npix, p.n_tile, 2, 1, stage_blocks) > kLimit) continue;
-                if (pixel_items(px) == 0) continue;
-                const long long items = pixel_items(px) * p.n_blocks;
-                const long long rounds = (items + sms - 1) / sms;
-                const int nbuf = 2 * px <= 512 ? 2 : 1;
-                const double mma_step = groups * ((px / groups) / 2.0 > 64.0 ? (px / groups) / 2.0 : 64.0);
-                const double tile_time = (double)p.pairs * (2 * mma_step + stage_cycles);
-                const double writeback = (nbuf == 1 ? 1.0 : 0.15) * (px / 128.0) * (3000.0 * p.n_tile / 128.0);
-                double cost = rounds * (tile_time + 0.5 * writeback);
-                // With one accumulator set the MMAs of an item wait for the whole write-back of the item before it
-                // (four warps, measured ~2000 cycles per 32-pixel block of 128 maps, ~1200 of 64); from the third round
-                // of items on that outweighs the wider MMAs (64 x 64 x 56 x 56 -> 128 maps, 3 x 3: 480-pixel items
-                // 69.1 us, 256-pixel items with two accumulator sets 64.6 us).
-                if (nbuf == 1 && rounds >= 3)
-                    cost += (double)(rounds - 2) * 0.75 * (px / 32.0) * (p.n_tile >= 128 ? 2000.0 : 1200.0);
-                // (items that leave half of the SMs idle are split in two along the channels further down)
-                if (items * 2 <= sms && p.cblks >= 2 && ksplit_allowed) cost = 0.5 * tile_time + writeback;
-                if (best_px == 0 || cost < best_cost) { best_px = px; best_cost = cost; }
-            }
-        } else {
-            const double mma_cycles = p.n_tile > 128 ? p.n_tile / 2 : 90;   // per 128-pixel tile and K step
-            for (int mt = 4; mt >= 1; mt >>= 1) {
-                if (forced_mt && mt != forced_mt) continue;
-                if (mt * set_cols > 512) continue;
-                const int npix = npix_of(mt * kTileM);
-                if (npix > 16000 || smem_need(2, npix, p.n_tile, 2, 1, 1) > kLimit) continue;
-                const long long items = (tiles + mt - 1) / mt * p.n_blocks;
-                const long long rounds = (items + sms - 1) / sms;
-                const int nbuf = (2 * mt * set_cols <= 512) ? 2 : 1;
-                const double tile_time = (double)p.pairs * (mt * 2 * mma_cycles + stage_cycles);
-                const double writeback = (nbuf == 1 ? 1.0 : 0.15) * mt * (3000.0 * p.n_tile / 128.0);
-                const double cost = rounds * (tile_time + 0.5 * writeback);
-                if (best_px == 0 || cost < best_cost) { best_px = mt * kTileM; best_cost = cost; }
-            }
+        // Any multiple of 32 pixels per item: the item size follows from the pixel count and the 148 SMs
+        // (64 x 32 x 32 pixels: 448 per item = 147 items in one round, where 512 would occupy 128 SMs).
+        // One or two MMAs of equal width cover the item per K step; an MMA narrower than 128 pixels is
+        // bound by its ~64-cycle issue cost.
+        for (int px = 512; px >= 64; px -= 32) {
+            if (forced_px && px != forced_px) continue;
+            const int groups = (px + 255) / 256;
+            if (px % (16 * groups)) continue;
+            const int npix = npix_of(px);
+            if (npix > 16000 || smem_need(2, npix, p.n_tile, 2, 1, stage_blocks) > kLimit) continue;
+            if (pixel_items(px) == 0) continue;
+            const long long items = pixel_items(px) * p.n_blocks;
+            const long long rounds = (items + sms - 1) / sms;
+            const int nbuf = 2 * px <= 512 ? 2 : 1;
+            const double mma_step = groups * ((px / groups) / 2.0 > 64.0 ? (px / groups) / 2.0 : 64.0);
+            const double tile_time = (double)p.pairs * (2 * mma_step + stage_cycles);
+            const double writeback = (nbuf == 1 ? 1.0 : 0.15) * (px / 128.0) * (3000.0 * p.n_tile / 128.0);
+            double cost = rounds * (tile_time + 0.5 * writeback);
+            // With one accumulator set the MMAs of an item wait for the whole write-back of the item before it
+            // (four warps, measured ~2000 cycles per 32-pixel block of 128 maps, ~1200 of 64); from the third round
+            // of items on that outweighs the wider MMAs (64 x 64 x 56 x 56 -> 128 maps, 3 x 3: 480-pixel items
+            // 69.1 us, 256-pixel items with two accumulator sets 64.6 us).
+            if (nbuf == 1 && rounds >= 3)
+                cost += (double)(rounds - 2) * 0.75 * (px / 32.0) * (p.n_tile >= 128 ? 2000.0 : 1200.0);
+            // (items that leave half of the SMs idle are split in two along the channels further down)
+            if (items * 2 <= sms && p.cblks >= 2 && ksplit_allowed) cost = 0.5 * tile_time + writeback;
+            if (best_px == 0 || cost < best_cost) { best_px = px; best_cost = cost; }
         }
         if (best_px == 0) return p;
         p.tile_px = best_px;
-        p.mt = (best_px + kTileM - 1) / kTileM;
         p.npix = npix_of(p.tile_px);
         // Filter stages: several taps per stage (up to 48 KB, trimmed below until three stages fit) so that the
         // single MMA-issuing thread pays its per-stage bookkeeping (barrier wait, commit: ~90 cycles, measured
@@ -426,11 +393,11 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         p.smem_bytes = smem_need(p.a_stages, p.npix, p.n_tile, p.b_stages, p.tps, p.cbg * stage_blocks) + extra;
     }
 
-    const int item_cols = p.swap ? p.tile_px : p.mt * p.n_tile;     // tensor-memory columns of one accumulator set
-    p.px_groups = p.swap ? (p.tile_px + 255) / 256 : p.mt;
+    const int item_cols = p.tile_px;     // tensor-memory columns of one accumulator set
+    p.px_groups = (p.tile_px + 255) / 256;
     {
         const int want = env_int("CONV2D_B200_TF32_PX_GROUPS", 0);
-        if (p.swap && want > 0 && want <= 2 && p.tile_px % (16 * want) == 0 && p.tile_px / want <= 256) p.px_groups = want;
+        if (want > 0 && want <= 2 && p.tile_px % (16 * want) == 0 && p.tile_px / want <= 256) p.px_groups = want;
     }
     if (p.pair_compact) p.px_groups = 1;
     p.nbuf = (2 * item_cols <= 512 && env_int("CONV2D_B200_TF32_NBUF", 2) != 1) ? 2 : 1;
@@ -449,7 +416,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     // (the filter ring gives up stages for it, down to two) and one item per block.
     p.cluster = 0;
     p.xchg_slots = 0;
-    if (p.ksplit == 2 && p.swap && !p.patch_w && !p.pair_taps && p.fold_r * p.fold_s == 1 && p.n_tile == 128 && !p.resident &&
+    if (p.ksplit == 2 && !p.patch_w && !p.pair_taps && p.fold_r * p.fold_s == 1 && p.n_tile == 128 && !p.resident &&
         items <= sms && env_int("CONV2D_B200_TF32_KSPLIT_CLUSTER", 1) != 0) {
         const int slots = (p.tile_px / 32 + 1) / 2;
         const size_t xb = xchg_area_bytes(slots);
