@@ -124,11 +124,11 @@ int describe_tensor_core_plan(const Shape& sh, bool b16, char* text, size_t text
     const double useful = 2.0 * out_px * sh.K * sh.C * sh.R * sh.S;
     return snprintf(text, text_bytes,
                     "tensor_core=1 kernel=general_tc addressing=%s filters_as=%s m_rows=%d tile_px=%d px_groups=%d acc_sets=%d items=%lld grid=%d "
-                    "ksplit=%d cluster=%d resident_filters=%d stacked_taps=%d stacked_compact=%d fold=%dx%d patch_w=%d smem_bytes=%zu "
+                    "ksplit=%d cluster=%d resident_filters=%d stacked_taps=%d stacked_compact=%d fold=%dx%d patch_w=%d crop=%d smem_bytes=%zu "
                     "mma_useful_px=%.4f mma_useful_flops=%.4f",
                     p.patch_w ? "patch" : "flat", "M", (int)rows, p.tile_px, p.px_groups, p.nbuf,
                     (long long)p.supertiles * p.n_blocks * p.ksplit, p.grid, p.ksplit, p.cluster, p.resident, p.pair_taps, p.pair_compact,
-                    p.fold_r, p.fold_s, p.patch_w, p.smem_bytes, out_px / cols, useful / issued);
+                    p.fold_r, p.fold_s, p.patch_w, p.crop, p.smem_bytes, out_px / cols, useful / issued);
 }
 
 namespace {
@@ -149,10 +149,10 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     if (env_int("CONV2D_B200_TF32_VERBOSE", 0) != 0)
         fprintf(stderr, "conv2d plan: n_tile %d n_blocks %d tile_px %d groups %d nbuf %d npix %d cblks %d taps %d stacked %d "
                 "fold %dx%d patch_w %d tw %d rows %d cols %d a_stages %d cbg %d b_stages %d tps %d resident %d ksplit %d "
-                "items %lld grid %d smem %zu\n",
+                "crop %d cost %.0f items %lld grid %d smem %zu\n",
                 p.n_tile, p.n_blocks, p.tile_px, p.px_groups, p.nbuf, p.npix, p.cblks, p.taps, p.pair_taps, p.fold_r, p.fold_s,
                 p.patch_w, p.patch_tw, p.patch_rows, p.patch_cols, p.a_stages, p.cbg, p.b_stages, p.tps, p.resident, p.ksplit,
-                (long long)p.supertiles * p.n_blocks * p.ksplit, p.grid, p.smem_bytes);
+                p.crop, p.cost, (long long)p.supertiles * p.n_blocks * p.ksplit, p.grid, p.smem_bytes);
     if (workspace_bytes < kStatusBytes + packed_floats(p) * sizeof(float)) return CONV2D_ERR_WORKSPACE;
     unsigned* status = static_cast<unsigned*>(workspace);
     float* wp = reinterpret_cast<float*>(static_cast<unsigned char*>(workspace) + kStatusBytes);
@@ -243,6 +243,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     a.vec_shift = a.vec == 4 ? 2 : (a.vec == 2 ? 1 : 0);
     a.pair_compact = p.pair_compact; a.cb_bytes = (int)p.cb_bytes;
     a.pair_taps = p.pair_taps; a.s_slots = p.s_slots; a.s_step = p.pair_taps ? 2 : 1; a.item_stride = p.tile_px - p.ovl;
+    a.crop = p.crop;
     a.div_HW = FastDiv(plan_h * plan_w); a.div_W = FastDiv(plan_w); a.div_npix = FastDiv(p.npix);
     a.div_qn = FastDiv(p.quad2 ? p.npix / 2 : (p.npix / 4 > 0 ? p.npix / 4 : 1)); a.div_patch_w = FastDiv(p.patch_w ? p.patch_w : 1);
     a.xchg_slots = p.xchg_slots;
@@ -269,7 +270,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     a.div_ksplit = FastDiv(p.ksplit); a.div_n_blocks = FastDiv(p.n_blocks);
     a.div_groups_lo = FastDiv(a.groups / p.ksplit > 0 ? a.groups / p.ksplit : 1);
     a.div_groups_hi = FastDiv((a.groups + p.ksplit - 1) / p.ksplit);
-    a.div_per_image = FastDiv(p.patch_w ? p.patch_rows * p.patch_cols : 1); a.div_patch_cols = FastDiv(p.patch_w ? p.patch_cols : 1);
+    a.div_per_image = FastDiv(p.patch_w ? p.patch_rows * p.patch_cols : (p.crop ? p.crop_items : 1)); a.div_patch_cols = FastDiv(p.patch_w ? p.patch_cols : 1);
     a.patch_item_rows = p.patch_w ? p.tile_px / p.patch_w : 0;
     // Failure-detection test hooks (host-side injection only): a short wait bound and one filter copy that is
     // never issued, so that a bounded wait expires and the time-out path can be checked without hanging anything.

@@ -68,6 +68,7 @@ struct KernelArgs {
                             // issued as an M = 64 MMA onto the same accumulator lanes (no zero-padded upper half)
     int cb_bytes;           // resident filters: bytes of one channel block of the bank (all taps)
     int item_stride;        // flat addressing: pixels between the starts of consecutive items (tile_px minus the overlap)
+    int crop;               // 1: items end with their image (div_per_image of them each), 0: they cut the whole sequence
     int ksplit;             // items per output tile (split of the contraction): 1 or 2
     int xchg_slots;         // cluster instances: 32-pixel blocks each block of a pair receives from its peer
     int xchg_bytes;         // ... and the bytes of the exchange area (rows + barriers) behind the transposition tiles
@@ -90,14 +91,17 @@ struct KernelArgs {
 
 // Where the staged pixel sequence of a work item lives in the image.
 //   flat  (PATCH = false): pixels of the whole batch numbered j = (n*H + h)*W + w; an item is the run
-//          [j0, j0 + tile_px) plus its halo; vertically adjacent taps are W pixels apart.
+//          [j0, j0 + tile_px) plus its halo; vertically adjacent taps are W pixels apart.  The windows of an image's last
+//          R - 1 rows wrap into the next image; where it pays the items leave them out (`crop`): they are equal
+//          parts of one image.
 //   patch (PATCH = true): an item is a rectangle of patch_rows... rows x patch_w columns of one image starting at
 //          (row0, col0), stored row after row with pitch patch_w (the staged halo adds R-1 rows); vertically adjacent
 //          taps are patch_w pixels apart.  Columns >= patch_tw of a patch row only feed outputs of the next patch and
 //          are dropped.  This keeps the halo small on wide images, for which the flat run would not fit on chip.
 struct ItemGeom {
     int j0;             // flat: first pixel
-    int n, row0, col0;  // patch: image and top-left corner
+    int n, row0, col0;  // patch: image and top-left corner; flat: image from whose first pixel row0 counts
+    int limit;          // flat: ... and the pixel at which the item's outputs end at the latest, counted from there, too
 };
 // Staged pixel jj -> (image n, offset inside one H*W plane); false when the pixel lies outside the batch / the image.
 template <bool PATCH>
@@ -127,10 +131,10 @@ __device__ __forceinline__ bool output_pixel(const KernelArgs& a, const ItemGeom
         q = g.col0 + pcol;
         return pcol < a.patch_tw && p < a.P && q < a.Q;
     }
-    const int j = g.j0 + jj;
-    if (j >= a.total_pix || jj >= a.item_stride) return false;       // (columns past the stride belong to the next item)
+    const int j = g.row0 + jj;
+    if (j >= g.limit || jj >= a.item_stride) return false;           // (columns past the stride belong to the next item)
     int off;
-    n = a.div_HW.divmod(j, off);
+    n = g.n + a.div_HW.divmod(j, off);
     p = a.div_W.divmod(off, q);
     return p < a.P && q < a.Q;
 }
@@ -363,8 +367,17 @@ __device__ __forceinline__ ItemInfo decode_item(const KernelArgs& a, int item)
     it.n_groups = a.div_ksplit.div((part + 1) * a.groups) - it.g_begin;
     // blocks stream the filter bank in rotated order (see kernel); n_groups is floor or ceil of groups / ksplit
     (it.n_groups == a.div_groups_lo.d ? a.div_groups_lo : a.div_groups_hi).divmod(rest, it.rot);
-    it.geom.j0 = it.supertile * a.item_stride;
-    it.geom.n = it.geom.row0 = it.geom.col0 = 0;
+    it.geom.j0 = it.geom.row0 = it.supertile * a.item_stride;
+    it.geom.n = it.geom.col0 = 0;
+    it.geom.limit = a.total_pix;
+    if (a.crop) {
+        int part;
+        it.geom.n = a.div_per_image.divmod(it.supertile, part);
+        it.geom.row0 = part * a.item_stride;
+        const int plane = (int)a.div_HW.d;
+        it.geom.limit = plane;
+        it.geom.j0 = it.geom.n * plane + it.geom.row0;
+    }
     if (a.patch_w) {
         int rem, pc;
         it.geom.n = a.div_per_image.divmod(it.supertile, rem);
@@ -578,7 +591,7 @@ general_tc_kernel(const KernelArgs a)
             uint32_t a_phase = 0, b_phase = 0, acc_phase0 = 0, acc_phase1 = 0;
             // diagnostics of block 0 (status words 2..5): cycles this thread waited for activations and for a
             // free accumulator set, its total cycles, its item count
-            long long wait_a = 0, wait_acc = 0, issue_cycles = 0;
+            long long wait_a = 0, wait_b = 0, wait_acc = 0, issue_cycles = 0;
             const long long t_begin = clock_now();
             if (kDiag && blockIdx.x == 0 && lane == 0) a.status[6] = (unsigned)(wall_ns() - *t_entry);   // ns from kernel entry to the start of the MMA loop
             int n_items = 0;
@@ -622,7 +635,9 @@ general_tc_kernel(const KernelArgs a)
                             if (a.resident) {
                                 b_lo = b_lo_fixed | ((smem_u32(b_smem + bank_at) >> 4) & 0x3FFFu);
                             } else {
+                                const long long tb = clock_now();
                                 if (!mbar_wait_bounded_warp(&b_full[bs], b_phase, abort_flag, a.max_polls)) { alive = false; break; }
+                                wait_b += clock_now() - tb;
                                 tc_fence_after_sync();
                                 b_lo = b_lo_fixed | ((smem_u32(b_smem + (size_t)bs * b_stage_bytes) >> 4) & 0x3FFFu);
                             }
@@ -693,7 +708,8 @@ general_tc_kernel(const KernelArgs a)
                 a.status[3] = (unsigned)wait_acc;
                 a.status[4] = (unsigned)(clock_now() - t_begin);
                 a.status[5] = (unsigned)n_items;
-                a.status[9] = (unsigned)issue_cycles;
+                a.status[9] = (unsigned)(issue_cycles - wait_b);
+                a.status[16] = (unsigned)wait_b;
                 a.status[7] = (unsigned)(wall_ns() - *t_entry);  // ns from kernel entry to the last MMA issued
             }
         }
@@ -920,7 +936,7 @@ general_tc_kernel(const KernelArgs a)
             // by one column (with the first column of the next block), and a map is the sum of two tile rows.
             constexpr bool stacked = STACK;         // (a template parameter: as a run-time flag it slowed the ordinary epilogue by 15 %)
             const int rpq = stacked ? 16 : a.n_tile / 4;    // maps per lane quarter: 32 (M = 128) or 16 (M = 64: lanes 0-15; stacked taps)
-            const int blocks = a.tile_px / 32;
+            const int blocks = (a.tile_px + 31) / 32;
             auto load_block = [&](uint32_t (&v0)[16], uint32_t (&v1)[16], uint32_t (&vx)[1], int b) {
                 tmem_ld16(lane_base + (uint32_t)(b * 32), v0);
                 tmem_ld16(lane_base + (uint32_t)(b * 32 + 16), v1);
