@@ -1150,6 +1150,80 @@ general_tc_kernel(const KernelArgs a)
                 if (lane == 0 && !helper) mbar_arrive(&acc_empty[buf]);
                 continue;
             }
+            if (STACK && (!VIRT || (a.vec >= 2 && !add))) {
+                // Stacked taps, two blocks to a pass as well.  The two rows of a map are added in registers: lanes l and l + 16 hold
+                // them, exchange a half of their columns (the right-hand taps' one column on) and each keep one half of the sums, so
+                // the tile is written and read once per map (64 x 128 x 32 x 32, 64 of 3 x 3: 33.0 -> 31.0 us; single pixels, 27 x 208 x
+                // 35 x 35: 35.0 -> 28.3.  On virtual images single pixels stay a block at a time: 48 x 384 x 46 x 31, 18 of 3 x 3 84 us, 98
+                // with two, as their producers, which load single pixels, too, then wait longer).
+                const int pairs = (blocks + 1) / 2, p_step = split ? 3 : 1;
+                const int kmax = min(16, a.K - nb * 64 - quarter * 16);            // maps of this quarter that exist
+                const bool up = lane >= 16;
+                auto fill = [&](int h) {                // the block in va0, va1, vax -> half h of the tile
+                    float4* row = reinterpret_cast<float4*>(tile + (lane & 15) * kStackPitch + (up ? 16 : 0) + 32 * h);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        float sum[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int i = 4 * q + e;
+                            const uint32_t give = up ? (i < 15 ? va0[(i + 1) & 15] : va1[0]) : va1[i];
+                            const uint32_t keep = up ? (i < 15 ? va1[(i + 1) & 15] : vax[0]) : va0[i];
+                            sum[e] = __uint_as_float(keep) + __uint_as_float(__shfl_xor_sync(0xffffffffu, give, 16));
+                        }
+                        row[q] = make_float4(sum[0], sum[1], sum[2], sum[3]);
+                    }
+                };
+                int bp = split ? share : 0;
+                if (bp < pairs) load_block(va0, va1, vax, 2 * bp);
+                while (bp < pairs) {
+                    const int b0 = 2 * bp;
+                    tmem_ld_wait();
+                    __syncwarp();                               // the previous pair has been read out
+                    fill(0);
+                    if (b0 + 1 < blocks) {
+                        load_block(va0, va1, vax, b0 + 1);
+                        tmem_ld_wait();
+                        fill(1);
+                    }
+                    __syncwarp();
+                    bp += p_step;
+                    if (bp < pairs) load_block(va0, va1, vax, 2 * bp);
+                    int n, p, q;                                // this lane's first pixel
+                    if (a.vec == 1 || add) {
+                        // single pixels: 32 of one map to an instruction
+                        for (int h = 0; h < 2; ++h)
+                            if (b0 + h < blocks && output_pixel<PATCH>(a, ii.geom, (b0 + h) * 32 + lane, n, p, q)) {
+                                float* o = a.y + (((size_t)n * a.K + nb * 64 + quarter * 16) * a.P + p) * a.Q + q;
+                                const float* src = tile + 32 * h + lane;
+#pragma unroll 8
+                                for (int r = 0; r < kmax; ++r, o += plane, src += kStackPitch) { if (add) atomicAdd(o, *src); else *o = *src; }
+                            }
+                    } else {
+                        // pairs or quads: each half of the warp stores one of the blocks
+                        const int half = lane >> 4, lanes_per_row = 32 >> a.vec_shift;
+                        const int row_sub = (lane & 15) >> (5 - a.vec_shift), pg = lane & (lanes_per_row - 1);
+                        if (b0 + half < blocks && output_pixel<PATCH>(a, ii.geom, (b0 + half) * 32 + pg * a.vec, n, p, q)) {
+                            float* o = a.y + (((size_t)n * a.K + nb * 64 + quarter * 16 + row_sub) * a.P + p) * a.Q + q;
+                            const float* src = tile + row_sub * kStackPitch + 32 * half + pg * a.vec;
+                            if (a.vec == 4) {
+#pragma unroll
+                                for (int r = 0; r < 16; r += 2, o += 2 * plane, src += 2 * kStackPitch)
+                                    if (r + row_sub < kmax) *reinterpret_cast<float4*>(o) = *reinterpret_cast<const float4*>(src);
+                            } else {
+#pragma unroll
+                                for (int r = 0; r < 16; ++r, o += plane, src += kStackPitch)
+                                    if (r < kmax) *reinterpret_cast<float2*>(o) = *reinterpret_cast<const float2*>(src);
+                            }
+                        }
+                    }
+                }
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0 && !helper) mbar_arrive(&acc_empty[buf]);
+                if (kDiag && blockIdx.x == 0 && warp == 4 && lane == 0) a.status[11] += (unsigned)(clock_now() - t_busy0);   // drained one item
+                continue;
+            }
             const int b_step = split ? 3 : 1;
             int b = split ? share : 0;
             if (b < blocks) load_block(va0, va1, vax, b);

@@ -41,6 +41,8 @@ constexpr int kMaxTaps = 256;                // taps left as descriptor shifts (
 constexpr size_t kBookBytes = 512 + kMaxTaps * 4;    // barriers, tensor-memory slot, flags + the table of tap shifts
 constexpr int kXposePitch = 36;             // floats per row of the epilogue's transposition tile (16-byte aligned, conflict-free)
 constexpr size_t kXposeBytes = (size_t)kEpilogueWarps * 32 * kXposePitch * 4;
+constexpr int kStackPitch = 68;             // ... of the tile of stacked taps: 16 maps x two 32-pixel blocks (conflict-free likewise)
+static_assert(16 * kStackPitch <= 32 * kXposePitch, "it lies in the same place");
 constexpr int kXchgBlockFloats = 32 * 32;   // exchange area of a two-block cluster: one 32-filter x 32-pixel block of partial sums
 // bytes of that area for `slots` 32-pixel blocks per lane quarter: blocks, then one barrier per (quarter, slot)
 constexpr size_t xchg_area_bytes(int slots) { return (size_t)kEpilogueWarps * slots * (kXchgBlockFloats * 4 + 8); }
@@ -222,14 +224,17 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     // an odd filter row as a 64-row slice that an M = 64 instruction adds onto the same accumulator lanes.  The bank
     // is then as large as the unstacked one, so a short contraction keeps its resident filters and still issues two
     // instructions per three taps instead of three at half rate (64 filters of 64 x 3 x 3 on 56 x 56 images).
-    // Measured on that shape: the MMA thread's issue time per 256-pixel item falls from 9.4k to 7.4k cycles, but the
-    // four write-back warps need 10.4k cycles for the item (8.9k unstacked: every map is the sum of two tile rows), and
-    // with two accumulator sets the slower of the two sets the pace: 36.5 -> 39.4 us.  Off by default
-    // (CONV2D_B200_TF32_PAIR_COMPACT = 1 turns it on) until the write-back is faster than the MMAs.
+    // 32 x 64 x 56 x 56, 64 of 3 x 3, padding 1: 29.8 -> 27.7 us (wholly stacked and streamed 28.7).  16-bit operands have half
+    // as many MMAs and are bound by what shared memory moves: off (64 x 128 x 32 x 32, 64 of 3 x 3 in bf16: 22.8 us, 24.8 stacked).
+    // The MMAs have to be what sets the pace: 36 pairs of tap and channel block (with fewer the write-back: 64 x 16 x 90 x 122, 19 of
+    // 3 x 3 57.6 -> 67.7 us; 5 x 48 x 74 x 74, 48 of 3 x 3 12.5 -> 13.9) whose pixels are loaded as quads (else the producers: 7 x 64 x 95 x 95, 48 of 3 x 3, padding 1 26.5 -> 30.8).
+    // CONV2D_B200_TF32_PAIR_COMPACT = 0 / 1: never / whenever possible.
+    const int compact_mode = env_int("CONV2D_B200_TF32_PAIR_COMPACT", b16 ? 0 : 2);
     p.pair_compact = 0;
     const size_t compact_cb_bytes = (size_t)r_eff * ((s_eff / 2) * 128 + (s_eff & 1) * 64) * kCB * 4;
     if (allow_compact && !p.pair_taps && st == 1 && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
-        !padded && (size_t)((c_eff + cbc - 1) / cbc) * compact_cb_bytes <= 152 * 1024 && env_int("CONV2D_B200_TF32_PAIR_COMPACT", 0) != 0) {
+        !padded && (size_t)((c_eff + cbc - 1) / cbc) * compact_cb_bytes <= 152 * 1024 && compact_mode != 0 &&
+        (compact_mode == 1 || ((long long)r_eff * s_eff * p.cblks >= 36 && (virt ? shape.W : sh.H * sh.W) % 4 == 0))) {
         p.pair_taps = 1;
         p.pair_compact = 1;
     }
@@ -267,6 +272,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     }
     if (virt) p.staged_ratio = (448.0 + flat_halo) / 448.0 * ((double)sh.H * sh.W) / ((double)sh.P * sh.Q);
     if (padded && !p.patch_w) return p;
+    if (p.pair_compact && p.patch_w && compact_mode != 1) return plan_with_patch_width(shape, b16, want_patch_w, false, virt, narrow);
     p.ovl = (p.pair_taps && !p.patch_w) ? 4 : 0;
     const long long halo = p.patch_w ? (long long)(r_eff - 1) * p.patch_w + (s_eff - 1) : flat_halo;
     // work items along the pixels for an item of px pixels (0: px is not possible in this mode)
@@ -324,7 +330,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         }
     }
 
-    if (p.pair_compact && !p.resident) return plan_with_patch_width(shape, b16, want_patch_w, false, virt);    // compact stacking needs the resident bank
+    if (p.pair_compact && !p.resident) return plan_with_patch_width(shape, b16, want_patch_w, false, virt, narrow);    // compact stacking needs the resident bank
     if (!p.resident) {
         // Streamed filters.  Measured: all SMs together draw filter stages from L2 at no more than
         // ~5-6 TB/s, i.e. a 8 KB stage costs ~120 cycles on top of the MMAs that consume it unless it is

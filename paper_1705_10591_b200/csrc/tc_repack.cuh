@@ -77,7 +77,8 @@ __global__ void repack_filters_kernel(const T* __restrict__ w, T* __restrict__ w
             const size_t row_elems = (size_t)(pairs * n_tile + odd * (n_tile / 2)) * kChunks * EPC;
             T* base = wp + (size_t)cb * ff.R * row_elems;
             const bool chan = vc < ff.C;
-            for (int r = 0; r < ff.R; ++r, base += row_elems) {
+            base += blockIdx.y * row_elems;                // (the rows are shared out over the grid's second dimension)
+            for (int r = blockIdx.y; r < ff.R; r += gridDim.y, base += gridDim.y * row_elems) {
                 for (int u = 0; u < pairs; ++u) {
                     T v = T(0);
                     if (k < K && chan) {
