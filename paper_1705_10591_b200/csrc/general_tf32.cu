@@ -172,26 +172,26 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
         const int bank_blocks = p.cblks / p.phases;
         const size_t tile_bytes = repack_tile_bytes(all_taps);
         const bool tiled = p.fold_r * p.fold_s == 1 && !p.mixed && tile_bytes <= kRepackTileLimit && p.n_tile % 8 == 0 && !p.pair_taps;
+        cudaError_t launched;
         if (tiled) {
             const dim3 grid((unsigned)(p.n_blocks * p.n_tile / 8), (unsigned)bank_blocks);
             int threads = (8 * kChunks * all_taps + 31) / 32 * 32;        // one 16-byte unit per thread in the store phase
             threads = threads < 128 ? 128 : (threads > 1024 ? 1024 : threads);
-            // (launched the ordinary way: it starts only when the previous call's kernel, which may still
-            // be reading the workspace, has finished; measured no gain from overlapping its launch)
-            if (b16)
-                repack_filters_tiled_kernel<unsigned short, 8><<<grid, threads, tile_bytes, stream>>>(
-                    static_cast<const unsigned short*>(w_any), reinterpret_cast<unsigned short*>(wp), status, sh.K, sh.C,
-                    all_taps, p.n_tile, bank_blocks, sh.S, 1, 0);
-            else
-                repack_filters_tiled_kernel<float, 4><<<grid, threads, tile_bytes, stream>>>(w, wp, status, sh.K, sh.C, all_taps,
-                                                                                             p.n_tile, bank_blocks, sh.S, p.phases > 1 ? sh.stride : 1, p.ext);
-        } else if (b16)
-            repack_filters_kernel<unsigned short, 8><<<dim3((unsigned)blocks, tap_rows), 256, 0, stream>>>(
-                static_cast<const unsigned short*>(w_any), reinterpret_cast<unsigned short*>(wp), status, sh.K, ff,
-                p.taps, p.n_tile, p.cblks, lanes, p.pair_taps + p.pair_compact);
-        else
-            repack_filters_kernel<float, 4><<<dim3((unsigned)blocks, tap_rows), 256, 0, stream>>>(w, wp, status, sh.K, ff, p.taps,
-                                                                                  p.n_tile, p.cblks, lanes, p.pair_taps + p.pair_compact);
+            launched = b16 ? launch_pdl(repack_filters_tiled_kernel<unsigned short, 8>, grid, dim3(threads), tile_bytes, stream,
+                                        static_cast<const unsigned short*>(w_any), reinterpret_cast<unsigned short*>(wp), status, sh.K, sh.C,
+                                        all_taps, p.n_tile, bank_blocks, sh.S, 1, 0)
+                           : launch_pdl(repack_filters_tiled_kernel<float, 4>, grid, dim3(threads), tile_bytes, stream, w, wp, status, sh.K, sh.C,
+                                        all_taps, p.n_tile, bank_blocks, sh.S, p.phases > 1 ? sh.stride : 1, p.ext);
+        } else {
+            const dim3 grid((unsigned)blocks, tap_rows);
+            const int stacked = p.pair_taps + p.pair_compact;
+            launched = b16 ? launch_pdl(repack_filters_kernel<unsigned short, 8>, grid, dim3(256), 0, stream,
+                                        static_cast<const unsigned short*>(w_any), reinterpret_cast<unsigned short*>(wp), status, sh.K, ff,
+                                        p.taps, p.n_tile, p.cblks, lanes, stacked)
+                           : launch_pdl(repack_filters_kernel<float, 4>, grid, dim3(256), 0, stream, w, wp, status, sh.K, ff, p.taps,
+                                        p.n_tile, p.cblks, lanes, stacked);
+        }
+        if (launched != cudaSuccess) return CONV2D_ERR_CUDA;
         count_launch();
         if (cudaGetLastError() != cudaSuccess) return CONV2D_ERR_CUDA;
     }

@@ -431,6 +431,7 @@ pointwise_tma_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
 __global__ void round_filters_tf32_kernel(const float4* __restrict__ w, float4* __restrict__ wp, long long n4,
                                           unsigned* __restrict__ status)
 {
+    grid_dep_wait();        // (the previous kernel on the stream may still be reading the workspace)
     grid_dep_launch();      // the convolution kernel may set itself up while this one runs
     if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / sizeof(unsigned)) status[threadIdx.x] = 0u;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -676,10 +677,8 @@ conv2d_status_t launch_pw(const void* x, const void* w, float* y, const Shape& s
             const long long n4 = (long long)sh.K * sh.C / 4;
             long long blocks = (n4 + 255) / 256;
             if (blocks > sm_count() * 8LL) blocks = sm_count() * 8LL;
-            // (launched the ordinary way: it starts only when the previous kernel on the stream, which may still be
-            // reading the workspace, has finished)
-            round_filters_tf32_kernel<<<(unsigned)blocks, 256, 0, stream>>>(static_cast<const float4*>(w), reinterpret_cast<float4*>(wp),
-                                                                            n4, static_cast<unsigned*>(workspace));
+            if (launch_pdl(round_filters_tf32_kernel, dim3((unsigned)blocks), dim3(256), 0, stream, static_cast<const float4*>(w),
+                           reinterpret_cast<float4*>(wp), n4, static_cast<unsigned*>(workspace)) != cudaSuccess) return CONV2D_ERR_CUDA;
             count_launch();
         }
         w = wp;

@@ -498,8 +498,8 @@ general_tc_kernel(const KernelArgs a)
     // Everything above touched only this block's shared and tensor memory; it may overlap the tail of the
     // preceding kernel on the stream (the filter re-ordering of this call, or the previous call).  From here
     // on global memory is read and written: every role waits for the preceding kernel first, except that the
-    // producers go ahead when that kernel is this call's own filter re-ordering.  It was launched the ordinary way,
-    // so everything before it on the stream had finished when it started, it does not touch the image, and the
+    // producers go ahead when that kernel is this call's own filter re-ordering.  That one lets this kernel start only after
+    // everything before it on the stream has finished, it does not touch the image, and the
     // image is read only: the first activation stages are then in flight while the filters are still being written.
     grid_dep_launch();
     if (!(a.early_x && producer_index(warp) >= 0)) grid_dep_wait();
