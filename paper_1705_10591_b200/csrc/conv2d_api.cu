@@ -32,6 +32,7 @@ conv2d_status_t make_shape(int N, int C, int H, int W, int K, int R, int S, Shap
 __global__ void pad_planes_kernel(const float* __restrict__ x, float* __restrict__ xp, int H, int W, int pad_h, int pad_w,
                                   unsigned* status_to_clear)
 {
+    ptx::grid_dep_wait();
     // (the fp32 path has no kernel that clears the status block in front of the workspace)
     if (status_to_clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / sizeof(unsigned))
         status_to_clear[threadIdx.x] = 0u;
@@ -56,6 +57,7 @@ template <bool ROUND>
 __global__ void space_to_depth_kernel(const float* __restrict__ x, float* __restrict__ x2, int H, int W,
                                       int pad_h, int pad_w, int st, int H2, int W2, unsigned* status_to_clear)
 {
+    ptx::grid_dep_wait();
     if (status_to_clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / sizeof(unsigned))
         status_to_clear[threadIdx.x] = 0u;
     // blockIdx.y = source plane (n, c); it produces the st*st planes (a, b) of the rewritten image
@@ -75,6 +77,7 @@ template <bool ROUND>
 __global__ void filters_to_depth_kernel(const float* __restrict__ w, float* __restrict__ w2, int K, int C, int R, int S,
                                         int st, int R2, int S2)
 {
+    ptx::grid_dep_wait();
     const long long total = (long long)K * C * st * st * R2 * S2;
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
@@ -300,9 +303,9 @@ conv2d_status_t conv2d_fwd_general_padded(const float* x, const float* w, float*
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     const int plane_p = (H + 2 * pad_h) * (W + 2 * pad_w);
     const dim3 grid((unsigned)((plane_p + 1023) / 1024 > 64 ? 64 : (plane_p + 1023) / 1024), (unsigned)(N * C));
-    pad_planes_kernel<<<grid, 256, 0, stream>>>(x, xp, H, W, pad_h, pad_w, own_status ? static_cast<unsigned*>(workspace) : nullptr);
+    if (launch_pdl(pad_planes_kernel, grid, dim3(256), 0, stream, x, xp, H, W, pad_h, pad_w, own_status ? static_cast<unsigned*>(workspace) : nullptr) != cudaSuccess)
+        return CONV2D_ERR_CUDA;
     count_launch(1);
-    if (cudaGetLastError() != cudaSuccess) return CONV2D_ERR_CUDA;
     return conv2d_fwd_general(xp, w, y, N, C, H + 2 * pad_h, W + 2 * pad_w, K, R, S, algo, workspace, inner, flags, cuda_stream);
 }
 
@@ -367,16 +370,16 @@ conv2d_status_t conv2d_fwd_general_strided(const float* x, const float* w, float
         const int work = stride * stride * g.H2 * g.W2;
         const dim3 grid((unsigned)((work + 1023) / 1024 > 64 ? 64 : (work + 1023) / 1024), (unsigned)(N * C));
         auto kernel = tensor_cores ? space_to_depth_kernel<true> : space_to_depth_kernel<false>;
-        kernel<<<grid, 256, 0, stream>>>(x, x2, H, W, pad_h, pad_w, stride, g.H2, g.W2,
-                                         own_status ? static_cast<unsigned*>(workspace) : nullptr);
+        if (launch_pdl(kernel, grid, dim3(256), 0, stream, x, x2, H, W, pad_h, pad_w, stride, g.H2, g.W2,
+                       own_status ? static_cast<unsigned*>(workspace) : nullptr) != cudaSuccess) return CONV2D_ERR_CUDA;
     }
     count_launch(1);
     if (!(flags & CONV2D_FLAG_WEIGHTS_PACKED)) {
         auto kernel = tensor_cores ? filters_to_depth_kernel<true> : filters_to_depth_kernel<false>;
-        kernel<<<blocks_for((long long)K * g.C2 * g.R2 * g.S2), 256, 0, stream>>>(w, w2, K, C, R, S, stride, g.R2, g.S2);
+        if (launch_pdl(kernel, dim3(blocks_for((long long)K * g.C2 * g.R2 * g.S2)), dim3(256), 0, stream, w, w2, K, C, R, S, stride, g.R2, g.S2) != cudaSuccess)
+            return CONV2D_ERR_CUDA;
         count_launch(1);
     }
-    if (cudaGetLastError() != cudaSuccess) return CONV2D_ERR_CUDA;
     return conv2d_fwd_general(x2, w2, y, N, g.C2, g.H2, g.W2, K, g.R2, g.S2, algo, workspace, inner, flags, cuda_stream);
 }
 

@@ -279,6 +279,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     a.rot = env_int("CONV2D_B200_TF32_ROT", b16 ? 1 : 0) != 0 ? 1 : 0;
     a.test_drop_stage = env_int("CONV2D_B200_TF32_TEST_DROP_STAGE", -1);
     a.tmem_cols = (unsigned)p.tmem_cols;
+    a.early_next = weights_packed ? 1 : 0;
     a.early_x = (!weights_packed && (p.ksplit == 1 || p.cluster) && env_int("CONV2D_B200_TF32_EARLY_X", 1) != 0) ? 1 : 0;
     if (p.ksplit > 1 && !p.cluster &&
         cudaMemsetAsync(y, 0, (size_t)sh.N * sh.K * sh.P * sh.Q * sizeof(float), stream) != cudaSuccess)

@@ -89,6 +89,7 @@ struct PwArgs {
     int wide;            // pairs only: an item spans two MMA widths of pixels and uses both accumulator sets at once, so
                          // that a filter chunk serves twice the pixels (no write-back under the next item's MMAs then)
     unsigned max_polls;  // bound of every barrier wait
+    int early_next;      // 1: the next kernel on the stream may be placed while this one runs (see launch_pdl)
     int test_drop_stage; // test hook: the activation stage with this ordinal is armed but never copied (-1: none)
     FastDiv div_apb, div_tiles, div_nb;
 };
@@ -194,7 +195,7 @@ pointwise_tma_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
     const uint32_t tmem = *tmem_slot;
     // Everything above touched only this block's (pair's) shared and tensor memory and may overlap the tail of the
     // preceding kernel on the stream; global memory is read and written from here on.
-    grid_dep_launch();
+    if (a.early_next) grid_dep_launch();
     grid_dep_wait();
     if (blockIdx.x == 0 && tid == 0) *a.status = 0u;       // (a block that gives up raises it at its very end)
 
@@ -431,7 +432,7 @@ pointwise_tma_kernel(const __grid_constant__ CUtensorMap map_w, const __grid_con
 __global__ void round_filters_tf32_kernel(const float4* __restrict__ w, float4* __restrict__ wp, long long n4,
                                           unsigned* __restrict__ status)
 {
-    grid_dep_wait();        // (the previous kernel on the stream may still be reading the workspace)
+    grid_dep_wait();        // (the previous call may still be reading the workspace)
     grid_dep_launch();      // the convolution kernel may set itself up while this one runs
     if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / sizeof(unsigned)) status[threadIdx.x] = 0u;
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -740,6 +741,7 @@ conv2d_status_t launch_pw(const void* x, const void* w, float* y, const Shape& s
     a.ksplit = p.ksplit; a.cpart = p.cpart;
     a.multi = multi ? 1 : 0;
     a.max_polls = (unsigned)env_int("CONV2D_B200_TF32_MAX_POLLS", 1 << 22);
+    a.early_next = weights_packed || !p.round_filters ? 1 : 0;
     a.test_drop_stage = env_int("CONV2D_B200_TF32_TEST_DROP_STAGE", -1);
     a.div_apb = FastDiv(p.apb); a.div_tiles = FastDiv(p.tiles); a.div_nb = FastDiv(p.n_units * p.ksplit);
     if (env_int("CONV2D_B200_TF32_VERBOSE", 0) != 0)

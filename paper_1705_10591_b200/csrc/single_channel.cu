@@ -258,6 +258,7 @@ __global__ void __launch_bounds__(kThreads)
 single_channel_packed_kernel(const float* __restrict__ x, const float* __restrict__ w, float* __restrict__ y,
                              int H, int W, int K, int P, int Q, int tile_h, int vec_ld, int vec_st)
 {
+    ptx::grid_dep_wait();
     constexpr int NV = (S + kVec - 1 + 3) / 4;          // float4 loads per window row
     constexpr int WC = 4 * NV;
     constexpr int WR = R - 1 + TR;
@@ -399,7 +400,8 @@ conv2d_status_t launch_packed(const float* x, const float* w, float* y, const Sh
     dim3 grid((sh.Q + kTileW - 1) / kTileW, (sh.P + tile_h - 1) / tile_h, sh.N);
     const int vec_ld = (sh.W % 4 == 0) && (reinterpret_cast<uintptr_t>(x) % 16 == 0);
     const int vec_st = (sh.Q % 4 == 0) && (reinterpret_cast<uintptr_t>(y) % 16 == 0);
-    kern<<<grid, kThreads, smem, stream>>>(x, w, y, sh.H, sh.W, sh.K, sh.P, sh.Q, tile_h, vec_ld, vec_st);
+    if (launch_pdl(kern, grid, dim3(kThreads), smem, stream, x, w, y, sh.H, sh.W, sh.K, sh.P, sh.Q, tile_h, vec_ld, vec_st) != cudaSuccess)
+        return CONV2D_ERR_CUDA;
     count_launch();
     return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
 }
@@ -444,6 +446,7 @@ single_channel_rows_kernel(const float* __restrict__ x, const float* __restrict_
                            int N, int H, int W, int K, int P, int Q, int band_h, int col_tiles, int items,
                            unsigned max_polls, int test_short_item)
 {
+    ptx::grid_dep_wait();
     constexpr int NV = (S + kVec - 1 + 3) / 4;
     constexpr int WC = 4 * NV;
     constexpr int WR = R - 1 + TR;
@@ -615,9 +618,9 @@ conv2d_status_t launch_rows(const float* x, const float* w, float* y, const Shap
     const int grid = (int)(items < sms ? items : sms);
     // Failure-detection test hooks (host-side injection only): a short wait bound and one item whose barrier
     // expects a row that is never copied, so that the wait expires and the time-out path can be checked.
-    kern<<<grid, kRowsThreads, smem, stream>>>(x, w, y, sh.N, sh.H, sh.W, sh.K, sh.P, sh.Q, band_h, col_tiles, (int)items,
-                                               (unsigned)env_int("CONV2D_B200_SC_MAX_POLLS", 1 << 22),
-                                               env_int("CONV2D_B200_SC_TEST_SHORT_ITEM", -1));
+    if (launch_pdl(kern, dim3(grid), dim3(kRowsThreads), smem, stream, x, w, y, sh.N, sh.H, sh.W, sh.K, sh.P, sh.Q, band_h, col_tiles, (int)items,
+                   (unsigned)env_int("CONV2D_B200_SC_MAX_POLLS", 1 << 22), env_int("CONV2D_B200_SC_TEST_SHORT_ITEM", -1)) != cudaSuccess)
+        return CONV2D_ERR_CUDA;
     count_launch();
     return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
 }
@@ -640,6 +643,7 @@ single_channel_rows_shift_kernel(const float* __restrict__ x, const float* __res
                                  int N, int H, int W, int K, int P, int Q, int band_h, int col_tiles, int items,
                                  unsigned max_polls, int test_short_item)
 {
+    ptx::grid_dep_wait();
     constexpr int WC = (S + kVec - 1 + 1) / 2 * 2;      // window columns, even
     constexpr int RS = R * S;
     constexpr int RS2 = (RS + 1) / 2;
@@ -809,9 +813,9 @@ conv2d_status_t launch_rows_shift(const float* x, const float* w, float* y, cons
     if (items > 0x7fffffffLL) return CONV2D_ERR_UNSUPPORTED;
     const int sms = sm_count();
     const int grid = (int)(items < sms ? items : sms);
-    kern<<<grid, kRowsThreads, smem, stream>>>(x, w, y, sh.N, sh.H, sh.W, sh.K, sh.P, sh.Q, band_h, col_tiles, (int)items,
-                                               (unsigned)env_int("CONV2D_B200_SC_MAX_POLLS", 1 << 22),
-                                               env_int("CONV2D_B200_SC_TEST_SHORT_ITEM", -1));
+    if (launch_pdl(kern, dim3(grid), dim3(kRowsThreads), smem, stream, x, w, y, sh.N, sh.H, sh.W, sh.K, sh.P, sh.Q, band_h, col_tiles, (int)items,
+                   (unsigned)env_int("CONV2D_B200_SC_MAX_POLLS", 1 << 22), env_int("CONV2D_B200_SC_TEST_SHORT_ITEM", -1)) != cudaSuccess)
+        return CONV2D_ERR_CUDA;
     count_launch();
     return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
 }

@@ -17,6 +17,7 @@
 // thread and tap read (half the broadcasts, 16 warps) were slower everywhere: 2049 x 2049, 32 maps of 5 x 5 165 -> 214.
 #include "common.cuh"
 #include "fastdiv.cuh"
+#include "ptx.cuh"
 
 namespace conv2d_b200 {
 namespace {
@@ -55,6 +56,7 @@ template <int RT, int S, int M, bool TURN>
 __global__ void __launch_bounds__(kMaxThreads, Residency<M>::kBlocks)
 single_channel_flat_kernel(const FlatArgs a)
 {
+    ptx::grid_dep_wait();
     constexpr int PB = M / 2;                             // pairs of maps
     constexpr int TF = M == 1 ? 2 : M;                    // floats per tap: (w, w), or one of every map
     extern __shared__ __align__(16) float smem[];
@@ -292,9 +294,9 @@ conv2d_status_t launch_flat(FlatArgs& a, const Shape& sh, cudaStream_t stream)
     static SmemLimit smem_done;
     if (best_smem > 48 * 1024 && raise_smem_limit(reinterpret_cast<const void*>(kern), best_smem, smem_done) != cudaSuccess)
         return CONV2D_ERR_CUDA;
-    kern<<<(unsigned)blocks, best_threads, best_smem, stream>>>(a);
+    if (launch_pdl(kern, dim3((unsigned)blocks), dim3(best_threads), best_smem, stream, a) != cudaSuccess) return CONV2D_ERR_CUDA;
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
+    return CONV2D_OK;
 }
 
 // Maps accumulated together: as many as a class fills.  More of them share the reads of a window row; empty ones cost

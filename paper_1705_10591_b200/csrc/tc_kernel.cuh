@@ -76,6 +76,7 @@ struct KernelArgs {
     int test_drop_stage;    // test hook: the filter copy with this ordinal is armed but never issued (-1: none)
     int early_x;            // 1: this call's filter re-ordering kernel directly precedes on the stream, so the image is
                             // final already and the producers need not wait for that kernel
+    int early_next;         // 1: the next kernel on the stream may be placed while this one runs (see launch_pdl)
     // Virtual images (VIRT kernels): zero padding and strides, see staged_pixel_virtual.  H, W, HW are those of the image
     // in memory; div_HW and div_W divide by the virtual plane and row, total_pix counts virtual pixels.
     int st, off_h, off_w;   // stride; rows and columns of zeros before the image in the virtual one (before the stride)
@@ -501,7 +502,7 @@ general_tc_kernel(const KernelArgs a)
     // producers go ahead when that kernel is this call's own filter re-ordering.  That one lets this kernel start only after
     // everything before it on the stream has finished, it does not touch the image, and the
     // image is read only: the first activation stages are then in flight while the filters are still being written.
-    grid_dep_launch();
+    if (a.early_next) grid_dep_launch();
     if (!(a.early_x && producer_index(warp) >= 0)) grid_dep_wait();
 
     // Work item -> (supertile, filter block); blocks rotate the order of the channel-block groups by the

@@ -10,14 +10,9 @@ namespace {
 using namespace ptx;
 
 // The kernels that prepare filters are launched while the kernel before them on the stream drains (256 filters of 256 x 3 x 3 for 32 x
-// 14 x 14: complete call 26.8 -> 25.5 us).  They wait for its end before they touch anything (it may be the previous call, still
+// 14 x 14: complete call 26.8 -> 25.4 us).  They wait for its end before they touch anything (it may be the previous call, still
 // reading the workspace), and only then let the convolution kernel set itself up: whatever precedes the call is complete when
 // that kernel's first block starts, so its producers may read the image at once.
-__device__ __forceinline__ void start_after_previous()
-{
-    grid_dep_wait();
-    grid_dep_launch();
-}
 
 // ---------------------------------------------------------------- filter re-ordering
 // wp[nb][cb][t][chunk][f][e] = tf32(w[nb*n_tile + f][cb*kCB + 4*chunk + e][t]), zero outside K, C.
@@ -58,7 +53,8 @@ __global__ void repack_filters_kernel(const T* __restrict__ w, T* __restrict__ w
                                       int K, FoldedFilter ff, int taps, int n_tile, int cblks, long long threads_total,
                                       int stacked)
 {
-    start_after_previous();
+    grid_dep_wait();        // (the previous call may still be reading the workspace)
+    grid_dep_launch();
     // the status block in front of the filters starts every (non-prepacked) call cleared
     if (blockIdx.x == 0 && threadIdx.x < kStatusBytes / sizeof(unsigned)) status[threadIdx.x] = 0u;
     const bool folded = ff.fold_r * ff.fold_s > 1 || ff.st > 1;
@@ -136,7 +132,8 @@ __global__ void repack_filters_tiled_kernel(const T* __restrict__ w, T* __restri
 {
     extern __shared__ __align__(16) unsigned char repack_smem[];
     T* tile = reinterpret_cast<T*>(repack_smem);                 // [8][cpb * taps]
-    start_after_previous();
+    grid_dep_wait();        // (the previous call may still be reading the workspace)
+    grid_dep_launch();
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kStatusBytes / sizeof(unsigned)) status[threadIdx.x] = 0u;
     constexpr int cpb = kChunks * EPC;                           // channels per block
     const int cb = blockIdx.y, k0 = blockIdx.x * 8, c0 = cb * cpb;
