@@ -350,6 +350,14 @@ __device__ __forceinline__ void store_units(const float (&v)[CNT][kCB], float4* 
     }
 }
 
+// The four pixels of a quad from number `turn` on, cyclically.
+__device__ __forceinline__ float4 turned(float4 v, int turn)
+{
+    if (turn & 1) v = make_float4(v.y, v.z, v.w, v.x);
+    if (turn & 2) v = make_float4(v.z, v.w, v.x, v.y);
+    return v;
+}
+
 // Work item -> (supertile, filter block, part of the contraction).  With ksplit = 2 two items share an
 // output tile, each contracts half of the channel-block groups and both add their partial sums into y
 // (zeroed beforehand); 0 + a + b does not depend on the order, so the result stays deterministic.
@@ -428,6 +436,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 general_tc_kernel(const KernelArgs a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
+    constexpr bool kEarlyLoads = B16 || STACK || M64 || CLUSTER;      // producers load before they wait for the stage (see there)
+    constexpr bool kTurn = STACK || M64;                  // quad producers: lanes start with different pixels (see there)
     const uint32_t a_block_bytes = (uint32_t)kCB * a.cstride * 4 * (VIRT && a.quad2 && !a.mixed ? 2 : 1);       // one channel block of a stage
     const uint32_t a_stage_bytes = a_block_bytes * (uint32_t)a.cbg;
     const uint32_t b_chunk_bytes = (uint32_t)kCB * a.n_tile * 4;        // one (channel block, tap)
@@ -740,7 +750,20 @@ general_tc_kernel(const KernelArgs a)
                 const uint32_t a_phase = next_phase;
                 if (++next_as == a.a_stages) { next_as = 0; next_phase ^= 1u; }
                 if ((kstage & (a.pgroups - 1)) != gid) continue;         // pgroups is 1, 2 or 4
-                if (!mbar_wait_bounded(&a_empty[as], a_phase ^ 1u, abort_flag, a.max_polls)) { alive = false; break; }
+                // The stage is waited for when the first loads are under way: they need registers only, and a ring of two stages
+                // has no time to spare for their latency (with the turned stores below 32 x 64 x 56 x 56, 64 of 3 x 3, padding 1: 27.7 -> 23.1 us;
+                // 64 x 128 x 32 x 32, 128 of 3 x 3 in bf16 24.8 -> 23.4).  Of 128 fp32 filters in blocks of their own the wait comes first
+                // (32 x 128 x 56 x 56, stride 2 30.5 us, 31.9 with the loads first; 28 x 45 x 100 x 100, 176 of 3 x 3 110 and 122).
+                if (!kEarlyLoads && !mbar_wait_bounded(&a_empty[as], a_phase ^ 1u, abort_flag, a.max_polls)) { alive = false; break; }
+                bool waited = false;
+                auto stage_free = [&]() {
+                    if (!kEarlyLoads) return true;
+                    if (!waited) {
+                        waited = true;
+                        if (!mbar_wait_bounded(&a_empty[as], a_phase ^ 1u, abort_flag, a.max_polls)) alive = false;
+                    }
+                    return alive;
+                };
                 float4* dst = reinterpret_cast<float4*>(a_smem + (size_t)as * a_stage_bytes);
                 int gr = grp + ii.rot;
                 if (gr >= ii.n_groups) gr -= ii.n_groups;
@@ -757,6 +780,8 @@ general_tc_kernel(const KernelArgs a)
                         int n, h, wc;
                         const bool in = staged_pixel_virtual(a, ii.geom, 2 * pq, n, h, wc) && (unsigned)wc < (unsigned)a.W && cb < a.cblks;
                         float4* d = dst + (size_t)g * (a_block_bytes >> 4) + 2 * pq;
+                        // (phases as channels: two pixels, 32 bytes of a chunk, per lane; four lanes of eight start with the second, see the quads below)
+                        const int second = kTurn ? (pq >> 2) & 1 : 0, turn = 2 * second;
                         if (a.mixed) {
                             // a chunk holds the four phases of a channel: two rows of the image
                             const int c0 = cb * kChunks;
@@ -769,11 +794,12 @@ general_tc_kernel(const KernelArgs a)
                                     if ((unsigned)(h + 1) < (unsigned)a.H) v[2 * c + 1] = __ldg(reinterpret_cast<const float4*>(src + (size_t)c * a.HW + a.W));
                                 }
                             }
+                            if (!stage_free()) break;
 #pragma unroll
                             for (int c = 0; c < kChunks; ++c) {
-                                const float4 r0 = v[2 * c], r1 = v[2 * c + 1];
-                                d[c * a.cstride] = make_float4(to_tf32_rna(r0.x), to_tf32_rna(r0.y), to_tf32_rna(r1.x), to_tf32_rna(r1.y));
-                                d[c * a.cstride + 1] = make_float4(to_tf32_rna(r0.z), to_tf32_rna(r0.w), to_tf32_rna(r1.z), to_tf32_rna(r1.w));
+                                const float4 r0 = turned(v[2 * c], turn), r1 = turned(v[2 * c + 1], turn);
+                                d[c * a.cstride + second] = make_float4(to_tf32_rna(r0.x), to_tf32_rna(r0.y), to_tf32_rna(r1.x), to_tf32_rna(r1.y));
+                                d[c * a.cstride + (second ^ 1)] = make_float4(to_tf32_rna(r0.z), to_tf32_rna(r0.w), to_tf32_rna(r1.z), to_tf32_rna(r1.w));
                             }
                         } else {
                             const Phase p = phase_of(a, phase_table, cb);
@@ -785,6 +811,7 @@ general_tc_kernel(const KernelArgs a)
                                 for (int e = 0; e < kCB; ++e)
                                     if (c0 + e < a.C) v[e] = __ldg(reinterpret_cast<const float4*>(src + (size_t)e * a.HW));
                             }
+                            if (!stage_free()) break;
 #pragma unroll
                             for (int ch = 0; ch < kChunks; ++ch) {
                                 float4* dc = d + ch * a.cstride;
@@ -810,7 +837,12 @@ general_tc_kernel(const KernelArgs a)
                         // would fall on the same banks write different chunks in the same instruction.  Measured:
                         // a gain with 16-bit operands (below) only; with fp32 inputs the rotation is left out,
                         // as it splits every 512-byte load instruction over four channel planes (slower from DRAM).
-                        const int rot = a.rot ? (pq >> 1) & 3 : 0;
+                        const int rot = !kTurn && a.rot ? (pq >> 1) & 3 : 0;
+                        // A lane's four pixels are 64 bytes of a chunk, so eight lanes that all stored their first would meet on two
+                        // of the eight 16-byte bank groups.  Each lane takes its pixels in turn from (lane / 2) % 4 on: eight lanes
+                        // then cover all groups.  That costs four selections per stored word, and pays where shared memory sets the pace
+                        // (at most 64 filters: 32 x 64 x 56 x 56, 64 of 3 x 3, padding 1 25.0 -> 23.1 us; but 32 x 256 x 14 x 14, 256 of 3 x 3 24.9 -> 25.3).
+                        const int turn = kTurn ? (pq >> 1) & 3 : 0;
                         float4 v[kCB];
 #pragma unroll
                         for (int e = 0; e < kCB; ++e) v[e] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -835,14 +867,32 @@ general_tc_kernel(const KernelArgs a)
                                     if (j < left) v[4 * ch + j] = __ldg(reinterpret_cast<const float4*>(sc + (size_t)j * a.HW));
                             }
                         }
+                        if (!stage_free()) break;
                         float4* d = dst + (size_t)g * kChunks * a.cstride + 4 * pq;
+                        if (kTurn) {
 #pragma unroll
-                        for (int ch = 0; ch < kChunks; ++ch) {
-                            float4* dc = d + ((ch + rot) & 3) * a.cstride;
-                            dc[0] = make_float4(to_tf32_rna(v[4 * ch].x), to_tf32_rna(v[4 * ch + 1].x), to_tf32_rna(v[4 * ch + 2].x), to_tf32_rna(v[4 * ch + 3].x));
-                            dc[1] = make_float4(to_tf32_rna(v[4 * ch].y), to_tf32_rna(v[4 * ch + 1].y), to_tf32_rna(v[4 * ch + 2].y), to_tf32_rna(v[4 * ch + 3].y));
-                            dc[2] = make_float4(to_tf32_rna(v[4 * ch].z), to_tf32_rna(v[4 * ch + 1].z), to_tf32_rna(v[4 * ch + 2].z), to_tf32_rna(v[4 * ch + 3].z));
-                            dc[3] = make_float4(to_tf32_rna(v[4 * ch].w), to_tf32_rna(v[4 * ch + 1].w), to_tf32_rna(v[4 * ch + 2].w), to_tf32_rna(v[4 * ch + 3].w));
+                            for (int ch = 0; ch < kChunks; ++ch, d += a.cstride) {
+                                float4 u[4];                       // pixel (i + turn) % 4
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) {
+                                    const float4 t = turned(v[4 * ch + j], turn);
+                                    reinterpret_cast<float*>(&u[0])[j] = to_tf32_rna(t.x);
+                                    reinterpret_cast<float*>(&u[1])[j] = to_tf32_rna(t.y);
+                                    reinterpret_cast<float*>(&u[2])[j] = to_tf32_rna(t.z);
+                                    reinterpret_cast<float*>(&u[3])[j] = to_tf32_rna(t.w);
+                                }
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) d[(i + turn) & 3] = u[i];
+                            }
+                        } else {
+#pragma unroll
+                            for (int ch = 0; ch < kChunks; ++ch) {
+                                float4* dc = d + ((ch + rot) & 3) * a.cstride;
+                                dc[0] = make_float4(to_tf32_rna(v[4 * ch].x), to_tf32_rna(v[4 * ch + 1].x), to_tf32_rna(v[4 * ch + 2].x), to_tf32_rna(v[4 * ch + 3].x));
+                                dc[1] = make_float4(to_tf32_rna(v[4 * ch].y), to_tf32_rna(v[4 * ch + 1].y), to_tf32_rna(v[4 * ch + 2].y), to_tf32_rna(v[4 * ch + 3].y));
+                                dc[2] = make_float4(to_tf32_rna(v[4 * ch].z), to_tf32_rna(v[4 * ch + 1].z), to_tf32_rna(v[4 * ch + 2].z), to_tf32_rna(v[4 * ch + 3].z));
+                                dc[3] = make_float4(to_tf32_rna(v[4 * ch].w), to_tf32_rna(v[4 * ch + 1].w), to_tf32_rna(v[4 * ch + 2].w), to_tf32_rna(v[4 * ch + 3].w));
+                            }
                         }
                     }
                 } else if (B16 && !FOLD && a.quad) {
@@ -870,6 +920,7 @@ general_tc_kernel(const KernelArgs a)
                                     if (j < left) v[8 * ch + j] = __ldg(reinterpret_cast<const uint2*>(sc));
                             }
                         }
+                        if (!stage_free()) break;
                         float4* d = dst + (size_t)g * kChunks * a.cstride + 4 * pq;
 #pragma unroll
                         for (int ch = 0; ch < kChunks; ++ch) {        // 8 channels per 16-byte unit; word k = channels 2k, 2k+1
@@ -891,8 +942,10 @@ general_tc_kernel(const KernelArgs a)
                 for (int first = 0; first < units; first += nthr * kUnitsPerThread) {
                     float v[kUnitsPerThread][kCB];
                     load_units<B16, FOLD, PATCH, VIRT>(v, a, phase_table, ii.geom, gr * a.cbg, first, wtid, nthr);
+                    if (!stage_free()) break;
                     store_units<B16>(v, dst, a, first, wtid, nthr);
                 }
+                if (!stage_free()) break;                    // (a thread without a unit of this stage, too)
                 fence_proxy_async_smem();
                 mbar_arrive(&a_full[as]);
             }
