@@ -54,6 +54,7 @@
 #include "tc_plan.cuh"
 #include "tc_repack.cuh"
 #include "tc_kernel.cuh"
+#include "tensor_map.cuh"
 
 namespace conv2d_b200 {
 
@@ -114,6 +115,7 @@ int describe_tensor_core_plan(const Shape& sh, bool b16, char* text, size_t text
     }
     const Plan p = make_plan(sh, b16);
     if (!p.ok) return snprintf(text, text_bytes, "tensor_core=0");
+    const Bank bank = bank_layout(p, sh);
     const double out_px = (double)sh.N * sh.P * sh.Q;
     const double cols = (double)p.supertiles * p.tile_px;
     const double rows = p.n_tile;                                       // rows of the M operand
@@ -124,14 +126,26 @@ int describe_tensor_core_plan(const Shape& sh, bool b16, char* text, size_t text
     const double useful = 2.0 * out_px * sh.K * sh.C * sh.R * sh.S;
     return snprintf(text, text_bytes,
                     "tensor_core=1 kernel=general_tc addressing=%s filters_as=%s m_rows=%d tile_px=%d px_groups=%d acc_sets=%d items=%lld grid=%d "
-                    "ksplit=%d cluster=%d resident_filters=%d stacked_taps=%d stacked_compact=%d fold=%dx%d patch_w=%d crop=%d smem_bytes=%zu "
+                    "ksplit=%d cluster=%d resident_filters=%d stacked_taps=%d stacked_compact=%d bank=%dx%d%s fold=%dx%d patch_w=%d crop=%d smem_bytes=%zu "
                     "mma_useful_px=%.4f mma_useful_flops=%.4f",
                     p.patch_w ? "patch" : "flat", "M", (int)rows, p.tile_px, p.px_groups, p.nbuf,
                     (long long)p.supertiles * p.n_blocks * p.ksplit, p.grid, p.ksplit, p.cluster, p.resident, p.pair_taps, p.pair_compact,
-                    p.fold_r, p.fold_s, p.patch_w, p.crop, p.smem_bytes, out_px / cols, useful / issued);
+                    bank.rows, bank.taps, bank.stacked ? "s" : "", p.fold_r, p.fold_s, p.patch_w, p.crop, p.smem_bytes, out_px / cols, useful / issued);
 }
 
 namespace {
+// A plain bank of 64 filters, `taps` taps behind one another ([chunk][filter][16 bytes]), as the pairs of taps (t, t + 1) that compact
+// stacking multiplies: a box is [chunk][quarter][tap of the pair][16 filters][16 bytes], so that rows 32q .. 32q + 15 of a chunk are
+// maps 16q .. 16q + 15 of the left-hand tap and the 16 after them the same maps of the right-hand one.
+bool pair_map_of(CUtensorMap* map, const float* bank, int taps)
+{
+    constexpr cuuint64_t tap = 64 * 16 * kChunks;
+    const cuuint64_t dims[5] = {64, 2, 4, (cuuint64_t)kChunks, (cuuint64_t)taps - 1};
+    const cuuint64_t strides[4] = {tap, 16 * 16, 64 * 16, tap};
+    const cuuint32_t box[5] = {64, 2, 4, (cuuint32_t)kChunks, 1};
+    return encode_map(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, bank, 5, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE);
+}
+
 // workspace_bytes: checked against the plan's need here, so that a call plans only once (the planner reads two
 // dozen environment switches and costs ~2 us); SIZE_MAX = the caller has checked already.
 conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* y, const Shape& sh, bool b16, bool fp16,
@@ -160,36 +174,35 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     if (!weights_packed) {
         const long long total = (long long)packed_floats(p);
         const FoldedFilter ff{sh.C, sh.R, sh.S, p.fold_r, p.fold_s, p.mixed ? sh.stride : 1, p.ext};
-        const long long lanes = (long long)p.n_blocks * p.cblks * kChunks * p.n_tile * (b16 ? 8 : 4);   // one thread per element of a tap's slice
+        const Bank bank = bank_layout(p, sh);
+        const long long lanes = (long long)p.n_blocks * p.cblks * kChunks * bank.rows * (b16 ? 8 : 4);   // one thread per element of a tap's slice
         long long blocks = (lanes + 255) / 256;
         if (blocks > sm_count() * 16LL) blocks = sm_count() * 16LL;
         // few blocks: the taps are shared out, too (64 filters of 3 x 7 x 7 with stride 2: 16 blocks whose threads walked
         // over 16 taps took 7.6 us)
         unsigned tap_rows = 1;
-        if (p.pair_compact) tap_rows = (unsigned)sh.R;        // (there the rows of taps are: 32 x 64 x 56 x 56, 64 of 3 x 3, complete call 33.3 -> 32.8 us)
-        else while (tap_rows * 2 <= (unsigned)p.taps && blocks * tap_rows * 2 <= sm_count() * 4LL) tap_rows *= 2;
-        const int all_taps = p.phases > 1 ? sh.R * sh.S : p.taps;
+        while (tap_rows * 2 <= (unsigned)bank.taps && blocks * tap_rows * 2 <= sm_count() * 4LL) tap_rows *= 2;
+        const int all_taps = p.phases > 1 ? sh.R * sh.S : bank.taps;
         const int bank_blocks = p.cblks / p.phases;
         const size_t tile_bytes = repack_tile_bytes(all_taps);
-        const bool tiled = p.fold_r * p.fold_s == 1 && !p.mixed && tile_bytes <= kRepackTileLimit && p.n_tile % 8 == 0 && !p.pair_taps;
+        const bool tiled = p.fold_r * p.fold_s == 1 && !p.mixed && tile_bytes <= kRepackTileLimit && !bank.stacked;
         cudaError_t launched;
         if (tiled) {
-            const dim3 grid((unsigned)(p.n_blocks * p.n_tile / 8), (unsigned)bank_blocks);
+            const dim3 grid((unsigned)(p.n_blocks * bank.rows / 8), (unsigned)bank_blocks);
             int threads = (8 * kChunks * all_taps + 31) / 32 * 32;        // one 16-byte unit per thread in the store phase
             threads = threads < 128 ? 128 : (threads > 1024 ? 1024 : threads);
             launched = b16 ? launch_pdl(repack_filters_tiled_kernel<unsigned short, 8>, grid, dim3(threads), tile_bytes, stream,
                                         static_cast<const unsigned short*>(w_any), reinterpret_cast<unsigned short*>(wp), status, sh.K, sh.C,
-                                        all_taps, p.n_tile, bank_blocks, sh.S, 1, 0)
+                                        all_taps, bank.rows, bank_blocks, sh.S, 1, 0)
                            : launch_pdl(repack_filters_tiled_kernel<float, 4>, grid, dim3(threads), tile_bytes, stream, w, wp, status, sh.K, sh.C,
-                                        all_taps, p.n_tile, bank_blocks, sh.S, p.phases > 1 ? sh.stride : 1, p.ext);
+                                        all_taps, bank.rows, bank_blocks, sh.S, p.phases > 1 ? sh.stride : 1, p.ext);
         } else {
             const dim3 grid((unsigned)blocks, tap_rows);
-            const int stacked = p.pair_taps + p.pair_compact;
             launched = b16 ? launch_pdl(repack_filters_kernel<unsigned short, 8>, grid, dim3(256), 0, stream,
                                         static_cast<const unsigned short*>(w_any), reinterpret_cast<unsigned short*>(wp), status, sh.K, ff,
-                                        p.taps, p.n_tile, p.cblks, lanes, stacked)
-                           : launch_pdl(repack_filters_kernel<float, 4>, grid, dim3(256), 0, stream, w, wp, status, sh.K, ff, p.taps,
-                                        p.n_tile, p.cblks, lanes, stacked);
+                                        bank.taps, bank.rows, p.cblks, lanes, bank.stacked)
+                           : launch_pdl(repack_filters_kernel<float, 4>, grid, dim3(256), 0, stream, w, wp, status, sh.K, ff, bank.taps,
+                                        bank.rows, p.cblks, lanes, bank.stacked);
         }
         if (launched != cudaSuccess) return CONV2D_ERR_CUDA;
         count_launch();
@@ -203,7 +216,7 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     if (cudaGetDevice(&dev_id) != cudaSuccess || dev_id < 0 || dev_id >= 64) return CONV2D_ERR_CUDA;
     bool& attr_set = attr_set_on[dev_id];
     if (!attr_set) {
-        void (*all[])(KernelArgs) = {general_tc_kernel<false, false, false, false>, general_tc_kernel<true, false, false, false>,
+        void (*all[])(KernelArgs, CUtensorMap) = {general_tc_kernel<false, false, false, false>, general_tc_kernel<true, false, false, false>,
                                      general_tc_kernel<false, true, false, false>,  general_tc_kernel<true, true, false, false>,
                                      general_tc_kernel<false, false, true, false>,  general_tc_kernel<true, false, true, false>,
                                      general_tc_kernel<false, false, false, true>,  general_tc_kernel<true, false, false, true>,
@@ -287,7 +300,9 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     // Programmatic dependent launch: the kernel's set-up (barriers, tensor-memory allocation) overlaps the
     // tail of whatever kernel precedes it on the stream; it waits for that kernel before it touches global memory.
     const bool fold = p.fold_r * p.fold_s > 1;
-    void (*kernel)(KernelArgs);
+    CUtensorMap pair_map{};
+    if (p.pair_compact && !pair_map_of(&pair_map, wp, p.cblks * sh.R * sh.S)) return CONV2D_ERR_UNSUPPORTED;
+    void (*kernel)(KernelArgs, CUtensorMap);
     if (p.n_tile == 64 && !p.pair_taps) {
         if (p.virt) kernel = general_tc_kernel<false, false, false, false, false, true, true>;
         else if (p.patch_w) kernel = b16 ? general_tc_kernel<true, false, true, false, false, false, true> : general_tc_kernel<false, false, true, false, false, false, true>;
@@ -303,9 +318,9 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     if (p.cluster) {
         kernel = p.virt ? general_tc_kernel<false, false, false, false, true, true>
                : b16 ? general_tc_kernel<true, false, false, false, true> : general_tc_kernel<false, false, false, false, true>;
-        if (launch_pdl_cluster(kernel, dim3((unsigned)p.grid), dim3(kThreads), p.smem_bytes, stream, 2u, a) != cudaSuccess)
+        if (launch_pdl_cluster(kernel, dim3((unsigned)p.grid), dim3(kThreads), p.smem_bytes, stream, 2u, a, pair_map) != cudaSuccess)
             return CONV2D_ERR_CUDA;
-    } else if (launch_pdl(kernel, dim3((unsigned)p.grid), dim3(kThreads), p.smem_bytes, stream, a) != cudaSuccess) return CONV2D_ERR_CUDA;
+    } else if (launch_pdl(kernel, dim3((unsigned)p.grid), dim3(kThreads), p.smem_bytes, stream, a, pair_map) != cudaSuccess) return CONV2D_ERR_CUDA;
     count_launch();
     return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
 }

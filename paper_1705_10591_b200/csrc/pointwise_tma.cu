@@ -32,11 +32,11 @@
 // Every wait is bounded; on expiry the block stops, frees its tensor memory and raises the status word.
 #include <algorithm>
 #include <cstdio>
-#include <cuda.h>
 
 #include "common.cuh"
 #include "fastdiv.cuh"
 #include "ptx.cuh"
+#include "tensor_map.cuh"
 
 namespace conv2d_b200 {
 namespace {
@@ -443,38 +443,6 @@ __global__ void round_filters_tf32_kernel(const float4* __restrict__ w, float4* 
 }
 
 // ---------------------------------------------------------------- host side
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// The driver's tensor-map encoder, looked up through the runtime so that the library does not link against the
-// driver (it must load on machines without one).
-EncodeTiledFn encode_tiled_fn()
-{
-    static EncodeTiledFn fn = []() -> EncodeTiledFn {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            return nullptr;
-        return reinterpret_cast<EncodeTiledFn>(p);
-    }();
-    return fn;
-}
-
-// Tensor of `rank` dimensions (innermost first), zeros for out-of-range elements.  `swizzle`: 128-byte rows
-// with 16-byte chunks swizzled (K-major operands, output tiles) or with 32-byte chunks (the MN-major TF32 operand).
-bool encode_map(CUtensorMap* map, CUtensorMapDataType type, const void* base, int rank, const cuuint64_t* dims,
-                const cuuint64_t* strides_bytes, const cuuint32_t* box, CUtensorMapSwizzle swizzle)
-{
-    EncodeTiledFn fn = encode_tiled_fn();
-    if (!fn) return false;
-    const cuuint32_t ones[4] = {1, 1, 1, 1};
-    return fn(map, type, (cuuint32_t)rank, const_cast<void*>(base), dims, strides_bytes, box, ones,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 struct PwPlan {
     bool ok;
     int m_rows, n_blocks, apb, a_item, tiles, cchunks, stages, grid;

@@ -174,6 +174,11 @@ __device__ __forceinline__ void tma_load_4d(void* smem_dst, const void* map, int
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
                  ::"r"(smem_u32(smem_dst)), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar) : "memory");
 }
+__device__ __forceinline__ void tma_load_5d(void* smem_dst, const void* map, int c0, int c1, int c2, int c3, int c4, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
+                 ::"r"(smem_u32(smem_dst)), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar) : "memory");
+}
 // The same loads for a pair of blocks that run two-SM MMAs (cta_group::2): the box lands in this block's shared
 // memory, the bytes are signalled on `cluster_bar`, a shared::cluster address that may name a barrier of the peer
 // block (the block that issues the pair's MMAs waits for both blocks' boxes on one barrier).

@@ -3,6 +3,7 @@
 #pragma once
 #include "tc_plan.cuh"
 #include "ptx.cuh"
+#include "tensor_map.cuh"
 #include "fastdiv.cuh"
 
 namespace conv2d_b200 {
@@ -423,6 +424,27 @@ __device__ __forceinline__ void issue_tap(uint32_t d, uint32_t px_lo, uint32_t f
 #undef CONV2D_GROUP_MMA
 }
 
+// The resident bank of compact stacking.  In the workspace the bank lies tap by tap, as for every layer of these filters (whether
+// they are stacked depends on the image, too); its slices of two taps are put together here, one box of the tensor
+// map (pair_map_of) each, a lane a slice.  147 KB of 64 filters of 64 x 3 x 3 arrive as early as a bank stored in slices
+// (2 x 56 x 56: 8.9 us either way); issued by one lane 0.6 us later, as 32 bulk copies of 256 bytes to a slice 10 us later.  Not inlined: in line
+// it costs the producers 2 to 10 % (128 x 64 x 56 x 56: 72.3 -> 74 us), whose registers are at the limit.
+__device__ __noinline__ void load_pairs(unsigned char* dst, const float* bank, const CUtensorMap* map, int rows, int S, uint64_t* full,
+                                        volatile uint32_t* abort_flag, int lane)
+{
+    constexpr uint32_t kTap = 64 * 16 * kChunks;
+    if (lane == 0) mbar_arrive_expect_tx(full, (uint32_t)(rows * S) * kTap);
+    __syncwarp();
+    const unsigned char* src = reinterpret_cast<const unsigned char*>(bank);
+    const int slots = (S + 1) / 2;
+    for (int i = lane; i < rows * slots; i += 32) {
+        const int r = i / slots, s = 2 * (i - r * slots), t = r * S + s;
+        if (s + 1 < S) tma_load_5d(dst + (size_t)t * kTap, map, 0, 0, 0, 0, t, smem_u32(full));
+        else bulk_g2s(dst + (size_t)t * kTap, src + (size_t)t * kTap, kTap, full);
+    }
+    if (*abort_flag) { uint32_t dummy = 0; mbar_wait_bounded(full, 0u, &dummy, 1u << 16); }
+}
+
 // CLUSTER: the two work items of a split contraction (ksplit = 2) run as a two-block cluster, one item per block.
 // Each block stores every other 32-pixel block of the tile: it sends its partial sums of the peer's blocks into the
 // peer's shared memory (distributed shared memory, plain stores) and adds what the peer sent to its own
@@ -433,7 +455,7 @@ __device__ __forceinline__ void issue_tap(uint32_t d, uint32_t px_lo, uint32_t f
 // run-time code it cost the 128-filter layers 1 %: more spills in roles that are at the register limit).
 template <bool B16, bool FOLD, bool PATCH, bool STACK, bool CLUSTER = false, bool VIRT = false, bool M64 = false>
 __global__ void __launch_bounds__(kThreads, 1)
-general_tc_kernel(const KernelArgs a)
+general_tc_kernel(const KernelArgs a, const __grid_constant__ CUtensorMap pair_map)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr bool kEarlyLoads = B16 || STACK || M64 || CLUSTER;      // producers load before they wait for the stage (see there)
@@ -444,6 +466,7 @@ general_tc_kernel(const KernelArgs a)
     const uint32_t b_stage_bytes = b_chunk_bytes * (uint32_t)a.tps;
     unsigned char* a_smem = smem;
     unsigned char* b_smem = smem + (size_t)a.a_stages * a_stage_bytes;
+    if (STACK) b_smem = smem + ((size_t)a.a_stages * a_stage_bytes + 127) / 128 * 128;       // (tensor-map copies write to multiples of 128 bytes; stages are multiples of 64)
     const int bank_blocks = VIRT ? a.cblks_c : a.cblks;                 // pieces of cb_bytes in a filter block's bank
     const size_t b_region_bytes = a.resident ? (size_t)bank_blocks * a.cb_bytes : (size_t)a.b_stages * b_stage_bytes;
     float* xpose = reinterpret_cast<float*>(b_smem + b_region_bytes);
@@ -521,7 +544,8 @@ general_tc_kernel(const KernelArgs a)
 
     if (warp == 0) {
         // ---------------- filters: global -> shared by bulk copy, up to `tps` taps of one channel block per stage
-        if (lane == 0) {
+        if (STACK && a.pair_compact) load_pairs(b_smem, a.wp, &pair_map, bank_blocks * a.R, a.S, &b_full[0], abort_flag, lane);
+        else if (lane == 0) {
             int s = 0, issued = 0;
             uint32_t ph = 0;
             bool alive = true;

@@ -38,7 +38,7 @@ constexpr int kMaxAStages = 4;
 constexpr int kUnitsPerThread = 3;          // (pixel, channel block) units a producer thread keeps in flight per pass
 constexpr size_t kSmemLimit = 227 * 1024;
 constexpr int kMaxTaps = 256;                // taps left as descriptor shifts (after folding)
-constexpr size_t kBookBytes = 512 + kMaxTaps * 4;    // barriers, tensor-memory slot, flags + the table of tap shifts
+constexpr size_t kBookBytes = 512 + kMaxTaps * 4;    // barriers, tensor-memory slot, flags, up to 64 bytes before a bank of stacked taps + the table of tap shifts
 constexpr int kXposePitch = 36;             // floats per row of the epilogue's transposition tile (16-byte aligned, conflict-free)
 constexpr size_t kXposeBytes = (size_t)kEpilogueWarps * 32 * kXposePitch * 4;
 constexpr int kStackPitch = 68;             // ... of the tile of stacked taps: 16 maps x two 32-pixel blocks (conflict-free likewise)
@@ -65,7 +65,7 @@ struct Plan {
     int cbg;          // channel blocks per activation stage
     int resident;     // 1: the whole filter block stays in shared memory for the life of the thread block
     int pair_taps;    // 1: at most 64 filters, horizontally adjacent taps stacked in one M = 128 operand (see make_plan)
-    int pair_compact; // 1 (with pair_taps): a lone last tap of a filter row is a 64-row slice issued as M = 64 (resident bank only)
+    int pair_compact; // 1 (with pair_taps): a lone last tap of a filter row is a 64-row slice issued as M = 64 (resident bank only, put together from the plain one)
     size_t cb_bytes;  // bytes of one channel block of the re-ordered bank (all taps of one filter block)
     int s_slots;      // shift-table entries per filter row: S, or ceil(S / 2) with stacked taps
     int ovl;          // pixels by which consecutive flat items overlap (4 with stacked taps, else 0)
@@ -537,6 +537,17 @@ Plan make_plan(const Shape& sh, bool b16 = false)
         if (q.ok && q.patch_w == wp && q.makespan < 0.95 * best.makespan) best = q;
     }
     return best;
+}
+
+// How the re-ordered filters lie in the workspace: `rows` filters to a tap and filter block, `taps` to a channel block.  A call with
+// packed filters may have another number and size of images and another padding than the one that packed them, so this (like the
+// fold and the order of the taps) must follow from the filters' own sizes and the operand type.  Compact stacking
+// depends on the image, too: it puts its pairs of taps together from the plain bank.
+struct Bank { int rows, taps, stacked; };
+Bank bank_layout(const Plan& p, const Shape& sh)
+{
+    if (p.pair_compact) return Bank{p.n_tile / 2, sh.R * sh.S, 0};
+    return Bank{p.n_tile, p.taps, p.pair_taps};
 }
 
 size_t packed_floats(const Plan& p)
