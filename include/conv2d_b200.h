@@ -48,7 +48,7 @@ typedef enum {
     CONV2D_ERR_WORKSPACE = 4,      /* workspace smaller than conv2d_fwd_workspace_size reports */
     CONV2D_ERR_UNSUPPORTED = 5,    /* no kernel instance for this algorithm/shape combination */
     CONV2D_ERR_ARCH = 6,           /* current device is not compute capability 10.x */
-    CONV2D_ERR_CUDA = 7,           /* a CUDA runtime call failed (cudaGetLastError is left set) */
+    CONV2D_ERR_CUDA = 7,           /* a CUDA runtime call failed; later calls do not depend on it (a launch's error is not left set) */
     CONV2D_ERR_DEVICE_TIMEOUT = 8  /* a bounded on-device wait expired; outputs of that launch are invalid */
 } conv2d_status_t;
 

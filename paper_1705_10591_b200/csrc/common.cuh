@@ -86,6 +86,24 @@ inline int env_int(const char* name, int dflt)
     return (v && *v) ? atoi(v) : dflt;
 }
 
+// Every launch reports its own error and takes it out of the runtime, and nothing else asks the runtime for the last error: a call
+// that failed (on a stream whose capture was broken, say) leaves nothing behind that the next valid call would find.
+inline cudaError_t own_error(cudaError_t e)
+{
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_ordinary(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    return own_error(cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...));
+}
+
 // Launch with programmatic stream serialization: the kernel may be scheduled while the preceding kernel on the
 // stream drains; it calls grid_dep_wait() before it touches global memory.  Without an earlier grid_dep_launch() in the preceding
 // kernel "while it drains" begins when its last block ends: the launch is hidden (64 x 64, 8 filters of 3 x 3, one channel: 4.15 ->
@@ -107,7 +125,7 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     attr[0].val.programmaticStreamSerializationAllowed = env_int("CONV2D_B200_TF32_PDL", 1) != 0 ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    return own_error(cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...));
 }
 
 // The same for a kernel whose blocks form clusters of `cluster_x` consecutive blocks.
@@ -129,7 +147,7 @@ cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    return own_error(cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...));
 }
 
 // Launchers.  Each returns CONV2D_OK, CONV2D_ERR_UNSUPPORTED (no instance) or CONV2D_ERR_CUDA.

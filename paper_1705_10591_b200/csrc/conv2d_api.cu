@@ -120,9 +120,9 @@ __global__ void latch_status_kernel(const unsigned* status, unsigned* timed_out)
 }
 cudaError_t latch_status(const void* workspace, unsigned* timed_out, cudaStream_t stream)
 {
-    latch_status_kernel<<<1, 1, 0, stream>>>(static_cast<const unsigned*>(workspace), timed_out);
-    count_launch();
-    return cudaGetLastError();
+    const cudaError_t e = launch_ordinary(latch_status_kernel, dim3(1), dim3(1), 0, stream, static_cast<const unsigned*>(workspace), timed_out);
+    if (e == cudaSuccess) count_launch();
+    return e;
 }
 
 conv2d_status_t check_device()
@@ -415,7 +415,7 @@ struct CopySet {
         auto event = [&](cudaEvent_t& e) { ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess; };
         event(begin); event(end);
         for (int i = 0; i < kMaxChunks; ++i) { event(arrived[i]); event(done[i]); }
-        if (!ok) { destroy(); (void)cudaGetLastError(); }      // (the call goes on without a set: its launches must not find the error)
+        if (!ok) { destroy(); (void)cudaGetLastError(); }      // (the call goes on without a set)
         return ok;
     }
     void destroy()

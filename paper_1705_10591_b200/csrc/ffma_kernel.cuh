@@ -354,9 +354,9 @@ conv2d_status_t launch_split(const float* x, const float* w, float* y, const Sha
     a.vec_st = (sh.Q % 4 == 0 && reinterpret_cast<uintptr_t>(y) % 16 == 0) ? 4
              : (sh.Q % 2 == 0 && reinterpret_cast<uintptr_t>(y) % 8 == 0) ? 2 : 1;
     a.div_groups = FastDiv(f.groups); a.div_sps = FastDiv(f.sps); a.div_P = FastDiv(sh.P); a.div_H = FastDiv(sh.H);
-    kern<<<dim3((unsigned)f.seg_blocks, (unsigned)f.kblocks), f.threads, f.smem, stream>>>(a);
+    if (launch_ordinary(kern, dim3((unsigned)f.seg_blocks, (unsigned)f.kblocks), dim3(f.threads), f.smem, stream, a) != cudaSuccess) return CONV2D_ERR_CUDA;
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
+    return CONV2D_OK;
 }
 
 // Length of the segments by estimated time (all of them give the same bits: an output's additions run over (c, r, s) in

@@ -44,9 +44,9 @@ conv2d_status_t launch_direct_fallback(const float* x, const float* w, float* y,
     const int threads = 256;
     long long blocks = (total + threads - 1) / threads;
     if (blocks > (long long)sm_count() * 64) blocks = (long long)sm_count() * 64;
-    direct_kernel<<<(unsigned)blocks, threads, 0, stream>>>(x, w, y, sh.C, sh.H, sh.W, sh.K, sh.R, sh.S, sh.P, sh.Q, total);
+    if (launch_ordinary(direct_kernel, dim3((unsigned)blocks), dim3(threads), 0, stream, x, w, y, sh.C, sh.H, sh.W, sh.K, sh.R, sh.S, sh.P, sh.Q, total) != cudaSuccess) return CONV2D_ERR_CUDA;
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
+    return CONV2D_OK;
 }
 
 namespace {

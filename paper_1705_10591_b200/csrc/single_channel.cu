@@ -241,9 +241,9 @@ conv2d_status_t launch_unit(const float* x, const float* w, float* y, const Shap
     if (raise_smem_limit(reinterpret_cast<const void*>(kern), smem, smem_done) != cudaSuccess) return CONV2D_ERR_CUDA;
     dim3 grid((sh.Q + TW - 1) / TW, (sh.P + tile_h - 1) / tile_h, sh.N);
     const int vec_st = (sh.Q % UNIT == 0) && (reinterpret_cast<uintptr_t>(y) % 16 == 0);
-    kern<<<grid, kThreads, smem, stream>>>(x, w, y, sh.H, sh.W, sh.K, sh.P, sh.Q, tile_h, vec_st);
+    if (launch_ordinary(kern, grid, dim3(kThreads), smem, stream, x, w, y, sh.H, sh.W, sh.K, sh.P, sh.Q, tile_h, vec_st) != cudaSuccess) return CONV2D_ERR_CUDA;
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
+    return CONV2D_OK;
 }
 
 // Packed-FMA variant.  B200 issues fp32 FMAs at full rate only as two-wide packed instructions
@@ -403,7 +403,7 @@ conv2d_status_t launch_packed(const float* x, const float* w, float* y, const Sh
     if (launch_pdl(kern, grid, dim3(kThreads), smem, stream, x, w, y, sh.H, sh.W, sh.K, sh.P, sh.Q, tile_h, vec_ld, vec_st) != cudaSuccess)
         return CONV2D_ERR_CUDA;
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
+    return CONV2D_OK;
 }
 
 template <int R, int S, int TR, int WSRC>
@@ -419,9 +419,9 @@ conv2d_status_t launch_instance(const float* x, const float* w, float* y, const 
     dim3 grid((sh.Q + kTileW - 1) / kTileW, (sh.P + tile_h - 1) / tile_h, sh.N);
     const int vec_ld = (sh.W % 4 == 0) && (reinterpret_cast<uintptr_t>(x) % 16 == 0);
     const int vec_st = (sh.Q % 4 == 0) && (reinterpret_cast<uintptr_t>(y) % 16 == 0);
-    kern<<<grid, kThreads, smem, stream>>>(x, w, y, sh.H, sh.W, sh.K, sh.P, sh.Q, tile_h, vec_ld, vec_st);
+    if (launch_ordinary(kern, grid, dim3(kThreads), smem, stream, x, w, y, sh.H, sh.W, sh.K, sh.P, sh.Q, tile_h, vec_ld, vec_st) != cudaSuccess) return CONV2D_ERR_CUDA;
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
+    return CONV2D_OK;
 }
 
 // Wide persistent variant for large images.
@@ -622,7 +622,7 @@ conv2d_status_t launch_rows(const float* x, const float* w, float* y, const Shap
                    (unsigned)env_int("CONV2D_B200_SC_MAX_POLLS", 1 << 22), env_int("CONV2D_B200_SC_TEST_SHORT_ITEM", -1)) != cudaSuccess)
         return CONV2D_ERR_CUDA;
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
+    return CONV2D_OK;
 }
 
 // Wide persistent variant for rows that are only 8-byte aligned (Q = 2 mod 4, e.g. 3 x 3 or 7 x 7 taps on
@@ -817,7 +817,7 @@ conv2d_status_t launch_rows_shift(const float* x, const float* w, float* y, cons
                    (unsigned)env_int("CONV2D_B200_SC_MAX_POLLS", 1 << 22), env_int("CONV2D_B200_SC_TEST_SHORT_ITEM", -1)) != cudaSuccess)
         return CONV2D_ERR_CUDA;
     count_launch();
-    return cudaGetLastError() == cudaSuccess ? CONV2D_OK : CONV2D_ERR_CUDA;
+    return CONV2D_OK;
 }
 
 // 3 x 3 and 5 x 5 filters on the kernels of this file.
