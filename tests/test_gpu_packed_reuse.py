@@ -8,7 +8,7 @@ import pytest
 LAYERS = [
     ((64, 64, 3, 3), [(2, 56, 56, 1), (2, 55, 55, 1), (1, 124, 128, 0), (8, 124, 128, 0), (1, 112, 112, 1), (2, 128, 128, 1), (3, 33, 47, 0), (2, 40, 260, 0)]),
     ((17, 50, 3, 3), [(3, 30, 33, 1), (3, 30, 32, 1), (1, 12, 12, 0), (40, 12, 13, 0)]),
-    ((48, 16, 19, 2), [(2, 40, 12, 0), (2, 41, 13, 0), (1, 24, 21, 1)]),                   # 38 pairs of tap and channel block
+    ((48, 16, 19, 2), [(20, 40, 12, 0), (20, 41, 13, 0), (1, 24, 21, 1)]),                   # 38 pairs of tap and channel block
     ((5, 33, 4, 3), [(2, 20, 24, 0), (2, 21, 25, 0), (2, 20, 24, 1)]),
     ((64, 96, 3, 3), [(2, 20, 24, 0), (2, 21, 25, 1), (1, 90, 130, 1)]),                   # wholly stacked
     ((130, 40, 3, 3), [(2, 20, 24, 0), (2, 21, 25, 1), (1, 90, 130, 1)]),
