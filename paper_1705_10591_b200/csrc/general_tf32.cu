@@ -226,7 +226,10 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
                                      general_tc_kernel<false, false, false, false, false, false, true>, general_tc_kernel<true, false, false, false, false, false, true>,
                                      general_tc_kernel<false, true, false, false, false, false, true>, general_tc_kernel<true, true, false, false, false, false, true>,
                                      general_tc_kernel<false, false, true, false, false, false, true>, general_tc_kernel<true, false, true, false, false, false, true>,
-                                     general_tc_kernel<false, false, false, false, false, true, true>};
+                                     general_tc_kernel<false, false, false, false, false, true, true>,
+                                     general_tc_kernel<false, false, false, false, false, true, false, 1>, general_tc_kernel<false, false, false, false, true, true, false, 2>,
+                                     general_tc_kernel<false, false, false, true, false, true, false, 1>,  general_tc_kernel<false, false, false, true, false, true, false, 2>,
+                                     general_tc_kernel<false, false, false, false, false, true, true, 1>,  general_tc_kernel<false, false, false, false, false, true, true, 2>};
         for (auto k : all)
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess)
             return CONV2D_ERR_CUDA;
@@ -299,15 +302,23 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     // Programmatic dependent launch: the kernel's set-up (barriers, tensor-memory allocation) overlaps the
     // tail of whatever kernel precedes it on the stream; it waits for that kernel before it touches global memory.
     const bool fold = p.fold_r * p.fold_s > 1;
+    // Single pixels of virtual images, at most 64 filters: loads come before the wait where every stage has a producer group of
+    // its own, which otherwise could not load until its one stage is free; with a stage to spare the groups keep closer together when
+    // they wait first.  Loads first against wait first, 660 random layers: stacked taps 0.94 (0.83 to 1.03) and 1.05 (0.99 to 1.14),
+    // others of 6 to 9 taps 0.96 and 1.02, of fewer 1.00 and 1.03.
+    const bool pix = p.virt && !a.quad && !a.quad2, ahead = a.pgroups == p.a_stages;
     CUtensorMap pair_map{};
     if (p.pair_compact && !pair_map_of(&pair_map, wp, p.cblks * sh.R * sh.S)) return CONV2D_ERR_UNSUPPORTED;
     void (*kernel)(KernelArgs, CUtensorMap);
     if (p.n_tile == 64 && !p.pair_taps) {
-        if (p.virt) kernel = general_tc_kernel<false, false, false, false, false, true, true>;
+        if (pix) kernel = ahead ? general_tc_kernel<false, false, false, false, false, true, true, 2> : general_tc_kernel<false, false, false, false, false, true, true, 1>;
+        else if (p.virt) kernel = general_tc_kernel<false, false, false, false, false, true, true>;
         else if (p.patch_w) kernel = b16 ? general_tc_kernel<true, false, true, false, false, false, true> : general_tc_kernel<false, false, true, false, false, false, true>;
         else if (fold) kernel = b16 ? general_tc_kernel<true, true, false, false, false, false, true> : general_tc_kernel<false, true, false, false, false, false, true>;
         else kernel = b16 ? general_tc_kernel<true, false, false, false, false, false, true> : general_tc_kernel<false, false, false, false, false, false, true>;
     }
+    else if (pix && p.pair_taps) kernel = ahead ? general_tc_kernel<false, false, false, true, false, true, false, 2> : general_tc_kernel<false, false, false, true, false, true, false, 1>;
+    else if (pix) kernel = general_tc_kernel<false, false, false, false, false, true, false, 1>;
     else if (p.virt) kernel = p.pair_taps ? general_tc_kernel<false, false, false, true, false, true> : general_tc_kernel<false, false, false, false, false, true>;
     else if (p.pair_taps && p.patch_w) kernel = b16 ? general_tc_kernel<true, false, true, true> : general_tc_kernel<false, false, true, true>;
     else if (p.pair_taps) kernel = b16 ? general_tc_kernel<true, false, false, true> : general_tc_kernel<false, false, false, true>;
@@ -315,7 +326,8 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
     else if (fold) kernel = b16 ? general_tc_kernel<true, true, false, false> : general_tc_kernel<false, true, false, false>;
     else kernel = b16 ? general_tc_kernel<true, false, false, false> : general_tc_kernel<false, false, false, false>;
     if (p.cluster) {
-        kernel = p.virt ? general_tc_kernel<false, false, false, false, true, true>
+        kernel = pix ? general_tc_kernel<false, false, false, false, true, true, false, 2>
+               : p.virt ? general_tc_kernel<false, false, false, false, true, true>
                : b16 ? general_tc_kernel<true, false, false, false, true> : general_tc_kernel<false, false, false, false, true>;
         if (launch_pdl_cluster(kernel, dim3((unsigned)p.grid), dim3(kThreads), p.smem_bytes, stream, 2u, a, pair_map) != cudaSuccess)
             return CONV2D_ERR_CUDA;

@@ -453,12 +453,15 @@ __device__ __noinline__ void load_pairs(unsigned char* dst, const float* bank, c
 // VIRT: zero padding and strides on virtual images (staged_pixel_virtual); flat addressing, fp32 operands.
 // M64: at most 64 filters without stacked taps (the write-back takes two blocks at a time; in instances of its own, since as
 // run-time code it cost the 128-filter layers 1 %: more spills in roles that are at the register limit).
-template <bool B16, bool FOLD, bool PATCH, bool STACK, bool CLUSTER = false, bool VIRT = false, bool M64 = false>
+// PIX (virtual images): 0: the producers load quads of pixels; 1, 2: single pixels, with 2 before they wait for the stage.  Instances of their
+// own: together in one, the quads' code made the single pixels slower (48 x 384 x 46 x 31, 18 of 3 x 3, padding 1: 88 us, 80 apart; 32 x 64 x
+// 55 x 55, 64 of 3 x 3, padding 1: 30.6 and 30.1; 50 x 175 x 52 x 52, 352 of 3 x 3, stride 3: 172 and 165).
+template <bool B16, bool FOLD, bool PATCH, bool STACK, bool CLUSTER = false, bool VIRT = false, bool M64 = false, int PIX = 0>
 __global__ void __launch_bounds__(kThreads, 1)
 general_tc_kernel(const KernelArgs a, const __grid_constant__ CUtensorMap pair_map)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    constexpr bool kEarlyLoads = B16 || STACK || M64 || CLUSTER;      // producers load before they wait for the stage (see there)
+    constexpr bool kEarlyLoads = PIX == 2 || (PIX == 0 && (B16 || STACK || M64 || CLUSTER));      // producers load before they wait for the stage (see there)
     constexpr bool kTurn = STACK || M64;                  // quad producers: lanes start with different pixels (see there)
     const uint32_t a_block_bytes = (uint32_t)kCB * a.cstride * 4 * (VIRT && a.quad2 && !a.mixed ? 2 : 1);       // one channel block of a stage
     const uint32_t a_stage_bytes = a_block_bytes * (uint32_t)a.cbg;
@@ -774,14 +777,13 @@ general_tc_kernel(const KernelArgs a, const __grid_constant__ CUtensorMap pair_m
                 const uint32_t a_phase = next_phase;
                 if (++next_as == a.a_stages) { next_as = 0; next_phase ^= 1u; }
                 if ((kstage & (a.pgroups - 1)) != gid) continue;         // pgroups is 1, 2 or 4
-                // The stage is waited for when the first loads are under way: they need registers only, and a ring of two stages
+                // The stage is waited for when the first loads are under way (kEarlyLoads): they need registers only, and a ring of two stages
                 // has no time to spare for their latency (with the turned stores below 32 x 64 x 56 x 56, 64 of 3 x 3, padding 1: 27.7 -> 23.1 us;
                 // 64 x 128 x 32 x 32, 128 of 3 x 3 in bf16 24.8 -> 23.4).  Of 128 fp32 filters in blocks of their own the wait comes first
                 // (32 x 128 x 56 x 56, stride 2 30.5 us, 31.9 with the loads first; 28 x 45 x 100 x 100, 176 of 3 x 3 110 and 122).
-                if (!kEarlyLoads && !mbar_wait_bounded(&a_empty[as], a_phase ^ 1u, abort_flag, a.max_polls)) { alive = false; break; }
-                bool waited = false;
+                bool waited = !kEarlyLoads;
+                if (waited && !mbar_wait_bounded(&a_empty[as], a_phase ^ 1u, abort_flag, a.max_polls)) { alive = false; break; }
                 auto stage_free = [&]() {
-                    if (!kEarlyLoads) return true;
                     if (!waited) {
                         waited = true;
                         if (!mbar_wait_bounded(&a_empty[as], a_phase ^ 1u, abort_flag, a.max_polls)) alive = false;
@@ -792,7 +794,7 @@ general_tc_kernel(const KernelArgs a, const __grid_constant__ CUtensorMap pair_m
                 int gr = grp + ii.rot;
                 if (gr >= ii.n_groups) gr -= ii.n_groups;
                 gr += ii.g_begin;
-                if (VIRT && a.quad2) {
+                if (VIRT && !PIX && a.quad2) {
                     // Stride 2: four adjacent pixels of an image row are two virtual pixels of both phases of that row.
                     const int qn = a.npix >> 1;
                     for (int i = wtid; i < qn * a.cbg; i += nthr) {
@@ -848,7 +850,7 @@ general_tc_kernel(const KernelArgs a, const __grid_constant__ CUtensorMap pair_m
                             }
                         }
                     }
-                } else if (!B16 && !FOLD && a.quad) {
+                } else if (!B16 && !FOLD && !PIX && (VIRT || a.quad)) {
                     // H*W a multiple of 4: a thread fetches 4 adjacent pixels of each of the 16 channels with
                     // 128-bit loads (a quarter of the load instructions, which otherwise crowd the SM's memory
                     // pipeline that the MMA instructions pass through as well) and writes four 16-channel units.
