@@ -58,6 +58,7 @@ struct Plan {
     int fold_r, fold_s;  // taps folded into the channel dimension: 1 or R rows, 1 or S columns
     int patch_w, patch_tw, patch_rows, patch_cols;   // patch addressing (patch_w = 0: flat pixel run), see ItemGeom
     int crop, crop_items;   // flat addressing: 1 = items end with their image, crop_items of them each
+    int may_crop;           // 1: such items were or can be considered
     int taps;
     int a_stages;
     int b_stages;
@@ -105,7 +106,8 @@ size_t smem_need(int a_stages, int npix, int n_tile, int b_stages, int tps, int 
 
 // b16: the operands are 16-bit floats, bf16 or fp16 (16-byte unit = 8 channels, 32 channels per staged block, K = 16 per MMA); the
 // byte layout of every stage is the same as for TF32 (16 channels of 4 bytes).
-Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool allow_compact = true, bool virt = false, bool narrow = false)
+Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool allow_compact = true, bool virt = false, bool narrow = false,
+                           bool allow_crop = true)
 {
     Plan p{};
     p.ok = false;
@@ -272,7 +274,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     }
     if (virt) p.staged_ratio = (448.0 + flat_halo) / 448.0 * ((double)sh.H * sh.W) / ((double)sh.P * sh.Q);
     if (padded && !p.patch_w) return p;
-    if (p.pair_compact && p.patch_w && compact_mode != 1) return plan_with_patch_width(shape, b16, want_patch_w, false, virt, narrow);
+    if (p.pair_compact && p.patch_w && compact_mode != 1) return plan_with_patch_width(shape, b16, want_patch_w, false, virt, narrow, allow_crop);
     p.ovl = (p.pair_taps && !p.patch_w) ? 4 : 0;
     const long long halo = p.patch_w ? (long long)(r_eff - 1) * p.patch_w + (s_eff - 1) : flat_halo;
     // work items along the pixels for an item of px pixels (0: px is not possible in this mode)
@@ -330,7 +332,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         }
     }
 
-    if (p.pair_compact && !p.resident) return plan_with_patch_width(shape, b16, want_patch_w, false, virt, narrow);    // compact stacking needs the resident bank
+    if (p.pair_compact && !p.resident) return plan_with_patch_width(shape, b16, want_patch_w, false, virt, narrow, allow_crop);    // compact stacking needs the resident bank
     if (!p.resident) {
         // Streamed filters.  Measured: all SMs together draw filter stages from L2 at no more than
         // ~5-6 TB/s, i.e. a 8 KB stage costs ~120 cycles on top of the MMAs that consume it unless it is
@@ -342,14 +344,16 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         const int forced_px = env_int("CONV2D_B200_TF32_TILE_PX", 0);
         const bool ksplit_allowed = env_int("CONV2D_B200_TF32_KSPLIT", 1) != 0;
         int best_px = 0;
-        double best_cost = 0;
+        double best_cost = 0, flat_bound = 0;          // (flat_...: of the best items of the whole run)
+        bool flat_adds = false;
         // Any multiple of 32 pixels per item: the item size follows from the pixel count and the 148 SMs
         // (64 x 32 x 32 pixels: 448 per item = 147 items in one round, where 512 would occupy 128 SMs).
         // One or two MMAs of equal width cover the item per K step; an MMA narrower than 128 pixels is
         // bound by its ~64-cycle issue cost.
         long long best_items = 0;
         // (CONV2D_B200_TF32_CROP = 0: never, 2: wherever they fit)
-        const int crop_mode = p.patch_w || p.fold_r * p.fold_s != 1 || sh.C < kCB || forced_px ? 0 : env_int("CONV2D_B200_TF32_CROP", 1);
+        p.may_crop = !(p.patch_w || p.fold_r * p.fold_s != 1 || sh.C < kCB || forced_px);
+        const int crop_mode = !p.may_crop || !allow_crop ? 0 : env_int("CONV2D_B200_TF32_CROP", 1);
         auto consider = [&](int px, int groups, long long px_items, long long npix, int crop, int crop_items) {
             if (npix > 16000 || smem_need(2, (int)npix, p.n_tile, 2, 1, stage_blocks) > kLimit || px_items <= 0) return;
             const long long items = px_items * p.n_blocks;
@@ -366,9 +370,18 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
             if (nbuf == 1 && rounds >= 3)
                 cost += (double)(rounds - 2) * 0.75 * (px / 32.0) * (p.n_tile >= 128 ? 2000.0 : 1200.0);
             // (items that leave half of the SMs idle are split in two along the channels further down)
-            if (items * 2 <= sms && p.cblks >= 2 && ksplit_allowed) cost = 0.5 * tile_time + writeback;
-            const bool forced = crop_mode >= 2 && crop != 0 && p.crop == 0;
-            if (best_px != 0 && !forced && !(cost < (crop != p.crop ? 0.96 : 1.0) * best_cost)) return;
+            const bool split = items * 2 <= sms && p.cblks >= 2 && ksplit_allowed;
+            if (split) cost = 0.5 * tile_time + writeback;
+            // Items of an image against those of the whole run: also counted are the zero-fill and the adds of a contraction that is
+            // split without a cluster (9000 cycles), and the producers (6 cycles per staged pixel and channel block) must
+            // not become what sets the pace (128 x 256 x 11 x 139, 6 of 3 x 3: 441 items of 448 pixels 140 us, 640 of 256 175 us).
+            const bool adds = split && (p.n_tile != 128 || p.pair_taps);
+            const double turns = split ? 0.5 : (double)rounds, staging = turns * 6.0 * npix * p.cblks;
+            const double bound = (turns * tile_time > staging ? turns * tile_time : staging) + (adds ? 9000.0 : 0.0);
+            if (crop && adds && !flat_adds) cost += 9000.0;
+            if (best_px != 0 && !(crop_mode >= 2 && crop != p.crop) &&
+                (!(cost < (crop != p.crop ? 0.96 : 1.0) * best_cost) || (crop && crop_mode < 2 && staging > flat_bound))) return;
+            if (!crop) { flat_adds = adds; flat_bound = bound; }
             best_px = px;
             best_cost = cost;
             p.cost = cost;
@@ -514,20 +527,29 @@ bool patches_beat_virtual(const Plan& v, const Plan& patch, const Shape& sh)
 // where both take two rounds of equal items).
 Plan make_plan(const Shape& sh, bool b16 = false)
 {
+    // (the choice between virtual images, their widths and patches is made between plans without cropped items: with them the
+    // estimates took virtual images for layers that patches do faster, 128 x 70 x 13 x 151, 32 of 4 x 4, padding 2: 93 -> 126 us)
+    auto cropped = [&](const Plan& p, bool narrow) {
+        return p.ok && p.may_crop ? plan_with_patch_width(sh, b16, 0, true, true, narrow) : p;
+    };
     if (sh.stride > 1) {
         // Rows of a multiple of four columns allow 128-bit stores; where two columns less let the busiest block do a tenth
         // less (28 columns of output need 30: 145 items of 192 pixels instead of 133 of 224), pairs are the better cut.
-        const Plan p = plan_with_patch_width(sh, b16, 0, true, true);
-        if (!p.ok || sh.stride != 2 || env_int("CONV2D_B200_TF32_NARROW", 1) == 0) return p;
-        const Plan q = plan_with_patch_width(sh, b16, 0, true, true, true);
-        return q.ok && q.makespan < 0.9 * p.makespan ? q : p;
+        Plan p = plan_with_patch_width(sh, b16, 0, true, true, false, false);
+        bool narrow = false;
+        if (p.ok && sh.stride == 2 && env_int("CONV2D_B200_TF32_NARROW", 1) != 0) {
+            const Plan q = plan_with_patch_width(sh, b16, 0, true, true, true, false);
+            narrow = q.ok && q.makespan < 0.9 * p.makespan;
+            if (narrow) p = q;
+        }
+        return cropped(p, narrow);
     }
     Plan best = plan_with_patch_width(sh, b16, 0);
     const int mode = env_int("CONV2D_B200_TF32_VIRT", 1);                 // 0 never, 1 by the rule, 2 always
     if (mode != 0 && (sh.pad_h != 0 || sh.pad_w != 0)) {
         // Padding: virtual images, unless their rows are so wide that patches stage far fewer pixels (and see above).
-        const Plan v = plan_with_patch_width(sh, b16, 0, true, true);
-        if (v.ok && (mode == 2 || !best.ok || !(v.staged_ratio > 1.75 * best.staged_ratio || patches_beat_virtual(v, best, sh)))) return v;
+        const Plan v = plan_with_patch_width(sh, b16, 0, true, true, false, false);
+        if (v.ok && (mode == 2 || !best.ok || !(v.staged_ratio > 1.75 * best.staged_ratio || patches_beat_virtual(v, best, sh)))) return cropped(v, false);
     }
     if (!best.ok || !best.patch_w || env_int("CONV2D_B200_TF32_PATCH_W", 0) != 0) return best;
     const int first = best.patch_w;
