@@ -69,7 +69,11 @@ typedef enum {
 enum {
     /* The workspace already holds the filters of this exact call (same w contents,
        K, C, R, S and algorithm) in the kernel's internal order, left there by an
-       earlier call: skip the re-ordering launch. */
+       earlier call: skip the re-ordering launch.  The number and size of the images
+       may be others than in that call, except with 1 x 1 filters (one order for H*W
+       a multiple of 4, another for the rest) and with strided layers whose windows do
+       not overlap (R, S <= stride: the order depends on the images).  Padding and
+       stride belong to the layer: the same in both calls. */
     CONV2D_FLAG_WEIGHTS_PACKED = 1u
 };
 
@@ -210,7 +214,8 @@ conv2d_status_t conv2d_fwd_general_padded(const float* x, const float* w, float*
  * the tensor cores with operands rounded to the nearest TF32 either way.
  * 1 <= stride <= 8.  Workspace from conv2d_fwd_strided_workspace_size; required, 16-byte aligned, status
  * block first; it has room for the rewritten image and filters whether or not the call needs them.  With
- * CONV2D_FLAG_WEIGHTS_PACKED the rewritten filters of the previous call are reused too.
+ * CONV2D_FLAG_WEIGHTS_PACKED the rewritten filters of the previous call are reused too, which must have had images of the
+ * same number and size where the call rewrites them.
  * algo is AUTO, FFMA or TF32; N * C must not exceed 65535 (CONV2D_ERR_UNSUPPORTED otherwise, checked before
  * anything is enqueued).
  */

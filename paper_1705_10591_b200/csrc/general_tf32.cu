@@ -193,9 +193,9 @@ conv2d_status_t launch_tensor_core(const void* x_any, const void* w_any, float* 
             threads = threads < 128 ? 128 : (threads > 1024 ? 1024 : threads);
             launched = b16 ? launch_pdl(repack_filters_tiled_kernel<unsigned short, 8>, grid, dim3(threads), tile_bytes, stream,
                                         static_cast<const unsigned short*>(w_any), reinterpret_cast<unsigned short*>(wp), status, sh.K, sh.C,
-                                        all_taps, bank.rows, bank_blocks, sh.S, 1, 0)
+                                        all_taps, bank.rows, bank_blocks, sh.S, 1)
                            : launch_pdl(repack_filters_tiled_kernel<float, 4>, grid, dim3(threads), tile_bytes, stream, w, wp, status, sh.K, sh.C,
-                                        all_taps, bank.rows, bank_blocks, sh.S, p.phases > 1 ? sh.stride : 1, p.ext);
+                                        all_taps, bank.rows, bank_blocks, sh.S, p.phases > 1 ? sh.stride : 1);
         } else {
             const dim3 grid((unsigned)blocks, tap_rows);
             launched = b16 ? launch_pdl(repack_filters_kernel<unsigned short, 8>, grid, dim3(256), 0, stream,

@@ -500,11 +500,12 @@ general_tc_kernel(const KernelArgs a, const __grid_constant__ CUtensorMap pair_m
         for (int t = tid; t < a.R * a.S; t += kThreads) {
             const int r = t / a.S, sx = t - r * a.S + a.ext, r2 = r / a.st, s2 = sx / a.st;
             if (a.quad2) {
-                // taps of column phase 1 read the second 16-channel block of the channel block
+                // taps of column phase 1 read the second 16-channel block of the channel block (the bank has those in even
+                // columns of the filter first, in whichever phase `ext` puts them)
                 const int pa = r - r2 * a.st, pb = sx - s2 * a.st, rows = (a.R - pa + 1) / 2;
-                const int cols0 = (a.S + a.ext + 1) / 2 - a.ext, cols1 = a.S - cols0;
-                const int base = (pa * (a.R / 2) + min(pa, a.R % 2)) * a.S + (pb ? rows * cols0 : 0);
-                tap_shift[base + r2 * (pb ? cols1 : cols0) + (pb ? s2 : s2 - a.ext)] =
+                const int odd = (sx - a.ext) & 1, even_cols = (a.S + 1) / 2;
+                const int base = (pa * (a.R / 2) + min(pa, a.R % 2)) * a.S + (odd ? rows * even_cols : 0);
+                tap_shift[base + r2 * (odd ? a.S / 2 : even_cols) + ((sx - a.ext) >> 1)] =
                     (uint32_t)(r2 * a.row_pitch + s2) + (pb ? (uint32_t)(kChunks * a.cstride) : 0u);
                 continue;
             }

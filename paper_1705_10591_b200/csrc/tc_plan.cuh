@@ -129,8 +129,18 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
             // Stride 2 with whole quads of columns: the zeros in front of a row are a multiple of four columns, so that four
             // adjacent pixels of the image are two virtual pixels of both phases of a row.  The taps then start `ext`
             // columns into their phases, and `shift0` virtual pixels further on.
-            p.quad2 = st == 2 && sh.W % 4 == 0 && sh.S >= 2 && sh.R >= 2 && env_int("CONV2D_B200_TF32_QUAD", 1) != 0 ? 1 : 0;
-            p.off_w = p.quad2 ? (sh.pad_w + 3) / 4 * 4 : sh.pad_w;
+            // Channel blocks: all phases of a 16-channel block after one another, each with its own taps -- or, with few
+            // channels, the phases of every channel as staged channels with all ceil(R/st) x ceil(S/st) taps (zero filters
+            // where a phase has none), where that takes fewer MMAs: 3 channels, 7 x 7, stride 2: 16 pairs instead of 49.
+            // The taps of such staged channels lie by `ext`, which therefore follows from the padding whether the rows are whole quads or not:
+            // filters packed for one width serve the others.
+            const bool two = st == 2 && sh.S >= 2 && sh.R >= 2;
+            const int shifted = two ? sh.pad_w % 2 : 0;
+            const long long apart = (long long)((sh.C + kCB - 1) / kCB) * sh.R * sh.S;
+            const long long together = ((long long)sh.C * st * st + kCB - 1) / kCB * ((sh.R + st - 1) / st) * ((sh.S + shifted + st - 1) / st);
+            p.mixed = together < apart ? 1 : 0;
+            p.quad2 = two && sh.W % 4 == 0 && env_int("CONV2D_B200_TF32_QUAD", 1) != 0 ? 1 : 0;
+            p.off_w = p.quad2 ? (sh.pad_w + 3) / 4 * 4 : p.mixed ? sh.pad_w + shifted : sh.pad_w;
             p.ext = (p.off_w - sh.pad_w) % st;
             p.shift0 = (p.off_w - sh.pad_w) / st;
             p.virt_h = sh.P + (sh.R + st - 1) / st - 1;
@@ -186,15 +196,8 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     const int r_eff = st > 1 ? (sh.R + st - 1) / st : sh.R / p.fold_r, s_eff = st > 1 ? (sh.S + p.ext + st - 1) / st : sh.S / p.fold_s;
     p.cblks = (c_eff + cbc - 1) / cbc;
     if (st > 1) {
-        // Channel blocks: all phases of a 16-channel block after one another, each with its own taps -- or, with few
-        // channels, the phases of every channel as staged channels with all ceil(R/st) x ceil(S/st) taps (zero filters
-        // where a phase has none), where that takes fewer MMAs: 3 channels, 7 x 7, stride 2: 16 pairs instead of 49.
-        const long long apart = (long long)p.cblks * sh.R * sh.S;
-        const long long together = ((long long)sh.C * st * st + cbc - 1) / cbc * r_eff * s_eff;
-        if (together < apart) {
-            p.mixed = 1;
+        if (p.mixed) {
             p.phases = p.phase_cols = 1;
-            if (st != 2) p.quad2 = 0;
             p.cblks = (int)(((long long)sh.C * st * st + cbc - 1) / cbc);
         } else {
             // (with quad2 the two phases of a row are one block of 32 staged channels with the taps of both)

@@ -99,7 +99,7 @@ __global__ void repack_filters_kernel(const T* __restrict__ w, T* __restrict__ w
 // 8 filters x EPC elements (128 bytes with fp32) per (tap, chunk): both sides coalesced.
 template <typename T, int EPC>
 __global__ void repack_filters_tiled_kernel(const T* __restrict__ w, T* __restrict__ wp, unsigned* __restrict__ status,
-                                            int K, int C, int taps, int n_tile, int cblks, int S, int st, int ext)
+                                            int K, int C, int taps, int n_tile, int cblks, int S, int st)
 {
     extern __shared__ __align__(16) unsigned char repack_smem[];
     T* tile = reinterpret_cast<T*>(repack_smem);                 // [8][cpb * taps]
@@ -162,11 +162,9 @@ __global__ void repack_filters_tiled_kernel(const T* __restrict__ w, T* __restri
         }
         int tt = t;                                       // place of the tap in the bank
         if (st > 1) {                                     // grouped by phase (r % st, s % st), see phase_of
-            const int r = t / S, s = t - r * S + ext, R = taps / S, pa = r % st, pb = s % st, end = S + ext;
-            const int first = pb < ext ? 1 : 0;
-            const int rows = (R - pa + st - 1) / st, cols = (end - pb + st - 1) / st - first;
-            tt = (pa * (R / st) + min(pa, R % st)) * S + rows * (pb * (end / st) + min(pb, end % st) - min(pb, ext))
-               + (r / st) * cols + s / st - first;
+            const int r = t / S, s = t - r * S, R = taps / S, pa = r % st, pb = s % st;
+            const int rows = (R - pa + st - 1) / st, cols = (S - pb + st - 1) / st;
+            tt = (pa * (R / st) + min(pa, R % st)) * S + rows * (pb * (S / st) + min(pb, S % st)) + (r / st) * cols + s / st;
         }
         *reinterpret_cast<uint4*>(dst + (((size_t)tt * kChunks + chunk) * n_tile + f0 + kk) * EPC) = v;
     }

@@ -22,13 +22,16 @@ def _values(shape, seed):
     return torch.empty(shape, device="cuda").normal_(generator=gen)
 
 
-def _call(x, w, pad, ws, flags):
+def _call(x, w, pad, ws, flags, stride=1):
     import torch
     import paper_1705_10591_b200 as lib
     (N, C, H, W), (K, _, R, S) = x.shape, w.shape
-    y = torch.full((N, K, H + 2 * pad - R + 1, W + 2 * pad - S + 1), float("nan"), device="cuda")
+    y = torch.full((N, K, (H + 2 * pad - R) // stride + 1, (W + 2 * pad - S) // stride + 1), float("nan"), device="cuda")
     stream = torch.cuda.current_stream().cuda_stream
-    if pad:
+    if stride > 1:
+        lib.conv2d_fwd_general_strided(x.data_ptr(), w.data_ptr(), y.data_ptr(), N, C, H, W, K, R, S, pad, pad, stride, lib.ALGO_TF32,
+                                       ws.data_ptr(), ws.numel(), flags, stream)
+    elif pad:
         lib.conv2d_fwd_general_padded(x.data_ptr(), w.data_ptr(), y.data_ptr(), N, C, H, W, K, R, S, pad, pad, lib.ALGO_TF32,
                                       ws.data_ptr(), ws.numel(), flags, stream)
     else:
@@ -54,6 +57,32 @@ def test_packed_filters_serve_other_images(layer, images):
         for x, im, y in zip(xs, images, expect):
             # (a contraction split between blocks that add into y: two sums in any order give the same bits)
             assert torch.equal(_call(x, w, im[3], ws, lib.FLAG_WEIGHTS_PACKED), y), (packer, im)
+
+
+# K, C, R, S, stride, padding; then N, H, W: rows of whole quads and others
+STRIDED = [
+    ((70, 33, 3, 3, 2, 1), [(2, 20, 24), (2, 21, 25), (3, 18, 27), (1, 40, 132)]), ((64, 48, 5, 5, 2, 1), [(2, 20, 24), (2, 21, 26)]),
+    ((40, 20, 4, 4, 2, 1), [(2, 20, 24), (2, 21, 25)]), ((40, 20, 2, 3, 2, 0), [(2, 20, 24), (2, 21, 25)]),
+    ((64, 3, 7, 7, 2, 3), [(2, 32, 32), (2, 33, 33), (1, 50, 46)]), ((33, 3, 4, 4, 2, 1), [(2, 32, 32), (2, 33, 33)]),
+    ((20, 4, 3, 2, 2, 1), [(2, 20, 24), (2, 21, 25)]), ((20, 17, 5, 4, 3, 1), [(2, 20, 24), (2, 21, 25)]),
+]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("layer,images", STRIDED)
+def test_packed_filters_of_strided_layers_serve_other_images(layer, images):
+    import torch
+    import paper_1705_10591_b200 as lib
+    K, C, R, S, stride, pad = layer
+    w = _values((K, C, R, S), 11)
+    size = max(lib.conv2d_fwd_strided_workspace_size(N, C, H, W, K, R, S, pad, pad, stride, lib.ALGO_TF32) for N, H, W in images)
+    xs = [_values((N, C, H, W), 12 + i) for i, (N, H, W) in enumerate(images)]
+    expect = [_call(x, w, pad, torch.zeros(size, dtype=torch.uint8, device="cuda"), 0, stride) for x in xs]
+    for i, packer in enumerate(images):
+        ws = torch.zeros(size, dtype=torch.uint8, device="cuda")
+        _call(xs[i], w, pad, ws, 0, stride)
+        for x, im, y in zip(xs, images, expect):
+            assert torch.equal(_call(x, w, pad, ws, lib.FLAG_WEIGHTS_PACKED, stride), y), (packer, im)
 
 
 @pytest.mark.parametrize("algo", [2, 3])
