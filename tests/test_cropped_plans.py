@@ -10,3 +10,13 @@ import pytest
 def test_cropped_items_are_taken_by_the_rule(layer, crop):
     import paper_1705_10591_b200 as lib
     assert lib.conv2d_fwd_plan_describe(*layer, lib.ALGO_TF32)["crop"] == crop
+
+
+def test_the_cropped_test_layers_take_cropped_items(monkeypatch):
+    import paper_1705_10591_b200 as lib
+    from test_gpu_cropped_images import CASES
+    monkeypatch.setenv("CONV2D_B200_TF32_CROP", "2")
+    monkeypatch.setenv("CONV2D_B200_TF32_RESIDENT", "0")
+    for case in CASES:
+        for algo in (lib.ALGO_TF32, lib.ALGO_16BIT):
+            assert lib.conv2d_fwd_plan_describe(*case, algo)["crop"] == 1, case

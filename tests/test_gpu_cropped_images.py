@@ -40,3 +40,21 @@ def test_cropped_items_on_virtual_images(oracle, monkeypatch):
         x, w = small_integers((N, C, H, W), 1705), small_integers((K, C, R, S), 1706)
         y_ref, _ = _reference(oracle, x, w, pad, pad, st)
         np.testing.assert_array_equal(run_strided(x, w, pad, pad, st, 2)[0].astype(np.float64), y_ref)
+
+
+@pytest.mark.parametrize("case", [
+    # at most 64 filters, no split: stores of quads, of pairs and of single pixels; blocks of 32 columns whose number is odd, the last one half full;
+    # more items than SMs
+    (80, 64, 16, 16, 64, 5, 5), (75, 64, 14, 14, 33, 5, 5), (80, 64, 15, 17, 64, 5, 5), (160, 64, 14, 16, 20, 5, 5), (160, 48, 14, 14, 64, 3, 3), (150, 40, 10, 18, 61, 3, 3),
+])
+def test_cropped_items_of_few_filters_exact_on_integers(oracle, monkeypatch, case):
+    import paper_1705_10591_b200 as lib
+    N, C, H, W, K, R, S = case
+    monkeypatch.setenv("CONV2D_B200_TF32_CROP", "2")
+    monkeypatch.setenv("CONV2D_B200_TF32_RESIDENT", "0")
+    x, w = small_integers((N, C, H, W), 1707), small_integers((K, C, R, S), 1708)
+    y_ref, _ = oracle.conv2d_oracle(x, w)
+    for entry, algo in (("general", 2), ("bf16", 3)):
+        plan = lib.conv2d_fwd_plan_describe(N, C, H, W, K, R, S, algo)
+        assert plan["crop"] == 1 and plan["ksplit"] == 1
+        np.testing.assert_array_equal(run_library(x, w, entry=entry, algo=algo).astype(np.float64), y_ref)

@@ -62,3 +62,57 @@ def test_calls_captured_in_a_cuda_graph_replay_correctly(oracle):
         np.testing.assert_array_equal(got, y_direct.cpu().numpy())
         if nbytes:
             lib.conv2d_get_status(ws.data_ptr(), torch.cuda.current_stream().cuda_stream)
+
+
+def test_captured_calls_whose_kernels_overlap():
+    """Calls of several kernels, each launched while the one before it ends, in a graph: an extended image, a rewritten stride, rounded
+    filters, one channel, filters packed before; after the stream has waited for another one, after a copy and after each other."""
+    import torch
+    import paper_1705_10591_b200 as lib
+
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(491)
+    N, C, H, K = 2, 24, 30, 40
+    x = torch.empty((N, C, H, H), device="cuda").normal_(generator=gen)
+    xw = torch.empty((N, 512, H, H), device="cuda").normal_(generator=gen)
+    w = torch.empty((K, C, 3, 3), device="cuda").normal_(generator=gen)
+    ww = torch.empty((K, 512, 1, 1), device="cuda").normal_(generator=gen)
+    ws = [torch.zeros(1 << 23, dtype=torch.uint8, device="cuda") for _ in range(4)]
+    ys = [torch.zeros((N, K * C, H, H), device="cuda") for _ in range(5)]
+    p, side_copy = x.data_ptr(), torch.empty_like(x)
+    size = ws[0].numel()
+    calls = [
+        lambda s: lib.conv2d_fwd_general_padded(p, w.data_ptr(), ys[0].data_ptr(), N, C, H, H, K, 3, 3, 1, 1, lib.ALGO_FFMA, ws[0].data_ptr(), size, 0, s),
+        lambda s: lib.conv2d_fwd_general_strided(p, w.data_ptr(), ys[1].data_ptr(), N, C, H, H, K, 3, 3, 1, 1, 2, lib.ALGO_FFMA, ws[1].data_ptr(), size, 0, s),
+        lambda s: lib.conv2d_fwd_general(xw.data_ptr(), ww.data_ptr(), ys[2].data_ptr(), N, 512, H, H, K, 1, 1, lib.ALGO_TF32, ws[2].data_ptr(), size, 0, s),
+        lambda s: lib.conv2d_fwd_single_channel(p, w.data_ptr(), ys[3].data_ptr(), N * C, H, H, K // 8, 3, 3, 0, 0, 0, s),
+        lambda s: lib.conv2d_fwd_general(p, w.data_ptr(), ys[4].data_ptr(), N, C, H, H, K, 3, 3, lib.ALGO_TF32, ws[3].data_ptr(), size, lib.FLAG_WEIGHTS_PACKED, s),
+    ]
+    lib.conv2d_fwd_general(p, w.data_ptr(), ys[4].data_ptr(), N, C, H, H, K, 3, 3, lib.ALGO_TF32, ws[3].data_ptr(), size, 0, 0)   # (packs)
+    torch.cuda.synchronize()
+    stream, other = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        for call in calls:
+            call(stream.cuda_stream)
+    stream.synchronize()
+    direct = [y.clone() for y in ys]
+    for order in (range(5), (4, 3, 2, 1, 0), (3, 4, 0, 2, 1)):
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            for y in ys:
+                y.zero_()
+            for i in order:
+                other.wait_stream(stream)                   # the call follows a join of two streams and a copy
+                with torch.cuda.stream(other):
+                    side_copy.copy_(x)
+                stream.wait_stream(other)
+                calls[i](stream.cuda_stream)
+            for i in order:
+                calls[i](stream.cuda_stream)
+        for y in ys:
+            y.fill_(float("nan"))
+        for _ in range(2):
+            graph.replay()
+        torch.cuda.synchronize()
+        for y, d in zip(ys, direct):
+            assert torch.equal(y, d)
