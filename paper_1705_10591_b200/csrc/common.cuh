@@ -107,11 +107,13 @@ cudaError_t launch_ordinary(void (*kernel)(KArgs...), dim3 grid, dim3 block, siz
 // Launch with programmatic stream serialization: the kernel may be scheduled while the preceding kernel on the
 // stream drains; it calls grid_dep_wait() before it touches global memory.  Without an earlier grid_dep_launch() in the preceding
 // kernel "while it drains" begins when its last block ends: the launch is hidden (64 x 64, 8 filters of 3 x 3, one channel: 4.15 ->
-// 2.8 us a call), and the blocks are spread over the SMs as ever.  With one they are placed wherever a block has ended or an SM
-// stands empty, as many as fit: right for kernels of one block per SM (packed filters, 3 % on average), wrong for many small
-// blocks (zero-extended images before the fp32 kernel, 29 x 160 x 18 x 17, 80 of 3 x 3: 96 -> 186 us), so a convolution that
-// finds its filters packed triggers early, as the next call is likely to be one, too, and one that had them re-ordered does not
-// (the re-ordering kernel of the next call: 36 x 32 x 36 x 42, 180 of 3 x 3, stride 2 21.4 -> 19.2 us without).
+// 2.8 us of the GPU's time a call), and the blocks are spread over the SMs as ever.  With one they are placed wherever a block has ended or
+// an SM stands empty, as many as fit: right for kernels of one block per SM (packed filters, 3 % on average).  A kernel that would itself trigger
+// early must not be of many small blocks (zero-extended images that do, before the fp32 kernel, 29 x 160 x 18 x 17, 80 of 3 x 3:
+// 96 -> 186 us), and a convolution triggers early only where it finds its filters packed or has none to prepare, as the next call is then
+// likely to be one, too (the re-ordering kernel of the next call otherwise: 36 x 32 x 36 x 42, 180 of 3 x 3, stride 2 21.4 -> 19.2 us without).
+// Small blocks that happen to follow such a call gain from the hidden launch all the same: a 1 x 1 layer and a zero-extended fp32 one,
+// one after the other, 49.5 us, with ordinary launches of the small blocks 51.4; of 24 such pairs of calls none is slower than with those.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args)
 {

@@ -7,8 +7,8 @@
 //   * GEMM view: M = a block of 128 (or 64) filters, N = the pixels of a work item, contraction over
 //     (channel, tap).  The accumulator block rAcc[F_T][W_T] of Algorithm 2 becomes a filters x pixels fp32
 //     tile in tensor memory (lanes = filters, columns = pixels); a work item is any multiple of 32 pixels
-//     up to 512, covered by one or two MMAs per K step.  (With the pixels as M a 128-filter problem needs
-//     twice as many instructions, and the single issuing thread is what limits the rate.)
+//     up to 512 (of 16 where items end with their image), covered by one or two MMAs per K step.  (With the
+//     pixels as M a 128-filter problem needs twice as many instructions.)
 //   * Flat addressing: pixels are numbered in one sequence j = (n*H + h)*W + w over the whole batch.  For
 //     tap (r,s) the input needed by output j is pixel j + r*W + s of the same channel, a pure shift.  Per
 //     block of channels ONE run of tile_px + (R-1)*W + (S-1) pixels is staged ("block plus halo to the
@@ -33,7 +33,7 @@
 //     (coalesced along pixels, 128-bit loads where the alignment allows), round fp32 to TF32 and write
 //     16-byte units.
 //   * Persistent blocks, one per SM, walk over the work items round-robin.  Warp roles: warp 0 streams
-//     filter stages, warp 1 (one thread) issues tcgen05.mma and owns the tensor-memory allocation, eight
+//     filter stages, warp 1 issues tcgen05.mma (one elected lane) and owns the tensor-memory allocation, eight
 //     warps stage activations (in up to four groups that fill different stages concurrently), four warps
 //     drain finished accumulators through a shared-memory transposition so that a store instruction
 //     writes adjacent outputs of one map (the coalesced write-back that Section 4.2 leaves out); for the
@@ -125,10 +125,10 @@ int describe_tensor_core_plan(const Shape& sh, bool b16, char* text, size_t text
     if (p.pair_compact) issued *= (double)p.cb_bytes / ((double)p.taps * kCB * p.n_tile * 4);    // lone taps are 64-row MMAs
     const double useful = 2.0 * out_px * sh.K * sh.C * sh.R * sh.S;
     return snprintf(text, text_bytes,
-                    "tensor_core=1 kernel=general_tc addressing=%s filters_as=%s m_rows=%d tile_px=%d px_groups=%d acc_sets=%d items=%lld grid=%d "
+                    "tensor_core=1 kernel=general_tc addressing=%s filters_as=M m_rows=%d tile_px=%d px_groups=%d acc_sets=%d items=%lld grid=%d "
                     "ksplit=%d cluster=%d resident_filters=%d stacked_taps=%d stacked_compact=%d bank=%dx%d%s fold=%dx%d patch_w=%d crop=%d smem_bytes=%zu "
                     "mma_useful_px=%.4f mma_useful_flops=%.4f",
-                    p.patch_w ? "patch" : "flat", "M", (int)rows, p.tile_px, p.px_groups, p.nbuf,
+                    p.patch_w ? "patch" : "flat", (int)rows, p.tile_px, p.px_groups, p.nbuf,
                     (long long)p.supertiles * p.n_blocks * p.ksplit, p.grid, p.ksplit, p.cluster, p.resident, p.pair_taps, p.pair_compact,
                     bank.rows, bank.taps, bank.stacked ? "s" : "", p.fold_r, p.fold_s, p.patch_w, p.crop, p.smem_bytes, out_px / cols, useful / issued);
 }

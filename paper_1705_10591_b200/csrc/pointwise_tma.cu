@@ -24,7 +24,7 @@
 // truncated, not rounded: |error| <= (2^-10 + 2^-10 + 2^-20) * sum|x*w| plus fp32 accumulation over at most 256
 // channels, (C + 1) * 2^-24 * sum|x*w|: below 1.97e-3 * sum|x*w|, inside the 2e-3 bound of CONV2D_ALGO_TF32.
 //
-// Persistent blocks, one per SM: warp 0 (one thread) issues the loads, warp 1 (one thread) the MMAs, warps 2-9
+// Persistent blocks, one per SM: warp 0 (one thread) issues the loads, warp 1 (one elected lane) the MMAs, warps 2-9
 // drain the accumulators, two per tensor-memory lane quarter.  Two accumulator sets: the write-back of item i runs
 // under the loads and MMAs of item i + 1, which is what an operation bound by memory traffic needs.
 // Work items are runs of `a_item` 32-pixel atoms of the flat atom sequence (image-major; an image has

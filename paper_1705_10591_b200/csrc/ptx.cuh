@@ -53,9 +53,9 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     return false;
 }
 
-// The warp forms below are for the warp that issues the MMAs: all 32 lanes run its loop and decide together, so that the
-// compiler sees warp-uniform values (a tcgen05.mma takes its operands from uniform registers; from the registers of one
-// diverged lane they are moved there for every instruction), and one elected lane's instructions take effect.
+// The warp forms below are for the warp that issues the MMAs: all 32 lanes run its loop and decide together, and one elected
+// lane's instructions take effect.  Measured, such a warp issues at the pipe's rate and a lane that runs the loop alone does not (see
+// the MMA loop of the general kernel); why is a guess: warp-uniform operands need no moves.
 // The lane that elect.sync picks (1 there, 0 elsewhere).
 __device__ __forceinline__ uint32_t elect_one()
 {
@@ -278,7 +278,7 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar, uint32_t elected)
                  "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
                  ::"r"(smem_u32(bar)), "r"(elected) : "memory");
 }
-// Two-SM MMAs, issued by one thread of the pair's first block.  D is 256 x N: rows 0-127 in the first block's tensor
+// Two-SM MMAs, issued by the elected lane of a warp of the pair's first block.  D is 256 x N: rows 0-127 in the first block's tensor
 // memory, rows 128-255 in the second's, N columns in both.  The descriptors are offsets that hold in both blocks:
 // each block's shared memory holds its 128 rows of A and its half of B's N rows at the same addresses.
 __device__ __forceinline__ void mma_tf32_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate, uint32_t elected)
@@ -295,7 +295,7 @@ __device__ __forceinline__ void mma_b16_pair(uint32_t d_tmem, uint64_t a_desc, u
         "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate), "r"(elected) : "memory");
 }
-// Arrives once on `bar` of this block when all two-SM MMAs issued so far by this thread have completed ...
+// Arrives once on `bar` of this block when all two-SM MMAs issued so far by the elected lane have completed ...
 __device__ __forceinline__ void mma_commit_pair(uint64_t* bar, uint32_t elected)
 {
     asm volatile("{\n\t.reg .pred e;\n\tsetp.ne.b32 e, %1, 0;\n\t"

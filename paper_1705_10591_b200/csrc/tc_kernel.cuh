@@ -427,7 +427,8 @@ __device__ __forceinline__ void issue_tap(uint32_t d, uint32_t px_lo, uint32_t f
 // The resident bank of compact stacking.  In the workspace the bank lies tap by tap, as for every layer of these filters (whether
 // they are stacked depends on the image, too); its slices of two taps are put together here, one box of the tensor
 // map (pair_map_of) each, a lane a slice.  147 KB of 64 filters of 64 x 3 x 3 arrive as early as a bank stored in slices
-// (2 x 56 x 56: 8.9 us either way); issued by one lane 0.6 us later, as 32 bulk copies of 256 bytes to a slice 10 us later.  Not inlined: in line
+// (2 x 56 x 56: 8.9 us either way); issued by one lane through a map with 256-byte L2 promotion 0.6 us later, as 32 bulk copies of 256 bytes
+// to a slice 10 us later.  Not inlined: in line
 // it costs the producers 2 to 10 % (128 x 64 x 56 x 56: 72.3 -> 74 us), whose registers are at the limit.
 __device__ __noinline__ void load_pairs(unsigned char* dst, const float* bank, const CUtensorMap* map, int rows, int S, uint64_t* full,
                                         volatile uint32_t* abort_flag, int lane)
@@ -608,9 +609,8 @@ general_tc_kernel(const KernelArgs a, const __grid_constant__ CUtensorMap pair_m
             }
         }
     } else if (warp == 1) {
-        // ---------------- MMA issue.  All 32 lanes run the loop and one elected lane issues: a tcgen05.mma takes its
-        // operands from uniform registers, which the compiler fills for nothing where the warp stays together, and with
-        // moves of their own for every instruction where one lane has gone its own way.  In a loop of this shape with a
+        // ---------------- MMA issue.  All 32 lanes run the loop and one elected lane issues, which is faster than a loop that one
+        // lane runs alone (presumably because warp-uniform operands need no moves).  In a loop of this shape with a
         // stage boundary every 6 to 10 MMAs, cycles per MMA of a lone lane / of the warp: N = 256 155 / 132, N = 224 (two
         // groups) 122 / 114, N = 176 139 / 99, N = 96 161 / 93 (the pipe's own: 128, 112, 88, 64).
         {

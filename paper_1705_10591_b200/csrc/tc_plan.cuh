@@ -15,11 +15,11 @@ constexpr int kProducers = kProducerWarps * 32;
 static_assert(kProducers == 256, "the producer group arithmetic assumes 256 producer threads");
 constexpr int kEpilogueWarps = 4;
 // Warp roles by warp index.  An SM has four warp schedulers and warp w is served by scheduler w % 4.  The
-// single thread that issues the MMAs (warp 1) must never wait for an issue slot behind arithmetic-heavy
+// warp that issues the MMAs (warp 1) must never wait for an issue slot behind arithmetic-heavy
 // warps -- measured: sharing its scheduler with two producer warps stretched each MMA issue from ~64 to
 // 120-180 cycles -- so scheduler 1 hosts only that warp, one epilogue warp and two warps that only wait.
 //   warp 0           filter copies (one thread)
-//   warp 1           MMA issue (one thread), owner of the tensor-memory allocation
+//   warp 1           MMA issue (all lanes run the loop, an elected one issues), owner of the tensor-memory allocation
 //   warps 4-7        epilogue, tensor-memory lane quarter = warp % 4
 //   warps 2,3,8,10,11,12,14,15   activation producers (schedulers 0, 2, 3)
 //   warps 9, 13      no work until the block's last item
@@ -50,7 +50,7 @@ constexpr size_t xchg_area_bytes(int slots) { return (size_t)kEpilogueWarps * sl
 struct Plan {
     int n_tile;       // filters per work item: 64 or 128 rows of the M operand
     int n_blocks;     // work-item columns over the filters
-    int tile_px;      // pixels per work item: any multiple of 32 up to 512
+    int tile_px;      // pixels per work item: any multiple of 32 up to 512 (of 16 where items end with their image)
     int px_groups;    // MMAs per K step (each covers n_mma = tile_px / px_groups pixels)
     int nbuf;         // accumulator sets in tensor memory (2: write-back overlaps the next item)
     int npix;         // staged pixel rows per channel chunk
@@ -161,8 +161,8 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     const long long total_pix = (long long)sh.N * sh.H * sh.W;
     if (total_pix >= (1LL << 31) - (1LL << 20)) return p;     // flat pixel indices stay within int32
     const int kp16 = (sh.K + 15) / 16 * 16;
-    // Operand roles.  One tcgen05.mma costs its issuing thread ~60 cycles whatever its size (measured), so
-    // an instruction must carry >= 128 cycles of tensor-pipe work to keep the pipe busy: N = 256.  For any
+    // Operand roles.  One tcgen05.mma takes the pipe 64 cycles for any N up to 128 and N / 2 beyond, and the warp that issues it ~90
+    // at least, so an instruction should have N = 192 to 256.  For any
     // filter count that is possible with the pixels as the N operand: M = a block of 128 filters (zero
     // padded), N = 256 pixels, accumulator lanes = filters.  It also halves the filter bytes an item streams
     // per pixel compared with 128 pixels x 256 filters.
@@ -217,11 +217,10 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     // S taps takes ceil(S / 2) instructions instead of S (an odd last tap has zeros in the upper half).  In the
     // flat pixel run the last column of an item has no right neighbour, so consecutive items overlap by 4 pixels.
     // It pays when the MMAs dominate an item: the stacked operand doubles the filter bytes per instruction (a bank
-    // that was resident in shared memory may have to be streamed) and every block of the write-back reads two tile
-    // rows per map.  Measured with 64 filters: 128 channels 5 x 5 on 32 x 32: 63.9 -> 46.8 us, 7 x 7: 110.5 ->
-    // 74.4 us, 3 x 3: 31.7 -> 28.6 us; 64 channels 5 x 5 on 64 x 64 in bf16 (50 pairs of tap and channel block):
-    // 24.3 -> 20.8 us; 64 channels 3 x 3 on 56 x 56 (36 pairs): 27.6 -> 30.6 us.  Hence from 48 (tap, channel block)
-    // pairs on.  CONV2D_B200_TF32_PAIR_TAPS = 0 / 2: never / whenever possible.
+    // that was resident in shared memory may have to be streamed).  Hence from 48 (tap, channel block) pairs on.  Stacked against
+    // not, means of 420 random layers: fp32 with quads 0.91 at 48 to 59 pairs, 0.76 at 60 to 71, 0.85 from 96 on, single
+    // pixels 0.86 to 1.06; below 48 fp32 0.97 to 0.99 (0.83 to 1.68) and 0.98 to 1.06.  (16-bit operands gain below 48, too: 0.90 to 0.93 from 24 on.)
+    // CONV2D_B200_TF32_PAIR_TAPS = 0 / 2: never / whenever possible.
     const int pair_mode = env_int("CONV2D_B200_TF32_PAIR_TAPS", 1);
     p.pair_taps = (st == 1 && kp16 <= 64 && p.fold_r * p.fold_s == 1 && s_eff >= 2 && pair_mode != 0 &&
                    (pair_mode == 2 || (long long)r_eff * s_eff * p.cblks >= 48)) ? 1 : 0;
@@ -232,7 +231,8 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     // 32 x 64 x 56 x 56, 64 of 3 x 3, padding 1: 29.8 -> 27.7 us (wholly stacked and streamed 28.7).  16-bit operands have half
     // as many MMAs and are bound by what shared memory moves: off (64 x 128 x 32 x 32, 64 of 3 x 3 in bf16: 22.8 us, 24.8 stacked).
     // The MMAs have to be what sets the pace: 36 pairs of tap and channel block (with fewer the write-back: 64 x 16 x 90 x 122, 19 of
-    // 3 x 3 57.6 -> 67.7 us; 5 x 48 x 74 x 74, 48 of 3 x 3 12.5 -> 13.9) whose pixels are loaded as quads (else the producers: 7 x 64 x 95 x 95, 48 of 3 x 3, padding 1 26.5 -> 30.8).
+    // 3 x 3 57.6 -> 67.7 us; 5 x 48 x 74 x 74, 48 of 3 x 3 12.5 -> 13.9), of which at most 38 fit (4 KB each): 3 x 3 on 49 to 64
+    // channels, 6 x 6 on up to 16, 4 x 3 on 33 to 48 and the like, whose pixels are loaded as quads (else the producers: 7 x 64 x 95 x 95, 48 of 3 x 3, padding 1 26.5 -> 30.8).
     // CONV2D_B200_TF32_PAIR_COMPACT = 0 / 1: never / whenever possible.
     const int compact_mode = env_int("CONV2D_B200_TF32_PAIR_COMPACT", b16 ? 0 : 2);
     p.pair_compact = 0;
@@ -339,7 +339,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     if (!p.resident) {
         // Streamed filters.  Measured: all SMs together draw filter stages from L2 at no more than
         // ~5-6 TB/s, i.e. a 8 KB stage costs ~120 cycles on top of the MMAs that consume it unless it is
-        // reused by several tiles.  More tiles per item (mt) amortise that; fewer tiles leave room for a
+        // reused by more pixels.  Larger items amortise that; smaller ones leave room for a
         // second accumulator set (hidden write-back) and balance better.  Cost in units of one tile's MMA
         // time: rounds x mt x (1 + stage cost / MMA time) + exposed write-back.
         const size_t kLimit = kSmemLimit - extra;
@@ -420,7 +420,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         p.tile_px = best_px;
         p.supertiles = best_items > 0x7fffffffLL ? -1 : (int)best_items;
         // Filter stages: several taps per stage (up to 48 KB, trimmed below until three stages fit) so that the
-        // single MMA-issuing thread pays its per-stage bookkeeping (barrier wait, commit: ~90 cycles, measured
+        // warp that issues the MMAs pays its per-stage bookkeeping (barrier wait, commit: ~200 cycles, measured
         // by varying the stage size) once per 16-48 MMAs; the ring should hold
         // 64-128 KB in flight to cover the L2 latency.
         p.a_stages = 2;
@@ -490,7 +490,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
     return p;
 }
 
-// Rough cycles of the busiest block: its MMAs with 400 for every filter stage that its one issuing thread hands over, its
+// Rough cycles of the busiest block: its MMAs with 400 for every filter stage (fitted when one lane alone ran the MMA loop), its
 // producers (6 cycles per staged pixel and channel block, 5 where they load quads, a round trip to memory per block at
 // least) and its write-back, which overlap for the most part; and the zero-fill and adds of a contraction split without a
 // cluster (4.5 us).  Fitted to the times of 2070 random padded layers on virtual images and in patches (standard deviation

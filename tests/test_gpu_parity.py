@@ -411,7 +411,7 @@ def test_compact_stacked_taps(oracle, monkeypatch, dims, entry):
     import paper_1705_10591_b200 as lib
     N, C, H, W, K, R, S = dims
     algo_q = ALGO_TF32 if entry == "general" else 3
-    monkeypatch.setenv("CONV2D_B200_TF32_PAIR_COMPACT", "1")       # (measured slower on the benchmark shape: off by default)
+    monkeypatch.setenv("CONV2D_B200_TF32_PAIR_COMPACT", "1")       # (wherever possible; by default a rule chooses)
     assert lib.conv2d_fwd_plan_describe(*dims, algo_q).get("stacked_compact") == 1, "meant to take compact stacking"
     xi, wi = small_integers((N, C, H, W), 481), small_integers((K, C, R, S), 482)
     yi_ref, _ = oracle.conv2d_oracle(xi, wi)
