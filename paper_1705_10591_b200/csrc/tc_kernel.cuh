@@ -12,8 +12,8 @@ namespace {
 
 using namespace ptx;
 
-// Tuning builds (-DCONV2D_B200_TC_DIAGNOSTICS) make the MMA-issuing thread of block 0 count its cycles and leave
-// them in status words 2-9.  The product build contains none of it: that thread's instruction stream is what
+// Tuning builds (-DCONV2D_B200_TC_DIAGNOSTICS) make the warp of block 0 that issues the MMAs count its cycles and leave
+// them in status words 2-9 and 16.  The product build contains none of it: that warp's instruction stream is what
 // bounds the heavy shapes, and a timer read with a memory clobber around every wait is not free.
 #ifdef CONV2D_B200_TC_DIAGNOSTICS
 constexpr bool kDiag = true;

@@ -340,8 +340,8 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         // Streamed filters.  Measured: all SMs together draw filter stages from L2 at no more than
         // ~5-6 TB/s, i.e. a 8 KB stage costs ~120 cycles on top of the MMAs that consume it unless it is
         // reused by more pixels.  Larger items amortise that; smaller ones leave room for a
-        // second accumulator set (hidden write-back) and balance better.  Cost in units of one tile's MMA
-        // time: rounds x mt x (1 + stage cost / MMA time) + exposed write-back.
+        // second accumulator set (hidden write-back) and balance better.  Cost in cycles: rounds x one item's
+        // MMA and stage time + exposed write-back.
         const size_t kLimit = kSmemLimit - extra;
         const double stage_cycles = chunk / 66.0;           // one (tap, channel block) of filters through L2
         const int forced_px = env_int("CONV2D_B200_TF32_TILE_PX", 0);
