@@ -71,9 +71,11 @@ enum {
        K, C, R, S and algorithm) in the kernel's internal order, left there by an
        earlier call: skip the re-ordering launch.  The number and size of the images
        may be others than in that call, except with 1 x 1 filters (one order for H*W
-       a multiple of 4, another for the rest) and with strided layers whose windows do
-       not overlap (R, S <= stride: the order depends on the images).  Padding and
-       stride belong to the layer: the same in both calls. */
+       a multiple of 4, another for the rest) and with strided layers that a call may
+       rewrite (the order depends on the images): FFMA, windows that do not overlap
+       (R, S <= stride), and images so wide that the rows a window spans do not fit on
+       chip ((ceil(R / stride) - 1) * (W + 2 * pad_w) / stride of about 600 and more).
+       Padding and stride belong to the layer: the same in both calls. */
     CONV2D_FLAG_WEIGHTS_PACKED = 1u
 };
 
@@ -206,7 +208,7 @@ conv2d_status_t conv2d_fwd_general_padded(const float* x, const float* w, float*
  *   y[n,k,p,q] = sum_{c,r,s} xz[n,c,stride*p+r-pad_h,stride*q+s-pad_w] * w[k,c,r,s],
  *   P = (H + 2*pad_h - R) / stride + 1, Q = (W + 2*pad_w - S) / stride + 1 (integer division), y [N][K][P][Q].
  * With the tensor-core algorithms the kernel stages the phases of the stride straight from x and multiplies each
- * with its own taps.  Otherwise (fp32, no such instance, or windows that do not overlap where an estimate finds the
+ * with its own taps.  Otherwise (fp32, no such instance: images too wide for it, or windows that do not overlap where an estimate finds the
  * 1 x 1 kernel faster on the rewritten image) the call rewrites the problem as a stride-1 convolution
  * over stride*stride times as many channels ("space to depth": channel (c,a,b) of the rewritten image holds the pixels
  * whose row is a and whose column is b modulo the stride; the filters are split the same way) with two extra kernels
