@@ -58,7 +58,7 @@ struct Plan {
     int fold_r, fold_s;  // taps folded into the channel dimension: 1 or R rows, 1 or S columns
     int patch_w, patch_tw, patch_rows, patch_cols;   // patch addressing (patch_w = 0: flat pixel run), see ItemGeom
     int crop, crop_items;   // flat addressing: 1 = items end with their image, crop_items of them each
-    int may_crop;           // 1: such items were or can be considered
+    int wants_crop;         // 1: the rule would choose such items, but this plan was made without them
     int taps;
     int a_stages;
     int b_stages;
@@ -355,8 +355,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
         // bound by its ~64-cycle issue cost.
         long long best_items = 0;
         // (CONV2D_B200_TF32_CROP = 0: never, 2: wherever they fit)
-        p.may_crop = !(p.patch_w || p.fold_r * p.fold_s != 1 || sh.C < kCB || forced_px);
-        const int crop_mode = !p.may_crop || !allow_crop ? 0 : env_int("CONV2D_B200_TF32_CROP", 1);
+        const int crop_mode = p.patch_w || p.fold_r * p.fold_s != 1 || sh.C < kCB || forced_px ? 0 : env_int("CONV2D_B200_TF32_CROP", 1);
         auto consider = [&](int px, int groups, long long px_items, long long npix, int crop, int crop_items) {
             if (npix > 16000 || smem_need(2, (int)npix, p.n_tile, 2, 1, stage_blocks) > kLimit || px_items <= 0) return;
             const long long items = px_items * p.n_blocks;
@@ -384,6 +383,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
             if (crop && adds && !flat_adds) cost += 9000.0;
             if (best_px != 0 && !(crop_mode >= 2 && crop != p.crop) &&
                 (!(cost < (crop != p.crop ? 0.96 : 1.0) * best_cost) || (crop && crop_mode < 2 && staging > flat_bound))) return;
+            if (crop && !allow_crop) { p.wants_crop = 1; return; }
             if (!crop) { flat_adds = adds; flat_bound = bound; }
             best_px = px;
             best_cost = cost;
@@ -407,7 +407,7 @@ Plan plan_with_patch_width(const Shape& shape, bool b16, int want_patch_w, bool 
             // a pattern; with few channels the producers set the pace, and more items stage more pixels (4 x 4 x 131 x 67, stride 2:
             // 14.9 -> 16.4 us).
             const long long plane = (long long)sh.H * sh.W, used = (long long)(sh.P - 1) * sh.W + sh.Q;
-            for (int m = 1; m <= 64; ++m) {
+            for (int m = 1; m <= 64 && !p.wants_crop; ++m) {
                 const long long cols = (used + m - 1) / m + p.ovl;
                 const int groups = cols > 256 ? 2 : 1;
                 const int n = (int)(((cols + groups - 1) / groups + 15) / 16 * 16);
@@ -531,9 +531,10 @@ bool patches_beat_virtual(const Plan& v, const Plan& patch, const Shape& sh)
 Plan make_plan(const Shape& sh, bool b16 = false)
 {
     // (the choice between virtual images, their widths and patches is made between plans without cropped items: with them the
-    // estimates took virtual images for layers that patches do faster, 128 x 70 x 13 x 151, 32 of 4 x 4, padding 2: 93 -> 126 us)
+    // estimates took virtual images for layers that patches do faster, 128 x 70 x 13 x 151, 32 of 4 x 4, padding 2: 93 -> 126 us);
+    // planned once more only where the rule chooses them)
     auto cropped = [&](const Plan& p, bool narrow) {
-        return p.ok && p.may_crop ? plan_with_patch_width(sh, b16, 0, true, true, narrow) : p;
+        return p.ok && p.wants_crop ? plan_with_patch_width(sh, b16, 0, true, true, narrow) : p;
     };
     if (sh.stride > 1) {
         // Rows of a multiple of four columns allow 128-bit stores; where two columns less let the busiest block do a tenth
